@@ -241,8 +241,20 @@ void build_basis(Ctx& c, const dft_basis_desc* b, const dft_grid_desc* g, const 
         c.n_tc_tiles = (int)((tc_tiles(c.K, 256).size() + tc_tiles(c.K, 128).size()) / 2);
         c.tile_cap = std::max(c.n_tc_tiles, 1 << 17);
     }
-    c.part_cap = std::max<long long>({2LL * cheb_step_parts(c.K), 2LL * c.tile_cap, 3LL * 1184, 2048, 592LL * 16}) + 64;
+    c.part_cap = std::max<long long>({2LL * c.tile_cap, 3LL * 1184, 2048, 592LL * 16}) + 64;
     c.pl_hist = c.p.mixer == DFT_MIX_PULAY ? (c.p.mix_history > 0 ? c.p.mix_history : 8) : 0;
+    c.gram_cap = 1 << 20;
+}
+
+// Expansion buffers beyond the scratch matrices X0, X1 and B that the FP64
+// path keeps: 2 sqrt(2 N_C) products need up to that many (k_poly.cu), fewer
+// only cost products.  At most 1 GiB, or as much again as the rest of the
+// workspace while the total stays below 96 GiB.
+int ps_extra_slots(const Ctx& c, size_t base) {
+    if (c.p.precision != DFT_PREC_FP64) return 0;
+    const size_t gib = size_t(1) << 30, K2 = ((size_t)c.K * c.K * sizeof(double) + 255) & ~size_t(255);
+    const size_t room = base < 96 * gib ? std::min(base, 96 * gib - base) : 0;
+    return (int)std::min<size_t>(128, std::max(gib, room) / K2);
 }
 
 // carve the workspace; with base == nullptr only the size is computed
@@ -314,7 +326,12 @@ size_t carve(Ctx& c, char* base) {
         o_cnt = L.off(sizeof(int) * 3 * (size_t)c.tile_cap);
         o_macc = L.off(sizeof(long long) * (size_t)c.cheb_cap);
     }
+    const size_t o_gram = L.off(sizeof(double) * (size_t)c.gram_cap);
+    c.ps_extra = ps_extra_slots(c, L.total);
+    std::vector<size_t> o_ps(c.ps_extra);
+    for (auto& o : o_ps) o = L.off(K2);
     if (base) {
+        c.d_gram = (double*)(base + o_gram);
         c.d_fn = (Fn*)(base + o_fn);
         c.d_tab = (double*)(base + o_tab);
         if (c.contracted) {
@@ -358,6 +375,10 @@ size_t carve(Ctx& c, char* base) {
             c.d_nlB = (double*)(base + o_nlb);
             c.d_nlEB = (double*)(base + o_nleb);
             c.d_VNL = (double*)(base + o_vnl);
+        }
+        if (c.p.precision == DFT_PREC_FP64) {
+            c.ps_slot = {c.d_X0, c.d_X1, c.d_B};
+            for (size_t o : o_ps) c.ps_slot.push_back((double*)(base + o));
         }
         if (c.Kp > 0) {
             for (int q = 0; q < 2; ++q) c.d_h16[q] = base + o_h16[q];
@@ -529,7 +550,7 @@ int auto_order(Ctx& c, double emin, double emax, cudaStream_t s) {
 // number of moments-pass steps j = 1..J with 2j + 1 <= N_C - 1
 inline int pass1_steps(int n_c) { return n_c >= 2 ? (n_c - 2) / 2 : 0; }
 
-// F~ = L^-1 F L^-T, spectral bounds, N_C, H_N, and m_0, m_1, m_2
+// F~ = L^-1 F L^-T, spectral bounds, N_C, H_N (mixed path: also m_0, m_1, m_2)
 void dm_prepare(Ctx& c, const double* F, cudaStream_t s, Timer* tm, int t0) {
     if (!c.have_chol) throw Error(DFT_EINVAL, "call dft_overlap_kinetic first");
     const int K = c.K;
@@ -559,20 +580,15 @@ void dm_prepare(Ctx& c, const double* F, cudaStream_t s, Timer* tm, int t0) {
     c.n_c_cur = n_c;
     launch_cos_table(4 * n_c, c.d_cos, s);
     if (tm) tm->mark(t0 + 2);
+    if (c.p.precision == DFT_PREC_FP64) return;
+    // split H_N into its 16-bit pair; trace and |H|^2 of the pair
     double m0 = (double)K;
     DFT_CUDA_CHECK(cudaMemcpyAsync(c.d_mom, &m0, sizeof(double), cudaMemcpyHostToDevice, s));
-    if (c.p.precision != DFT_PREC_FP64) {
-        // split H_N into its 16-bit pair; trace and |H|^2 of the pair
-        tc_split_h(c, s);
-        tc_init(c, nullptr, s);
-        DFT_CUDA_CHECK(cudaMemcpyAsync(c.d_mom + 1, c.d_scal + SCAL_TRACE, sizeof(double), cudaMemcpyDeviceToDevice, s));
-        DFT_CUDA_CHECK(cudaMemcpyAsync(c.d_scal + SCAL_TRACE, c.d_scal + SCAL_TRACE + 1, sizeof(double),
-                                       cudaMemcpyDeviceToDevice, s));
-    } else {
-        launch_cheb_init(K, c.d_H, c.d_X0, c.d_X1, nullptr, nullptr, s);
-        launch_trace(K, c.d_H, c.d_mom + 1, s);
-        launch_frob_dot((long long)K * K, c.d_H, c.d_H, c.d_part, c.d_scal + SCAL_TRACE, s);
-    }
+    tc_split_h(c, s);
+    tc_init(c, nullptr, s);
+    DFT_CUDA_CHECK(cudaMemcpyAsync(c.d_mom + 1, c.d_scal + SCAL_TRACE, sizeof(double), cudaMemcpyDeviceToDevice, s));
+    DFT_CUDA_CHECK(cudaMemcpyAsync(c.d_scal + SCAL_TRACE, c.d_scal + SCAL_TRACE + 1, sizeof(double),
+                                   cudaMemcpyDeviceToDevice, s));
     DFT_CUDA_CHECK(cudaMemsetAsync(c.d_scal + SCAL_TRACE + 1, 0, sizeof(double), s));
     if (n_c > 2) launch_moment_reduce(1, c.d_scal + SCAL_TRACE, c.d_mom, 2, -1, m0, c.d_mom + 1, s);
 }
@@ -625,7 +641,7 @@ int tc_pass2_tuned(TcBatch& b, int total_k, int Lmax, cudaStream_t s) {
     return l;
 }
 
-// moments pass of one system: m_l = Tr T_l(H_N), l < N_C, by doubling
+// moments of one system: m_l = Tr T_l(H_N), l < N_C (mixed path by doubling)
 void dm_pass1(Ctx& c, cudaStream_t s) {
     const int K = c.K, n_c = c.n_c_cur, J = pass1_steps(n_c);
     if (c.p.precision != DFT_PREC_FP64) {
@@ -645,16 +661,7 @@ void dm_pass1(Ctx& c, cudaStream_t s) {
         }
         return;
     }
-    const double m0 = (double)K;
-    int nparts = cheb_step_parts(K);
-    double* cur = c.d_X1;
-    double* prev = c.d_X0;
-    for (int j = 1; j <= J; ++j) {
-        launch_cheb_step_fp64(K, c.d_H, cur, prev, nullptr, nullptr, 0, c.d_part, c.d_flags, s);
-        std::swap(cur, prev);
-        launch_moment_reduce(nparts, c.d_part, c.d_mom, (2 * j + 2 < n_c) ? 2 * j + 2 : -1, 2 * j + 1, m0,
-                             c.d_mom + 1, s);
-    }
+    ps64_pass1(c, true, s);
 }
 
 // mu from 2 sum_l a_l(mu) m_l = N_e (Eq. 2.8), then the coefficients
@@ -688,13 +695,7 @@ void dm_pass2(Ctx& c, cudaStream_t s) {
         tc_rho_finish(c, s);
         return;
     }
-    launch_cheb_init(K, c.d_H, c.d_X0, c.d_X1, c.d_rho, c.d_coef, s);
-    double* cur = c.d_X1;
-    double* prev = c.d_X0;
-    for (int l = 2; l < n_c; ++l) {
-        launch_cheb_step_fp64(K, c.d_H, cur, prev, c.d_rho, c.d_coef, l, nullptr, c.d_flags, s);
-        std::swap(cur, prev);
-    }
+    ps64_pass2(c, s);
 }
 
 // P = L^-T rho L^-1, electron count, status flags

@@ -74,6 +74,15 @@ struct TcCfg {
     int epf = 0;        // 1: prefetch the epilogue's rows into L2 before the last chunks
     int flow = 0;       // 1: one cooperative launch per pass, tiles wait on block counters (256-wide tiles)
 };
+
+// how a Chebyshev expansion of n_c terms is evaluated (k_poly.cu): babies
+// T_1 .. T_s, giants T_{qs}, q <= Q; direct: the giants are kept, else
+// Clenshaw's recurrence in T_s
+struct PsPlan {
+    int n_c = 0, s = 1, Q = 0;
+    bool direct = false;
+};
+
 struct Ctx {
     // problem
     int K = 0, n_atoms = 0;
@@ -118,9 +127,16 @@ struct Ctx {
     double* d_Linv = nullptr;
     double* d_A = nullptr;       // K x K scratch (Fock / transformed Fock)
     double* d_H = nullptr;       // normalised Hamiltonian H_N
-    double* d_X0 = nullptr;
+    double* d_X0 = nullptr;      // scratch: expansion buffers, column route
     double* d_X1 = nullptr;
     double* d_rho = nullptr;
+    // expansion buffers of the FP64 path (K x K each) and the plan of the
+    // density matrix in progress
+    std::vector<double*> ps_slot;
+    int ps_extra = 0;            // of them, those carved for this purpose alone
+    PsPlan ps;
+    double* d_gram = nullptr;    // partial Gram sums [gram_cap]
+    long long gram_cap = 0;
     double* d_B = nullptr;       // K x K scratch
     double* d_P = nullptr;       // K x K density matrix of the last SCF step
     double* d_F = nullptr;       // K x K Fock matrix of the SCF step
@@ -295,15 +311,19 @@ void launch_moment_weights(int n_c, int M, const double* cos_tab, const double* 
                            cudaStream_t s);
 void launch_mu_bisect(int M, const double* cos_tab, const double* wk, double beta, double n_e,
                       double* scal, int* flags, cudaStream_t s);
-void launch_cheb_init(int K, const double* H, double* X0, double* X1, double* rho,
-                      const double* coef, cudaStream_t s);
-// X_next (written over Xprev) = 2 H Xcur - Xprev; rho += coef[l] X_next (if rho);
-// moment partials (if part): <Xn, Xn>, <Xn, Xcur>
-void launch_cheb_step_fp64(int K, const double* H, const double* Xcur, double* Xprev, double* rho,
-                           const double* coef, int l, double* part, int* flags, cudaStream_t s);
-int cheb_step_parts(int K);
 void launch_moment_reduce(int nparts, const double* part, double* mom, int idx_even, int idx_odd,
                           double m0, const double* m1, cudaStream_t s);
+
+// ---- grouped evaluation of the expansion (k_poly.cu) ----
+PsPlan ps_plan(int n_c, int nslot, bool prefer_direct);
+// m_l, l < n_c, from the traces and Gram sums D ((Q + 1) x s)
+void launch_ps_moments(int K, const PsPlan& p, const double* D, double* mom, cudaStream_t s);
+// c_qr of the C_q from a_l; work holds (Q + 1) s doubles
+void launch_ps_coefs(const PsPlan& p, const double* a, double* c, double* work, cudaStream_t s);
+// FP64 path: babies and giants of H_N and the moments into d_mom; then
+// rho = sum_l a_l T_l into d_rho from the coefficients in d_coef
+void ps64_pass1(Ctx& c, bool moments, cudaStream_t s);
+void ps64_pass2(Ctx& c, cudaStream_t s);
 
 // ---- tensor-core Chebyshev path (k_cheb_tc.cu) ----
 int tc_pad(int K);

@@ -1,8 +1,6 @@
 // Chebyshev engine (Supp. B): expansion coefficients of the Fermi-Dirac
 // function, Chebyshev moments, the chemical potential by bisection on the
-// electron count (Eq. 2.8), and the FP64 three-term recurrence
-// X_{l+1} = 2 H_N X_l - X_{l-1} with the coefficient-weighted sum fused into
-// the product's epilogue.
+// electron count (Eq. 2.8).
 #include "dft_internal.cuh"
 
 #include <algorithm>
@@ -122,97 +120,6 @@ __global__ void __launch_bounds__(1024) k_mu_bisect(int M, const double* __restr
     if (threadIdx.x == 0) scal[SCAL_MU] = 0.5 * (lo + hi);
 }
 
-// X0 = I, X1 = H, rho = a0 I + a1 H (rho may be null: moments pass)
-__global__ void k_cheb_init(int K, const double* __restrict__ H, double* X0, double* X1, double* rho,
-                            const double* __restrict__ a) {
-    long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (long long)K * K) return;
-    double id = (e / K == e % K) ? 1.0 : 0.0;
-    double h = H[e];
-    X0[e] = id;
-    X1[e] = h;
-    if (rho) rho[e] = a[0] * id + a[1] * h;
-}
-
-constexpr int CK = 16;
-
-// One Chebyshev step on a CB x CB tile: C = H Xcur; Xn = 2C - Xprev (stored over
-// Xprev); rho += a_l Xn; optional moment partials <Xn,Xn>, <Xn,Xcur>.  The
-// FP64 pipe is the limit, so small K uses 32 x 32 tiles to give every SM work.
-template <int CB>
-__global__ void __launch_bounds__(256) k_cheb_step_fp64(int K, const double* __restrict__ H,
-                                                        const double* __restrict__ Xc, double* __restrict__ Xp,
-                                                        double* __restrict__ rho, const double* __restrict__ a,
-                                                        int l, double* __restrict__ part, int* flags) {
-    constexpr int TM = CB / 16;
-    __shared__ double As[CK][CB + 1];
-    __shared__ double Bs[CK][CB + 1];
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    const int m0 = blockIdx.y * CB, n0 = blockIdx.x * CB;
-    double acc[TM][TM] = {};
-    for (int k0 = 0; k0 < K; k0 += CK) {
-        for (int e = threadIdx.x; e < CB * CK; e += 256) {
-            int kk = e % CK, mm = e / CK;
-            int gm = m0 + mm, gk = k0 + kk;
-            As[kk][mm] = (gm < K && gk < K) ? H[(long long)gm * K + gk] : 0.0;
-            int nn = e % CB, kb = e / CB;
-            int gn = n0 + nn, gk2 = k0 + kb;
-            Bs[kb][nn] = (gn < K && gk2 < K) ? Xc[(long long)gk2 * K + gn] : 0.0;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < CK; ++kk) {
-            double av[TM], bv[TM];
-#pragma unroll
-            for (int i = 0; i < TM; ++i) av[i] = As[kk][ty + 16 * i];
-#pragma unroll
-            for (int j = 0; j < TM; ++j) bv[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-            for (int i = 0; i < TM; ++i)
-#pragma unroll
-                for (int j = 0; j < TM; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-    const double al = rho ? a[l] : 0.0;
-    double s_nn = 0.0, s_nc = 0.0;
-    bool bad = false;
-#pragma unroll
-    for (int i = 0; i < TM; ++i) {
-        int gm = m0 + ty + 16 * i;
-        if (gm >= K) continue;
-#pragma unroll
-        for (int j = 0; j < TM; ++j) {
-            int gn = n0 + tx + 16 * j;
-            if (gn >= K) continue;
-            long long e = (long long)gm * K + gn;
-            double xn = 2.0 * acc[i][j] - Xp[e];
-            Xp[e] = xn;
-            bad |= !(fabs(xn) <= 4.0);
-            if (rho) rho[e] = fma(al, xn, rho[e]);
-            if (part) {
-                s_nn = fma(xn, xn, s_nn);
-                s_nc = fma(xn, Xc[e], s_nc);
-            }
-        }
-    }
-    if (bad) atomicExch(&flags[FLAG_SPECTRUM], 1);
-    if (part) {
-        s_nn = block_sum<256>(s_nn);
-        s_nc = block_sum<256>(s_nc);
-        if (threadIdx.x == 0) {
-            int b = blockIdx.y * gridDim.x + blockIdx.x;
-            part[2 * b] = s_nn;
-            part[2 * b + 1] = s_nc;
-        }
-    }
-}
-
-inline int fp64_tile(int K) {
-    int nb = (K + 63) / 64;
-    return nb * nb < 2 * 152 ? 32 : 64;
-}
-
 // m_{even} = 2 <Xn,Xn> - m0, m_{odd} = 2 <Xn,Xc> - m1 (T_{2l} = 2T_l^2 - 1,
 // T_{2l+1} = 2 T_{l+1} T_l - T_1), partials summed in a fixed order
 __global__ void __launch_bounds__(256) k_moment_reduce(int np, const double* __restrict__ part, double* mom,
@@ -258,28 +165,6 @@ void launch_mu_bisect(int M, const double* cos_tab, const double* wk, double bet
                       int* flags, cudaStream_t s) {
     k_mu_bisect<<<1, 1024, 0, s>>>(M, cos_tab, wk, beta, n_e, scal, flags);
     check_launch("mu_bisect");
-}
-
-void launch_cheb_init(int K, const double* H, double* X0, double* X1, double* rho, const double* coef,
-                      cudaStream_t s) {
-    k_cheb_init<<<blocks_for((long long)K * K, 256), 256, 0, s>>>(K, H, X0, X1, rho, coef);
-    check_launch("cheb_init");
-}
-
-int cheb_step_parts(int K) {
-    int cb = fp64_tile(K);
-    int nb = (K + cb - 1) / cb;
-    return nb * nb;
-}
-
-void launch_cheb_step_fp64(int K, const double* H, const double* Xcur, double* Xprev, double* rho,
-                           const double* coef, int l, double* part, int* flags, cudaStream_t s) {
-    int cb = fp64_tile(K);
-    int nb = (K + cb - 1) / cb;
-    dim3 grid(nb, nb);
-    if (cb == 32) k_cheb_step_fp64<32><<<grid, 256, 0, s>>>(K, H, Xcur, Xprev, rho, coef, l, part, flags);
-    else k_cheb_step_fp64<64><<<grid, 256, 0, s>>>(K, H, Xcur, Xprev, rho, coef, l, part, flags);
-    check_launch("cheb_step_fp64");
 }
 
 void launch_moment_reduce(int nparts, const double* part, double* mom, int idx_even, int idx_odd, double m0,
