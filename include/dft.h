@@ -28,12 +28,10 @@
  *  - Device pointers must be 16-byte aligned (DFT_EINVAL otherwise).
  *
  * Environment (mixed-precision paths)
- *  - DFT_AUTOTUNE_CACHE: JSON file that keeps the tensor-core launch shape
- *    tuned per (precision, size bucket, batch size); read at the first
- *    tuned launch, rewritten after each tuning.
- *  - DFT_AUTOTUNE_OFF: any value disables tuning (the default shape runs).
- *  - DFT_TC_SHAPE="bk,persist,bn[,streamk[,pf[,epf[,flow]]]]": forces one
- *    launch shape and disables tuning: k-block 32 or 64; 0 = one CTA per
+ *  - DFT_TC_SHAPE="bk,persist,bn[,streamk[,pf[,epf[,flow]]]]": runs the
+ *    Chebyshev sum as the plain three-term recurrence with this launch
+ *    shape of its tensor-core step (unset: the grouped evaluation of
+ *    dft_density_matrix): k-block 32 or 64; 0 = one CTA per
  *    tile, 1 or 2 = that many persistent CTAs per SM; tile width 256, or 128
  *    with bk = 32; streamk 1 = equal chunk ranges per CTA on a cooperative
  *    grid (256-wide tiles); pf = L2 prefetch distance of operand k-blocks
@@ -212,7 +210,10 @@ dft_status dft_nonlocal_matrix(dft_ctx* ctx, double* VNL, void* stream);
  * by the Chebyshev recurrence of Supp. B in the symmetric form
  * F~ = L^-1 F L^-T, X_0 = I, X_{l+1} = 2 H_N X_l - X_{l-1}, H_N = (F~ - Ebar)/dE,
  * P = L^-T rho L^-1 with rho = sum_l a_l(mu) X_l, and mu fixed by
- * 2 Tr[P S] = N_e (Eq. 2.8) from the Chebyshev moments.  P (device, K x K)
+ * 2 Tr[P S] = N_e (Eq. 2.8) from the Chebyshev moments.  The sum and the
+ * moments are evaluated from products of X_r, r < s, and X_{qs} (about
+ * 2 sqrt(2 N_C) matrix products; Liang, Baer et al., J. Comput. Phys. 194,
+ * 575 (2004)) with s chosen by N_C and the workspace.  P (device, K x K)
  * is written; info (host, may be NULL) receives mu, the bounds and N_C.
  * Mixed precisions: the two congruences run as split-FP16 tensor-core
  * products (about 22 bits; FP64 results), and unless params.skip_correction
@@ -312,11 +313,10 @@ dft_status dft_scf_step(dft_ctx* ctx, double* n_in_out, double* v_ks_out, double
  * per-system stages (potential, Fock matrix, bounds and N_C before the
  * recurrence; back-transform, collocation, energy and mixing after it) run
  * concurrently on per-context streams driven by host threads and are joined
- * to `stream`.  The two Chebyshev passes of all systems are merged into
- * tensor-core launches over the tiles of every system still inside its own
- * N_C, so ragged K share the SMs: one cooperative launch per pass with the
- * dataflow launch shape; otherwise one launch per recurrence step, captured
- * once in a CUDA graph and replayed while the step counts stay the same.
+ * to `stream`.  The products of all systems' Chebyshev expansions are merged
+ * into tensor-core launches, level by level (with DFT_TC_SHAPE, the steps of
+ * their recurrences: one cooperative launch per pass or one launch per step
+ * replayed from a CUDA graph), so ragged K share the SMs.
  * ctxs[0] holds the batch tables (system table, tensor maps, tile lists)
  * and the graphs.  n_in_out[q]: device density of system q, updated as by
  * dft_scf_step; infos (host, may be NULL) receives n results (stage times

@@ -275,9 +275,11 @@ size_t carve(Ctx& c, char* base) {
     size_t o_tp = L.off(sizeof(int) * (c.n_tiles + 1));
     size_t o_tf = L.off(sizeof(int) * std::max<long long>(1, c.tile_nnz));
     size_t o_xyz = L.off(sizeof(double) * 3 * c.n_atoms);
-    size_t o_S = L.off(K2), o_T = L.off(K2), o_Li = L.off(K2), o_A = L.off(K2), o_H = L.off(K2);
-    size_t o_X0 = L.off(K2), o_X1 = L.off(K2), o_rho = L.off(K2), o_B = L.off(K2), o_P = L.off(K2);
-    size_t o_F = L.off(K2);
+    size_t o_S = L.off(K2), o_T = L.off(K2), o_Li = L.off(K2), o_A = L.off(K2), o_F = L.off(K2);
+    size_t o_rho = L.off(K2);
+    // from here to the end of P: free while the mixed path's expansion runs
+    size_t o_H = L.off(K2), o_X0 = L.off(K2), o_X1 = L.off(K2), o_B = L.off(K2), o_P = L.off(K2);
+    const std::pair<size_t, size_t> free_mat(o_H, L.total);
     size_t o_vec = L.off(sizeof(double) * 4 * c.K);
     size_t o_scal = L.off(sizeof(double) * SCAL_COUNT);
     size_t o_coef = L.off(sizeof(double) * (5 * (size_t)c.cheb_cap + 64));
@@ -288,9 +290,11 @@ size_t carve(Ctx& c, char* base) {
     size_t o_flags = L.off(sizeof(int) * FLAG_COUNT);
     size_t o_vloc = L.off(G), o_nion = L.off(G), o_vks = L.off(G), o_nout = L.off(G), o_gtmp = L.off(G);
     size_t o_fr = L.off(sizeof(double) * c.nfft_r);
-    size_t o_fo = L.off(sizeof(double) * c.nfft_r);
     size_t o_gh = L.off(sizeof(double) * c.nfft_c);
+    // the transform and its inverse are free between Poisson solves
+    size_t o_fo = L.off(sizeof(double) * c.nfft_r);
     size_t o_fc = L.off(sizeof(cufftDoubleComplex) * c.nfft_c);
+    const std::pair<size_t, size_t> free_fft(o_fo, L.total);
     size_t o_kw = L.off(sizeof(double) * nkc);
     size_t o_kc = L.off(sizeof(cufftDoubleComplex) * nkc);
     size_t o_pl = c.pl_hist > 0 ? L.off(sizeof(double) * 2 * (size_t)c.pl_hist * c.ng) : 0;
@@ -310,13 +314,16 @@ size_t carve(Ctx& c, char* base) {
     }
     size_t o_h16[2] = {0, 0}, o_x16[4] = {0, 0, 0, 0}, o_rtc = 0, o_tiles = 0, o_systab = 0, o_maps = 0;
     size_t o_cst = 0, o_skf = 0, o_skb = 0, o_cnt = 0, o_macc = 0, o_li16[2] = {0, 0}, o_lt16[2] = {0, 0};
+    std::pair<size_t, size_t> free_tc(0, 0);
     if (c.Kp > 0) {
         size_t P16 = (size_t)c.Kp * c.Kp * 2;
-        for (auto& o : o_h16) o = L.off(P16);
-        for (auto& o : o_x16) o = L.off(P16);
         for (auto& o : o_li16) o = L.off(P16);
         for (auto& o : o_lt16) o = L.off(P16);
+        free_tc.first = L.total;
+        for (auto& o : o_h16) o = L.off(P16);
+        for (auto& o : o_x16) o = L.off(P16);
         o_rtc = L.off((size_t)c.Kp * c.Kp * sizeof(double));
+        free_tc.second = L.total;
         o_systab = L.off(sizeof(TcSys) * TC_MAX_SYS);
         o_maps = L.off(sizeof(CUtensorMap) * TC_MAPS_PER_SYS * TC_MAX_SYS);
         o_tiles = L.off(sizeof(TcTile) * (size_t)c.tile_cap);
@@ -330,6 +337,26 @@ size_t carve(Ctx& c, char* base) {
     c.ps_extra = ps_extra_slots(c, L.total);
     std::vector<size_t> o_ps(c.ps_extra);
     for (auto& o : o_ps) o = L.off(K2);
+    // expansion slots of the mixed path: scratch that is free while the
+    // expansion runs (T_1 = slot 0 is split from d_H, so the pairs come first),
+    // then buffers of their own, at most an eighth of the workspace, or as much
+    // again while the total stays below 1.6 GB; 2 sqrt(2 N_C) products use up
+    // to about 110
+    std::vector<size_t> o_pst;
+    size_t o_pmaps = 0, o_pslots = 0, o_psys = 0, o_pitems = 0, o_ppairs = 0;
+    if (c.Kp > 0) {
+        const size_t sb = pst_slot_bytes(c.Kp), small = 1600000000;
+        for (const auto& r : {free_tc, free_mat, free_fft})
+            for (size_t o = r.first; o + sb <= r.second; o += sb) o_pst.push_back(o);
+        const size_t extra = std::max(L.total / 8, L.total < small ? std::min(L.total, small - L.total) : 0);
+        for (size_t used = sb; used <= extra && o_pst.size() < 112; used += sb) o_pst.push_back(L.off(sb));
+        if (o_pst.size() > 160) o_pst.resize(160);
+        o_pmaps = L.off(sizeof(CUtensorMap) * 4 * o_pst.size());
+        o_pslots = L.off(sizeof(void*) * o_pst.size());
+        o_psys = L.off(sizeof(PstSys) * TC_MAX_SYS);
+        o_pitems = L.off(sizeof(PstItem) * PST_ITEM_CAP);
+        o_ppairs = L.off(sizeof(int2) * PST_ITEM_CAP);
+    }
     if (base) {
         c.d_gram = (double*)(base + o_gram);
         c.d_fn = (Fn*)(base + o_fn);
@@ -381,6 +408,13 @@ size_t carve(Ctx& c, char* base) {
             for (size_t o : o_ps) c.ps_slot.push_back((double*)(base + o));
         }
         if (c.Kp > 0) {
+            c.pst_slot.clear();
+            for (size_t o : o_pst) c.pst_slot.push_back(base + o);
+            c.d_pst_maps = (CUtensorMap*)(base + o_pmaps);
+            c.d_pst_slots = (void**)(base + o_pslots);
+            c.d_pst_sys = (PstSys*)(base + o_psys);
+            c.d_pst_items = (PstItem*)(base + o_pitems);
+            c.d_pst_pairs = (int2*)(base + o_ppairs);
             for (int q = 0; q < 2; ++q) c.d_h16[q] = base + o_h16[q];
             for (int q = 0; q < 4; ++q) c.d_x16[q] = base + o_x16[q];
             for (int q = 0; q < 2; ++q) {
@@ -550,7 +584,7 @@ int auto_order(Ctx& c, double emin, double emax, cudaStream_t s) {
 // number of moments-pass steps j = 1..J with 2j + 1 <= N_C - 1
 inline int pass1_steps(int n_c) { return n_c >= 2 ? (n_c - 2) / 2 : 0; }
 
-// F~ = L^-1 F L^-T, spectral bounds, N_C, H_N (mixed path: also m_0, m_1, m_2)
+// F~ = L^-1 F L^-T, spectral bounds, N_C, H_N (the plain recurrence: also m_0, m_1, m_2)
 void dm_prepare(Ctx& c, const double* F, cudaStream_t s, Timer* tm, int t0) {
     if (!c.have_chol) throw Error(DFT_EINVAL, "call dft_overlap_kinetic first");
     const int K = c.K;
@@ -581,6 +615,12 @@ void dm_prepare(Ctx& c, const double* F, cudaStream_t s, Timer* tm, int t0) {
     launch_cos_table(4 * n_c, c.d_cos, s);
     if (tm) tm->mark(t0 + 2);
     if (c.p.precision == DFT_PREC_FP64) return;
+    TcCfg shape;
+    c.recurrence = tc_forced_shape(shape);
+    if (!c.recurrence) {
+        pst_split_h(c, s);
+        return;
+    }
     // split H_N into its 16-bit pair; trace and |H|^2 of the pair
     double m0 = (double)K;
     DFT_CUDA_CHECK(cudaMemcpyAsync(c.d_mom, &m0, sizeof(double), cudaMemcpyHostToDevice, s));
@@ -593,63 +633,23 @@ void dm_prepare(Ctx& c, const double* F, cudaStream_t s, Timer* tm, int t0) {
     if (n_c > 2) launch_moment_reduce(1, c.d_scal + SCAL_TRACE, c.d_mom, 2, -1, m0, c.d_mom + 1, s);
 }
 
-// In-flight tuning of the tensor-core launch shape on the weighted pass
-// (the dominant one): while the shape of this (precision, size, batch) is
-// untuned, the first steps l = 2, 3, ... run each candidate shape on two
-// rounds of real steps (two per-step launches, or one dataflow launch of
-// eight steps), timed by events, and the fastest per step (minimum over
-// rounds) is kept for the rest of the pass and for later calls; no step is
-// repeated.  Returns the first step not yet run.
-int tc_pass2_tuned(TcBatch& b, int total_k, int Lmax, cudaStream_t s) {
-    int l = 2;
-    TcCfg cand[12];
-    const int nc = tc_candidates(b, cand);
-    const int per = 2, per_flow = 8, rounds = 2;
-    int need = 0;
-    for (int i = 0; i < nc; ++i) need += rounds * (cand[i].flow ? per_flow : per);
-    if (tc_needs_tuning(b, total_k) && Lmax - 2 >= need + 8) {
-        float best_ms[12];
-        for (float& x : best_ms) x = 1e30f;
-        cudaEvent_t e0, e1;
-        DFT_CUDA_CHECK(cudaEventCreate(&e0));
-        DFT_CUDA_CHECK(cudaEventCreate(&e1));
-        for (int r = 0; r < rounds; ++r)
-            for (int i = 0; i < nc; ++i) {
-                b.cfg = cand[i];
-                const int n = cand[i].flow ? per_flow : per;
-                DFT_CUDA_CHECK(cudaEventRecord(e0, s));
-                if (cand[i].flow) {
-                    tc_run_flow(b, l, n, 1, 1, s);
-                    l += n;
-                } else {
-                    for (int k = 0; k < n; ++k, ++l) tc_step_batch(b, l, (l + 1) & 1, 1, s);
-                }
-                DFT_CUDA_CHECK(cudaEventRecord(e1, s));
-                DFT_CUDA_CHECK(cudaEventSynchronize(e1));
-                float ms = 0.f;
-                DFT_CUDA_CHECK(cudaEventElapsedTime(&ms, e0, e1));
-                best_ms[i] = std::min(best_ms[i], ms / n);
-            }
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-        int best = 0;
-        for (int i = 1; i < nc; ++i)
-            if (best_ms[i] < best_ms[best]) best = i;
-        tc_record(b, total_k, cand[best], best_ms, nc);
+// first pass of one system: the matrices of the expansion and, if wanted, the
+// moments m_l = Tr T_l(H_N), l < N_C (the plain recurrence by doubling)
+void dm_pass1(Ctx& c, bool moments, cudaStream_t s) {
+    if (c.p.precision != DFT_PREC_FP64 && !c.recurrence) {
+        Ctx* cp = &c;
+        const int m = moments ? 1 : 0;
+        pst_pass1(&cp, 1, &m, s);
+        return;
     }
-    b.cfg = tc_tuned(b, total_k);
-    return l;
-}
-
-// moments of one system: m_l = Tr T_l(H_N), l < N_C (mixed path by doubling)
-void dm_pass1(Ctx& c, cudaStream_t s) {
-    const int K = c.K, n_c = c.n_c_cur, J = pass1_steps(n_c);
     if (c.p.precision != DFT_PREC_FP64) {
+        if (!moments) return;
+        const int J = pass1_steps(c.n_c_cur);
         Ctx* cp = &c;
         int lim = J + 1, last = J;
         TcBatch b = tc_batch(c, &cp, 1, &lim, &last, s);
         tc_set_limits(b, &cp, &lim, &last, s);
-        b.cfg = tc_tuned(b, K);
+        tc_forced_shape(b.cfg);
         if (b.cfg.flow) {
             tc_run_flow(b, 1, J, 0, 2, s);
             tc_moments_from_fixed(b, J, s);
@@ -661,7 +661,7 @@ void dm_pass1(Ctx& c, cudaStream_t s) {
         }
         return;
     }
-    ps64_pass1(c, true, s);
+    ps64_pass1(c, moments, s);
 }
 
 // mu from 2 sum_l a_l(mu) m_l = N_e (Eq. 2.8), then the coefficients
@@ -681,17 +681,22 @@ void dm_mu_fixed(Ctx& c, double mu, cudaStream_t s) {
 
 // weighted pass of one system: rho = sum_l a_l X_l
 void dm_pass2(Ctx& c, cudaStream_t s) {
-    const int K = c.K, n_c = c.n_c_cur;
+    const int n_c = c.n_c_cur;
+    if (c.p.precision != DFT_PREC_FP64 && !c.recurrence) {
+        Ctx* cp = &c;
+        pst_pass2(&cp, 1, s);
+        return;
+    }
     if (c.p.precision != DFT_PREC_FP64) {
         tc_init(c, c.d_coef, s);
         Ctx* cp = &c;
         int lim = n_c, last = 0;
         TcBatch b = tc_batch(c, &cp, 1, &lim, &last, s);
         tc_set_limits(b, &cp, &lim, &last, s);
-        const int l0 = tc_pass2_tuned(b, K, n_c, s);
-        if (b.cfg.flow) tc_run_flow(b, l0, n_c - l0, 1, 1, s);
+        tc_forced_shape(b.cfg);
+        if (b.cfg.flow) tc_run_flow(b, 2, n_c - 2, 1, 1, s);
         else
-            for (int l = l0; l < n_c; ++l) tc_step_batch(b, l, (l + 1) & 1, 1, s);
+            for (int l = 2; l < n_c; ++l) tc_step_batch(b, l, (l + 1) & 1, 1, s);
         tc_rho_finish(c, s);
         return;
     }
@@ -746,12 +751,9 @@ void dm_finish(Ctx& c, double* P, dft_info* info, cudaStream_t s) {
 void density_matrix_impl(Ctx& c, const double* F, double* P, dft_info* info, cudaStream_t s, Timer* tm,
                          int t0, const double* mu_fixed = nullptr) {
     dm_prepare(c, F, s, tm, t0);
-    if (mu_fixed) {
-        dm_mu_fixed(c, *mu_fixed, s);
-    } else {
-        dm_pass1(c, s);
-        dm_mu(c, s);
-    }
+    dm_pass1(c, mu_fixed == nullptr, s);
+    if (mu_fixed) dm_mu_fixed(c, *mu_fixed, s);
+    else dm_mu(c, s);
     if (tm) tm->mark(t0 + 3);
     dm_pass2(c, s);
     if (tm) tm->mark(t0 + 4);
@@ -946,6 +948,7 @@ dft_status dft_init_basis(dft_ctx** ctx, const dft_basis_desc* basis, const dft_
             DFT_CUDA_CHECK(cudaMemsetAsync(c->d_x16[0], 0, (size_t)c->Kp * c->Kp * 2 * 4, s));
             tc_setup(*c);
             cg_setup(*c);
+            pst_setup(*c, s);
         }
         launch_build_tables(*c, s);
         if (c->contracted) {
@@ -1173,55 +1176,63 @@ dft_status dft_scf_step_batched(dft_ctx* const* ctxs, int n, double* const* n_in
             dm_prepare(c, c.d_F, as, nullptr, 0);
         });
         tm.mark(1);
-        // moments pass over all systems: one dataflow launch, or one launch per
-        // step replayed from a CUDA graph
-        std::vector<int> lim(n), last(n);
-        int Jmax = 0, Lmax = 0;
-        for (int q = 0; q < n; ++q) {
-            int J = pass1_steps(cs[q]->n_c_cur);
-            lim[q] = J + 1;
-            last[q] = J;
-            Jmax = std::max(Jmax, J);
-            Lmax = std::max(Lmax, cs[q]->n_c_cur);
-        }
-        TcBatch b = tc_batch(lead, cs.data(), n, lim.data(), last.data(), s);
-        tc_set_limits(b, cs.data(), lim.data(), last.data(), s);
-        int total_k = 0;
-        for (int q = 0; q < n; ++q) total_k += cs[q]->K;
-        b.cfg = tc_tuned(b, total_k);
-        const long long gkey1 = batch_key(b);
-        if (b.cfg.flow) {
-            tc_run_flow(b, 1, Jmax, 0, 2, s);
-            tc_moments_from_fixed(b, Jmax, s);
+        if (!lead.recurrence) {
+            const std::vector<int> want(n, 1);
+            pst_pass1(cs.data(), n, want.data(), s);
+            tm.mark(2);
+            fork_systems(cs, s, [&](Ctx& c, int, cudaStream_t as) { dm_mu(c, as); });
+            tm.mark(3);
+            pst_pass2(cs.data(), n, s);
+            tm.mark(4);
         } else {
-            run_graph(lead, 0, Jmax, gkey1, s, [&](cudaStream_t gs) {
-                for (int j = 1; j <= Jmax; ++j) {
-                    tc_step_batch(b, j, j & 1, 2, gs);
-                    tc_moment_reduce_batch(b, j, gs);
-                }
-            });
+            // moments pass over all systems: one dataflow launch, or one launch per
+            // step replayed from a CUDA graph
+            std::vector<int> lim(n), last(n);
+            int Jmax = 0, Lmax = 0;
+            for (int q = 0; q < n; ++q) {
+                int J = pass1_steps(cs[q]->n_c_cur);
+                lim[q] = J + 1;
+                last[q] = J;
+                Jmax = std::max(Jmax, J);
+                Lmax = std::max(Lmax, cs[q]->n_c_cur);
+            }
+            TcBatch b = tc_batch(lead, cs.data(), n, lim.data(), last.data(), s);
+            tc_set_limits(b, cs.data(), lim.data(), last.data(), s);
+            tc_forced_shape(b.cfg);
+            const long long gkey1 = batch_key(b);
+            if (b.cfg.flow) {
+                tc_run_flow(b, 1, Jmax, 0, 2, s);
+                tc_moments_from_fixed(b, Jmax, s);
+            } else {
+                run_graph(lead, 0, Jmax, gkey1, s, [&](cudaStream_t gs) {
+                    for (int j = 1; j <= Jmax; ++j) {
+                        tc_step_batch(b, j, j & 1, 2, gs);
+                        tc_moment_reduce_batch(b, j, gs);
+                    }
+                });
+            }
+            tm.mark(2);
+            for (int q = 0; q < n; ++q) {
+                dm_mu(*cs[q], s);
+                tc_init(*cs[q], cs[q]->d_coef, s);
+                lim[q] = cs[q]->n_c_cur;
+                last[q] = 0;
+            }
+            tc_set_limits(b, cs.data(), lim.data(), last.data(), s);
+            tm.mark(3);
+            const int l0 = 2;
+            const long long gkey2 = batch_key(b) * 65536 + l0;
+            if (b.cfg.flow) {
+                tc_run_flow(b, l0, Lmax - l0, 1, 1, s);
+            } else {
+                run_graph(lead, 1, Lmax - l0, gkey2, s, [&](cudaStream_t gs) {
+                    for (int l = l0; l < Lmax; ++l) tc_step_batch(b, l, (l + 1) & 1, 1, gs);
+                });
+            }
+            tm.mark(4);
         }
-        tm.mark(2);
-        for (int q = 0; q < n; ++q) {
-            dm_mu(*cs[q], s);
-            tc_init(*cs[q], cs[q]->d_coef, s);
-            lim[q] = cs[q]->n_c_cur;
-            last[q] = 0;
-        }
-        tc_set_limits(b, cs.data(), lim.data(), last.data(), s);
-        tm.mark(3);
-        const int l0 = tc_pass2_tuned(b, total_k, Lmax, s);
-        const long long gkey2 = batch_key(b) * 65536 + l0;
-        if (b.cfg.flow) {
-            tc_run_flow(b, l0, Lmax - l0, 1, 1, s);
-        } else {
-            run_graph(lead, 1, Lmax - l0, gkey2, s, [&](cudaStream_t gs) {
-                for (int l = l0; l < Lmax; ++l) tc_step_batch(b, l, (l + 1) & 1, 1, gs);
-            });
-        }
-        tm.mark(4);
         fork_systems(cs, s, [&](Ctx& c, int q, cudaStream_t as) {
-            tc_rho_finish(c, as);
+            if (c.recurrence) tc_rho_finish(c, as);
             dm_finish(c, c.d_P, &loc[q], as);
             c.mu_hist[1] = c.mu_hist[0];
             c.mu_hist[0] = c.mu_last;

@@ -64,7 +64,7 @@ struct TcFlow {
     int bias = 0;   // added to the producer's counter targets (0; 1 only to test the waits' expiry)
 };
 
-// launch configuration of the tensor-core step (chosen by the autotuner)
+// launch shape of the recurrence's tensor-core step (DFT_TC_SHAPE)
 struct TcCfg {
     int bk = 32;        // k-block width: 32, 64 or 16 (64 and 16 only with 256-wide tiles)
     int persist = 0;    // 0: one CTA per tile; p > 0: p CTAs per SM, strided tile loop
@@ -82,6 +82,25 @@ struct PsPlan {
     int n_c = 0, s = 1, Q = 0;
     bool direct = false;
 };
+
+// one system of a tensor-core product launch (k_poly_tc.cu) and one product:
+// out = alpha sum_{first <= q < last} A_q B_q - prev (a pair) + add (FP32
+// planes) on its slots; mode: PST_*
+struct PstSys {
+    int K, nb;                   // basis size, 256-blocks per side
+    const CUtensorMap* maps;     // 4 per slot
+    void* const* slot;
+    int* flags;
+};
+struct PstItem {
+    int sys, first, last;
+    int prev, add, out;          // slots, -1: none
+    int mode;
+    float limit;                 // > 0: FLAG_SPECTRUM beyond it
+    int tile0;                   // first tile of this product in the launch
+};
+enum { PST_ALPHA2 = 1, PST_IDENT = 2, PST_OUT_F32 = 4 };   // alpha = 2; prev = I; FP32 planes out
+constexpr int PST_ITEM_CAP = 16384;
 
 struct Ctx {
     // problem
@@ -135,6 +154,16 @@ struct Ctx {
     std::vector<double*> ps_slot;
     int ps_extra = 0;            // of them, those carved for this purpose alone
     PsPlan ps;
+    // expansion slots of the mixed path (upper blocks of a split pair each,
+    // k_poly_tc.cu), their tensor maps and table on the device, and the
+    // launch tables of a batch led by this context
+    std::vector<void*> pst_slot;
+    CUtensorMap* d_pst_maps = nullptr;
+    void** d_pst_slots = nullptr;
+    PstSys* d_pst_sys = nullptr;
+    PstItem* d_pst_items = nullptr;
+    int2* d_pst_pairs = nullptr;
+    bool recurrence = false;     // this density matrix runs the plain three-term recurrence
     double* d_gram = nullptr;    // partial Gram sums [gram_cap]
     long long gram_cap = 0;
     double* d_B = nullptr;       // K x K scratch
@@ -201,7 +230,6 @@ struct Ctx {
     int* d_cnt = nullptr;        // dataflow: block-pair counters of a batch led by this context [3 x tile_cap]
     long long* d_macc = nullptr; // dataflow: fixed-point moment sums of this system [cheb_cap]
     int n_c_cur = 0;             // Chebyshev order of the density matrix in progress
-    TcCfg tc_cfg;                // launch shape chosen for this system
     double e_bounds[2] = {0, 0}; // its spectral bounds
     cudaGraphExec_t graph_exec[2] = {nullptr, nullptr};   // batched recurrence loops
     int graph_count[2] = {0, 0};
@@ -315,7 +343,7 @@ void launch_moment_reduce(int nparts, const double* part, double* mom, int idx_e
                           double m0, const double* m1, cudaStream_t s);
 
 // ---- grouped evaluation of the expansion (k_poly.cu) ----
-PsPlan ps_plan(int n_c, int nslot, bool prefer_direct);
+PsPlan ps_plan(int n_c, int nslot, bool prefer_direct, int nroll);
 // m_l, l < n_c, from the traces and Gram sums D ((Q + 1) x s)
 void launch_ps_moments(int K, const PsPlan& p, const double* D, double* mom, cudaStream_t s);
 // c_qr of the C_q from a_l; work holds (Q + 1) s doubles
@@ -325,7 +353,15 @@ void launch_ps_coefs(const PsPlan& p, const double* a, double* c, double* work, 
 void ps64_pass1(Ctx& c, bool moments, cudaStream_t s);
 void ps64_pass2(Ctx& c, cudaStream_t s);
 
-// ---- tensor-core Chebyshev path (k_cheb_tc.cu) ----
+// the same in split 16-bit form on the tensor cores, for n systems at once
+// (k_poly_tc.cu); moments[q] = 0: no moments wanted of system q
+size_t pst_slot_bytes(int Kp);
+void pst_setup(Ctx& c, cudaStream_t s);
+void pst_split_h(Ctx& c, cudaStream_t s);
+void pst_pass1(Ctx* const* cs, int n, const int* moments, cudaStream_t s);
+void pst_pass2(Ctx* const* cs, int n, cudaStream_t s);
+
+// ---- three-term recurrence on the tensor cores (k_cheb_tc.cu) ----
 int tc_pad(int K);
 std::vector<int> tc_tiles(int K, int bn);   // (row tile, column tile) pairs reaching the upper triangle
 void tc_setup(Ctx& c);
@@ -342,13 +378,8 @@ struct TcBatch {
     bool bf = false;
     TcCfg cfg;
 };
-// in-flight tuning: the first steps of a pass run each candidate on real
-// steps, the fastest is kept per (precision, K bucket, systems) and cached
-// (optionally in the JSON file named by DFT_AUTOTUNE_CACHE)
-TcCfg tc_tuned(const TcBatch& b, int total_k);
-bool tc_needs_tuning(const TcBatch& b, int total_k);
-void tc_record(const TcBatch& b, int total_k, TcCfg best, const float* ms, int ncand);
-int tc_candidates(const TcBatch& b, TcCfg* out);   // at most 8
+// launch shape of DFT_TC_SHAPE; false: unset or malformed (no recurrence)
+bool tc_forced_shape(TcCfg& c);
 int tc_streamk_grid(const TcBatch& b);             // 0 where stream-K does not apply
 // fill leader's batch area with the given systems (pass lim/mom_last per system)
 TcBatch tc_batch(Ctx& leader, Ctx* const* sys, int nsys, const int* lim, const int* mom_last, cudaStream_t s);

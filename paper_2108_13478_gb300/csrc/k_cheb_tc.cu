@@ -1,4 +1,6 @@
-// Tensor-core Chebyshev step (Supp. B) for sm_103a: X_{l+1} = 2 H_N X_l - X_{l-1}
+// Tensor-core Chebyshev step (Supp. B) for sm_103a, the plain three-term
+// recurrence (run when DFT_TC_SHAPE names its launch shape; otherwise the
+// grouped evaluation of k_poly_tc.cu runs): X_{l+1} = 2 H_N X_l - X_{l-1}
 // with the product on tcgen05 (FP32 accumulation in tensor memory) in the split
 // form H X ~ H_hi X_hi + H_hi X_lo + H_lo X_hi, where every operand is stored as
 // a pair of 16-bit floats (hi = round(x), lo = round(x - hi)).  With FP16 the
@@ -43,10 +45,6 @@
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
-#include <fstream>
-#include <map>
-#include <mutex>
-#include <sstream>
 
 namespace dft {
 namespace tc {
@@ -1436,7 +1434,7 @@ void tc_step_batch(const TcBatch& b, int l, int cur, int mode, cudaStream_t s) {
         return;
     }
     const Ctx& L = *b.leader;
-    // launch shape (tuned): one CTA per tile, with the hardware handing tiles
+    // launch shape: one CTA per tile, with the hardware handing tiles
     // to SMs as they free up, or a persistent grid of `persist` CTAs per SM
     // walking the tile list with a fixed stride
     const int v = b.cfg.bn == 128 ? 1 : 0;
@@ -1597,86 +1595,8 @@ void tc_rho_finish(const Ctx& c, cudaStream_t s) {
     check_launch("rho_mirror");
 }
 
-// ---- autotuner of the tensor-core launch configuration ----
-namespace {
-std::mutex g_tune_mu;
-std::map<std::string, TcCfg> g_tuned;
-std::map<std::string, std::vector<float>> g_tune_ms;   // candidate times of the tuning run (diagnostics)
-bool g_tune_loaded = false;
-
-std::string tune_key(const TcBatch& b, int total_k) {
-    // quarter-octave buckets of the summed basis size
-    int bucket = (int)std::lround(4.0 * std::log2((double)std::max(total_k, 1)));
-    std::ostringstream o;
-    o << (b.bf ? "bf16x3" : "fp16x3") << "_kb" << bucket << "_n" << b.nsys;
-    return o.str();
-}
-
-// cache file: one entry per line, `"key": [bk, persist, bn, streamk, flow, ms...],`
-// inside braces (entries without bn are 256-wide, without streamk tile mode;
-// ms are the candidates' times per step)
-void tune_load() {
-    if (g_tune_loaded) return;
-    g_tune_loaded = true;
-    const char* path = std::getenv("DFT_AUTOTUNE_CACHE");
-    if (!path) return;
-    std::ifstream f(path);
-    std::string line;
-    while (std::getline(f, line)) {
-        size_t q0 = line.find('"'), q1 = line.find('"', q0 + 1), lb = line.find('[', q1 + 1);
-        if (q0 == std::string::npos || q1 == std::string::npos || lb == std::string::npos) continue;
-        TcCfg c;
-        int n = std::sscanf(line.c_str() + lb, "[%d, %d, %d, %d, %d", &c.bk, &c.persist, &c.bn, &c.streamk, &c.flow);
-        if (n == 2) c.bn = 256;
-        if (n < 4) c.streamk = 0;
-        if (n < 5) c.flow = 0;
-        if (n >= 2 && (c.bk == 32 || c.bk == 64 || (c.bk == 16 && c.bn == 256)) && c.persist >= 0 && c.persist <= 2 &&
-            (c.bn == 256 || (c.bn == 128 && c.bk == 32)) && (c.streamk == 0 || (c.streamk == 1 && c.bn == 256)) &&
-            (c.flow == 0 || c.flow == 1))
-            g_tuned[line.substr(q0 + 1, q1 - q0 - 1)] = c;
-    }
-}
-
-void tune_save() {
-    const char* path = std::getenv("DFT_AUTOTUNE_CACHE");
-    if (!path) return;
-    std::ofstream f(path);
-    f << "{\n";
-    size_t i = 0;
-    for (auto& kv : g_tuned)
-    {
-        f << "  \"" << kv.first << "\": [" << kv.second.bk << ", " << kv.second.persist << ", " << kv.second.bn << ", "
-          << kv.second.streamk << ", " << kv.second.flow;
-        auto it = g_tune_ms.find(kv.first);
-        if (it != g_tune_ms.end())
-            for (float m : it->second) f << ", " << m;
-        f << "]" << (++i < g_tuned.size() ? "," : "") << "\n";
-    }
-    f << "}\n";
-}
-}  // namespace
-
-int tc_candidates(const TcBatch& b, TcCfg* out) {
-    const TcCfg c[8] = {{32, 0, 256, 0}, {64, 0, 256, 0}, {32, 1, 256, 0}, {64, 1, 256, 0},
-                        {32, 0, 128, 0}, {32, 2, 128, 0}, {32, 0, 256, 1}, {64, 0, 256, 1}};
-    int n = 0;
-    for (int i = 0; i < 6; ++i) out[n++] = c[i];
-    // stream-K only where it applies and where it can balance a ragged last wave
-    if (tc_streamk_grid(b) == std::min(num_sms(), TC_SK_MAX_CTAS)) {
-        out[n++] = c[6];
-        out[n++] = c[7];
-    }
-    for (int bk : {32, 64}) {
-        TcCfg f;
-        f.bk = bk;
-        f.flow = 1;
-        out[n++] = f;
-    }
-    return n;
-}
-
 // launch shape forced through DFT_TC_SHAPE="bk,persist,bn[,streamk[,pf[,epf[,flow]]]]"
-static bool forced_shape(TcCfg& c) {
+bool tc_forced_shape(TcCfg& c) {
     const char* e = std::getenv("DFT_TC_SHAPE");
     if (!e) return false;
     TcCfg f;
@@ -1693,30 +1613,6 @@ static bool forced_shape(TcCfg& c) {
         return false;
     c = f;
     return true;
-}
-
-bool tc_needs_tuning(const TcBatch& b, int total_k) {
-    TcCfg f;
-    if (std::getenv("DFT_AUTOTUNE_OFF") || forced_shape(f)) return false;
-    std::lock_guard<std::mutex> lock(g_tune_mu);
-    tune_load();
-    return g_tuned.find(tune_key(b, total_k)) == g_tuned.end();
-}
-
-TcCfg tc_tuned(const TcBatch& b, int total_k) {
-    TcCfg f;
-    if (forced_shape(f)) return f;
-    std::lock_guard<std::mutex> lock(g_tune_mu);
-    tune_load();
-    auto it = g_tuned.find(tune_key(b, total_k));
-    return it == g_tuned.end() ? TcCfg{} : it->second;
-}
-
-void tc_record(const TcBatch& b, int total_k, TcCfg best, const float* ms, int n) {
-    std::lock_guard<std::mutex> lock(g_tune_mu);
-    g_tuned[tune_key(b, total_k)] = best;
-    g_tune_ms[tune_key(b, total_k)] = std::vector<float>(ms, ms + n);
-    tune_save();
 }
 
 }  // namespace dft

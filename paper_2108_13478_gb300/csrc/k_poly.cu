@@ -322,10 +322,10 @@ inline int upper_tiles(int K, int tb) {
 }  // namespace
 
 // Baby count and plan for n_c terms on nslot buffers: s + 2 Q products, Q =
-// (n_c - 1) / s.  Direct: s - 1 babies (T_1 = H_N has its own storage), the
+// (n_c - 1) / s.  Direct: s - 1 babies (T_1 = H_N is not counted), the
 // giants G_2 .. G_Q and PS_CQ buffers for the C_q and the partial sums of the
-// weighted products.  Clenshaw: the babies T_2 .. T_s and two rolling buffers.
-PsPlan ps_plan(int n_c, int nslot, bool prefer_direct) {
+// weighted products.  Clenshaw: the babies T_2 .. T_s and nroll buffers.
+PsPlan ps_plan(int n_c, int nslot, bool prefer_direct, int nroll) {
     PsPlan p;
     p.n_c = n_c;
     int best = 1 << 30;
@@ -334,7 +334,7 @@ PsPlan ps_plan(int n_c, int nslot, bool prefer_direct) {
         const int Q = (n_c - 1) / s;
         const int cost = s + 2 * Q;
         const int need_d = (s - 1) + std::max(0, Q - 1) + (Q > 0 ? PS_CQ + 1 : 0);
-        const int need_c = (s - 1) + 2;
+        const int need_c = (s - 1) + nroll;
         const bool fits_d = need_d <= nslot && Q <= PS_MAX_Q, fits_c = need_c <= nslot;
         if (cost < best && (fits_d || fits_c)) {
             best = cost;
@@ -445,7 +445,7 @@ double growth_limit(int l, int n_c) {
 
 // babies, giants and (with moments) m_l; the plan is kept in c.ps
 void ps64_pass1(Ctx& c, bool moments, cudaStream_t st) {
-    c.ps = ps_plan(c.n_c_cur, (int)c.ps_slot.size(), upper_tiles(c.K, 32) < 4 * 152);
+    c.ps = ps_plan(c.n_c_cur, (int)c.ps_slot.size(), upper_tiles(c.K, 32) < 4 * 152, 2);
     const PsPlan& p = c.ps;
     Ps64 e{c, p, st};
     const int s = p.s, Q = p.Q;

@@ -1,0 +1,1039 @@
+// The grouped Chebyshev expansion (k_poly.cu) on the tensor cores: products
+// of symmetric polynomials of H_N in the split 16-bit form
+//   A B ~ A_hi B_hi + A_hi B_lo + A_lo B_hi   (hi = round(x), lo = round(x - hi))
+// on tcgen05 with FP32 accumulation, for one or many systems per launch.
+//
+// Storage.  Every matrix is symmetric, so a buffer ("slot") keeps the 256 x
+// 256 blocks (a, b), a <= b, only (diagonal blocks whole), folded into a
+// rectangle of R = nb / 2 + 1 block rows (nb = Kp / 256 blocks per side): block row a
+// < R lies in place, block row a >= R, which has nb - a blocks, fills the
+// free left end of block row nb - a.  Half the bytes of full storage: twice
+// as many babies fit the workspace, more operand tiles stay in L2, and no
+// mirror is written.  A slot holds the hi plane and then the lo plane; the same two planes
+// can hold FP32 values as their upper and lower 16 bits.  An
+// operand tile whose k block lies left of the diagonal is read transposed:
+// as rows of k (MN-major operand, 128-byte swizzle, one 3-D TMA box), the
+// others K-major (64-byte swizzle).
+//
+// Kernel k_pst_prod: persistent, one CTA per SM, one 128 x 256 output tile
+// at a time: warp 0 lane 0 drives the TMA loads of the four operand tiles of
+// each 32-wide k-block into a 4-stage ring of 48 KB, warp 1 owns the 512
+// tensor-memory columns and lane 0 issues the MMAs, eight epilogue warps add
+// each finished unit of SUB k-blocks from one of two accumulators into FP32
+// registers (round to nearest; the tensor core's own FP32 accumulation leans
+// towards zero with every addition, so its chains are kept short) and then
+// write x = alpha A B - prev + add straight from registers: a thread's 16 columns are
+// one 32-byte sector per plane, so no staging is needed, the ring stays with the
+// producer and the next tile's loads and first two units run under the
+// epilogue.  Every wait is bounded; on expiry the CTA sets FLAG_TIMEOUT,
+// drains what it issued and returns.
+//
+// Density matrix at K = 1230, tail 1e-5 (N_C ~ 1410, direct plan): 118.9 ms
+// with the recurrence of k_cheb_tc.cu, 7.4 ms with this (error of P against
+// an exact eigensolve 3.7e-5 -> 2.5e-5); SCF cycle at K = 4650 (Clenshaw plan,
+// s = 34, 112 products) 677 -> 165 ms.
+#include "ps_plan.cuh"
+#include "tc_ptx.cuh"
+
+#include <algorithm>
+#include <cmath>
+
+namespace dft {
+namespace {
+
+using namespace tc;
+
+constexpr int BM = 128, BN = 256, BK = 32, STAGES = 4;
+constexpr int SUB = 2;   // k-blocks per accumulator promotion: chains of 12 additions
+constexpr int A_BYTES = BM * BK * 2, B_BYTES = BN * BK * 2;
+constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;
+constexpr int NEPI = 256, NTHREADS = 64 + NEPI, CPT = 128;
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
+constexpr int TMEM_COLS = 2 * BN;
+constexpr int SMS = 152;
+// pairs hold x * SC: the low half of an FP16 pair of x itself would be a
+// subnormal number for the elements of order K^-1/2 that most of a T_l
+// consists of (2^-25 absolute); scaled, the pair keeps 22 bits down to
+// 2^-27.  |T_l| <= 4 and the b_q stay far below 65504 / SC.
+constexpr float SC = 1024.0f, ISC = 1.0f / SC;
+
+// folded place of block (a, b), a <= b
+__device__ __forceinline__ void fold(int a, int b, int nb, int& row, int& col) {
+    const bool in_place = a <= nb / 2;
+    row = in_place ? a : nb - a;
+    col = in_place ? b : b - a;
+}
+
+// tile u of a system: blocks (p, q) row by row, both 128-row tiles of a block
+// together; row tiles beyond K are left out
+__device__ __forceinline__ void tile_at(int u, int nb, int mt, int& i, int& j) {
+    int p = 0;
+    for (;; ++p) {
+        const int rows = min(2, mt - 2 * p), n = (nb - p) * rows;
+        if (u < n) {
+            j = p + u / rows;
+            i = 2 * p + u % rows;
+            return;
+        }
+        u -= n;
+    }
+}
+
+__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+        ::"r"(smem_u32(dst)), "l"(map), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
+        : "memory");
+}
+
+// descriptor of an MN-major operand in 128-byte swizzle: 64-element groups of
+// the M (N) index 32 k-rows x 128 bytes = 4096 bytes apart (leading offset),
+// groups of 8 k-rows 1024 bytes apart (stride offset)
+__device__ __forceinline__ uint64_t smem_desc_mn(const void* p) {
+    const uint64_t addr = (uint64_t)(smem_u32(p) & 0x3FFFF) >> 4;
+    return addr | ((uint64_t)(BK * 128 >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
+}
+
+// one product of a launch as the roles walk it
+struct Work {
+    PstItem it;
+    const PstSys* S;
+    int i, j, p, nk;   // row tile, column block, row block, k-blocks per operand pair
+};
+__device__ __forceinline__ Work work_at(int t, const PstItem* __restrict__ items, int nitems,
+                                        const PstSys* __restrict__ sys) {
+    int a = 0, b = nitems;   // last item with tile0 <= t
+    while (b - a > 1) {
+        const int m = (a + b) >> 1;
+        if (items[m].tile0 <= t) a = m;
+        else b = m;
+    }
+    Work w;
+    w.it = items[a];
+    w.S = sys + w.it.sys;
+    tile_at(t - w.it.tile0, w.S->nb, (w.S->K + BM - 1) / BM, w.i, w.j);
+    w.p = w.i >> 1;
+    w.nk = (w.S->K + BK - 1) / BK;
+    return w;
+}
+
+template <bool BF>
+__global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restrict__ sys,
+                                                          const PstItem* __restrict__ items, int nitems,
+                                                          const int2* __restrict__ pairs, int ntiles) {
+    using T = typename H16<BF>::T;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint64_t* full = (uint64_t*)(smem + STAGES * STAGE_BYTES);
+    uint64_t* empty = full + STAGES;
+    uint64_t* accfull = empty + STAGES;
+    uint64_t* accempty = accfull + 2;
+    uint64_t* drain = accempty + 2;
+    uint32_t* tmem_slot = (uint32_t*)(drain + 1);
+    volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
+    static_assert((2 * STAGES + 5) * 8 + 8 <= 256, "barriers exceed their area");
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int a = 0; a < 2; ++a) {
+            mbar_init(&accfull[a], 1);
+            mbar_init(&accempty[a], NEPI);
+        }
+        mbar_init(drain, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    auto sAh = [&](int s) { return smem + s * STAGE_BYTES; };
+    auto sAl = [&](int s) { return smem + s * STAGE_BYTES + A_BYTES; };
+    auto sBh = [&](int s) { return smem + s * STAGE_BYTES + 2 * A_BYTES; };
+    auto sBl = [&](int s) { return smem + s * STAGE_BYTES + 2 * A_BYTES + B_BYTES; };
+
+    if (warp == 0) {
+        if (lane == 0) {
+            long long g = 0;   // k-blocks issued by this CTA
+            for (int t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x) {
+                const Work w = work_at(t, items, nitems, sys);
+                const int nb = w.S->nb, lo_row = (nb / 2 + 1) * 256;
+                for (int q = w.it.first; q < w.it.last && !*abort_flag; ++q) {
+                    const int2 ab = pairs[q];
+                    const CUtensorMap* ma = w.S->maps + 4 * ab.x;
+                    const CUtensorMap* mb = w.S->maps + 4 * ab.y;
+                    for (int kb = 0; kb < w.nk; ++kb, ++g) {
+                        const int s = (int)(g % STAGES);
+                        const int kq = kb >> 3, kx = (kb & 7) * BK;   // 256-block of k, offset inside
+                        int ar, ac, br, bc;
+                        fold(min(w.p, kq), max(w.p, kq), nb, ar, ac);
+                        fold(min(w.j, kq), max(w.j, kq), nb, br, bc);
+                        if (!mbar_wait(&empty[s], (uint32_t)((g / STAGES) & 1) ^ 1u)) {
+                            *abort_flag = 1;
+                            break;
+                        }
+                        mbar_expect_tx(&full[s], STAGE_BYTES);
+                        if (kq >= w.p) {
+                            const int y = ar * 256 + (w.i & 1) * BM, x = ac * 256 + kx;
+                            tma_load_2d(sAh(s), ma + 0, x, y, &full[s]);
+                            tma_load_2d(sAl(s), ma + 0, x, y + lo_row, &full[s]);
+                        } else {
+                            const int y = ar * 256 + kx, z = ac * 4 + (w.i & 1) * 2;
+                            tma_load_3d(sAh(s), ma + 2, 0, y, z, &full[s]);
+                            tma_load_3d(sAl(s), ma + 2, 0, y + lo_row, z, &full[s]);
+                        }
+                        if (kq >= w.j) {
+                            const int y = br * 256, x = bc * 256 + kx;
+                            tma_load_2d(sBh(s), mb + 1, x, y, &full[s]);
+                            tma_load_2d(sBl(s), mb + 1, x, y + lo_row, &full[s]);
+                        } else {
+                            const int y = br * 256 + kx, z = bc * 4;
+                            tma_load_3d(sBh(s), mb + 3, 0, y, z, &full[s]);
+                            tma_load_3d(sBl(s), mb + 3, 0, y + lo_row, z, &full[s]);
+                        }
+                    }
+                }
+            }
+            if (*abort_flag) {
+                // the last load issued into each stage must land before exit
+                for (long long q = (g > STAGES ? g - STAGES : 0); q < g; ++q)
+                    mbar_wait(&full[q % STAGES], (uint32_t)((q / STAGES) & 1));
+            }
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        if (lane == 0) {
+            const uint32_t idesc0 = (1u << 4) | ((BF ? 1u : 0u) << 7) | ((BF ? 1u : 0u) << 10) |
+                                    ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+            long long g = 0, u = 0;   // k-blocks and units of this CTA
+            for (int t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x) {
+                const Work w = work_at(t, items, nitems, sys);
+                const int nkt = w.nk * (w.it.last - w.it.first);
+                int kb = 0;   // within the operand pair
+                for (int k0 = 0; k0 < nkt && !*abort_flag; k0 += SUB, ++u) {
+                    const int a = (int)(u & 1);
+                    if (!mbar_wait(&accempty[a], (uint32_t)(((u >> 1) & 1) ^ 1))) {
+                        *abort_flag = 1;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint32_t d = tmem + (uint32_t)(a * BN);
+                    bool first = true;
+                    for (int k = k0; k < min(nkt, k0 + SUB); ++k, ++g) {
+                        const int s = (int)(g % STAGES);
+                        if (*abort_flag || !mbar_wait(&full[s], (uint32_t)((g / STAGES) & 1))) {
+                            *abort_flag = 1;
+                            break;
+                        }
+                        tc_fence_after();
+                        const int kq = kb >> 3;
+                        if (++kb == w.nk) kb = 0;
+                        const bool at = kq < w.p, bt = kq < w.j;   // operand read transposed
+                        const uint32_t idesc = idesc0 | ((at ? 1u : 0u) << 15) | ((bt ? 1u : 0u) << 16);
+                        const uint64_t ah = at ? smem_desc_mn(sAh(s)) : smem_desc<BK * 2>(sAh(s));
+                        const uint64_t al = at ? smem_desc_mn(sAl(s)) : smem_desc<BK * 2>(sAl(s));
+                        const uint64_t bh = bt ? smem_desc_mn(sBh(s)) : smem_desc<BK * 2>(sBh(s));
+                        const uint64_t bl = bt ? smem_desc_mn(sBl(s)) : smem_desc<BK * 2>(sBl(s));
+                        // 16 k: 32 bytes along a K-major row, 16 rows of 128 bytes MN-major
+                        const uint64_t as = at ? 128 : 2, bs = bt ? 128 : 2;
+#pragma unroll
+                        for (int kk = 0; kk < BK / 16; ++kk) {
+                            umma_f16(d, ah + kk * as, bh + kk * bs, idesc, first ? 0u : 1u);
+                            umma_f16(d, ah + kk * as, bl + kk * bs, idesc, 1u);
+                            umma_f16(d, al + kk * as, bh + kk * bs, idesc, 1u);
+                            first = false;
+                        }
+                        umma_commit(&empty[s]);
+                    }
+                    umma_commit(&accfull[a]);
+                }
+            }
+            if (*abort_flag) {
+                // every MMA this thread issued must finish before tensor memory is freed
+                umma_commit(drain);
+                mbar_wait(drain, 0);
+            }
+        }
+        __syncwarp();
+    } else {
+        const int quad = warp & 3, half = (warp - 2) >> 2;
+        const int r_loc = 32 * quad + lane;
+        long long u = 0;
+        bool ok = true;
+        for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+            const Work w = work_at(t, items, nitems, sys);
+            const PstSys& S = *w.S;
+            const int nunit = (w.nk * (w.it.last - w.it.first) + SUB - 1) / SUB;
+            float R[CPT];
+#pragma unroll
+            for (int i = 0; i < CPT; ++i) R[i] = 0.0f;
+            for (int q = 0; q < nunit; ++q, ++u) {
+                const int a = (int)(u & 1);
+                const bool got = mbar_wait(&accfull[a], (uint32_t)((u >> 1) & 1));
+                ok = __all_sync(0xffffffffu, got && !*abort_flag);
+                if (!ok) break;
+                tc_fence_after();
+                tmem_add_groups<CPT / 16>(tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(a * BN + half * CPT), R);
+                tc_fence_before();
+                mbar_arrive(&accempty[a]);
+            }
+            if (!ok) {
+                *abort_flag = 1;
+                if (lane == 0) atomicExch(&S.flags[FLAG_TIMEOUT], 1);
+                break;
+            }
+            int fr, fc;
+            fold(w.p, w.j, S.nb, fr, fc);
+            const int ld = S.nb * 256;
+            const size_t plane = (size_t)(S.nb / 2 + 1) * 256 * ld;
+            const size_t e0 = (size_t)(fr * 256 + (w.i & 1) * BM + r_loc) * ld + fc * 256 + half * CPT;
+            const int r = w.i * BM + r_loc, c0 = w.j * BN + half * CPT;   // global row, first column
+            const bool diag = w.p == w.j, f32_out = (w.it.mode & PST_OUT_F32) != 0;
+            const float alpha = ((w.it.mode & PST_ALPHA2) ? 2.0f : 1.0f) * (ISC * ISC);
+            const uint16_t* pv = w.it.prev >= 0 ? (const uint16_t*)S.slot[w.it.prev] + e0 : nullptr;
+            const uint16_t* ad = w.it.add >= 0 ? (const uint16_t*)S.slot[w.it.add] + e0 : nullptr;
+            uint16_t* out = (uint16_t*)S.slot[w.it.out] + e0;
+            // the whole block, for the mirror inside a diagonal block
+            uint16_t* blk = (uint16_t*)S.slot[w.it.out] + (size_t)(fr * 256) * ld + fc * 256;
+            const float limit = w.it.limit;
+            bool bad = false;
+            uint4 nh, nl, ah4, al4;
+            const uint4 z4 = make_uint4(0, 0, 0, 0);
+            nh = pv ? *(const uint4*)pv : z4;
+            nl = pv ? *(const uint4*)(pv + plane) : z4;
+            ah4 = ad ? *(const uint4*)ad : z4;
+            al4 = ad ? *(const uint4*)(ad + plane) : z4;
+#pragma unroll
+            for (int c8 = 0; c8 < CPT / 8; ++c8) {
+                const uint32_t ph[4] = {nh.x, nh.y, nh.z, nh.w}, pl[4] = {nl.x, nl.y, nl.z, nl.w};
+                const uint32_t gh[4] = {ah4.x, ah4.y, ah4.z, ah4.w}, gl[4] = {al4.x, al4.y, al4.z, al4.w};
+                if (c8 + 1 < CPT / 8) {
+                    // the next 8 columns in flight while these are updated
+                    if (pv) {
+                        nh = *(const uint4*)(pv + 8 * (c8 + 1));
+                        nl = *(const uint4*)(pv + plane + 8 * (c8 + 1));
+                    }
+                    if (ad) {
+                        ah4 = *(const uint4*)(ad + 8 * (c8 + 1));
+                        al4 = *(const uint4*)(ad + plane + 8 * (c8 + 1));
+                    }
+                }
+                uint32_t hw[4], lw[4];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const int sh = 16 * (e & 1), c = c0 + 8 * c8 + e;
+                    float x = alpha * R[8 * c8 + e];
+                    if (pv)
+                        x = fmaf(-ISC, H16<BF>::to_f(from_bits16<T>(ph[e >> 1] >> sh)) +
+                                           H16<BF>::to_f(from_bits16<T>(pl[e >> 1] >> sh)), x);
+                    if (ad) x += __uint_as_float((((gh[e >> 1] >> sh) & 0xffffu) << 16) | ((gl[e >> 1] >> sh) & 0xffffu));
+                    if ((w.it.mode & PST_IDENT) && c == r && r < S.K) x -= 1.0f;
+                    bad |= !(fabsf(x) <= limit) && r < S.K && c < S.K && c >= r;
+                    uint32_t h, l;
+                    if (f32_out) {
+                        h = __float_as_uint(x) >> 16;
+                        l = __float_as_uint(x) & 0xffffu;
+                    } else {
+                        x *= SC;
+                        const T th = H16<BF>::from_f(x);
+                        h = bits16(th);
+                        l = bits16(H16<BF>::from_f(x - H16<BF>::to_f(th)));
+                    }
+                    if (e & 1) {
+                        hw[e >> 1] |= h << 16;
+                        lw[e >> 1] |= l << 16;
+                    } else {
+                        hw[e >> 1] = h;
+                        lw[e >> 1] = l;
+                    }
+                    if (diag && c >= r && !f32_out) {
+                        // both triangles of a diagonal block from its upper one
+                        const int br = r - w.p * 256, bc = c - w.p * 256;
+                        blk[(size_t)br * ld + bc] = (uint16_t)h;
+                        blk[plane + (size_t)br * ld + bc] = (uint16_t)l;
+                        blk[(size_t)bc * ld + br] = (uint16_t)h;
+                        blk[plane + (size_t)bc * ld + br] = (uint16_t)l;
+                    }
+                }
+                if (!diag || f32_out) {
+                    *(uint4*)(out + 8 * c8) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+                    *(uint4*)(out + plane + 8 * c8) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+                }
+            }
+            if (bad && limit > 0.0f) atomicExch(&S.flags[FLAG_SPECTRUM], 1);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+    }
+}
+
+// FP64 symmetric matrix -> pair in a slot, zero beyond K
+template <bool BF>
+__global__ void __launch_bounds__(256) k_pst_split(int K, int nb, const double* __restrict__ A, uint16_t* slot) {
+    using T = typename H16<BF>::T;
+    int a = 0, t = blockIdx.x;   // block (a, b)
+    while (t >= nb - a) {
+        t -= nb - a;
+        ++a;
+    }
+    const int b = a + t;
+    int fr, fc;
+    fold(a, b, nb, fr, fc);
+    const size_t ld = (size_t)nb * 256, plane = (size_t)(nb / 2 + 1) * 256 * ld;
+    const int c = threadIdx.x, gc = b * 256 + c;
+    for (int r = blockIdx.y * 16; r < (int)blockIdx.y * 16 + 16; ++r) {
+        const int gr = a * 256 + r;
+        const double x = gr < K && gc < K ? A[(long long)gr * K + gc] * (double)SC : 0.0;
+        const T h = H16<BF>::from_d(x);
+        const T l = H16<BF>::from_d(x - (double)H16<BF>::to_f(h));
+        uint16_t* o = slot + (size_t)(fr * 256 + r) * ld + fc * 256 + c;
+        o[0] = (uint16_t)bits16(h);
+        o[plane] = (uint16_t)bits16(l);
+    }
+}
+
+// four consecutive elements of a pair (scaled back)
+template <bool BF>
+__device__ __forceinline__ float4 pair4(const uint16_t* p, size_t plane) {
+    using T = typename H16<BF>::T;
+    const uint2 h = *(const uint2*)p, l = *(const uint2*)(p + plane);
+    auto f = [](uint32_t a, uint32_t b) { return ISC * (H16<BF>::to_f(from_bits16<T>(a)) + H16<BF>::to_f(from_bits16<T>(b))); };
+    return make_float4(f(h.x, l.x), f(h.x >> 16, l.x >> 16), f(h.y, l.y), f(h.y >> 16, l.y >> 16));
+}
+
+// block blockIdx.x of the upper block triangle
+__device__ __forceinline__ void block_at(int t, int nb, int& a, int& b) {
+    a = 0;
+    while (t >= nb - a) {
+        t -= nb - a;
+        ++a;
+    }
+    b = a + t;
+}
+
+// C_q = sum_{r<s} c_qr T_r (T_0 = I) for up to 8 q at once, each to a slot, as
+// a pair (operand) or as FP32 planes.  HBM-bound: the babies are read once
+// per 8 q; 4 consecutive elements per thread, FP32 FMA chains of s terms.
+template <bool BF>
+__global__ void __launch_bounds__(256) k_pst_combine(int K, int nb, int s, PstList T, PstOut out, int q0, int nq,
+                                                     const double* __restrict__ c, int f32) {
+    using H = typename H16<BF>::T;
+    __shared__ float4 cf[PS_MAX_S][2];
+    const int qb = blockIdx.z * 8, n = min(8, nq - qb);
+    for (int e = threadIdx.x; e < s * 8; e += 256) {
+        const int r = e >> 3, q = e & 7;
+        ((float*)cf)[e] = q < n ? (float)c[(long long)(q0 + qb + q) * s + r] : 0.0f;
+    }
+    __syncthreads();
+    int a, b, fr, fc;
+    block_at(blockIdx.x, nb, a, b);
+    fold(a, b, nb, fr, fc);
+    const size_t ld = (size_t)nb * 256, plane = (size_t)(nb / 2 + 1) * 256 * ld;
+    const int lr = blockIdx.y * 4 + (threadIdx.x >> 6), lc = (threadIdx.x & 63) * 4;
+    if (a * 256 + (int)blockIdx.y * 4 >= (K + 31) / 32 * 32) return;   // beyond every operand's k range
+    const size_t e0 = (size_t)(fr * 256 + lr) * ld + fc * 256 + lc;
+    float acc[8][4];
+    const int gr = a * 256 + lr, gc = b * 256 + lc;
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc[q][k] = (gr == gc + k && gr < K) ? ((const float*)cf)[q] : 0.0f;
+#pragma unroll 2
+    for (int r = 1; r < s; ++r) {
+        const float4 x = pair4<BF>((const uint16_t*)T.p[r] + e0, plane);
+        const float4 c0 = cf[r][0], c1 = cf[r][1];
+        const float w[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            acc[q][0] = fmaf(w[q], x.x, acc[q][0]);
+            acc[q][1] = fmaf(w[q], x.y, acc[q][1]);
+            acc[q][2] = fmaf(w[q], x.z, acc[q][2]);
+            acc[q][3] = fmaf(w[q], x.w, acc[q][3]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        if (q >= n) break;
+        uint32_t h[4], l[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float x = acc[q][k];
+            if (f32) {
+                h[k] = __float_as_uint(x) >> 16;
+                l[k] = __float_as_uint(x) & 0xffffu;
+            } else {
+                const H th = H16<BF>::from_f(x * SC);
+                h[k] = bits16(th);
+                l[k] = bits16(H16<BF>::from_f(x * SC - H16<BF>::to_f(th)));
+            }
+        }
+        uint16_t* o = (uint16_t*)out.p[qb + q] + e0;
+        *(uint2*)o = make_uint2(h[0] | (h[1] << 16), h[2] | (h[3] << 16));
+        *(uint2*)(o + plane) = make_uint2(l[0] | (l[1] << 16), l[2] | (l[3] << 16));
+    }
+}
+
+// partial Gram sums <G_q, T_r>: CTA blockIdx.x takes rows blockIdx.x,
+// + gridDim.x, ... of all blocks; off-diagonal blocks count twice.  64 x 64
+// pairs per CTA; per 64 columns of a row FP32 FMA chains, then FP64.
+template <bool BF>
+__global__ void __launch_bounds__(256) k_pst_gram(int K, int nb, PstList G, int nq, PstList T, int s,
+                                                  double* __restrict__ part) {
+    __shared__ __align__(16) float g[64][68], t[64][68];
+    const int qb = blockIdx.y * 64, rb = blockIdx.z * 64;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const size_t ld = (size_t)nb * 256, plane = (size_t)(nb / 2 + 1) * 256 * ld;
+    double acc[4][4] = {};
+    const bool live = qb + 4 * ty < nq;
+    const int nblk = nb * (nb + 1) / 2;
+    for (int w = blockIdx.x; w < nblk * 256; w += gridDim.x) {
+        int a, b, fr, fc;
+        block_at(w >> 8, nb, a, b);
+        const int lr = w & 255;
+        if (a * 256 + lr >= K) continue;
+        fold(a, b, nb, fr, fc);
+        const float wt = a == b ? 1.0f : 2.0f;
+        for (int x0 = 0; x0 < 256 && b * 256 + x0 < K; x0 += 64) {
+            const size_t e0 = (size_t)(fr * 256 + lr) * ld + fc * 256 + x0;
+            __syncthreads();
+            for (int e = threadIdx.x; e < 64 * 16; e += 256) {
+                const int m = e >> 4, c = (e & 15) * 4, gc = b * 256 + x0 + c;
+                float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
+                if (qb + m < nq) x = pair4<BF>((const uint16_t*)G.p[qb + m] + e0 + c, plane);
+                if (rb + m < s && rb + m > 0) y = pair4<BF>((const uint16_t*)T.p[rb + m] + e0 + c, plane);
+                g[c][m] = gc < K ? wt * x.x : 0.f;
+                g[c + 1][m] = gc + 1 < K ? wt * x.y : 0.f;
+                g[c + 2][m] = gc + 2 < K ? wt * x.z : 0.f;
+                g[c + 3][m] = gc + 3 < K ? wt * x.w : 0.f;
+                t[c][m] = gc < K ? y.x : 0.f;
+                t[c + 1][m] = gc + 1 < K ? y.y : 0.f;
+                t[c + 2][m] = gc + 2 < K ? y.z : 0.f;
+                t[c + 3][m] = gc + 3 < K ? y.w : 0.f;
+            }
+            __syncthreads();
+            if (!live) continue;
+            float f[4][4] = {};
+#pragma unroll 8
+            for (int c = 0; c < 64; ++c) {
+                const float4 x = *(const float4*)&g[c][4 * ty], y = *(const float4*)&t[c][4 * tx];
+                const float xa[4] = {x.x, x.y, x.z, x.w}, ya[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) f[i][j] = fmaf(xa[i], ya[j], f[i][j]);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] += (double)f[i][j];
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int q = qb + 4 * ty + i, r = rb + 4 * tx + j;
+            if (q < nq && r < s) part[((long long)blockIdx.x * nq + q) * s + r] = acc[i][j];
+        }
+}
+
+// out[y * stride] = Tr of matrix y of the list
+template <bool BF>
+__global__ void __launch_bounds__(128) k_pst_trace(int K, int nb, PstList L, double* __restrict__ out, int stride) {
+    using H = typename H16<BF>::T;
+    __shared__ double red[4];
+    const size_t ld = (size_t)nb * 256, plane = (size_t)(nb / 2 + 1) * 256 * ld;
+    const uint16_t* X = (const uint16_t*)L.p[blockIdx.x];
+    double x = 0.0;
+    for (int i = threadIdx.x; i < K; i += 128) {
+        int fr, fc;
+        fold(i >> 8, i >> 8, nb, fr, fc);
+        const size_t e = (size_t)(fr * 256 + (i & 255)) * ld + fc * 256 + (i & 255);
+        x += (double)H16<BF>::to_f(from_bits16<H>(X[e])) + (double)H16<BF>::to_f(from_bits16<H>(X[e + plane]));
+    }
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
+    __syncthreads();
+    if (threadIdx.x == 0) out[(long long)blockIdx.x * stride] = (double)ISC * (red[0] + red[1] + red[2] + red[3]);
+}
+
+// rho (K x K, FP64, both triangles) = [C_0 or rho] + sum of np FP32 partial
+// products - b2: C_0 = sum_r c_0r T_r in FP32 FMA chains of 8 terms added in FP64
+template <bool BF>
+__global__ void __launch_bounds__(256) k_pst_finish(int K, int nb, int s, PstList T, const double* __restrict__ c,
+                                                    PstOut part, int np, const uint16_t* b2, int first,
+                                                    double* __restrict__ rho) {
+    using H = typename H16<BF>::T;
+    __shared__ double sh[32][33];
+    __shared__ float cf[PS_MAX_S];
+    const int nt = (K + 31) / 32;
+    int ti, tj;
+    block_at(blockIdx.x, nt, ti, tj);
+    for (int r = threadIdx.x; r < s; r += 256) cf[r] = (float)c[r];
+    __syncthreads();
+    int fr, fc;
+    fold(ti >> 3, tj >> 3, nb, fr, fc);
+    const size_t ld = (size_t)nb * 256, plane = (size_t)(nb / 2 + 1) * 256 * ld;
+    const int lc = threadIdx.x & 31;
+    auto pr = [](const uint16_t* p, size_t pl) {
+        return ISC * (H16<BF>::to_f(from_bits16<H>(*p)) + H16<BF>::to_f(from_bits16<H>(p[pl])));
+    };
+    for (int lr = threadIdx.x >> 5; lr < 32; lr += 8) {
+        const int gr = ti * 32 + lr, gc = tj * 32 + lc;
+        double x = 0.0;
+        if (gr < K && gc < K) {
+            const size_t e = (size_t)(fr * 256 + (gr & 255)) * ld + fc * 256 + (gc & 255);
+            if (first) {
+                if (gr == gc) x = c[0];
+                for (int r0 = 1; r0 < s; r0 += 8) {
+                    float f = 0.0f;
+                    for (int r = r0; r < min(s, r0 + 8); ++r) f = fmaf(cf[r], pr((const uint16_t*)T.p[r] + e, plane), f);
+                    x += (double)f;
+                }
+            } else {
+                x = rho[(long long)gr * K + gc];
+            }
+            for (int p = 0; p < np; ++p) {
+                const uint16_t* q = (const uint16_t*)part.p[p] + e;
+                x += (double)__uint_as_float(((uint32_t)q[0] << 16) | q[plane]);
+            }
+            if (b2) x -= (double)pr(b2 + e, plane);
+            if (gc >= gr) rho[(long long)gr * K + gc] = x;
+        }
+        sh[lc][lr] = x;
+    }
+    __syncthreads();
+    for (int lr = threadIdx.x >> 5; lr < 32; lr += 8) {
+        const int gr = tj * 32 + lr, gc = ti * 32 + lc;
+        if (gr < K && gc < K && gr > gc) rho[(long long)gr * K + gc] = sh[lr][lc];
+    }
+}
+
+__global__ void k_pst_gram_sum(int nsplit, int n, const double* __restrict__ part, double* __restrict__ D) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= n) return;
+    double x = 0.0;
+    for (int p = 0; p < nsplit; ++p) x += part[(long long)p * n + e];
+    D[e] = x;
+}
+
+int row_tiles(int K) { return (K + BM - 1) / BM; }
+int sys_tiles(const Ctx& c) {
+    const int nb = c.Kp / 256, mt = row_tiles(c.K);
+    int n = 0;
+    for (int p = 0; p < nb; ++p) n += (nb - p) * std::max(0, std::min(2, mt - 2 * p));
+    return n;
+}
+
+double growth_limit(int l, int n_c) {
+    if (l >= n_c - 1 || n_c < 3) return 4.0;
+    return std::cosh(std::acosh(4.0) * (double)l / (n_c - 1));
+}
+
+// One call's product launches: items are queued level by level (all systems
+// of the batch together) and uploaded once per flush.
+struct Queue {
+    Ctx& lead;
+    cudaStream_t st;
+    bool bf;
+    std::vector<PstItem> items;
+    std::vector<int2> pairs;
+    struct Launch { int first, n, tiles; };
+    std::vector<Launch> launches;
+    int open = 0;
+
+    Queue(Ctx& l, cudaStream_t s) : lead(l), st(s), bf(l.p.precision == DFT_PREC_BF16X3) {}
+    void add(int sys, const Ctx& c, std::initializer_list<int2> ab, int prev, int add_, int out, int mode, double limit) {
+        PstItem it{};
+        it.sys = sys;
+        it.first = (int)pairs.size();
+        for (const int2& x : ab) pairs.push_back(x);
+        finish_item(it, c, prev, add_, out, mode, limit);
+    }
+    void finish_item(PstItem& it, const Ctx& c, int prev, int add_, int out, int mode, double limit) {
+        it.last = (int)pairs.size();
+        it.prev = prev;
+        it.add = add_;
+        it.out = out;
+        it.mode = mode;
+        it.limit = (float)limit;
+        if (launches.empty() || !open) {
+            launches.push_back({(int)items.size(), 0, 0});
+            open = 1;
+        }
+        it.tile0 = launches.back().tiles;
+        launches.back().tiles += sys_tiles(c);
+        launches.back().n++;
+        items.push_back(it);
+    }
+    void close() { open = 0; }   // the next item starts a new launch
+    void upload() {
+        if (items.empty()) return;
+        if ((long long)items.size() > PST_ITEM_CAP || (long long)pairs.size() > PST_ITEM_CAP)
+            throw Error(DFT_EINTERNAL, "expansion items exceed their buffer");
+        DFT_CUDA_CHECK(cudaMemcpyAsync(lead.d_pst_items, items.data(), sizeof(PstItem) * items.size(),
+                                       cudaMemcpyHostToDevice, st));
+        DFT_CUDA_CHECK(cudaMemcpyAsync(lead.d_pst_pairs, pairs.data(), sizeof(int2) * pairs.size(),
+                                       cudaMemcpyHostToDevice, st));
+    }
+    void launch(size_t k) {
+        const Launch& l = launches[k];
+        const int grid = std::min(l.tiles, SMS);
+        if (bf) k_pst_prod<true><<<grid, NTHREADS, SMEM_BYTES, st>>>(lead.d_pst_sys, lead.d_pst_items + l.first, l.n, lead.d_pst_pairs, l.tiles);
+        else k_pst_prod<false><<<grid, NTHREADS, SMEM_BYTES, st>>>(lead.d_pst_sys, lead.d_pst_items + l.first, l.n, lead.d_pst_pairs, l.tiles);
+        check_launch("pst_prod");
+    }
+    void run() {
+        upload();
+        for (size_t k = 0; k < launches.size(); ++k) launch(k);
+        items.clear();
+        pairs.clear();
+        launches.clear();
+        open = 0;
+    }
+};
+
+// slots of one system: babies T_1 .. T_s at 0 .. s - 1; direct plan: giants
+// G_2 .. G_Q at s .. s + Q - 2, then C_q and partial sums; Clenshaw plan: two
+// rolling buffers, then C_q (and giants on their way to the Gram sums)
+struct View {
+    Ctx& c;
+    const PsPlan& p;
+    explicit View(Ctx& x) : c(x), p(x.ps) {}
+    int baby(int r) const { return r - 1; }
+    int giant(int q) const { return q == 1 ? p.s - 1 : p.s + q - 2; }
+    int extra(int i) const { return p.s + (p.direct ? std::max(0, p.Q - 1) : 0) + i; }
+    int nextra() const { return (int)c.pst_slot.size() - extra(0); }
+    PstList babies() const {
+        PstList T{};
+        for (int r = 1; r < p.s; ++r) T.p[r] = c.pst_slot[baby(r)];
+        return T;
+    }
+};
+
+template <class A, class B>
+void pick(bool bf, A&& a, B&& b) {
+    if (bf) a();
+    else b();
+}
+
+void gram(Ctx& c, int q0, const std::vector<int>& slots, cudaStream_t st) {
+    const View v(c);
+    const int s = v.p.s, nb = c.Kp / 256;
+    const bool bf = c.p.precision == DFT_PREC_BF16X3;
+    double* D = c.d_wk;
+    const PstList T = v.babies();
+    for (size_t k = 0; k < slots.size(); k += PS_MAX_S) {
+        const int nq = (int)std::min<size_t>(PS_MAX_S, slots.size() - k);
+        PstList G{};
+        for (int q = 0; q < nq; ++q) G.p[q] = c.pst_slot[slots[k + q]];
+        if ((long long)nq * s > c.gram_cap) throw Error(DFT_EINTERNAL, "Gram partials exceed their buffer");
+        const int tiles = ((nq + 63) / 64) * ((s + 63) / 64);
+        const int nsplit = (int)std::max<long long>(
+            1, std::min<long long>({(long long)nb * (nb + 1) / 2 * 256, 4LL * SMS / tiles, c.gram_cap / ((long long)nq * s)}));
+        const dim3 grid(nsplit, (nq + 63) / 64, (s + 63) / 64);
+        double* Dq = D + (long long)(q0 + k) * s;
+        if (s > 1) {
+            pick(bf, [&] { k_pst_gram<true><<<grid, 256, 0, st>>>(c.K, nb, G, nq, T, s, c.d_gram); },
+                 [&] { k_pst_gram<false><<<grid, 256, 0, st>>>(c.K, nb, G, nq, T, s, c.d_gram); });
+            k_pst_gram_sum<<<(nq * s + 255) / 256, 256, 0, st>>>(nsplit, nq * s, c.d_gram, Dq);
+        }
+        pick(bf, [&] { k_pst_trace<true><<<nq, 128, 0, st>>>(c.K, nb, G, Dq, s); },
+             [&] { k_pst_trace<false><<<nq, 128, 0, st>>>(c.K, nb, G, Dq, s); });
+        check_launch("pst_gram", 3);
+    }
+}
+
+void combine(Ctx& c, const double* cf, int q0, int nq, const std::vector<int>& out, bool f32, cudaStream_t st) {
+    const View v(c);
+    const int nb = c.Kp / 256;
+    PstOut o{};
+    for (int q = 0; q < nq; ++q) o.p[q] = c.pst_slot[out[q]];
+    const PstList T = v.babies();
+    const dim3 grid(nb * (nb + 1) / 2, 64, (nq + 7) / 8);
+    pick(c.p.precision == DFT_PREC_BF16X3,
+         [&] { k_pst_combine<true><<<grid, 256, 0, st>>>(c.K, nb, v.p.s, T, o, q0, nq, cf, f32 ? 1 : 0); },
+         [&] { k_pst_combine<false><<<grid, 256, 0, st>>>(c.K, nb, v.p.s, T, o, q0, nq, cf, f32 ? 1 : 0); });
+    check_launch("pst_combine");
+}
+
+void finish(Ctx& c, const double* cf, const std::vector<int>& part, int b2, bool first, cudaStream_t st) {
+    const View v(c);
+    const int nt = (c.K + 31) / 32;
+    PstOut o{};
+    for (size_t q = 0; q < part.size(); ++q) o.p[q] = c.pst_slot[part[q]];
+    const PstList T = v.babies();
+    const uint16_t* b = b2 >= 0 ? (const uint16_t*)c.pst_slot[b2] : nullptr;
+    const int np = (int)part.size();
+    pick(c.p.precision == DFT_PREC_BF16X3,
+         [&] { k_pst_finish<true><<<nt * (nt + 1) / 2, 256, 0, st>>>(c.K, c.Kp / 256, v.p.s, T, cf, o, np, b, first, c.d_rho); },
+         [&] { k_pst_finish<false><<<nt * (nt + 1) / 2, 256, 0, st>>>(c.K, c.Kp / 256, v.p.s, T, cf, o, np, b, first, c.d_rho); });
+    check_launch("pst_finish");
+}
+
+double* coef_ps(Ctx& c) { return c.d_coef + c.n_c_cur; }
+
+}  // namespace
+
+size_t pst_slot_bytes(int Kp) {
+    const size_t nb = Kp / 256;
+    return (nb / 2 + 1) * 256 * (size_t)Kp * 4;
+}
+
+// tensor maps of every slot (K-major boxes of 128 and 256 rows, transposed
+// boxes of 128 and 256 columns; both planes are rows of one map) and the slot
+// table, uploaded once
+void pst_setup(Ctx& c, cudaStream_t st) {
+    const int n = (int)c.pst_slot.size(), nb = c.Kp / 256;
+    std::vector<CUtensorMap> maps(4 * (size_t)n);
+    const cuuint64_t rows = (cuuint64_t)(nb / 2 + 1) * 256 * 2, ld = (cuuint64_t)c.Kp;
+    for (int k = 0; k < n; ++k) {
+        for (int v = 0; v < 2; ++v) {
+            cuuint64_t dims[2] = {ld, rows}, strides[1] = {ld * 2};
+            cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)(v ? BN : BM)}, es[2] = {1, 1};
+            CUresult r = encode_fn()(&maps[4 * k + v], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, c.pst_slot[k], dims, strides,
+                                     box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+                                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+            if (r != CUDA_SUCCESS) throw Error(DFT_ECUDA, "cuTensorMapEncodeTiled (slot) failed");
+        }
+        for (int v = 0; v < 2; ++v) {
+            cuuint64_t dims[3] = {64, rows, ld / 64}, strides[2] = {ld * 2, 128};
+            cuuint32_t box[3] = {64, (cuuint32_t)BK, (cuuint32_t)((v ? BN : BM) / 64)}, es[3] = {1, 1, 1};
+            CUresult r = encode_fn()(&maps[4 * k + 2 + v], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, c.pst_slot[k], dims,
+                                     strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+            if (r != CUDA_SUCCESS) throw Error(DFT_ECUDA, "cuTensorMapEncodeTiled (transposed slot) failed");
+        }
+    }
+    DFT_CUDA_CHECK(cudaMemcpyAsync(c.d_pst_maps, maps.data(), sizeof(CUtensorMap) * maps.size(), cudaMemcpyHostToDevice, st));
+    DFT_CUDA_CHECK(cudaMemcpyAsync(c.d_pst_slots, c.pst_slot.data(), sizeof(void*) * n, cudaMemcpyHostToDevice, st));
+    DFT_CUDA_CHECK(cudaStreamSynchronize(st));   // the host staging goes out of scope
+    DFT_CUDA_CHECK(cudaFuncSetAttribute(k_pst_prod<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
+    DFT_CUDA_CHECK(cudaFuncSetAttribute(k_pst_prod<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
+}
+
+// T_1 = H_N (from c.d_H, which is free afterwards)
+void pst_split_h(Ctx& c, cudaStream_t st) {
+    const int nb = c.Kp / 256;
+    const dim3 grid(nb * (nb + 1) / 2, 16);
+    uint16_t* t1 = (uint16_t*)c.pst_slot[0];
+    pick(c.p.precision == DFT_PREC_BF16X3, [&] { k_pst_split<true><<<grid, 256, 0, st>>>(c.K, nb, c.d_H, t1); },
+         [&] { k_pst_split<false><<<grid, 256, 0, st>>>(c.K, nb, c.d_H, t1); });
+    check_launch("pst_split");
+}
+
+// Babies, giants and moments of every system (T_1 in place).  moments[q] = 0:
+// the coefficients of system q are already fixed, so only the spectrum check
+// is left of the moments' giants.
+void pst_pass1(Ctx* const* cs, int n, const int* moments, cudaStream_t st) {
+    Ctx& lead = *cs[0];
+    std::vector<PstSys> tab(n);
+    for (int k = 0; k < n; ++k) {
+        Ctx& c = *cs[k];
+        const int nslot = (int)c.pst_slot.size();
+        // T_1 takes a slot here; one product's tiles below two waves: direct
+        c.ps = ps_plan(c.n_c_cur, nslot - 1, sys_tiles(c) < 2 * SMS, 6);
+        tab[k] = PstSys{c.K, c.Kp / 256, c.d_pst_maps, c.d_pst_slots, c.d_flags};
+    }
+    DFT_CUDA_CHECK(cudaMemcpyAsync(lead.d_pst_sys, tab.data(), sizeof(PstSys) * n, cudaMemcpyHostToDevice, st));
+    Queue Q(lead, st);
+    // doubling of every system's X_1 .. X_top, level by level together
+    auto doubling = [&](auto&& top_of, auto&& slot_of, auto&& limit_of) {
+        for (int m = 1;; m *= 2) {
+            bool any = false;
+            for (int k = 0; k < n; ++k) {
+                const int top = top_of(k);
+                for (int j = 1; j <= std::min(m, top - m); ++j) {
+                    Q.add(k, *cs[k], {make_int2(slot_of(k, m), slot_of(k, j))}, m > j ? slot_of(k, m - j) : -1, -1,
+                          slot_of(k, m + j), PST_ALPHA2 | (m == j ? PST_IDENT : 0), limit_of(k, m + j));
+                    any = true;
+                }
+            }
+            Q.close();
+            if (!any) break;
+        }
+    };
+    doubling([&](int k) { const PsPlan& p = cs[k]->ps; return p.Q > 0 ? p.s : p.s - 1; },
+             [&](int k, int r) { return View(*cs[k]).baby(r); }, [&](int, int) { return 4.0; });
+    doubling([&](int k) { const PsPlan& p = cs[k]->ps; return p.direct ? p.Q : 0; },
+             [&](int k, int q) { return View(*cs[k]).giant(q); },
+             [&](int k, int q) { const PsPlan& p = cs[k]->ps; return q == p.Q ? growth_limit(p.Q * p.s, p.n_c) : 4.0; });
+    Q.run();
+    for (int k = 0; k < n; ++k) {
+        Ctx& c = *cs[k];
+        const PsPlan& p = c.ps;
+        const View v(c);
+        const int s = p.s, nb = c.Kp / 256;
+        const bool bf = c.p.precision == DFT_PREC_BF16X3;
+        if (moments[k] && s > 1) {
+            PstList L{};
+            for (int r = 1; r < s; ++r) L.p[r - 1] = c.pst_slot[v.baby(r)];
+            pick(bf, [&] { k_pst_trace<true><<<s - 1, 128, 0, st>>>(c.K, nb, L, c.d_wk + 1, 1); },
+                 [&] { k_pst_trace<false><<<s - 1, 128, 0, st>>>(c.K, nb, L, c.d_wk + 1, 1); });
+            check_launch("pst_trace");
+        }
+        if (p.direct && moments[k] && p.Q > 0) {
+            std::vector<int> g;
+            for (int q = 1; q <= p.Q; ++q) g.push_back(v.giant(q));
+            gram(c, 1, g, st);
+        }
+        if (!p.direct && p.Q > 1) {
+            const int r0 = v.extra(0), nring = v.nextra(), ts = v.baby(s);
+            if (moments[k]) {
+                // giants G_2 .. G_Q in a ring of nring buffers; the Gram sums take up
+                // to nring - 2 at a time, so that the babies are read less often
+                std::vector<int> at(p.Q + 1, ts);
+                for (int q = 2; q <= p.Q; ++q) at[q] = r0 + (q - 2) % nring;
+                for (int q = 1; q < p.Q; ++q) {
+                    Q.add(k, c, {make_int2(ts, at[q])}, q > 1 ? at[q - 1] : -1, -1, at[q + 1],
+                          PST_ALPHA2 | (q == 1 ? PST_IDENT : 0), q + 1 == p.Q ? growth_limit(p.Q * s, p.n_c) : 4.0);
+                    Q.close();
+                }
+                Q.upload();
+                int done = 1;   // giants 1 .. done - 1 are in the Gram sums
+                for (int q = 1; q <= p.Q; ++q) {
+                    const int have = q - done + 1;
+                    if (q == p.Q || have >= std::max(1, nring - 2)) {
+                        gram(c, done, std::vector<int>(at.begin() + done, at.begin() + q + 1), st);
+                        done = q + 1;
+                    }
+                    if (q < p.Q) Q.launch(q - 1);
+                }
+                Q.items.clear();
+                Q.pairs.clear();
+                Q.launches.clear();
+                Q.open = 0;
+            } else {
+                // T_{2^i s} up to the order of the expansion: the spectrum check
+                int cur = ts, l = s;
+                for (int i = 0; 2 * l <= p.n_c - 1; ++i) {
+                    Q.add(k, c, {make_int2(cur, cur)}, -1, -1, r0 + (i & 1), PST_ALPHA2 | PST_IDENT,
+                          growth_limit(2 * l, p.n_c));
+                    Q.close();
+                    cur = r0 + (i & 1);
+                    l *= 2;
+                }
+                Q.run();
+            }
+        }
+        if (moments[k]) launch_ps_moments(c.K, p, c.d_wk, c.d_mom, st);
+    }
+}
+
+// rho = sum_l a_l T_l of every system (coefficients in its d_coef) into d_rho
+void pst_pass2(Ctx* const* cs, int n, cudaStream_t st) {
+    Ctx& lead = *cs[0];
+    Queue Q(lead, st);
+    for (int k = 0; k < n; ++k) {
+        Ctx& c = *cs[k];
+        launch_ps_coefs(c.ps, c.d_coef, coef_ps(c), coef_ps(c) + (long long)(c.ps.Q + 1) * c.ps.s, st);
+    }
+    // direct plans: chunks of giants, all systems' products of a chunk together
+    std::vector<int> at(n, 1);
+    for (bool any = true; any;) {
+        any = false;
+        std::vector<std::vector<int>> part(n);
+        int total = 0;
+        for (int k = 0; k < n; ++k)
+            if (cs[k]->ps.direct) total += sys_tiles(*cs[k]);
+        for (int k = 0; k < n; ++k) {
+            Ctx& c = *cs[k];
+            const PsPlan& p = c.ps;
+            const View v(c);
+            if (!p.direct || at[k] > p.Q) continue;
+            any = true;
+            const int left = p.Q - at[k] + 1, spare = v.nextra();
+            // about four waves of tiles over the batch; fewer giants per FP32 sum also
+            // mean less rounding
+            const int want = std::max(1, std::min(left, 4 * SMS / std::max(1, total) + 1));
+            const int np = std::max(1, std::min({want, spare / 2, PS_MAX_ITEMS}));
+            const int nq = std::min({left, spare - np, PS_MAX_ITEMS});
+            std::vector<int> cq;
+            for (int q = 0; q < nq; ++q) cq.push_back(v.extra(q));
+            combine(c, coef_ps(c), at[k], nq, cq, false, st);
+            const int npu = std::min(np, nq);
+            for (int y = 0; y < npu; ++y) {
+                PstItem it{};
+                it.sys = k;
+                it.first = (int)Q.pairs.size();
+                for (int q = (int)((long long)nq * y / npu); q < (int)((long long)nq * (y + 1) / npu); ++q)
+                    Q.pairs.push_back(make_int2(v.giant(at[k] + q), cq[q]));
+                part[k].push_back(v.extra(nq + y));
+                Q.finish_item(it, c, -1, -1, part[k].back(), PST_OUT_F32, 0.0);
+            }
+        }
+        if (!any) break;
+        Q.run();
+        for (int k = 0; k < n; ++k) {
+            Ctx& c = *cs[k];
+            if (part[k].empty()) continue;
+            const bool first = at[k] == 1;
+            const int left = c.ps.Q - at[k] + 1, spare = View(c).nextra();
+            const int want = std::max(1, std::min(left, 4 * SMS / std::max(1, total) + 1));
+            const int np = std::max(1, std::min({want, spare / 2, PS_MAX_ITEMS}));
+            at[k] += std::min({left, spare - np, PS_MAX_ITEMS});
+            finish(c, coef_ps(c), part[k], -1, first, st);
+        }
+    }
+    for (int k = 0; k < n; ++k) {
+        Ctx& c = *cs[k];
+        const PsPlan& p = c.ps;
+        const View v(c);
+        if (p.Q == 0) {
+            finish(c, coef_ps(c), {}, -1, true, st);
+            continue;
+        }
+        if (p.direct) continue;
+        // Clenshaw in T_s: b_q = C_q + 2 T_s b_{q+1} - b_{q+2}, C_q formed W at a time
+        const int W = std::min(8, v.nextra() - 2), ts = v.baby(p.s);
+        int b1 = v.extra(0), b2 = v.extra(1);
+        combine(c, coef_ps(c), p.Q, 1, {b1}, false, st);
+        std::vector<int> add_at(p.Q + 1);
+        bool have2 = false;
+        for (int q = p.Q - 1; q >= 1; --q) {
+            add_at[q] = v.extra(2 + (p.Q - 1 - q) % W);
+            Q.add(k, c, {make_int2(ts, b1)}, have2 ? b2 : -1, add_at[q], b2, PST_ALPHA2, 0.0);
+            Q.close();
+            std::swap(b1, b2);
+            have2 = true;
+        }
+        const int tail = v.extra(2);
+        Q.add(k, c, {make_int2(ts, b1)}, -1, -1, tail, PST_OUT_F32, 0.0);
+        Q.upload();
+        int l = 0;
+        for (int q = p.Q - 1; q >= 1; --q, ++l) {
+            if ((p.Q - 1 - q) % W == 0) {
+                // C_{q - m + 1} .. C_q, lowest first
+                const int m = std::min(W, q);
+                std::vector<int> o;
+                for (int i = 0; i < m; ++i) o.push_back(add_at[q - m + 1 + i]);
+                combine(c, coef_ps(c), q - m + 1, m, o, true, st);
+            }
+            Q.launch(l);
+        }
+        Q.launch(l);
+        finish(c, coef_ps(c), {tail}, have2 ? b2 : -1, true, st);
+        Q.items.clear();
+        Q.pairs.clear();
+        Q.launches.clear();
+        Q.open = 0;
+    }
+}
+
+}  // namespace dft

@@ -27,4 +27,13 @@ struct Ps64Items {
     int ident[PS_MAX_ITEMS];
 };
 
+
+// ---- split 16-bit path (k_poly_tc.cu) ----
+struct PstList {
+    const void* p[PS_MAX_S];
+};
+struct PstOut {
+    void* p[PS_MAX_ITEMS];
+};
+
 }  // namespace dft

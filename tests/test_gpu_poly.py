@@ -45,3 +45,26 @@ def test_fp64_expansion_matches_the_oracle_at_every_grouping(name, orders):
         # the requirement of the FP64 path; rounding errors grow with the order
         assert err < 1e-9 * max(1.0, np.max(np.abs(ref["P"])))
         assert abs(info.n_e_trace - s.n_electrons) < 1e-8 * s.n_electrons
+
+
+@pytest.mark.parametrize("name,orders", [("tiny8", (2, 3, 5, 40, 700, 6000)), ("tiny37", (2, 33, 1500, 7000)),
+                                         ("cluster64", (1400,))])
+def test_split_expansion_matches_the_oracle_at_every_grouping(name, orders):
+    """One, two and three 256-blocks per side (operands read in place and
+    transposed, folded block rows, ragged last blocks), direct and Clenshaw
+    plans; the gate of the mixed path's density matrices, 1e-4 of max|P|."""
+    s, F, S, lo, hi = problem(name)
+    Fd = torch.from_numpy(F).cuda()
+    for n_c in orders:
+        beta = n_c / (2.0 * (hi - lo))
+        ref = dm.dm_cheb(F, S, s.n_electrons, beta, lo, hi, n_c, m_nodes=4 * n_c)
+        ctx = dft.Context(s, e_min=lo, e_max=hi, cheb_order=n_c, kT=1.0 / beta, precision=dft.DFT_PREC_FP16X3,
+                          skip_correction=1)
+        ctx.overlap_kinetic()
+        P, info = ctx.density_matrix(Fd)
+        ctx.close()
+        err = float(np.max(np.abs(P.cpu().numpy() - ref["P"]))) / np.max(np.abs(ref["P"]))
+        print(f"{name} split N_C {n_c}: max|dP| / max|P| {err:.2e}, N_e {info.n_e_trace:.6f}, dmu {info.mu - ref['mu']:.1e}")
+        assert info.spectrum_ok == 1
+        assert err < 1e-4
+        assert abs(info.n_e_trace - s.n_electrons) < 1e-4 * s.n_electrons
