@@ -4,16 +4,18 @@
 // on tcgen05 with FP32 accumulation, for one or many systems per launch.
 //
 // Storage.  Every matrix is symmetric, so a buffer ("slot") keeps the 256 x
-// 256 blocks (a, b), a <= b, only (diagonal blocks whole), folded into a
-// rectangle of R = nb / 2 + 1 block rows (nb = Kp / 256 blocks per side): block row a
-// < R lies in place, block row a >= R, which has nb - a blocks, fills the
-// free left end of block row nb - a.  Half the bytes of full storage: twice
-// as many babies fit the workspace, more operand tiles stay in L2, and no
-// mirror is written.  A slot holds the hi plane and then the lo plane; the same two planes
-// can hold FP32 values as their upper and lower 16 bits.  An
-// operand tile whose k block lies left of the diagonal is read transposed:
-// as rows of k (MN-major operand, 128-byte swizzle, one 3-D TMA box), the
-// others K-major (64-byte swizzle).
+// 256 blocks (a, b), a <= b, only (diagonal blocks whole), each transposed
+// (rows of b, columns of a), folded into a rectangle of R = nb / 2 + 1 block
+// rows (nb = Kp / 256 blocks per side): block row a < R lies in place, block
+// row a >= R, which has nb - a blocks, fills the free left end of block row
+// nb - a.  Half the bytes of full storage: twice as many babies fit the
+// workspace, more operand tiles stay in L2, and no mirror is written.  A slot
+// holds the hi plane and then the lo plane; the same two planes can hold FP32
+// values as their upper and lower 16 bits.  An operand tile whose k block lies
+// on or right of the diagonal is read as rows of k (MN-major operand, 128-byte
+// swizzle, one 3-D TMA box), the others K-major (64-byte swizzle); both run
+// at the same speed.  The transposition makes a warp's 32 rows of one output
+// column contiguous, so the epilogue needs no staging.
 //
 // Kernel k_pst_prod: persistent, one CTA per SM, one 128 x 256 output tile
 // at a time: warp 0 lane 0 drives the TMA loads of the four operand tiles of
@@ -22,10 +24,12 @@
 // each finished unit of SUB k-blocks from one of two accumulators into FP32
 // registers (round to nearest; the tensor core's own FP32 accumulation leans
 // towards zero with every addition, so its chains are kept short) and then
-// write x = alpha A B - prev + add straight from registers: a thread's 16 columns are
-// one 32-byte sector per plane, so no staging is needed, the ring stays with the
-// producer and the next tile's loads and first two units run under the
-// epilogue.  Every wait is bounded; on expiry the CTA sets FLAG_TIMEOUT,
+// write x = alpha A B - prev + add straight from registers: neighbouring lanes
+// swap one of two columns, so that a lane moves two rows of one column per
+// 32-bit access and a warp whole sectors (with one row per lane and 16-byte
+// accesses along the row the epilogue took 60 of 100 us per tile at K =
+// 2000).  The ring stays with the producer, and the next tile's loads and
+// first two units run under the epilogue.  Every wait is bounded; on expiry the CTA sets FLAG_TIMEOUT,
 // drains what it issued and returns.
 //
 // Density matrix at K = 1230, tail 1e-5 (N_C ~ 1410, direct plan): 118.9 ms
@@ -44,11 +48,23 @@ namespace {
 using namespace tc;
 
 constexpr int BM = 128, BN = 256, BK = 32, STAGES = 4;
-constexpr int SUB = 2;   // k-blocks per accumulator promotion: chains of 12 additions
+// k-blocks per accumulator promotion: chains of 24 additions.  Promoting every
+// 2 costs 0.4 us per promotion (16 products at K = 2000: 440 against 389 us)
+// for an error of P of 2.5e-5 instead of 2.7e-5 (K = 1230)
+constexpr int SUB = 4;
 constexpr int A_BYTES = BM * BK * 2, B_BYTES = BN * BK * 2;
 constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;
-constexpr int NEPI = 256, NTHREADS = 64 + NEPI, CPT = 128;
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
+// warps 0 .. 3: producer, MMA issuer and two idle ones, so that the eight
+// epilogue warps are whole warpgroups and can take the registers these do not
+// need (384 x 168 at launch = 128 x 40 + 256 x 232)
+constexpr int NEPI = 256, NTHREADS = 128 + NEPI, CPT = 128;
+// behind the ring: barriers, the launch's item table (the first ITEM_SMEM
+// items; reading it from global memory at each tile cost 4 us per tile) and
+// one 16 x 32 transposition buffer per epilogue warp
+constexpr int ITEM_SMEM = 384;
+constexpr int TR_WORDS = 16 * 33;
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256 + ITEM_SMEM * (int)sizeof(PstItem) + 8 * TR_WORDS * 4;
+static_assert(SMEM_BYTES <= 232448, "shared memory of one CTA");
 constexpr int TMEM_COLS = 2 * BN;
 constexpr int SMS = 152;
 // pairs hold x * SC: the low half of an FP16 pair of x itself would be a
@@ -100,8 +116,7 @@ struct Work {
     const PstSys* S;
     int i, j, p, nk;   // row tile, column block, row block, k-blocks per operand pair
 };
-__device__ __forceinline__ Work work_at(int t, const PstItem* __restrict__ items, int nitems,
-                                        const PstSys* __restrict__ sys) {
+__device__ __forceinline__ Work work_at(int t, const PstItem* items, int nitems, const PstSys* __restrict__ sys) {
     int a = 0, b = nitems;   // last item with tile0 <= t
     while (b - a > 1) {
         const int m = (a + b) >> 1;
@@ -119,7 +134,7 @@ __device__ __forceinline__ Work work_at(int t, const PstItem* __restrict__ items
 
 template <bool BF>
 __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restrict__ sys,
-                                                          const PstItem* __restrict__ items, int nitems,
+                                                          const PstItem* __restrict__ items_g, int nitems,
                                                           const int2* __restrict__ pairs, int ntiles) {
     using T = typename H16<BF>::T;
     extern __shared__ uint8_t smem_raw[];
@@ -132,8 +147,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
     uint32_t* tmem_slot = (uint32_t*)(drain + 1);
     volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
     static_assert((2 * STAGES + 5) * 8 + 8 <= 256, "barriers exceed their area");
+    PstItem* items_s = (PstItem*)(smem + STAGES * STAGE_BYTES + 256);
+    uint32_t* tr_all = (uint32_t*)(items_s + ITEM_SMEM);
+    const PstItem* items = nitems <= ITEM_SMEM ? items_s : items_g;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (nitems <= ITEM_SMEM)
+        for (int e = threadIdx.x; e < nitems * (int)(sizeof(PstItem) / 4); e += NTHREADS)
+            ((int*)items_s)[e] = ((const int*)items_g)[e];
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(&full[s], 1);
@@ -141,7 +162,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(&accfull[a], 1);
-            mbar_init(&accempty[a], NEPI);
+            mbar_init(&accempty[a], NEPI / 32);   // one arrival per warp: 256 arrivals took longer than a unit's MMAs
         }
         mbar_init(drain, 1);
         *abort_flag = 0;
@@ -164,6 +185,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
     auto sBh = [&](int s) { return smem + s * STAGE_BYTES + 2 * A_BYTES; };
     auto sBl = [&](int s) { return smem + s * STAGE_BYTES + 2 * A_BYTES + B_BYTES; };
 
+    if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
     if (warp == 0) {
         if (lane == 0) {
             long long g = 0;   // k-blocks issued by this CTA
@@ -185,7 +208,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
                             break;
                         }
                         mbar_expect_tx(&full[s], STAGE_BYTES);
-                        if (kq >= w.p) {
+                        if (kq < w.p) {
                             const int y = ar * 256 + (w.i & 1) * BM, x = ac * 256 + kx;
                             tma_load_2d(sAh(s), ma + 0, x, y, &full[s]);
                             tma_load_2d(sAl(s), ma + 0, x, y + lo_row, &full[s]);
@@ -194,7 +217,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
                             tma_load_3d(sAh(s), ma + 2, 0, y, z, &full[s]);
                             tma_load_3d(sAl(s), ma + 2, 0, y + lo_row, z, &full[s]);
                         }
-                        if (kq >= w.j) {
+                        if (kq < w.j) {
                             const int y = br * 256, x = bc * 256 + kx;
                             tma_load_2d(sBh(s), mb + 1, x, y, &full[s]);
                             tma_load_2d(sBl(s), mb + 1, x, y + lo_row, &full[s]);
@@ -240,7 +263,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
                         tc_fence_after();
                         const int kq = kb >> 3;
                         if (++kb == w.nk) kb = 0;
-                        const bool at = kq < w.p, bt = kq < w.j;   // operand read transposed
+                        const bool at = kq >= w.p, bt = kq >= w.j;   // MN-major operand
                         const uint32_t idesc = idesc0 | ((at ? 1u : 0u) << 15) | ((bt ? 1u : 0u) << 16);
                         const uint64_t ah = at ? smem_desc_mn(sAh(s)) : smem_desc<BK * 2>(sAh(s));
                         const uint64_t al = at ? smem_desc_mn(sAl(s)) : smem_desc<BK * 2>(sAl(s));
@@ -267,15 +290,47 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
             }
         }
         __syncwarp();
+    }
     } else {
-        const int quad = warp & 3, half = (warp - 2) >> 2;
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 232;");
+        const int quad = warp & 3, half = (warp - 4) >> 2;
         const int r_loc = 32 * quad + lane;
+        uint32_t* tr = tr_all + (warp - 4) * TR_WORDS;
         long long u = 0;
         bool ok = true;
         for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
             const Work w = work_at(t, items, nitems, sys);
             const PstSys& S = *w.S;
-            const int nunit = (w.nk * (w.it.last - w.it.first) + SUB - 1) / SUB;
+            const int nunit = (w.nk * (w.it.last - w.it.first) + SUB - 1) / SUB, K = S.K, nb = S.nb;
+            int fr, fc;
+            fold(w.p, w.j, nb, fr, fc);
+            const int ld = nb * 256;
+            const size_t plane = (size_t)(nb / 2 + 1) * 256 * ld;
+            // this lane's 32-bit words: rows r & ~1, r | 1 (stored columns) of output
+            // column c + (lane & 1) (stored row)
+            const bool odd = lane & 1;
+            const size_t e0 = (size_t)(fr * 256 + half * CPT + odd) * ld + fc * 256 + (w.i & 1) * BM + (r_loc & ~1);
+            const int r = w.i * BM + r_loc, c0 = w.j * BN + half * CPT;   // global row, first column
+            const bool diag = w.p == w.j, f32_out = (w.it.mode & PST_OUT_F32) != 0, ident = (w.it.mode & PST_IDENT) != 0 && r < K;
+            const float alpha = ((w.it.mode & PST_ALPHA2) ? 2.0f : 1.0f) * (ISC * ISC);
+            const uint16_t* pv = w.it.prev >= 0 ? (const uint16_t*)S.slot[w.it.prev] + e0 : nullptr;
+            const uint16_t* ad = w.it.add >= 0 ? (const uint16_t*)S.slot[w.it.add] + e0 : nullptr;
+            uint16_t* out = (uint16_t*)S.slot[w.it.out] + e0;
+            const float limit = w.it.limit;
+            bool bad = false;
+            constexpr int EB = 16;   // columns per batch, the next one's loads in flight
+            uint32_t nh[EB / 2], nl[EB / 2], mh[EB / 2], ml[EB / 2];
+            auto fetch = [&](int cb) {
+#pragma unroll
+                for (int k = 0; k < EB / 2; ++k) {
+                    const size_t o = (size_t)(cb + 2 * k) * ld;
+                    nh[k] = pv ? *(const uint32_t*)(pv + o) : 0u;
+                    nl[k] = pv ? *(const uint32_t*)(pv + plane + o) : 0u;
+                    mh[k] = ad ? *(const uint32_t*)(ad + o) : 0u;
+                    ml[k] = ad ? *(const uint32_t*)(ad + plane + o) : 0u;
+                }
+            };
+            fetch(0);   // arrives under the products
             float R[CPT];
 #pragma unroll
             for (int i = 0; i < CPT; ++i) R[i] = 0.0f;
@@ -287,91 +342,116 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
                 tc_fence_after();
                 tmem_add_groups<CPT / 16>(tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(a * BN + half * CPT), R);
                 tc_fence_before();
-                mbar_arrive(&accempty[a]);
+                __syncwarp();
+                if (lane == 0 && q + 1 < nunit) mbar_arrive(&accempty[a]);
             }
             if (!ok) {
                 *abort_flag = 1;
                 if (lane == 0) atomicExch(&S.flags[FLAG_TIMEOUT], 1);
                 break;
             }
-            int fr, fc;
-            fold(w.p, w.j, S.nb, fr, fc);
-            const int ld = S.nb * 256;
-            const size_t plane = (size_t)(S.nb / 2 + 1) * 256 * ld;
-            const size_t e0 = (size_t)(fr * 256 + (w.i & 1) * BM + r_loc) * ld + fc * 256 + half * CPT;
-            const int r = w.i * BM + r_loc, c0 = w.j * BN + half * CPT;   // global row, first column
-            const bool diag = w.p == w.j, f32_out = (w.it.mode & PST_OUT_F32) != 0;
-            const float alpha = ((w.it.mode & PST_ALPHA2) ? 2.0f : 1.0f) * (ISC * ISC);
-            const uint16_t* pv = w.it.prev >= 0 ? (const uint16_t*)S.slot[w.it.prev] + e0 : nullptr;
-            const uint16_t* ad = w.it.add >= 0 ? (const uint16_t*)S.slot[w.it.add] + e0 : nullptr;
-            uint16_t* out = (uint16_t*)S.slot[w.it.out] + e0;
-            // the whole block, for the mirror inside a diagonal block
-            uint16_t* blk = (uint16_t*)S.slot[w.it.out] + (size_t)(fr * 256) * ld + fc * 256;
-            const float limit = w.it.limit;
-            bool bad = false;
-            uint4 nh, nl, ah4, al4;
-            const uint4 z4 = make_uint4(0, 0, 0, 0);
-            nh = pv ? *(const uint4*)pv : z4;
-            nl = pv ? *(const uint4*)(pv + plane) : z4;
-            ah4 = ad ? *(const uint4*)ad : z4;
-            al4 = ad ? *(const uint4*)(ad + plane) : z4;
+            // the sums go back to the last unit's accumulator, which stays with the
+            // epilogue until they are used up, so that the update is a short loop
+            // (unrolled over 128 registers it was 90 KB of code per tile, and
+            // fetching it took 30 us)
+            const int a_last = (int)((u - 1) & 1);
+            const uint32_t tacc = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(a_last * BN + half * CPT);
+            tc_fence_after();
 #pragma unroll
-            for (int c8 = 0; c8 < CPT / 8; ++c8) {
-                const uint32_t ph[4] = {nh.x, nh.y, nh.z, nh.w}, pl[4] = {nl.x, nl.y, nl.z, nl.w};
-                const uint32_t gh[4] = {ah4.x, ah4.y, ah4.z, ah4.w}, gl[4] = {al4.x, al4.y, al4.z, al4.w};
-                if (c8 + 1 < CPT / 8) {
-                    // the next 8 columns in flight while these are updated
+            for (int q = 0; q < CPT / 16; ++q) tmem_st16(tacc + 16 * q, &R[16 * q]);
+            tmem_wait_st();
+#pragma unroll 1
+            for (int cb = 0; cb < CPT; cb += EB) {
+                static_assert(EB == 16, "one tensor-memory load per batch");
+                uint32_t av[16];
+                tmem_ld16(tacc + cb, av);
+                uint32_t ph[EB / 2], pl[EB / 2], gh[EB / 2], gl[EB / 2];
+#pragma unroll
+                for (int k = 0; k < EB / 2; ++k) {
+                    ph[k] = nh[k];
+                    pl[k] = nl[k];
+                    gh[k] = mh[k];
+                    gl[k] = ml[k];
+                }
+                if (cb + EB < CPT) fetch(cb + EB);
+#pragma unroll
+                for (int k = 0; k < EB / 2; ++k) {
+                    // columns c, c + 1 of this lane's row: one from its own words, one from
+                    // the neighbour's
+                    uint32_t own[2];
+                    float x[2];
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) x[u] = alpha * __uint_as_float(av[2 * k + u]);
                     if (pv) {
-                        nh = *(const uint4*)(pv + 8 * (c8 + 1));
-                        nl = *(const uint4*)(pv + plane + 8 * (c8 + 1));
+                        const uint32_t qh = __shfl_xor_sync(0xffffffffu, ph[k], 1);
+                        const uint32_t ql = __shfl_xor_sync(0xffffffffu, pl[k], 1);
+                        const uint32_t h0 = odd ? qh >> 16 : ph[k], h1 = odd ? ph[k] >> 16 : qh;
+                        const uint32_t l0 = odd ? ql >> 16 : pl[k], l1 = odd ? pl[k] >> 16 : ql;
+                        x[0] = fmaf(-ISC, H16<BF>::to_f(from_bits16<T>(h0)) + H16<BF>::to_f(from_bits16<T>(l0)), x[0]);
+                        x[1] = fmaf(-ISC, H16<BF>::to_f(from_bits16<T>(h1)) + H16<BF>::to_f(from_bits16<T>(l1)), x[1]);
                     }
                     if (ad) {
-                        ah4 = *(const uint4*)(ad + 8 * (c8 + 1));
-                        al4 = *(const uint4*)(ad + plane + 8 * (c8 + 1));
+                        const uint32_t qh = __shfl_xor_sync(0xffffffffu, gh[k], 1);
+                        const uint32_t ql = __shfl_xor_sync(0xffffffffu, gl[k], 1);
+                        const uint32_t f0 = odd ? __byte_perm(ql, qh, 0x7632) : __byte_perm(gl[k], gh[k], 0x5410);
+                        const uint32_t f1 = odd ? __byte_perm(gl[k], gh[k], 0x7632) : __byte_perm(ql, qh, 0x5410);
+                        x[0] += __uint_as_float(f0);
+                        x[1] += __uint_as_float(f1);
                     }
-                }
-                uint32_t hw[4], lw[4];
 #pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const int sh = 16 * (e & 1), c = c0 + 8 * c8 + e;
-                    float x = alpha * R[8 * c8 + e];
-                    if (pv)
-                        x = fmaf(-ISC, H16<BF>::to_f(from_bits16<T>(ph[e >> 1] >> sh)) +
-                                           H16<BF>::to_f(from_bits16<T>(pl[e >> 1] >> sh)), x);
-                    if (ad) x += __uint_as_float((((gh[e >> 1] >> sh) & 0xffffu) << 16) | ((gl[e >> 1] >> sh) & 0xffffu));
-                    if ((w.it.mode & PST_IDENT) && c == r && r < S.K) x -= 1.0f;
-                    bad |= !(fabsf(x) <= limit) && r < S.K && c < S.K && c >= r;
-                    uint32_t h, l;
-                    if (f32_out) {
-                        h = __float_as_uint(x) >> 16;
-                        l = __float_as_uint(x) & 0xffffu;
-                    } else {
-                        x *= SC;
-                        const T th = H16<BF>::from_f(x);
-                        h = bits16(th);
-                        l = bits16(H16<BF>::from_f(x - H16<BF>::to_f(th)));
+                    for (int u = 0; u < 2; ++u) {
+                        const int c = c0 + cb + 2 * k + u;
+                        if (ident && c == r) x[u] -= 1.0f;
+                        bad |= !(fabsf(x[u]) <= limit) && r < K && c < K && (!diag || c >= r);
+                        if (f32_out) {
+                            own[u] = __byte_perm(__float_as_uint(x[u]), 0, 0x1032);   // upper half first
+                        } else {
+                            const float y = x[u] * SC;
+                            const T th = H16<BF>::from_f(y);
+                            own[u] = bits16(th) | (bits16(H16<BF>::from_f(y - H16<BF>::to_f(th))) << 16);
+                        }
                     }
-                    if (e & 1) {
-                        hw[e >> 1] |= h << 16;
-                        lw[e >> 1] |= l << 16;
-                    } else {
-                        hw[e >> 1] = h;
-                        lw[e >> 1] = l;
+                    const uint32_t mine = odd ? own[1] : own[0];
+                    const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? own[0] : own[1], 1);
+                    const uint32_t e = odd ? got : mine, o = odd ? mine : got;   // even and odd row of my column
+                    const size_t at = (size_t)(cb + 2 * k) * ld;
+                    const uint32_t eh = __byte_perm(e, o, 0x5410), el = __byte_perm(e, o, 0x7632);
+                    const int c = c0 + cb + 2 * k + odd;
+                    if (!diag || c >= (r | 1)) {
+                        *(uint32_t*)(out + at) = eh;
+                        *(uint32_t*)(out + plane + at) = el;
+                    } else if (c == (r & ~1)) {
+                        out[at] = (uint16_t)eh;
+                        out[plane + at] = (uint16_t)el;
                     }
-                    if (diag && c >= r && !f32_out) {
-                        // both triangles of a diagonal block from its upper one
-                        const int br = r - w.p * 256, bc = c - w.p * 256;
-                        blk[(size_t)br * ld + bc] = (uint16_t)h;
-                        blk[plane + (size_t)br * ld + bc] = (uint16_t)l;
-                        blk[(size_t)bc * ld + br] = (uint16_t)h;
-                        blk[plane + (size_t)bc * ld + br] = (uint16_t)l;
+                    if (diag) {
+                        tr[(2 * k) * 33 + lane] = own[0];
+                        tr[(2 * k + 1) * 33 + lane] = own[1];
                     }
                 }
-                if (!diag || f32_out) {
-                    *(uint4*)(out + 8 * c8) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-                    *(uint4*)(out + plane + 8 * c8) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+                if (diag) {
+                    // the lower triangle of a diagonal block mirrors the upper one (left to
+                    // their own rounding errors the two triangles drift apart, and the
+                    // antisymmetric part grows exponentially along a recurrence): 2 rows x 16
+                    // columns per access
+                    __syncwarp();
+                    uint16_t* row = (uint16_t*)S.slot[w.it.out] + (size_t)(fr * 256 + (w.i & 1) * BM + 32 * quad) * ld +
+                                    fc * 256 + half * CPT + cb + (lane & 15);
+#pragma unroll 4
+                    for (int q = 0; q < 16; ++q) {
+                        const int rr = 2 * q + (lane >> 4);
+                        const uint32_t v = tr[(lane & 15) * 33 + rr];
+                        if (c0 + cb + (lane & 15) > w.i * BM + 32 * quad + rr) {
+                            row[(size_t)rr * ld] = (uint16_t)v;
+                            row[plane + (size_t)rr * ld] = (uint16_t)(v >> 16);
+                        }
+                    }
+                    __syncwarp();
                 }
             }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&accempty[a_last]);
             if (bad && limit > 0.0f) atomicExch(&S.flags[FLAG_SPECTRUM], 1);
         }
     }
@@ -396,9 +476,9 @@ __global__ void __launch_bounds__(256) k_pst_split(int K, int nb, const double* 
     int fr, fc;
     fold(a, b, nb, fr, fc);
     const size_t ld = (size_t)nb * 256, plane = (size_t)(nb / 2 + 1) * 256 * ld;
-    const int c = threadIdx.x, gc = b * 256 + c;
+    const int c = threadIdx.x, gc = a * 256 + c;
     for (int r = blockIdx.y * 16; r < (int)blockIdx.y * 16 + 16; ++r) {
-        const int gr = a * 256 + r;
+        const int gr = b * 256 + r;
         const double x = gr < K && gc < K ? A[(long long)gr * K + gc] * (double)SC : 0.0;
         const T h = H16<BF>::from_d(x);
         const T l = H16<BF>::from_d(x - (double)H16<BF>::to_f(h));
@@ -408,13 +488,17 @@ __global__ void __launch_bounds__(256) k_pst_split(int K, int nb, const double* 
     }
 }
 
-// four consecutive elements of a pair (scaled back)
+// four consecutive elements of a pair, as stored and scaled back
+template <bool BF>
+__device__ __forceinline__ float4 pair4_raw(uint2 h, uint2 l) {
+    using T = typename H16<BF>::T;
+    auto f = [](uint32_t a, uint32_t b) { return H16<BF>::to_f(from_bits16<T>(a)) + H16<BF>::to_f(from_bits16<T>(b)); };
+    return make_float4(f(h.x, l.x), f(h.x >> 16, l.x >> 16), f(h.y, l.y), f(h.y >> 16, l.y >> 16));
+}
 template <bool BF>
 __device__ __forceinline__ float4 pair4(const uint16_t* p, size_t plane) {
-    using T = typename H16<BF>::T;
-    const uint2 h = *(const uint2*)p, l = *(const uint2*)(p + plane);
-    auto f = [](uint32_t a, uint32_t b) { return ISC * (H16<BF>::to_f(from_bits16<T>(a)) + H16<BF>::to_f(from_bits16<T>(b))); };
-    return make_float4(f(h.x, l.x), f(h.x >> 16, l.x >> 16), f(h.y, l.y), f(h.y >> 16, l.y >> 16));
+    const float4 x = pair4_raw<BF>(*(const uint2*)p, *(const uint2*)(p + plane));
+    return make_float4(ISC * x.x, ISC * x.y, ISC * x.z, ISC * x.w);
 }
 
 // block blockIdx.x of the upper block triangle
@@ -446,15 +530,15 @@ __global__ void __launch_bounds__(256) k_pst_combine(int K, int nb, int s, PstLi
     fold(a, b, nb, fr, fc);
     const size_t ld = (size_t)nb * 256, plane = (size_t)(nb / 2 + 1) * 256 * ld;
     const int lr = blockIdx.y * 4 + (threadIdx.x >> 6), lc = (threadIdx.x & 63) * 4;
-    if (a * 256 + (int)blockIdx.y * 4 >= (K + 31) / 32 * 32) return;   // beyond every operand's k range
+    if (b * 256 + (int)blockIdx.y * 4 >= (K + 31) / 32 * 32) return;   // beyond every operand's k range
     const size_t e0 = (size_t)(fr * 256 + lr) * ld + fc * 256 + lc;
     float acc[8][4];
-    const int gr = a * 256 + lr, gc = b * 256 + lc;
+    const int gr = b * 256 + lr, gc = a * 256 + lc;
 #pragma unroll
     for (int q = 0; q < 8; ++q)
 #pragma unroll
         for (int k = 0; k < 4; ++k) acc[q][k] = (gr == gc + k && gr < K) ? ((const float*)cf)[q] : 0.0f;
-#pragma unroll 2
+#pragma unroll 4
     for (int r = 1; r < s; ++r) {
         const float4 x = pair4<BF>((const uint16_t*)T.p[r] + e0, plane);
         const float4 c0 = cf[r][0], c1 = cf[r][1];
@@ -489,68 +573,114 @@ __global__ void __launch_bounds__(256) k_pst_combine(int K, int nb, int s, PstLi
     }
 }
 
-// partial Gram sums <G_q, T_r>: CTA blockIdx.x takes rows blockIdx.x,
-// + gridDim.x, ... of all blocks; off-diagonal blocks count twice.  64 x 64
-// pairs per CTA; per 64 columns of a row FP32 FMA chains, then FP64.
+// partial Gram sums <G_q, T_r>, 8 x 8 pairs per CTA (blockIdx.x: 8 babies,
+// blockIdx.z: 8 giants) over the 4-element groups of CTA column blockIdx.y;
+// off-diagonal blocks count twice.  HBM-bound where few giants are at hand
+// (each baby is read once per 8 giants; the CTAs of one column, adjacent in
+// launch order, share the giants' elements in L2), so nothing is staged: every thread keeps its 64 FP32
+// FMA chains (at most GRAM_GROUPS x 4 products long) and the chains meet in
+// FP64.
+constexpr int GRAM_GROUPS = 32;   // 4-element groups per thread
 template <bool BF>
 __global__ void __launch_bounds__(256) k_pst_gram(int K, int nb, PstList G, int nq, PstList T, int s,
                                                   double* __restrict__ part) {
-    __shared__ __align__(16) float g[64][68], t[64][68];
-    const int qb = blockIdx.y * 64, rb = blockIdx.z * 64;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    __shared__ double red[8][64];
+    const int rb = blockIdx.x * 8, qb = blockIdx.z * 8;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const size_t ld = (size_t)nb * 256, plane = (size_t)(nb / 2 + 1) * 256 * ld;
-    double acc[4][4] = {};
-    const bool live = qb + 4 * ty < nq;
-    const int nblk = nb * (nb + 1) / 2;
-    for (int w = blockIdx.x; w < nblk * 256; w += gridDim.x) {
+    const long long ngroup = (long long)(nb * (nb + 1) / 2) * 16384;   // per block 256 rows of 64 groups
+    float f[8][8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+#pragma unroll
+        for (int r = 0; r < 8; ++r) f[q][r] = 0.0f;
+    // the block of a CTA's groups is one: 256 x GRAM_GROUPS divides 16384
+    static_assert(16384 % (256 * GRAM_GROUPS) == 0, "a CTA's groups must lie in one block");
+    for (long long base = (long long)blockIdx.y * 256 * GRAM_GROUPS; base < ngroup;
+         base += (long long)gridDim.y * 256 * GRAM_GROUPS) {
         int a, b, fr, fc;
-        block_at(w >> 8, nb, a, b);
-        const int lr = w & 255;
-        if (a * 256 + lr >= K) continue;
+        block_at((int)(base >> 14), nb, a, b);
         fold(a, b, nb, fr, fc);
-        const float wt = a == b ? 1.0f : 2.0f;
-        for (int x0 = 0; x0 < 256 && b * 256 + x0 < K; x0 += 64) {
-            const size_t e0 = (size_t)(fr * 256 + lr) * ld + fc * 256 + x0;
-            __syncthreads();
-            for (int e = threadIdx.x; e < 64 * 16; e += 256) {
-                const int m = e >> 4, c = (e & 15) * 4, gc = b * 256 + x0 + c;
-                float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
-                if (qb + m < nq) x = pair4<BF>((const uint16_t*)G.p[qb + m] + e0 + c, plane);
-                if (rb + m < s && rb + m > 0) y = pair4<BF>((const uint16_t*)T.p[rb + m] + e0 + c, plane);
-                g[c][m] = gc < K ? wt * x.x : 0.f;
-                g[c + 1][m] = gc + 1 < K ? wt * x.y : 0.f;
-                g[c + 2][m] = gc + 2 < K ? wt * x.z : 0.f;
-                g[c + 3][m] = gc + 3 < K ? wt * x.w : 0.f;
-                t[c][m] = gc < K ? y.x : 0.f;
-                t[c + 1][m] = gc + 1 < K ? y.y : 0.f;
-                t[c + 2][m] = gc + 2 < K ? y.z : 0.f;
-                t[c + 3][m] = gc + 3 < K ? y.w : 0.f;
+        const float wt = a == b ? 1.0f : 2.0f;   // the pairs' scale is taken out at the end
+#pragma unroll 1
+        for (int g = 0; g < GRAM_GROUPS; ++g) {
+            const int e = (int)(base & 16383) + g * 256 + threadIdx.x;
+            const int lr = e >> 6, lc = (e & 63) * 4, gc = a * 256 + lc;
+            if (b * 256 + lr >= K || gc >= K) continue;
+            const size_t at = (size_t)(fr * 256 + lr) * ld + fc * 256 + lc;
+            const int live = min(4, K - gc);
+            // every list entry is a valid slot (the host pads them), so all loads of a
+            // group are issued before the first is used
+            float4 x[8];
+            uint2 hx[8], lx[8], hy[4], ly[4];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const uint16_t* g_ = (const uint16_t*)G.p[qb + q] + at;
+                hx[q] = *(const uint2*)g_;
+                lx[q] = *(const uint2*)(g_ + plane);
             }
-            __syncthreads();
-            if (!live) continue;
-            float f[4][4] = {};
-#pragma unroll 8
-            for (int c = 0; c < 64; ++c) {
-                const float4 x = *(const float4*)&g[c][4 * ty], y = *(const float4*)&t[c][4 * tx];
-                const float xa[4] = {x.x, x.y, x.z, x.w}, ya[4] = {y.x, y.y, y.z, y.w};
+            auto fetch = [&](int r0) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+                for (int r = 0; r < 4; ++r) {
+                    const uint16_t* t_ = (const uint16_t*)T.p[rb + r0 + r] + at;
+                    hy[r] = *(const uint2*)t_;
+                    ly[r] = *(const uint2*)(t_ + plane);
+                }
+            };
+            fetch(0);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) f[i][j] = fmaf(xa[i], ya[j], f[i][j]);
+            for (int q = 0; q < 8; ++q) {
+                x[q] = pair4_raw<BF>(hx[q], lx[q]);
+                x[q].x *= wt;
+                x[q].y *= wt;
+                x[q].z *= wt;
+                x[q].w *= wt;
+                if (live < 4) {   // beyond K the slots may hold anything
+                    if (live < 2) x[q].y = 0.f;
+                    if (live < 3) x[q].z = 0.f;
+                    x[q].w = 0.f;
+                }
             }
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int r0 = 0; r0 < 8; r0 += 4) {
+                float4 y[4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] += (double)f[i][j];
+                for (int r = 0; r < 4; ++r) {
+                    y[r] = pair4_raw<BF>(hy[r], ly[r]);
+                    if (live < 4) {
+                        if (live < 2) y[r].y = 0.f;
+                        if (live < 3) y[r].z = 0.f;
+                        y[r].w = 0.f;
+                    }
+                }
+                if (r0 == 0) fetch(4);
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int q = 0; q < 8; ++q)
+                        f[q][r0 + r] = fmaf(x[q].x, y[r].x, fmaf(x[q].y, y[r].y, fmaf(x[q].z, y[r].z, fmaf(x[q].w, y[r].w, f[q][r0 + r]))));
+            }
         }
     }
+    // sums over the warp's lanes: chains of four lanes in FP32, then FP64
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int q = 0; q < 8; ++q)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int q = qb + 4 * ty + i, r = rb + 4 * tx + j;
-            if (q < nq && r < s) part[((long long)blockIdx.x * nq + q) * s + r] = acc[i][j];
+        for (int r = 0; r < 8; ++r) {
+            float v = f[q][r];
+            v += __shfl_xor_sync(0xffffffffu, v, 16);
+            v += __shfl_xor_sync(0xffffffffu, v, 8);
+            double d = (double)v;
+            for (int o = 4; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+            if (lane == 0) red[warp][q * 8 + r] = d;
         }
+    __syncthreads();
+    if (threadIdx.x < 64) {
+        const int q = qb + (threadIdx.x >> 3), r = rb + (threadIdx.x & 7);
+        double d = 0.0;
+        for (int w = 0; w < 8; ++w) d += red[w][threadIdx.x];
+        if (q < nq && r < s) part[((long long)blockIdx.y * nq + q) * s + r] = d * ((double)ISC * ISC);
+    }
 }
 
 // out[y * stride] = Tr of matrix y of the list
@@ -594,43 +724,51 @@ __global__ void __launch_bounds__(256) k_pst_finish(int K, int nb, int s, PstLis
     auto pr = [](const uint16_t* p, size_t pl) {
         return ISC * (H16<BF>::to_f(from_bits16<H>(*p)) + H16<BF>::to_f(from_bits16<H>(p[pl])));
     };
+    // lanes along the row index gr (contiguous in the slots), element (gr, gc), gc >= gr
     for (int lr = threadIdx.x >> 5; lr < 32; lr += 8) {
-        const int gr = ti * 32 + lr, gc = tj * 32 + lc;
+        const int gr = ti * 32 + lc, gc = tj * 32 + lr;
         double x = 0.0;
         if (gr < K && gc < K) {
-            const size_t e = (size_t)(fr * 256 + (gr & 255)) * ld + fc * 256 + (gc & 255);
+            const size_t e = (size_t)(fr * 256 + (gc & 255)) * ld + fc * 256 + (gr & 255);
             if (first) {
                 if (gr == gc) x = c[0];
                 for (int r0 = 1; r0 < s; r0 += 8) {
+                    float y[8];
+#pragma unroll
+                    for (int r = 0; r < 8; ++r) y[r] = r0 + r < s ? pr((const uint16_t*)T.p[r0 + r] + e, plane) : 0.0f;
                     float f = 0.0f;
-                    for (int r = r0; r < min(s, r0 + 8); ++r) f = fmaf(cf[r], pr((const uint16_t*)T.p[r] + e, plane), f);
+#pragma unroll
+                    for (int r = 0; r < 8; ++r) f = r0 + r < s ? fmaf(cf[r0 + r], y[r], f) : f;
                     x += (double)f;
                 }
             } else {
-                x = rho[(long long)gr * K + gc];
+                x = rho[(long long)gc * K + gr];
             }
             for (int p = 0; p < np; ++p) {
                 const uint16_t* q = (const uint16_t*)part.p[p] + e;
                 x += (double)__uint_as_float(((uint32_t)q[0] << 16) | q[plane]);
             }
             if (b2) x -= (double)pr(b2 + e, plane);
-            if (gc >= gr) rho[(long long)gr * K + gc] = x;
+            if (gc >= gr) rho[(long long)gc * K + gr] = x;
         }
         sh[lc][lr] = x;
     }
     __syncthreads();
     for (int lr = threadIdx.x >> 5; lr < 32; lr += 8) {
-        const int gr = tj * 32 + lr, gc = ti * 32 + lc;
-        if (gr < K && gc < K && gr > gc) rho[(long long)gr * K + gc] = sh[lr][lc];
+        const int gr = ti * 32 + lr, gc = tj * 32 + lc;
+        if (gr < K && gc < K && gc > gr) rho[(long long)gr * K + gc] = sh[lr][lc];
     }
 }
 
-__global__ void k_pst_gram_sum(int nsplit, int n, const double* __restrict__ part, double* __restrict__ D) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+// D[e] = sum of the partials, one warp per entry, in a fixed order
+__global__ void __launch_bounds__(256) k_pst_gram_sum(int nsplit, int n, const double* __restrict__ part,
+                                                      double* __restrict__ D) {
+    const int e = (blockIdx.x * 256 + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (e >= n) return;
     double x = 0.0;
-    for (int p = 0; p < nsplit; ++p) x += part[(long long)p * n + e];
-    D[e] = x;
+    for (int p = lane; p < nsplit; p += 32) x += part[(long long)p * n + e];
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+    if (lane == 0) D[e] = x;
 }
 
 int row_tiles(int K) { return (K + BM - 1) / BM; }
@@ -720,9 +858,10 @@ struct View {
     int giant(int q) const { return q == 1 ? p.s - 1 : p.s + q - 2; }
     int extra(int i) const { return p.s + (p.direct ? std::max(0, p.Q - 1) : 0) + i; }
     int nextra() const { return (int)c.pst_slot.size() - extra(0); }
+    // T_0 = I is not stored: its entry, and those behind the last, hold T_1's slot
     PstList babies() const {
-        PstList T{};
-        for (int r = 1; r < p.s; ++r) T.p[r] = c.pst_slot[baby(r)];
+        PstList T;
+        for (int r = 0; r < PS_MAX_S; ++r) T.p[r] = c.pst_slot[baby(r > 0 && r < p.s ? r : 1)];
         return T;
     }
 };
@@ -741,18 +880,19 @@ void gram(Ctx& c, int q0, const std::vector<int>& slots, cudaStream_t st) {
     const PstList T = v.babies();
     for (size_t k = 0; k < slots.size(); k += PS_MAX_S) {
         const int nq = (int)std::min<size_t>(PS_MAX_S, slots.size() - k);
-        PstList G{};
-        for (int q = 0; q < nq; ++q) G.p[q] = c.pst_slot[slots[k + q]];
+        PstList G;
+        for (int q = 0; q < PS_MAX_S; ++q) G.p[q] = c.pst_slot[slots[k + std::min(q, nq - 1)]];
         if ((long long)nq * s > c.gram_cap) throw Error(DFT_EINTERNAL, "Gram partials exceed their buffer");
-        const int tiles = ((nq + 63) / 64) * ((s + 63) / 64);
+        // chains of GRAM_GROUPS groups while the partial sums fit their buffer
         const int nsplit = (int)std::max<long long>(
-            1, std::min<long long>({(long long)nb * (nb + 1) / 2 * 256, 4LL * SMS / tiles, c.gram_cap / ((long long)nq * s)}));
-        const dim3 grid(nsplit, (nq + 63) / 64, (s + 63) / 64);
+            1, std::min<long long>({(long long)nb * (nb + 1) / 2 * (16384 / (256 * GRAM_GROUPS)),
+                                    c.gram_cap / ((long long)nq * s), 65535LL}));
+        const dim3 grid((s + 7) / 8, nsplit, (nq + 7) / 8);
         double* Dq = D + (long long)(q0 + k) * s;
         if (s > 1) {
             pick(bf, [&] { k_pst_gram<true><<<grid, 256, 0, st>>>(c.K, nb, G, nq, T, s, c.d_gram); },
                  [&] { k_pst_gram<false><<<grid, 256, 0, st>>>(c.K, nb, G, nq, T, s, c.d_gram); });
-            k_pst_gram_sum<<<(nq * s + 255) / 256, 256, 0, st>>>(nsplit, nq * s, c.d_gram, Dq);
+            k_pst_gram_sum<<<(nq * s + 7) / 8, 256, 0, st>>>(nsplit, nq * s, c.d_gram, Dq);
         }
         pick(bf, [&] { k_pst_trace<true><<<nq, 128, 0, st>>>(c.K, nb, G, Dq, s); },
              [&] { k_pst_trace<false><<<nq, 128, 0, st>>>(c.K, nb, G, Dq, s); });
