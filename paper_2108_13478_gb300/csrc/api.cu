@@ -274,6 +274,7 @@ size_t carve(Ctx& c, char* base) {
     }
     size_t o_tp = L.off(sizeof(int) * (c.n_tiles + 1));
     size_t o_tf = L.off(sizeof(int) * std::max<long long>(1, c.tile_nnz));
+    size_t o_to = L.off(sizeof(int) * c.n_tiles);
     size_t o_xyz = L.off(sizeof(double) * 3 * c.n_atoms);
     size_t o_S = L.off(K2), o_T = L.off(K2), o_Li = L.off(K2), o_A = L.off(K2), o_F = L.off(K2);
     size_t o_rho = L.off(K2);
@@ -369,6 +370,7 @@ size_t carve(Ctx& c, char* base) {
         }
         c.d_tile_ptr = (int*)(base + o_tp);
         c.d_tile_fn = (int*)(base + o_tf);
+        c.d_tile_order = (int*)(base + o_to);
         c.d_xyz = (double*)(base + o_xyz);
         c.d_S = (double*)(base + o_S); c.d_T = (double*)(base + o_T); c.d_Linv = (double*)(base + o_Li);
         c.d_A = (double*)(base + o_A); c.d_H = (double*)(base + o_H);
@@ -932,6 +934,11 @@ dft_status dft_init_basis(dft_ctx** ctx, const dft_basis_desc* basis, const dft_
             DFT_CUDA_CHECK(cudaMemcpyAsync(c->d_term_par, par.data(), sizeof(int) * c->Kt, cudaMemcpyHostToDevice, s));
         }
         DFT_CUDA_CHECK(cudaMemcpyAsync(c->d_tile_ptr, tp.data(), sizeof(int) * tp.size(), cudaMemcpyHostToDevice, s));
+        c->grid_split = grid_split(*c, tp.data());
+        std::vector<int> order(c->n_tiles);
+        for (long long t = 0; t < c->n_tiles; ++t) order[t] = (int)t;
+        std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return tp[x + 1] - tp[x] > tp[y + 1] - tp[y]; });
+        DFT_CUDA_CHECK(cudaMemcpyAsync(c->d_tile_order, order.data(), sizeof(int) * order.size(), cudaMemcpyHostToDevice, s));
         if (!tf.empty())
             DFT_CUDA_CHECK(cudaMemcpyAsync(c->d_tile_fn, tf.data(), sizeof(int) * tf.size(), cudaMemcpyHostToDevice, s));
         DFT_CUDA_CHECK(cudaMemcpyAsync(c->d_xyz, c->xyz_host.data(), sizeof(double) * c->xyz_host.size(),

@@ -18,8 +18,6 @@ namespace dft {
 // grid tile edge (points per axis) used by collocation and quadrature
 constexpr int TILE = 8;
 constexpr int TILE_PTS = TILE * TILE * TILE;
-// functions per chunk staged in shared memory
-constexpr int FCH = 32;
 
 // one basis function (a Cartesian primitive), device layout
 struct Fn {
@@ -96,10 +94,11 @@ struct PstItem {
     int sys, first, last;
     int prev, add, out;          // slots, -1: none
     int mode;
+    int sub;                     // k-blocks per accumulator promotion
     float limit;                 // > 0: FLAG_SPECTRUM beyond it
     int tile0;                   // first tile of this product in the launch
 };
-enum { PST_ALPHA2 = 1, PST_IDENT = 2, PST_OUT_F32 = 4 };   // alpha = 2; prev = I; FP32 planes out
+enum { PST_ALPHA2 = 1, PST_IDENT = 2, PST_OUT_F32 = 4, PST_FINE = 8 };   // alpha = 2; prev = I; FP32 planes out; shortest accumulation chains
 constexpr int PST_ITEM_CAP = 16384;
 
 struct Ctx {
@@ -140,6 +139,8 @@ struct Ctx {
     double* d_Mt = nullptr;      //   term-level K_t x K_t scratch
     int* d_tile_ptr = nullptr;   // [n_tiles + 1]
     int* d_tile_fn = nullptr;    // [tile_nnz]
+    int* d_tile_order = nullptr; // [n_tiles], longest lists first
+    int grid_split = 1;          // blocks per tile of the grid kernels
     double* d_xyz = nullptr;     // [n_atoms * 3]
     double* d_S = nullptr;       // K x K
     double* d_T = nullptr;
@@ -294,6 +295,7 @@ void launch_nonlocal(const Ctx& c, cudaStream_t s);
 // FP64 kernels on the FP64 path, FP32 arithmetic (FP64 in and out) on the mixed path
 void launch_collocate(const Ctx& c, const double* P, double* n, cudaStream_t s);
 void launch_quadrature(const Ctx& c, const double* v, double* V, cudaStream_t s);
+int grid_split(const Ctx& c, const int* tile_ptr);   // from the host's list offsets
 void launch_gaussian_sum(const Ctx& c, double amp, double width, double* out, cudaStream_t s);
 
 // ---- dense FP64 linear algebra (k_linalg.cu) ----
@@ -343,7 +345,7 @@ void launch_moment_reduce(int nparts, const double* part, double* mom, int idx_e
                           double m0, const double* m1, cudaStream_t s);
 
 // ---- grouped evaluation of the expansion (k_poly.cu) ----
-PsPlan ps_plan(int n_c, int nslot, bool prefer_direct, int nroll);
+PsPlan ps_plan(int n_c, int nslot, double seq, double par, int nroll);
 // m_l, l < n_c, from the traces and Gram sums D ((Q + 1) x s)
 void launch_ps_moments(int K, const PsPlan& p, const double* D, double* mom, cudaStream_t s);
 // c_qr of the C_q from a_l; work holds (Q + 1) s doubles

@@ -59,7 +59,12 @@ struct Out {
     __half* hi = nullptr;   // split output (Kp stride), or
     __half* lo = nullptr;
     double* f64 = nullptr;  // FP64 output, K x K (ld K), symmetric when upper
+    float scale = 1.0f;     // applied to the product (a power of two)
 };
+// rho's pair holds RHO_SCALE rho: most of its elements are far below 1, where
+// the low half of an unscaled FP16 pair is subnormal (2^-25 absolute, which
+// the back-transform amplifies); |rho| <= 1
+constexpr float RHO_SCALE = 1024.0f;
 
 // tile t of the launch -> (row tile i, column tile j); upper: only tiles with
 // j >= i / 2 (those reaching the upper triangle); col_major walks columns in
@@ -197,13 +202,19 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm3_tc(const __grid_constant_
                     tc_fence_after();
                     const uint64_t ah = smem_desc<BK * 2>(sAh(s)), al = smem_desc<BK * 2>(sAl(s));
                     const uint64_t bh = smem_desc<BK * 2>(sBh(s)), bl = smem_desc<BK * 2>(sBl(s));
+                    // the small cross products first: additions to the accumulator lose
+                    // bits in proportion to what it holds already
 #pragma unroll
                     for (int kk = 0; kk < BK / 16; ++kk) {
                         const uint64_t off = (uint64_t)(kk * 2);   // 32 bytes per 16-element k step
-                        umma_f16(d, ah + off, bh + off, idesc, first ? 0u : 1u);
-                        umma_f16(d, ah + off, bl + off, idesc, 1u);
+                        umma_f16(d, ah + off, bl + off, idesc, first ? 0u : 1u);
                         umma_f16(d, al + off, bh + off, idesc, 1u);
                         first = false;
+                    }
+#pragma unroll
+                    for (int kk = 0; kk < BK / 16; ++kk) {
+                        const uint64_t off = (uint64_t)(kk * 2);
+                        umma_f16(d, ah + off, bh + off, idesc, 1u);
                     }
                     umma_commit(&empty[s]);
                 }
@@ -239,6 +250,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm3_tc(const __grid_constant_
         } else {
             const int r = m0 + r_loc;
             const int c0 = n0 + half * CPT;
+#pragma unroll
+            for (int i = 0; i < CPT; ++i) R[i] *= out.scale;
             if (out.hi) {
                 // re-split into an FP16 pair, 8 columns per 16-byte store
                 bool big = false;
@@ -287,13 +300,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm3_tc(const __grid_constant_
 
 // FP64 K x K (leading dimension ld, transposed if trans) -> FP16 pair Kp x Kp,
 // zero-padded; FLAG_RANGE if an element is outside the pair's range
-__global__ void k_split16(int K, int Kp, const double* __restrict__ A, int ld, int trans, __half* __restrict__ hi,
+__global__ void k_split16(int K, int Kp, const double* __restrict__ A, int ld, int trans, double scale, __half* __restrict__ hi,
                           __half* __restrict__ lo, int* __restrict__ flags) {
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (long long)Kp * Kp) return;
     const int i = (int)(e / Kp), j = (int)(e % Kp);
     double x = 0.0;
-    if (i < K && j < K) x = trans ? A[(long long)j * ld + i] : A[(long long)i * ld + j];
+    if (i < K && j < K) x = scale * (trans ? A[(long long)j * ld + i] : A[(long long)i * ld + j]);
     if (!(fabs(x) < (double)SPLIT_MAX)) {
         atomicExch(&flags[FLAG_RANGE], 1);
         x = 0.0;
@@ -396,9 +409,9 @@ void gemm(const Ctx& c, const CUtensorMap* a, const CUtensorMap* b, int kr, bool
     check_launch("gemm3_tc");
 }
 
-void split(const Ctx& c, const double* A, bool trans, void* hi, void* lo, cudaStream_t s) {
+void split(const Ctx& c, const double* A, bool trans, void* hi, void* lo, cudaStream_t s, double scale = 1.0) {
     const long long n = (long long)c.Kp * c.Kp;
-    k_split16<<<blocks_for(n, 256), 256, 0, s>>>(c.K, c.Kp, A, c.K, trans ? 1 : 0, (__half*)hi, (__half*)lo, c.d_flags);
+    k_split16<<<blocks_for(n, 256), 256, 0, s>>>(c.K, c.Kp, A, c.K, trans ? 1 : 0, scale, (__half*)hi, (__half*)lo, c.d_flags);
     check_launch("split16");
 }
 
@@ -431,12 +444,15 @@ void cg_transform_f(const Ctx& c, const double* F, double* Ft, cudaStream_t s) {
     cg::gemm(c, c.tm_xn, c.tm_li[1], cg::KR_COL_END, true, ft, s);
 }
 
-void cg_split_rho(const Ctx& c, cudaStream_t s) { cg::split(c, c.d_rho, false, c.d_x16[0], c.d_x16[1], s); }
+void cg_split_rho(const Ctx& c, cudaStream_t s) {
+    cg::split(c, c.d_rho, false, c.d_x16[0], c.d_x16[1], s, cg::RHO_SCALE);
+}
 
 void cg_correct_rho(const Ctx& c, cudaStream_t s) {
     // rho^2 on the upper tiles, mirrored, into the FP64 scratch d_B
     cg::Out r2;
     r2.f64 = c.d_B;
+    r2.scale = 1.0f / (cg::RHO_SCALE * cg::RHO_SCALE);
     cg::gemm(c, c.tm_xn, c.tm_x[0], cg::KR_FULL, true, r2, s);
     const int np = 592;
     cg::k_corr_norms<<<np, 256, 0, s>>>(c.K, c.d_rho, c.d_part);
@@ -453,6 +469,7 @@ void cg_back_transform(const Ctx& c, double* P, cudaStream_t s) {
     cg::Out g2;
     g2.hi = (__half*)c.d_x16[2];
     g2.lo = (__half*)c.d_x16[3];
+    g2.scale = 1.0f / cg::RHO_SCALE;
     cg::gemm(c, c.tm_lt[0], c.tm_x[0], cg::KR_ROW_START, false, g2, s);
     cg::Out p;
     p.f64 = P;

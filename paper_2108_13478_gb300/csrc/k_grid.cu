@@ -8,6 +8,8 @@
 // phi_a(r_g) costs two multiplications (Supp. A.1).
 #include "dft_internal.cuh"
 
+#include <algorithm>
+
 namespace dft {
 namespace {
 
@@ -35,193 +37,337 @@ __global__ void k_build_tables(const Fn* __restrict__ fn, int K, int W, double o
     tab[idx] = val;
 }
 
-// stage the 8-point slices of NCH functions' tables for the tile at t0
-template <typename R, int NCH = FCH>
-__device__ __forceinline__ void stage_slices(const Fn* __restrict__ fn, const double* __restrict__ tab,
-                                             int W, const int* __restrict__ list, int n_t, int c0,
-                                             const int t0[3], R (*sx)[TILE], R (*sy)[TILE],
-                                             R (*sz)[TILE]) {
-    for (int e = threadIdx.x; e < NCH * 3 * TILE; e += blockDim.x) {
-        int fl = e / (3 * TILE);
-        int d = (e / TILE) % 3;
-        int q = e % TILE;
+// Collocation and quadrature of one 8^3 tile run as small matrix products over
+// pairs (ca <= cb) of chunks of CH functions of the tile's list, plane by plane
+// (z fixed, 64 points): FP32 with CH = 64 and 8 x 8 sums per thread, so that 4
+// shared-memory reads of 16 bytes feed 64 multiply-adds (the FMA pipe is the
+// limit, not shared memory); FP64 with CH = 32 and 4 x 4.  A block has two
+// groups of 64 threads, one per half of the z planes; both groups share the
+// chunk's x, y, z slices.  Only ca <= cb is computed: half of the products
+// of the full double sum.  Tiles are launched by falling list length, so that
+// the last blocks to run are short ones.
+template <typename R>
+struct GridCfg {
+    static constexpr int TI = sizeof(R) == 4 ? 8 : 4;   // sums per thread and side
+    static constexpr int CH = 8 * TI;                   // functions per chunk
+    static constexpr int V = TI / 2;                    // elements per 16-byte access
+    struct __align__(16) Vec { R v[V]; };
+};
+
+__device__ __forceinline__ void group_sync(int g) { asm volatile("bar.sync %0, 64;" ::"r"(1 + g) : "memory"); }
+
+// the 8-point slices of CH functions' tables for the tile at t0 (zero outside
+// the windows and beyond the list), [axis][function][point]
+template <typename R, int CH>
+__device__ __forceinline__ void stage_slices(const Fn* __restrict__ fn, const double* __restrict__ tab, int W,
+                                             const int* __restrict__ list, int n_t, int c0, const int t0[3],
+                                             R (*s)[CH][TILE]) {
+    for (int e = threadIdx.x; e < CH * 3 * TILE; e += blockDim.x) {
+        const int q = e % TILE, fl = (e / TILE) % CH, d = e / (TILE * CH);
         double val = 0.0;
         if (c0 + fl < n_t) {
-            int f = list[c0 + fl];
-            int i = t0[d] + q;
-            int lo = fn[f].lo[d], hi = fn[f].hi[d];
+            const int f = list[c0 + fl];
+            const int i = t0[d] + q;
+            const int lo = fn[f].lo[d], hi = fn[f].hi[d];
             if (i >= lo && i <= hi) val = tab[((long long)f * 3 + d) * W + (i - lo)];
         }
-        if (d == 0) sx[fl][q] = (R)val;
-        else if (d == 1) sy[fl][q] = (R)val;
-        else sz[fl][q] = (R)val;
+        s[d][fl][q] = (R)val;
     }
 }
 
-// n(r_g) = sum_a 2 phi_a(r_g) sum_b phi_b(r_g) P_ba for the points of one tile
-// (Eq. A.5 summed over the columns a).  256 threads, 2 points each.  R is the
-// arithmetic type (double on the FP64 path, float on the mixed path); inputs
-// and output stay double.
+// TI x TI sums over NK terms: acc_ij += A[k][i of ty] B[k][j of tx], rows of
+// pitch pa, pb; thread indexes i: V ty + (0..V-1) and CH / 2 + V ty + (0..V-1)
+template <typename R, int NK>
+__device__ __forceinline__ void tile_product(const R* A, int pa, const R* B, int pb, int ty, int tx,
+                                             R (&acc)[GridCfg<R>::TI][GridCfg<R>::TI]) {
+    using C = GridCfg<R>;
+    using Vec = typename C::Vec;
+#pragma unroll 4
+    for (int k = 0; k < NK; ++k) {
+        R a[C::TI], b[C::TI];
+        *(Vec*)&a[0] = *(const Vec*)(A + k * pa + C::V * ty);
+        *(Vec*)&a[C::V] = *(const Vec*)(A + k * pa + C::CH / 2 + C::V * ty);
+        *(Vec*)&b[0] = *(const Vec*)(B + k * pb + C::V * tx);
+        *(Vec*)&b[C::V] = *(const Vec*)(B + k * pb + C::CH / 2 + C::V * tx);
+#pragma unroll
+        for (int i = 0; i < C::TI; ++i)
+#pragma unroll
+            for (int j = 0; j < C::TI; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+    }
+}
+// function (point) of sum i of thread row (column) t
 template <typename R>
-__global__ void __launch_bounds__(256) k_collocate(
+__device__ __forceinline__ int sum_at(int t, int i) {
+    using C = GridCfg<R>;
+    return (i / C::V) * (C::CH / 2) + C::V * t + i % C::V;
+}
+
+// n(r_g) = 2 sum_ab P_ab phi_a phi_b for the points of one tile (Eq. A.5): per
+// chunk pair and plane Y[q][a] = sum_b phi_b(q) Q_ba, n(q) += sum_a phi_a(q) Y[q][a],
+// Q = P_ba + P_ab off the chunk diagonal (P need not be symmetric), P on it.
+// FP32 sums are at most CH long and meet in FP64.  Double: the 64 points of a
+// plane go through 4 x 4 sums in two halves.
+template <typename R>
+struct CollSmem {
+    using C = GridCfg<R>;
+    static constexpr int NB = 32;   // functions of chunk b staged at a time
+    R w[2][NB][64];           // phi_b of the group's plane
+    R P[C::CH][C::CH + 16 / sizeof(R)];
+    R xy[64][C::CH];          // x y of chunk a
+    R sa[3][C::CH][TILE], sb[3][C::CH][TILE];
+    double n[TILE_PTS];
+    int la[C::CH], lb[C::CH];
+};
+template <typename R>
+__global__ void __launch_bounds__(128, sizeof(R) == 4 ? 3 : 2) k_collocate(
     const Fn* __restrict__ fn, const double* __restrict__ tab, int W, const int* __restrict__ tile_ptr,
-    const int* __restrict__ tile_fn, int ntx, int nty, int nx, int ny, int nz, int K,
+    const int* __restrict__ tile_fn, const int* __restrict__ tile_order, int ntx, int nty, int nx, int ny, int nz, int K,
     const double* __restrict__ P, double* __restrict__ n_out) {
-    __shared__ R sxa[FCH][TILE], sya[FCH][TILE], sza[FCH][TILE];
-    __shared__ R sxb[FCH][TILE], syb[FCH][TILE], szb[FCH][TILE];
-    __shared__ __align__(16) R sP[FCH][FCH];
-    const int t = blockIdx.x;
-    const int tx = t % ntx, ty = (t / ntx) % nty, tz = t / (ntx * nty);
-    const int t0[3] = {tx * TILE, ty * TILE, tz * TILE};
+    using C = GridCfg<R>;
+    constexpr int TI = C::TI, CH = C::CH, NB = CollSmem<R>::NB;
+    extern __shared__ __align__(16) uint8_t smem_raw[];
+    CollSmem<R>& s = *(CollSmem<R>*)smem_raw;
+    const int t = tile_order[blockIdx.x];
+    const int tx_ = t % ntx, ty_ = (t / ntx) % nty, tz_ = t / (ntx * nty);
+    const int t0[3] = {tx_ * TILE, ty_ * TILE, tz_ * TILE};
     const int* list = tile_fn + tile_ptr[t];
     const int n_t = tile_ptr[t + 1] - tile_ptr[t];
-    const int px = threadIdx.x & 7, py = (threadIdx.x >> 3) & 7, pz0 = threadIdx.x >> 6, pz1 = pz0 + 4;
-    double acc0 = 0.0, acc1 = 0.0;
-    for (int ca = 0; ca < n_t; ca += FCH) {
-        R y0[FCH], y1[FCH];
-#pragma unroll
-        for (int j = 0; j < FCH; ++j) { y0[j] = (R)0; y1[j] = (R)0; }
-        for (int cb = 0; cb < n_t; cb += FCH) {
+    const int g = threadIdx.x >> 6, u = threadIdx.x & 63, tx = u & 7, ty = u >> 3;
+    // planes of this block (gridDim.y blocks share a tile), and of this group
+    const int nz_block = TILE / gridDim.y, nz_group = nz_block / 2, z0 = blockIdx.y * nz_block + g * nz_group;
+    for (int p = threadIdx.x; p < TILE_PTS; p += 128) s.n[p] = 0.0;
+    for (int ca = 0; ca < n_t; ca += CH) {
+        __syncthreads();
+        stage_slices<R, CH>(fn, tab, W, list, n_t, ca, t0, s.sa);
+        for (int e = threadIdx.x; e < CH; e += 128) s.la[e] = ca + e < n_t ? list[ca + e] : -1;
+        __syncthreads();
+        for (int e = threadIdx.x; e < 64 * CH; e += 128) {
+            const int f = e % CH, q = e / CH;
+            s.xy[q][f] = s.sa[0][f][q & 7] * s.sa[1][f][q >> 3];
+        }
+        for (int cb = ca; cb < n_t; cb += CH) {
             __syncthreads();
-            stage_slices(fn, tab, W, list, n_t, cb, t0, sxb, syb, szb);
-            for (int e = threadIdx.x; e < FCH * FCH; e += blockDim.x) {
-                int i = e / FCH, j = e % FCH;
-                double v = 0.0;
-                if (cb + i < n_t && ca + j < n_t) v = P[(long long)list[cb + i] * K + list[ca + j]];
-                sP[i][j] = (R)v;
+            stage_slices<R, CH>(fn, tab, W, list, n_t, cb, t0, s.sb);
+            for (int e = threadIdx.x; e < CH; e += 128) s.lb[e] = cb + e < n_t ? list[cb + e] : -1;
+            __syncthreads();
+            // 8 loads in flight per thread (they are scattered runs of a few functions)
+            for (int e0 = threadIdx.x; e0 < CH * CH; e0 += 128 * 8) {
+                double x[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const int e = e0 + 128 * k, fa = s.la[e % CH], fb = s.lb[e / CH];
+                    x[k] = fa >= 0 && fb >= 0 ? P[(long long)fb * K + fa] : 0.0;
+                }
+#pragma unroll
+                for (int k = 0; k < 8; ++k) s.P[(e0 + 128 * k) / CH][(e0 + 128 * k) % CH] = (R)x[k];
+            }
+            if (ca != cb) {
+                __syncthreads();
+                for (int e0 = threadIdx.x; e0 < CH * CH; e0 += 128 * 8) {
+                    double x[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const int e = e0 + 128 * k, fa = s.la[e / CH], fb = s.lb[e % CH];
+                        x[k] = fa >= 0 && fb >= 0 ? P[(long long)fa * K + fb] : 0.0;
+                    }
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) s.P[(e0 + 128 * k) % CH][(e0 + 128 * k) / CH] += (R)x[k];
+                }
             }
             __syncthreads();
-#pragma unroll 2
-            for (int i = 0; i < FCH; ++i) {
-                R pxy = sxb[i][px] * syb[i][py];
-                R pb0 = pxy * szb[i][pz0];
-                R pb1 = pxy * szb[i][pz1];
+            for (int z = z0; z < z0 + nz_group; ++z) {
+#pragma unroll 1
+                for (int q0 = 0; q0 < 64; q0 += CH) {   // CH points at a time
+                    R Y[TI][TI];
 #pragma unroll
-                for (int j = 0; j < FCH; ++j) {
-                    R pv = sP[i][j];
-                    y0[j] = fma(pb0, pv, y0[j]);
-                    y1[j] = fma(pb1, pv, y1[j]);
+                    for (int i = 0; i < TI; ++i)
+#pragma unroll
+                        for (int j = 0; j < TI; ++j) Y[i][j] = (R)0;
+#pragma unroll 1
+                    for (int b0 = 0; b0 < CH; b0 += NB) {
+                        if (q0 == 0 || CH > NB) {
+                            group_sync(g);
+                            // this thread's point of the plane
+                            const int x = u & 7, y = u >> 3;
+#pragma unroll 8
+                            for (int b = 0; b < NB; ++b)
+                                s.w[g][b][u] = s.sb[0][b0 + b][x] * s.sb[1][b0 + b][y] * s.sb[2][b0 + b][z];
+                            group_sync(g);
+                        }
+                        tile_product<R, NB>(&s.w[g][0][q0], 64, &s.P[b0][0], CH + 16 / sizeof(R), ty, tx, Y);
+                    }
+                    R za[TI];
+#pragma unroll
+                    for (int j = 0; j < TI; ++j) za[j] = s.sa[2][sum_at<R>(tx, j)][z];
+#pragma unroll
+                    for (int i = 0; i < TI; ++i) {
+                        const int q = q0 + sum_at<R>(ty, i);
+                        R c = (R)0, xa[TI];
+                        *(typename C::Vec*)&xa[0] = *(const typename C::Vec*)&s.xy[q][C::V * tx];
+                        *(typename C::Vec*)&xa[C::V] = *(const typename C::Vec*)&s.xy[q][CH / 2 + C::V * tx];
+#pragma unroll
+                        for (int j = 0; j < TI; ++j) c = fma(xa[j] * za[j], Y[i][j], c);
+                        for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+                        if (tx == 0) s.n[64 * z + q] += (double)c;
+                    }
                 }
             }
         }
-        __syncthreads();
-        stage_slices(fn, tab, W, list, n_t, ca, t0, sxa, sya, sza);
-        __syncthreads();
-        R c0 = (R)0, c1 = (R)0;
-#pragma unroll
-        for (int j = 0; j < FCH; ++j) {
-            R pxy = sxa[j][px] * sya[j][py];
-            c0 = fma(pxy * sza[j][pz0], y0[j], c0);
-            c1 = fma(pxy * sza[j][pz1], y1[j], c1);
-        }
-        acc0 += (double)c0;
-        acc1 += (double)c1;
     }
-    int gx = t0[0] + px, gy = t0[1] + py;
-    if (gx < nx && gy < ny) {
-        int gz0 = t0[2] + pz0, gz1 = t0[2] + pz1;
-        if (gz0 < nz) n_out[((long long)gz0 * ny + gy) * nx + gx] = 2.0 * acc0;
-        if (gz1 < nz) n_out[((long long)gz1 * ny + gy) * nx + gx] = 2.0 * acc1;
+    __syncthreads();
+    for (int p = blockIdx.y * nz_block * 64 + threadIdx.x; p < (int)(blockIdx.y + 1) * nz_block * 64; p += 128) {
+        const int gx = t0[0] + (p & 7), gy = t0[1] + ((p >> 3) & 7), gz = t0[2] + (p >> 6);
+        if (gx < nx && gy < ny && gz < nz) n_out[((long long)gz * ny + gy) * nx + gx] = 2.0 * s.n[p];
     }
 }
 
 // V_ab += h^3 sum_{g in tile} phi_a v phi_b for all pairs of the tile's list
-// (Eq. A.6).  Chunks of QCH = 64 functions, chunk pairs (ca <= cb), the
-// off-diagonal chunk blocks mirrored.  Per block of QPTS points, the values
-// phi_a(g) and v(g) phi_b(g) of both chunks are formed in shared memory once;
-// each thread then accumulates a 4 x 4 register block of pairs (a = ty + 16 i,
-// b = tx + 16 j), two shared-memory reads per four multiply-adds.  Every pair
-// sums its points in the order g = 0 .. 511.  Contributions of different
-// tiles meet as integers: each is rounded to a multiple of 2^-48 and added
-// with a 64-bit integer atomic into V's own storage, so the sum is exact and
-// independent of the order in which tiles finish (the result is the same bit
-// for bit on every run and in every batch); k_fixed_to_double then turns the
-// integers into doubles in place.  Rounding each tile's contribution costs
+// (Eq. A.6): per chunk pair and plane G_ab = sum_q (x y)_a(q) w_b(q) with w =
+// v phi_b, V_ab += z_a G_ab.  Contributions of different tiles meet as
+// integers: each is rounded to a multiple of 2^-48 and added with a 64-bit
+// integer atomic into the upper triangle of V's own storage (the lists ascend,
+// so la <= lb is fa <= fb), so the sum is exact and independent of the order
+// in which tiles finish (the result is the same bit for bit on every run and
+// in every batch); k_fixed_to_double then turns the integers into doubles and
+// mirrors them.  Rounding each tile's contribution costs
 // at most 2^-49 (1.8e-15; ~1e-12 over the ~10^3 tiles two diffuse functions
 // share); partial sums must stay within +-2^15 (|V| is O(10) for potentials
 // of tens of hartree).
-constexpr int QCH = 64;
 constexpr double QFIX = 281474976710656.0;   // 2^48
 template <typename R>
-__global__ void __launch_bounds__(256) k_quadrature(
+struct QuadSmem {
+    using C = GridCfg<R>;
+    R w[2][64][C::CH];        // v phi_b of the group's plane; the group's sums at the end
+    R xy[64][C::CH];          // x y of chunk a
+    R sa[3][C::CH][TILE], sb[3][C::CH][TILE];
+    R v[TILE_PTS];
+    int la[C::CH], lb[C::CH];
+};
+template <typename R>
+__global__ void __launch_bounds__(128, sizeof(R) == 4 ? 3 : 2) k_quadrature(
     const Fn* __restrict__ fn, const double* __restrict__ tab, int W, const int* __restrict__ tile_ptr,
-    const int* __restrict__ tile_fn, int ntx, int nty, int nx, int ny, int nz, int K, double h3,
+    const int* __restrict__ tile_fn, const int* __restrict__ tile_order, int ntx, int nty, int nx, int ny, int nz, int K, double h3,
     const double* __restrict__ v, double* __restrict__ V) {
-    constexpr int QPTS = sizeof(R) == 4 ? 32 : 16;
-    __shared__ R sxa[QCH][TILE], sya[QCH][TILE], sza[QCH][TILE];
-    __shared__ R sxb[QCH][TILE], syb[QCH][TILE], szb[QCH][TILE];
-    __shared__ R sv[TILE_PTS];
-    __shared__ R pa[QPTS][QCH], pb[QPTS][QCH];
-    const int t = blockIdx.x;
-    const int tx = t % ntx, ty_ = (t / ntx) % nty, tz = t / (ntx * nty);
-    const int t0[3] = {tx * TILE, ty_ * TILE, tz * TILE};
+    using C = GridCfg<R>;
+    constexpr int TI = C::TI, CH = C::CH;
+    extern __shared__ __align__(16) uint8_t smem_raw[];
+    QuadSmem<R>& s = *(QuadSmem<R>*)smem_raw;
+    const int t = tile_order[blockIdx.x];
+    const int tx_ = t % ntx, ty_ = (t / ntx) % nty, tz_ = t / (ntx * nty);
+    const int t0[3] = {tx_ * TILE, ty_ * TILE, tz_ * TILE};
     const int* list = tile_fn + tile_ptr[t];
     const int n_t = tile_ptr[t + 1] - tile_ptr[t];
     if (n_t == 0) return;
-    for (int p = threadIdx.x; p < TILE_PTS; p += blockDim.x) {
-        int gx = t0[0] + (p & 7), gy = t0[1] + ((p >> 3) & 7), gz = t0[2] + (p >> 6);
-        sv[p] = (R)((gx < nx && gy < ny && gz < nz) ? v[((long long)gz * ny + gy) * nx + gx] : 0.0);
+    for (int p = threadIdx.x; p < TILE_PTS; p += 128) {
+        const int gx = t0[0] + (p & 7), gy = t0[1] + ((p >> 3) & 7), gz = t0[2] + (p >> 6);
+        s.v[p] = (R)((gx < nx && gy < ny && gz < nz) ? v[((long long)gz * ny + gy) * nx + gx] : 0.0);
     }
-    const int ux = threadIdx.x & 15, uy = threadIdx.x >> 4;   // b = ux + 16 j, a = uy + 16 i
-    for (int ca = 0; ca < n_t; ca += QCH) {
+    const int g = threadIdx.x >> 6, u = threadIdx.x & 63, tx = u & 7, ty = u >> 3;
+    const int nch = (n_t + CH - 1) / CH, npair = nch * (nch + 1) / 2;
+    // this block's run of chunk pairs (gridDim.y blocks share a tile), in row order
+    const int p_end = (int)((long long)npair * (blockIdx.y + 1) / gridDim.y);
+    int pair = (int)((long long)npair * blockIdx.y / gridDim.y);
+    if (pair >= p_end) return;
+    int ia = 0, ib = pair;
+    while (ib >= nch - ia) {
+        ib -= nch - ia;
+        ++ia;
+    }
+    ib += ia;
+    for (; pair < p_end; ++ia, ib = ia) {
+        const int ca = ia * CH;
         __syncthreads();
-        stage_slices<R, QCH>(fn, tab, W, list, n_t, ca, t0, sxa, sya, sza);
-        for (int cb = ca; cb < n_t; cb += QCH) {
+        stage_slices<R, CH>(fn, tab, W, list, n_t, ca, t0, s.sa);
+        for (int e = threadIdx.x; e < CH; e += 128) s.la[e] = ca + e < n_t ? list[ca + e] : -1;
+        __syncthreads();
+        for (int e = threadIdx.x; e < 64 * CH; e += 128) {
+            const int f = e % CH, q = e / CH;
+            s.xy[q][f] = s.sa[0][f][q & 7] * s.sa[1][f][q >> 3];
+        }
+        for (; ib < nch && pair < p_end; ++ib, ++pair) {
+            const int cb = ib * CH;
             __syncthreads();
-            stage_slices<R, QCH>(fn, tab, W, list, n_t, cb, t0, sxb, syb, szb);
-            R acc[4][4];
+            stage_slices<R, CH>(fn, tab, W, list, n_t, cb, t0, s.sb);
+            for (int e = threadIdx.x; e < CH; e += 128) s.lb[e] = cb + e < n_t ? list[cb + e] : -1;
+            __syncthreads();
+            R acc[TI][TI];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < TI; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = (R)0;
-            for (int p0 = 0; p0 < TILE_PTS; p0 += QPTS) {
-                __syncthreads();
-                for (int e = threadIdx.x; e < QPTS * QCH; e += blockDim.x) {
-                    int pp = e / QCH, f = e % QCH;
-                    int p = p0 + pp;
-                    int x = p & 7, y = (p >> 3) & 7, z = p >> 6;
-                    pa[pp][f] = sxa[f][x] * sya[f][y] * sza[f][z];
-                    pb[pp][f] = sxb[f][x] * syb[f][y] * szb[f][z] * sv[p];
+                for (int j = 0; j < TI; ++j) acc[i][j] = (R)0;
+            for (int z = 4 * g; z < 4 * g + 4; ++z) {
+                group_sync(g);
+                {
+                    // one function of chunk b per thread (two threads each in FP64), its points of the plane
+                    const int f = u % CH, y0 = (u / CH) * (TILE * CH / 64);
+                    const R zb = s.sb[2][f][z];
+                    R x[TILE];
+#pragma unroll
+                    for (int k = 0; k < TILE; ++k) x[k] = s.sb[0][f][k] * zb;
+#pragma unroll 2
+                    for (int y = y0; y < y0 + TILE * CH / 64; ++y) {
+                        const R yb = s.sb[1][f][y];
+#pragma unroll
+                        for (int k = 0; k < TILE; ++k) s.w[g][8 * y + k][f] = x[k] * (yb * s.v[64 * z + 8 * y + k]);
+                    }
                 }
-                __syncthreads();
-#pragma unroll 4
-                for (int pp = 0; pp < QPTS; ++pp) {
-                    R va[4], vb[4];
+                group_sync(g);
+                R G[TI][TI];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) va[i] = pa[pp][uy + 16 * i];
+                for (int i = 0; i < TI; ++i)
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) vb[j] = pb[pp][ux + 16 * j];
+                    for (int j = 0; j < TI; ++j) G[i][j] = (R)0;
+                tile_product<R, 64>(&s.xy[0][0], CH, &s.w[g][0][0], CH, ty, tx, G);
 #pragma unroll
-                    for (int i = 0; i < 4; ++i)
+                for (int i = 0; i < TI; ++i) {
+                    const R za = s.sa[2][sum_at<R>(ty, i)][z];
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) acc[i][j] = fma(va[i], vb[j], acc[i][j]);
+                    for (int j = 0; j < TI; ++j) acc[i][j] = fma(za, G[i][j], acc[i][j]);
                 }
             }
+            group_sync(g);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int la = ca + uy + 16 * i;
-                if (la >= n_t) continue;
-                const int fa = list[la];
+            for (int i = 0; i < TI; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int lb = cb + ux + 16 * j;
-                    if (lb >= n_t) continue;
-                    const int fb = list[lb];
-                    const unsigned long long q = (unsigned long long)llrint(h3 * (double)acc[i][j] * QFIX);
-                    atomicAdd((unsigned long long*)&V[(long long)fa * K + fb], q);
-                    if (ca != cb) atomicAdd((unsigned long long*)&V[(long long)fb * K + fa], q);
-                }
+                for (int j = 0; j < TI; ++j) s.w[g][sum_at<R>(ty, i)][sum_at<R>(tx, j)] = acc[i][j];
+            __syncthreads();
+            for (int e = threadIdx.x; e < CH * CH; e += 128) {
+                const int a = e / CH, b = e % CH, fa = s.la[a], fb = s.lb[b];
+                if (fa < 0 || fb < 0 || fa > fb) continue;
+                const R sum = s.w[0][a][b] + s.w[1][a][b];
+                const unsigned long long q = (unsigned long long)llrint(h3 * (double)sum * QFIX);
+                atomicAdd((unsigned long long*)&V[(long long)fa * K + fb], q);
             }
         }
     }
 }
 
-// V's 64-bit integer sums (units of 2^-44) -> doubles, in place
-__global__ void k_fixed_to_double(long long n, double* V) {
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    const long long q = reinterpret_cast<const long long*>(V)[e];
-    V[e] = (double)q * (1.0 / QFIX);
+// V's 64-bit integer sums (units of 2^-48, upper triangle) -> doubles, both triangles
+__global__ void __launch_bounds__(256) k_fixed_to_double(int K, double* V) {
+    __shared__ double sh[32][33];
+    const int nb = (K + 31) / 32;
+    int ti = 0, tj = blockIdx.x;
+    while (tj >= nb - ti) {
+        tj -= nb - ti;
+        ++ti;
+    }
+    tj += ti;
+    const int c = threadIdx.x & 31;
+    for (int r = threadIdx.x >> 5; r < 32; r += 8) {
+        const int i = ti * 32 + r, j = tj * 32 + c;
+        double x = 0.0;
+        if (i < K && j < K && j >= i) {
+            const long long e = (long long)i * K + j;
+            x = (double)reinterpret_cast<const long long*>(V)[e] * (1.0 / QFIX);
+            V[e] = x;
+        }
+        sh[c][r] = x;
+    }
+    __syncthreads();
+    for (int r = threadIdx.x >> 5; r < 32; r += 8) {
+        const int i = tj * 32 + r, j = ti * 32 + c;
+        if (i < K && j < K && i > j) V[(long long)i * K + j] = sh[r][c];
+    }
 }
 
 // out(r_g) = sum_C amp exp(-|r_g - R_C|^2 / w^2), terms below 1e-30 |amp| dropped
@@ -244,6 +390,24 @@ __global__ void k_gaussian_sum(const double* __restrict__ xyz, int n_atoms, int 
 
 }  // namespace
 
+// Blocks per grid tile: a tile's work grows with the square of its list, and a
+// small cluster has few tiles, so tiles are split (collocation by planes,
+// quadrature by chunk pairs) until the longest takes at most a third of what an SM
+// gets on average (K = 240 in FP64: 343 tiles, the longest lists of 432 terms
+// against 170 on average)
+int grid_split(const Ctx& c, const int* tile_ptr) {
+    const int ch = c.p.precision == DFT_PREC_FP64 ? GridCfg<double>::CH : GridCfg<float>::CH;
+    double total = 0.0, longest = 0.0;
+    for (long long t = 0; t < c.n_tiles; ++t) {
+        const double n = (tile_ptr[t + 1] - tile_ptr[t] + ch - 1) / ch, w = n * (n + 1) / 2;
+        total += w;
+        longest = std::max(longest, w);
+    }
+    int s = 1;
+    while (s < 8 && longest / s > total / 152.0 / 3.0) s *= 2;
+    return s;
+}
+
 void launch_build_tables_for(const Ctx& c, const Fn* fn, int count, int W, double* tab, cudaStream_t s) {
     long long total = (long long)count * 3 * W;
     if (total == 0) return;
@@ -255,18 +419,27 @@ void launch_build_tables_for(const Ctx& c, const Fn* fn, int count, int W, doubl
 
 void launch_build_tables(const Ctx& c, cudaStream_t s) { launch_build_tables_for(c, c.d_fn, c.Kt, c.tab_w, c.d_tab, s); }
 
+namespace {
+template <class Kern>
+void allow_smem(Kern k, size_t bytes) {
+    DFT_CUDA_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+}
+}  // namespace
+
 void launch_collocate(const Ctx& c, const double* P, double* n, cudaStream_t s) {
     // contracted functions: collocate their terms with P_t = C^T P C
     if (c.contracted) {
         launch_expand(c, P, c.d_Mt, s);
         P = c.d_Mt;
     }
-    if (c.p.precision == DFT_PREC_FP64)
-        k_collocate<double><<<(unsigned)c.n_tiles, 256, 0, s>>>(c.d_fn, c.d_tab, c.tab_w, c.d_tile_ptr, c.d_tile_fn,
-                                                                c.ntile[0], c.ntile[1], c.n[0], c.n[1], c.n[2], c.Kt, P, n);
-    else
-        k_collocate<float><<<(unsigned)c.n_tiles, 256, 0, s>>>(c.d_fn, c.d_tab, c.tab_w, c.d_tile_ptr, c.d_tile_fn,
-                                                               c.ntile[0], c.ntile[1], c.n[0], c.n[1], c.n[2], c.Kt, P, n);
+    auto go = [&](auto kern, size_t bytes) {
+        allow_smem(kern, bytes);
+        const dim3 grid((unsigned)c.n_tiles, std::min(c.grid_split, 4));   // by planes, at least one per thread group
+        kern<<<grid, 128, bytes, s>>>(c.d_fn, c.d_tab, c.tab_w, c.d_tile_ptr, c.d_tile_fn, c.d_tile_order, c.ntile[0],
+                                      c.ntile[1], c.n[0], c.n[1], c.n[2], c.Kt, P, n);
+    };
+    if (c.p.precision == DFT_PREC_FP64) go(k_collocate<double>, sizeof(CollSmem<double>));
+    else go(k_collocate<float>, sizeof(CollSmem<float>));
     check_launch("collocate");
 }
 
@@ -275,16 +448,15 @@ void launch_quadrature(const Ctx& c, const double* v, double* V, cudaStream_t s)
     double* Vq = c.contracted ? c.d_Mt : V;
     const int K = c.Kt;
     DFT_CUDA_CHECK(cudaMemsetAsync(Vq, 0, sizeof(double) * (size_t)K * K, s));
-    if (c.p.precision == DFT_PREC_FP64)
-        k_quadrature<double><<<(unsigned)c.n_tiles, 256, 0, s>>>(c.d_fn, c.d_tab, c.tab_w, c.d_tile_ptr, c.d_tile_fn,
-                                                                 c.ntile[0], c.ntile[1], c.n[0], c.n[1], c.n[2], K,
-                                                                 c.h * c.h * c.h, v, Vq);
-    else
-        k_quadrature<float><<<(unsigned)c.n_tiles, 256, 0, s>>>(c.d_fn, c.d_tab, c.tab_w, c.d_tile_ptr, c.d_tile_fn,
-                                                                c.ntile[0], c.ntile[1], c.n[0], c.n[1], c.n[2], K,
-                                                                c.h * c.h * c.h, v, Vq);
-    const long long n = (long long)K * K;
-    k_fixed_to_double<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, Vq);
+    auto go = [&](auto kern, size_t bytes) {
+        allow_smem(kern, bytes);
+        kern<<<dim3((unsigned)c.n_tiles, c.grid_split), 128, bytes, s>>>(c.d_fn, c.d_tab, c.tab_w, c.d_tile_ptr, c.d_tile_fn, c.d_tile_order, c.ntile[0],
+                                                     c.ntile[1], c.n[0], c.n[1], c.n[2], K, c.h * c.h * c.h, v, Vq);
+    };
+    if (c.p.precision == DFT_PREC_FP64) go(k_quadrature<double>, sizeof(QuadSmem<double>));
+    else go(k_quadrature<float>, sizeof(QuadSmem<float>));
+    const long long nb = (K + 31) / 32;
+    k_fixed_to_double<<<(unsigned)(nb * (nb + 1) / 2), 256, 0, s>>>(K, Vq);
     check_launch("quadrature", 2);
     if (c.contracted) launch_contract(c, c.d_Mt, V, s);
 }

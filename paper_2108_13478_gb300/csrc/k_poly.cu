@@ -10,9 +10,11 @@
 //   c_qr = 2 a_{qs+r} with a_{qs-r} -= a_{qs+r};
 //   m_{qs+r} = Tr T_{qs+r} = 2 <G_q, T_r> - m_{qs-r}  (moments without a product).
 //
-// Babies and giants come by doubling, T_{m+j} = 2 T_m T_j - T_{m-j}, so each
-// launch computes m products at once and the whole expansion takes about
-// 2 log2(sqrt(N_C)) dependent launches ("direct" plan).  Where the
+// The babies come by the three-term recurrence, one product after the other:
+// by doubling (T_{2m} = 2 T_m^2 - I) their rounding errors no longer act as a
+// shift of the energies, and in a basis with a well-conditioned overlap P was
+// off by 70 times as much.  The giants come by doubling, G_{m+j} = 2 G_m G_j -
+// G_{m-j}, m products per launch, with no such loss ("direct" plan).  Where the
 // workspace cannot hold the giants, they roll in two buffers and the sum is
 // taken by Clenshaw's recurrence in T_s, b_q = C_q + 2 T_s b_{q+1} - b_{q+2},
 // rho = C_0 + T_s b_1 - b_2 ("Clenshaw" plan: same number of products, one
@@ -22,7 +24,7 @@
 // the limit of every kernel here).  All operands are symmetric polynomials
 // of H_N, so products are formed on upper tiles and mirrored.  Whole density
 // matrix at tail 1e-10 (N_C ~ 2900), the three-term recurrence with full
-// products before and this now: K = 80 134 -> 6.7 ms, K = 370 559 -> 17.7 ms,
+// products before and this now: K = 80 134 -> 8.8 ms, K = 370 559 -> 20.0 ms,
 // error against an exact eigensolve 6e-14 relative on both sides.
 #include "dft_internal.cuh"
 #include "ps_plan.cuh"
@@ -325,42 +327,33 @@ inline int upper_tiles(int K, int tb) {
 // (n_c - 1) / s.  Direct: s - 1 babies (T_1 = H_N is not counted), the
 // giants G_2 .. G_Q and PS_CQ buffers for the C_q and the partial sums of the
 // weighted products.  Clenshaw: the babies T_2 .. T_s and nroll buffers.
-PsPlan ps_plan(int n_c, int nslot, bool prefer_direct, int nroll) {
+// seq: time of a product that has a launch to itself, par: its share of a
+// launch of many; babies and all products of a Clenshaw plan are of the first
+// kind, so a small matrix takes fewer babies and more giants.  Below PS_MIN_S
+// babies the giants' rounding errors would outgrow the recurrence's.
+PsPlan ps_plan(int n_c, int nslot, double seq, double par, int nroll) {
     PsPlan p;
     p.n_c = n_c;
-    int best = 1 << 30;
+    double best = 1e300;
     const int smax = std::min(n_c, PS_MAX_S);
-    for (int s = 1; s <= smax; ++s) {
-        const int Q = (n_c - 1) / s;
-        const int cost = s + 2 * Q;
-        const int need_d = (s - 1) + std::max(0, Q - 1) + (Q > 0 ? PS_CQ + 1 : 0);
-        const int need_c = (s - 1) + nroll;
-        const bool fits_d = need_d <= nslot && Q <= PS_MAX_Q, fits_c = need_c <= nslot;
-        if (cost < best && (fits_d || fits_c)) {
-            best = cost;
-            p.s = s;
-            p.Q = Q;
-            p.direct = fits_d;
-        }
-    }
-    // where one product leaves SMs idle, a direct plan within a quarter of the
-    // best product count beats a Clenshaw plan: the products of a level share
-    // a launch
-    if (!p.direct && prefer_direct) {
-        int bd = 1 << 30;
-        PsPlan d = p;
-        for (int s = 1; s <= smax; ++s) {
+    for (int pass = 0; pass < 2 && best > 1e299; ++pass)   // second pass: fewer babies than PS_MIN_S
+        for (int s = pass == 0 ? std::min(PS_MIN_S, smax) : 1; s <= smax; ++s) {
             const int Q = (n_c - 1) / s;
             const int need_d = (s - 1) + std::max(0, Q - 1) + (Q > 0 ? PS_CQ + 1 : 0);
-            if (need_d <= nslot && Q <= PS_MAX_Q && s + 2 * Q < bd) {
-                bd = s + 2 * Q;
-                d.s = s;
-                d.Q = Q;
-                d.direct = true;
+            const int need_c = (s - 1) + nroll;
+            if (need_d <= nslot && Q <= PS_MAX_Q && s * seq + 2 * Q * par < best) {
+                best = s * seq + 2 * Q * par;
+                p.s = s;
+                p.Q = Q;
+                p.direct = true;
+            }
+            if (need_c <= nslot && (s + 2 * Q) * seq < best) {
+                best = (s + 2 * Q) * seq;
+                p.s = s;
+                p.Q = Q;
+                p.direct = false;
             }
         }
-        if (d.direct && bd <= best + best / 4) p = d;
-    }
     return p;
 }
 
@@ -445,13 +438,23 @@ double growth_limit(int l, int n_c) {
 
 // babies, giants and (with moments) m_l; the plan is kept in c.ps
 void ps64_pass1(Ctx& c, bool moments, cudaStream_t st) {
-    c.ps = ps_plan(c.n_c_cur, (int)c.ps_slot.size(), upper_tiles(c.K, 32) < 4 * 152, 2);
+    const double waves = upper_tiles(c.K, 16) / 152.0;
+    c.ps = ps_plan(c.n_c_cur, (int)c.ps_slot.size(), std::ceil(waves), waves, 2);
     const PsPlan& p = c.ps;
     Ps64 e{c, p, st};
     const int s = p.s, Q = p.Q;
     // T_s is needed as soon as there is a giant
     const int top = Q > 0 ? s : s - 1;
-    e.doubling(top, [&](int r) { return e.baby(r); }, 4.0);
+    for (int r = 1; r < top; ++r) {
+        Ps64Items it{};
+        it.A[0] = c.d_H;
+        it.B[0] = e.baby(r);
+        it.prev[0] = r > 1 ? e.baby(r - 1) : nullptr;
+        it.ident[0] = r == 1;
+        it.out[0] = const_cast<double*>(e.baby(r + 1));
+        it.first[1] = 1;
+        e.products(it, 1, 2.0, 4.0);
+    }
     double* D = c.d_wk;   // (Q + 1) s doubles, consumed before the moment weights are written there
     if (moments && s > 1) {
         PsList L{};

@@ -48,10 +48,13 @@ namespace {
 using namespace tc;
 
 constexpr int BM = 128, BN = 256, BK = 32, STAGES = 4;
-// k-blocks per accumulator promotion: chains of 24 additions.  Promoting every
-// 2 costs 0.4 us per promotion (16 products at K = 2000: 440 against 389 us)
-// for an error of P of 2.5e-5 instead of 2.7e-5 (K = 1230)
-constexpr int SUB = 4;
+// k-blocks per accumulator promotion (PstItem::sub).  Longer chains lean
+// further towards zero.  Error of P at K = 370 / 1230 against an exact
+// eigensolve with 1, 2 and 4 in all products: 1.2e-5 / 2.4e-5, 1.3e-5 / 2.5e-5,
+// 1.8e-5 / 2.8e-5 (the recurrence this replaced: 2.3e-5 / 3.6e-5); a density
+// matrix at K = 2000 takes 10.7, 10.3 and 9.9 ms.  The babies' bias acts as a
+// scale of H_N on every term, so they, and everything where K is small, take 1.
+constexpr int SUB_FINE = 1, SUB = 2, SUB_FINE_K = 2048;
 constexpr int A_BYTES = BM * BK * 2, B_BYTES = BN * BK * 2;
 constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;
 // warps 0 .. 3: producer, MMA issuer and two idle ones, so that the eight
@@ -245,7 +248,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
                 const Work w = work_at(t, items, nitems, sys);
                 const int nkt = w.nk * (w.it.last - w.it.first);
                 int kb = 0;   // within the operand pair
-                for (int k0 = 0; k0 < nkt && !*abort_flag; k0 += SUB, ++u) {
+                for (int k0 = 0; k0 < nkt && !*abort_flag; k0 += w.it.sub, ++u) {
                     const int a = (int)(u & 1);
                     if (!mbar_wait(&accempty[a], (uint32_t)(((u >> 1) & 1) ^ 1))) {
                         *abort_flag = 1;
@@ -254,7 +257,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
                     tc_fence_after();
                     const uint32_t d = tmem + (uint32_t)(a * BN);
                     bool first = true;
-                    for (int k = k0; k < min(nkt, k0 + SUB); ++k, ++g) {
+                    for (int k = k0; k < min(nkt, k0 + w.it.sub); ++k, ++g) {
                         const int s = (int)(g % STAGES);
                         if (*abort_flag || !mbar_wait(&full[s], (uint32_t)((g / STAGES) & 1))) {
                             *abort_flag = 1;
@@ -271,13 +274,16 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
                         const uint64_t bl = bt ? smem_desc_mn(sBl(s)) : smem_desc<BK * 2>(sBl(s));
                         // 16 k: 32 bytes along a K-major row, 16 rows of 128 bytes MN-major
                         const uint64_t as = at ? 128 : 2, bs = bt ? 128 : 2;
+                        // the small cross products first: additions to the accumulator lose bits
+                        // in proportion to what it holds already
 #pragma unroll
                         for (int kk = 0; kk < BK / 16; ++kk) {
-                            umma_f16(d, ah + kk * as, bh + kk * bs, idesc, first ? 0u : 1u);
-                            umma_f16(d, ah + kk * as, bl + kk * bs, idesc, 1u);
+                            umma_f16(d, ah + kk * as, bl + kk * bs, idesc, first ? 0u : 1u);
                             umma_f16(d, al + kk * as, bh + kk * bs, idesc, 1u);
                             first = false;
                         }
+#pragma unroll
+                        for (int kk = 0; kk < BK / 16; ++kk) umma_f16(d, ah + kk * as, bh + kk * bs, idesc, 1u);
                         umma_commit(&empty[s]);
                     }
                     umma_commit(&accfull[a]);
@@ -301,7 +307,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
         for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
             const Work w = work_at(t, items, nitems, sys);
             const PstSys& S = *w.S;
-            const int nunit = (w.nk * (w.it.last - w.it.first) + SUB - 1) / SUB, K = S.K, nb = S.nb;
+            const int nunit = (w.nk * (w.it.last - w.it.first) + w.it.sub - 1) / w.it.sub, K = S.K, nb = S.nb;
             int fr, fc;
             fold(w.p, w.j, nb, fr, fc);
             const int ld = nb * 256;
@@ -809,7 +815,8 @@ struct Queue {
         it.prev = prev;
         it.add = add_;
         it.out = out;
-        it.mode = mode;
+        it.mode = mode & ~PST_FINE;
+        it.sub = (mode & PST_FINE) || c.K <= SUB_FINE_K ? SUB_FINE : SUB;
         it.limit = (float)limit;
         if (launches.empty() || !open) {
             launches.push_back({(int)items.size(), 0, 0});
@@ -987,8 +994,9 @@ void pst_pass1(Ctx* const* cs, int n, const int* moments, cudaStream_t st) {
     for (int k = 0; k < n; ++k) {
         Ctx& c = *cs[k];
         const int nslot = (int)c.pst_slot.size();
-        // T_1 takes a slot here; one product's tiles below two waves: direct
-        c.ps = ps_plan(c.n_c_cur, nslot - 1, sys_tiles(c) < 2 * SMS, 6);
+        // T_1 takes a slot here
+        const double waves = sys_tiles(c) / (double)SMS;
+        c.ps = ps_plan(c.n_c_cur, nslot - 1, std::ceil(waves), waves, 6);
         tab[k] = PstSys{c.K, c.Kp / 256, c.d_pst_maps, c.d_pst_slots, c.d_flags};
     }
     DFT_CUDA_CHECK(cudaMemcpyAsync(lead.d_pst_sys, tab.data(), sizeof(PstSys) * n, cudaMemcpyHostToDevice, st));
@@ -1009,8 +1017,19 @@ void pst_pass1(Ctx* const* cs, int n, const int* moments, cudaStream_t st) {
             if (!any) break;
         }
     };
-    doubling([&](int k) { const PsPlan& p = cs[k]->ps; return p.Q > 0 ? p.s : p.s - 1; },
-             [&](int k, int r) { return View(*cs[k]).baby(r); }, [&](int, int) { return 4.0; });
+    for (int r = 1;; ++r) {
+        bool any = false;
+        for (int k = 0; k < n; ++k) {
+            const PsPlan& p = cs[k]->ps;
+            if (r >= (p.Q > 0 ? p.s : p.s - 1)) continue;
+            const View v(*cs[k]);
+            Q.add(k, *cs[k], {make_int2(v.baby(1), v.baby(r))}, r > 1 ? v.baby(r - 1) : -1, -1, v.baby(r + 1),
+                  PST_FINE | PST_ALPHA2 | (r == 1 ? PST_IDENT : 0), 4.0);
+            any = true;
+        }
+        Q.close();
+        if (!any) break;
+    }
     doubling([&](int k) { const PsPlan& p = cs[k]->ps; return p.direct ? p.Q : 0; },
              [&](int k, int q) { return View(*cs[k]).giant(q); },
              [&](int k, int q) { const PsPlan& p = cs[k]->ps; return q == p.Q ? growth_limit(p.Q * p.s, p.n_c) : 4.0; });

@@ -7,6 +7,7 @@
 namespace dft {
 
 constexpr int PS_MAX_S = 128;      // babies per plan, matrices per Gram or combination launch
+constexpr int PS_MIN_S = 24;
 constexpr int PS_MAX_Q = 1024;     // giants of a direct plan
 constexpr int PS_MAX_ITEMS = 32;   // products per launch
 constexpr int PS_CQ = 8;           // buffers a direct plan keeps for C_q and partial sums
