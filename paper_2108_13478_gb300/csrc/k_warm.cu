@@ -14,6 +14,9 @@
 
 #include <cuda_fp16.h>
 
+#include <algorithm>
+#include <cmath>
+
 namespace dft {
 namespace {
 
@@ -23,7 +26,19 @@ constexpr double RC = 8.0, RCUT = 12.0;
 constexpr int OW1 = 0, OB1 = OW1 + NH * ND, OW2 = OB1 + NH, OB2 = OW2 + NH * NH, OW3 = OB2 + NH,
               OB3 = OW3 + NH * NH, OW4 = OB3 + NH, OB4 = OW4 + NO * NH, NPARAM = OB4 + NO;
 
-__device__ __forceinline__ double width(int k) { return 0.5 * pow(6.0, k / 15.0); }
+// 1 / w_k^2 as the kernels use it, from the host (each thread computing the 16
+// powers for itself took 4 of the 4.7 ms of a training step at 47 atoms)
+struct Widths {
+    float iw2[NO];
+};
+Widths widths() {
+    Widths w;
+    for (int k = 0; k < NO; ++k) {
+        const double wk = 0.5 * std::pow(6.0, k / 15.0);
+        w.iw2[k] = (float)(1.0 / (wk * wk));
+    }
+    return w;
+}
 
 // one block of ND threads per atom, thread k summing component k over the
 // neighbours (distances and the cutoff function in FP64, the Gaussians in
@@ -84,38 +99,49 @@ __global__ void __launch_bounds__(NH) k_mlp_forward(const double* __restrict__ G
     }
 }
 
-// v0 = v_start + sum over atoms within RCUT of sum_k c_Ak exp(-r^2/w_k^2)
-__global__ void k_assemble(const double* __restrict__ xyz, int n, const double* __restrict__ coef, int nx, int ny,
-                           int nz, double ox, double oy, double oz, double h, const double* __restrict__ v_start,
-                           double* __restrict__ v0) {
-    long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= (long long)nx * ny * nz) return;
-    int ix = (int)(g % nx), iy = (int)((g / nx) % ny), iz = (int)(g / ((long long)nx * ny));
-    double x = ox + h * ix, y = oy + h * iy, z = oz + h * iz;
-    double inv_w2[NO];
-#pragma unroll
-    for (int k = 0; k < NO; ++k) {
-        double wk = width(k);
-        inv_w2[k] = 1.0 / (wk * wk);
-    }
-    // per atom the 16 Gaussians in FP32 (exp on the FP32 units), the sum over
-    // atoms in FP64
-    float iw2[NO];
-#pragma unroll
-    for (int k = 0; k < NO; ++k) iw2[k] = (float)inv_w2[k];
+// v0 = v_start + sum over atoms within RCUT of sum_k c_Ak exp(-r^2/w_k^2).
+// Atoms are sorted out in FP32 (with a margin above its rounding error), the
+// distance of those left is FP64, the 16 Gaussians FP32, the sum over atoms FP64.
+__global__ void __launch_bounds__(256) k_assemble(const double* __restrict__ xyz, int n, const double* __restrict__ coef,
+                                                  int nx, int ny, int nz, double ox, double oy, double oz, double h,
+                                                  Widths wd, const double* __restrict__ v_start, double* __restrict__ v0) {
+    constexpr int NA = 64;   // atoms staged at a time
+    __shared__ float4 af[NA];
+    __shared__ double ad[NA][3];
+    __shared__ float cf[NA][NO];
+    const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool in = g < (long long)nx * ny * nz;
+    const int ix = (int)(g % nx), iy = (int)((g / nx) % ny), iz = (int)(g / ((long long)nx * ny));
+    const double x = ox + h * ix, y = oy + h * iy, z = oz + h * iz;
+    // positions relative to the box, so that FP32 resolves 1e-5 bohr in boxes of any place
+    const float xf = (float)(h * ix), yf = (float)(h * iy), zf = (float)(h * iz);
+    constexpr float far2 = (float)(RCUT * RCUT) * 1.0001f + 0.01f;
     double s = 0.0;
-    for (int a = 0; a < n; ++a) {
-        double dx = x - xyz[3 * a], dy = y - xyz[3 * a + 1], dz = z - xyz[3 * a + 2];
-        double r2 = dx * dx + dy * dy + dz * dz;
-        if (r2 >= RCUT * RCUT) continue;
-        const double* c = coef + (long long)a * NO;
-        const float r2f = (float)r2;
-        float sa = 0.0f;
+    for (int a0 = 0; a0 < n; a0 += NA) {
+        const int m = min(NA, n - a0);
+        __syncthreads();
+        for (int e = threadIdx.x; e < m; e += blockDim.x) {
+            const double* p = xyz + 3 * (a0 + e);
+            af[e] = make_float4((float)(p[0] - ox), (float)(p[1] - oy), (float)(p[2] - oz), 0.f);
+            for (int d = 0; d < 3; ++d) ad[e][d] = p[d];
+        }
+        for (int e = threadIdx.x; e < m * NO; e += blockDim.x) cf[e / NO][e % NO] = (float)coef[(long long)a0 * NO + e];
+        __syncthreads();
+        for (int a = 0; a < m && in; ++a) {
+            const float4 q = af[a];
+            const float fx = xf - q.x, fy = yf - q.y, fz = zf - q.z;
+            if (fx * fx + fy * fy + fz * fz > far2) continue;
+            const double dx = x - ad[a][0], dy = y - ad[a][1], dz = z - ad[a][2];
+            const double r2 = dx * dx + dy * dy + dz * dz;
+            if (r2 >= RCUT * RCUT) continue;
+            const float r2f = (float)r2;
+            float sa = 0.0f;
 #pragma unroll
-        for (int k = 0; k < NO; ++k) sa = fmaf((float)c[k], expf(-r2f * iw2[k]), sa);
-        s += (double)sa;
+            for (int k = 0; k < NO; ++k) sa = fmaf(cf[a][k], expf(-r2f * wd.iw2[k]), sa);
+            s += (double)sa;
+        }
     }
-    v0[g] = (v_start ? v_start[g] : 0.0) + s;
+    if (in) v0[g] = (v_start ? v_start[g] : 0.0) + s;
 }
 
 template <int BS>
@@ -133,42 +159,70 @@ __device__ double block_sum(double v) {
     return r;
 }
 
-// dc_Ak = scale * sum over points within RCUT of atom A of resid * exp(-r^2/w_k^2)
+// part[A][slab][k] = sum over the points of z slab blockIdx.y within RCUT of
+// atom A = blockIdx.x of resid * exp(-r^2/w_k^2): warps over rows, lanes along
+// x, chains of at most 8 FP32 products before they meet in FP64 (16 FP64
+// multiply-adds per point kept the FP64 pipe busy for twice the Gaussians' time)
 __global__ void __launch_bounds__(256) k_assemble_adjoint(const double* __restrict__ xyz, const double* __restrict__ resid,
                                                           int nx, int ny, int nz, double ox, double oy, double oz,
-                                                          double h, double scale, double* __restrict__ dc) {
+                                                          double h, Widths wd, double* __restrict__ part) {
     const int a = blockIdx.x;
-    const double X = xyz[3 * a], Y = xyz[3 * a + 1], Z = xyz[3 * a + 2];
+    const double c[3] = {xyz[3 * a], xyz[3 * a + 1], xyz[3 * a + 2]}, o[3] = {ox, oy, oz};
     int lo[3], hi[3];
-    const double c[3] = {X, Y, Z}, o[3] = {ox, oy, oz};
     const int nn[3] = {nx, ny, nz};
     for (int d = 0; d < 3; ++d) {
         lo[d] = max(0, (int)ceil((c[d] - RCUT - o[d]) / h));
         hi[d] = min(nn[d] - 1, (int)floor((c[d] + RCUT - o[d]) / h));
     }
-    double inv_w2[NO], acc[NO];
+    double acc[NO];
+    float f[NO];
 #pragma unroll
     for (int k = 0; k < NO; ++k) {
-        double wk = width(k);
-        inv_w2[k] = 1.0 / (wk * wk);
         acc[k] = 0.0;
+        f[k] = 0.0f;
     }
-    const long long ex = hi[0] - lo[0] + 1, ey = hi[1] - lo[1] + 1, ez = hi[2] - lo[2] + 1;
-    const long long tot = (ex > 0 && ey > 0 && ez > 0) ? ex * ey * ez : 0;
-    for (long long q = threadIdx.x; q < tot; q += blockDim.x) {
-        int ix = lo[0] + (int)(q % ex), iy = lo[1] + (int)((q / ex) % ey), iz = lo[2] + (int)(q / (ex * ey));
-        double dx = ox + h * ix - X, dy = oy + h * iy - Y, dz = oz + h * iz - Z;
-        double r2 = dx * dx + dy * dy + dz * dz;
-        if (r2 >= RCUT * RCUT) continue;
-        double rv = resid[((long long)iz * ny + iy) * nx + ix];
-        const float r2f = (float)r2;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int ey = hi[1] - lo[1] + 1, ez = hi[2] - lo[2] + 1;
+    const int z0 = ez > 0 ? (int)((long long)ez * blockIdx.y / gridDim.y) : 0;
+    const int z1 = ez > 0 ? (int)((long long)ez * (blockIdx.y + 1) / gridDim.y) : 0;
+    const int rows = ey > 0 ? (z1 - z0) * ey : 0;
+    int held = 0;
+    for (int row = warp; row < rows; row += 8) {
+        const int iz = lo[2] + z0 + row / ey, iy = lo[1] + row % ey;
+        const double dy = oy + h * iy - c[1], dz = oz + h * iz - c[2];
+        const double q = dy * dy + dz * dz;
+        if (q >= RCUT * RCUT) continue;
+        const double* rv = resid + ((long long)iz * ny + iy) * nx;
+        for (int ix = lo[0] + lane; ix <= hi[0]; ix += 32) {
+            const double dx = ox + h * ix - c[0];
+            const double r2 = dx * dx + q;
+            if (r2 >= RCUT * RCUT) continue;
+            const float r2f = (float)r2, v = (float)rv[ix];
 #pragma unroll
-        for (int k = 0; k < NO; ++k) acc[k] = fma(rv, (double)expf(-r2f * (float)inv_w2[k]), acc[k]);
+            for (int k = 0; k < NO; ++k) f[k] = fmaf(v, expf(-r2f * wd.iw2[k]), f[k]);
+            if (++held == 8) {
+                held = 0;
+#pragma unroll
+                for (int k = 0; k < NO; ++k) {
+                    acc[k] += (double)f[k];
+                    f[k] = 0.0f;
+                }
+            }
+        }
     }
     for (int k = 0; k < NO; ++k) {
-        double v = block_sum<256>(acc[k]);
-        if (threadIdx.x == 0) dc[(long long)a * NO + k] = scale * v;
+        const double v = block_sum<256>(acc[k] + (double)f[k]);
+        if (threadIdx.x == 0) part[((long long)a * gridDim.y + blockIdx.y) * NO + k] = v;
     }
+}
+
+// dc_Ak = scale * the slabs' sums in order
+__global__ void k_adjoint_sum(int n, int slabs, double scale, const double* __restrict__ part, double* __restrict__ dc) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= n * NO) return;
+    double s = 0.0;
+    for (int q = 0; q < slabs; ++q) s += part[((long long)(e / NO) * slabs + q) * NO + e % NO];
+    dc[e] = scale * s;
 }
 
 // dL/dtheta accumulated (FP32 atomics) from dL/dc of every atom
@@ -293,7 +347,7 @@ void warm_forward(Ctx& c, const void* state, const double* v_start, double* v0, 
     k_mlp_forward<<<c.n_atoms, NH, 0, s>>>(c.d_wdesc, c.n_atoms, st_w16(const_cast<void*>(state)), c.d_wcoef,
                                            keep ? c.d_wz : nullptr);
     k_assemble<<<blocks_for(c.ng, 256), 256, 0, s>>>(c.d_xyz, c.n_atoms, c.d_wcoef, c.n[0], c.n[1], c.n[2],
-                                                     c.origin[0], c.origin[1], c.origin[2], c.h, v_start, v0);
+                                                     c.origin[0], c.origin[1], c.origin[2], c.h, widths(), v_start, v0);
     check_launch("warm_forward", 3);
 }
 
@@ -304,10 +358,13 @@ double warm_accumulate(Ctx& c, void* state, const double* v_start, const double*
     int np = (int)std::min<long long>(592, (c.ng + 255) / 256);
     k_sq_diff<<<np, 256, 0, s>>>(c.ng, c.d_nout, v_target, c.d_gtmp, c.d_part);
     k_sum<<<1, 256, 0, s>>>(np, c.d_part, h3, c.d_scal + SCAL_RES);
-    k_assemble_adjoint<<<c.n_atoms, 256, 0, s>>>(c.d_xyz, c.d_gtmp, c.n[0], c.n[1], c.n[2], c.origin[0], c.origin[1],
-                                                 c.origin[2], c.h, 2.0 * h3, c.d_wdc);
+    // enough slabs for about four blocks per SM; their sums in the Gram buffer, which is idle here
+    const int slabs = (int)std::max<long long>(1, std::min<long long>({16, 4 * 152 / c.n_atoms + 1, c.gram_cap / (NO * (long long)c.n_atoms)}));
+    k_assemble_adjoint<<<dim3(c.n_atoms, slabs), 256, 0, s>>>(c.d_xyz, c.d_gtmp, c.n[0], c.n[1], c.n[2], c.origin[0],
+                                                              c.origin[1], c.origin[2], c.h, widths(), c.d_gram);
+    k_adjoint_sum<<<blocks_for((long long)c.n_atoms * NO, 256), 256, 0, s>>>(c.n_atoms, slabs, 2.0 * h3, c.d_gram, c.d_wdc);
     k_mlp_backward<<<c.n_atoms, NH, 0, s>>>(c.d_wdesc, st_w16(state), c.d_wz, c.d_wdc, st_grad(state));
-    check_launch("warm_accumulate", 4);
+    check_launch("warm_accumulate", 5);
     double L = 0.0;
     DFT_CUDA_CHECK(cudaMemcpyAsync(&L, c.d_scal + SCAL_RES, sizeof(double), cudaMemcpyDeviceToHost, s));
     DFT_CUDA_CHECK(cudaStreamSynchronize(s));
