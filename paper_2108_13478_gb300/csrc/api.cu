@@ -286,7 +286,7 @@ size_t carve(Ctx& c, char* base) {
     size_t o_coef = L.off(sizeof(double) * (5 * (size_t)c.cheb_cap + 64));
     size_t o_mom = L.off(sizeof(double) * c.cheb_cap);
     size_t o_cos = L.off(sizeof(double) * 16 * (size_t)c.cheb_cap);
-    size_t o_wk = L.off(sizeof(double) * 4 * (size_t)c.cheb_cap);
+    size_t o_wk = L.off(sizeof(double) * (8 * (size_t)c.cheb_cap + 16));
     size_t o_part = L.off(sizeof(double) * c.part_cap);
     size_t o_flags = L.off(sizeof(int) * FLAG_COUNT);
     size_t o_vloc = L.off(G), o_nion = L.off(G), o_vks = L.off(G), o_nout = L.off(G), o_gtmp = L.off(G);
@@ -670,7 +670,7 @@ void dm_pass1(Ctx& c, bool moments, cudaStream_t s) {
 void dm_mu(Ctx& c, cudaStream_t s) {
     const int n_c = c.n_c_cur, M = 4 * n_c;
     launch_moment_weights(n_c, M, c.d_cos, c.d_mom, c.d_wk, s);
-    launch_mu_bisect(M, c.d_cos, c.d_wk, c.p.beta, c.p.n_electrons, c.d_scal, c.d_flags, s);
+    launch_mu_bisect(M, c.d_cos, c.d_wk, c.p.beta, c.p.n_electrons, c.d_part, c.d_scal, c.d_flags, s);
     launch_cheb_coeffs(n_c, M, c.d_cos, c.d_scal, c.p.beta, 0.0, false, c.d_coef, s);
 }
 

@@ -329,9 +329,11 @@ void launch_trace(int K, const double* X, double* out, cudaStream_t s);
 void launch_identity(int K, double* X, cudaStream_t s);
 // Lanczos on symmetric A: writes padded bounds to scal[SCAL_EMIN], scal[SCAL_EMAX]
 void lanczos_bounds(const Ctx& c, const double* A, int steps, cudaStream_t s);
-// the same with explicit buffers (vec: 4 K doubles, scal: SCAL_COUNT doubles)
+// the same with explicit buffers (vec: 4 K doubles, scal: SCAL_COUNT doubles,
+// state: TRI_STATE_DOUBLES)
+constexpr int TRI_STATE_DOUBLES = 4200;
 void lanczos_bounds_at(int K, const double* A, int steps, unsigned long long seed, double* vec, double* scal,
-                       cudaStream_t s);
+                       double* state, cudaStream_t s);
 
 // ---- Chebyshev engine (k_cheb.cu) ----
 void launch_cos_table(int M, double* cos_tab, cudaStream_t s);
@@ -339,7 +341,9 @@ void launch_cheb_coeffs(int n_c, int M, const double* cos_tab, const double* sca
                         double mu_override, bool use_override, double* coef, cudaStream_t s);
 void launch_moment_weights(int n_c, int M, const double* cos_tab, const double* mom, double* wk,
                            cudaStream_t s);
-void launch_mu_bisect(int M, const double* cos_tab, const double* wk, double beta, double n_e,
+constexpr int MU_STATE_DOUBLES = 160;
+// wk: M weights, then room for M + 1 suffix sums
+void launch_mu_bisect(int M, const double* cos_tab, double* wk, double beta, double n_e, double* state,
                       double* scal, int* flags, cudaStream_t s);
 void launch_moment_reduce(int nparts, const double* part, double* mom, int idx_even, int idx_odd,
                           double m0, const double* m1, cudaStream_t s);

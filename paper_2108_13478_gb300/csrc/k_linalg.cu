@@ -7,6 +7,8 @@
 // and L^-1 is kept, which gives the same operator to roundoff.
 #include "dft_internal.cuh"
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cmath>
 
@@ -72,12 +74,13 @@ __global__ void __launch_bounds__(256) k_dgemm(int M, int N, int Kd, double alph
     }
 }
 
-// Square K x K products with a triangular factor: the k range of each 64 x 64
+// Square K x K products with a triangular factor: the k range of each GB x GB
+// (64, or 32 where 64 would leave SMs idle: K < ~800)
 // output tile is cut to where the triangular operand is nonzero, and with
 // UPPER only tiles on or above the diagonal are computed (symmetric results,
 // mirrored afterwards).  KR: 0 full, 1 k < end of row tile, 2 k < end of
 // column tile, 3 k >= start of row tile, 4 k >= start of column tile.
-template <bool TA, bool TB, int KR, bool UPPER>
+template <int GB, bool TA, bool TB, int KR, bool UPPER>
 __global__ void __launch_bounds__(256) k_dgemm_tri(int K, const double* __restrict__ A, const double* __restrict__ B,
                                                    double* __restrict__ C) {
     if (UPPER && blockIdx.x < blockIdx.y) return;
@@ -90,7 +93,8 @@ __global__ void __launch_bounds__(256) k_dgemm_tri(int K, const double* __restri
     if (KR == 2) khi = min(K, n0 + GB);
     if (KR == 3) klo = m0;
     if (KR == 4) klo = n0;
-    double acc[4][4] = {};
+    constexpr int TM = GB / 16;
+    double acc[TM][TM] = {};
     for (int k0 = klo; k0 < khi; k0 += GK) {
         for (int e = threadIdx.x; e < GB * GK; e += 256) {
             int mm, kk;
@@ -111,24 +115,24 @@ __global__ void __launch_bounds__(256) k_dgemm_tri(int K, const double* __restri
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < GK; ++kk) {
-            double a[4], b[4];
+            double a[TM], b[TM];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
+            for (int i = 0; i < TM; ++i) a[i] = As[kk][ty + 16 * i];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
+            for (int j = 0; j < TM; ++j) b[j] = Bs[kk][tx + 16 * j];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < TM; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+                for (int j = 0; j < TM; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < TM; ++i) {
         int gm = m0 + ty + 16 * i;
         if (gm >= K) continue;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < TM; ++j) {
             int gn = n0 + tx + 16 * j;
             if (gn < K) C[(long long)gm * K + gn] = acc[i][j];
         }
@@ -390,42 +394,147 @@ __global__ void __launch_bounds__(256) k_gemv(int K, const double* __restrict__ 
 
 // single CTA: alpha_j = w.v_j; w -= alpha v_j + beta_j v_{j-1}; (twice, for
 // local orthogonality); beta_{j+1} = |w|; v_{j+1} = w / beta_{j+1}
-__global__ void __launch_bounds__(1024) k_lanczos_update(int K, int j, double* w, const double* vj,
+// (NT threads: each FP64 warp instruction takes 16 clocks of the SM, so the
+// reductions cost in proportion to the warps; a small K takes few)
+template <int NT>
+__global__ void __launch_bounds__(NT) k_lanczos_update(int K, int j, double* w, const double* vj,
                                                          const double* vjm1, double* vnext, double* scal) {
     __shared__ double sh;
     double s = 0.0;
-    for (int i = threadIdx.x; i < K; i += 1024) s = fma(w[i], vj[i], s);
-    s = block_sum<1024>(s);
+    for (int i = threadIdx.x; i < K; i += NT) s = fma(w[i], vj[i], s);
+    s = block_sum<NT>(s);
     if (threadIdx.x == 0) sh = s;
     __syncthreads();
     double alpha = sh;
     double beta = scal[SCAL_BETA + j];
-    for (int i = threadIdx.x; i < K; i += 1024) w[i] = w[i] - alpha * vj[i] - (j > 0 ? beta * vjm1[i] : 0.0);
+    for (int i = threadIdx.x; i < K; i += NT) w[i] = w[i] - alpha * vj[i] - (j > 0 ? beta * vjm1[i] : 0.0);
     __syncthreads();
     // second pass against v_j (cheap reorthogonalisation)
     s = 0.0;
-    for (int i = threadIdx.x; i < K; i += 1024) s = fma(w[i], vj[i], s);
-    s = block_sum<1024>(s);
+    for (int i = threadIdx.x; i < K; i += NT) s = fma(w[i], vj[i], s);
+    s = block_sum<NT>(s);
     if (threadIdx.x == 0) sh = s;
     __syncthreads();
     double c = sh;
     alpha += c;
     s = 0.0;
-    for (int i = threadIdx.x; i < K; i += 1024) {
+    for (int i = threadIdx.x; i < K; i += NT) {
         double v = w[i] - c * vj[i];
         w[i] = v;
         s = fma(v, v, s);
     }
-    s = block_sum<1024>(s);
+    s = block_sum<NT>(s);
     if (threadIdx.x == 0) sh = sqrt(s);
     __syncthreads();
     double bn = sh;
     double inv = bn > 0.0 ? 1.0 / bn : 0.0;
-    for (int i = threadIdx.x; i < K; i += 1024) vnext[i] = w[i] * inv;
+    for (int i = threadIdx.x; i < K; i += NT) vnext[i] = w[i] * inv;
     if (threadIdx.x == 0) {
         scal[SCAL_ALPHA + j] = alpha;
         scal[SCAL_BETA + j + 1] = bn;
     }
+}
+
+// The whole Lanczos run of a small matrix as one launch of a cluster of CL
+// CTAs: each holds all of v_j and v_{j-1} and owns every CL-th run of rows; per step three
+// cluster barriers, after the partial sums of alpha, of the correction c and of
+// |w|^2 (published with the CTA's part of w) have been written to all CTAs.
+// 64 steps as 128 launches took 0.65 ms at K = 370 (and, with a batch's host
+// threads launching together, several ms of the driver's lock).
+constexpr int LC_CL = 8, LC_THREADS = 128, LC_MAX_K = 448;   // K: a CTA's rows of A stay in its shared memory
+__global__ void __cluster_dims__(LC_CL, 1, 1) __launch_bounds__(LC_THREADS)
+    k_lanczos_cluster(int K, int m, unsigned long long seed, const double* __restrict__ A, double* scal) {
+    namespace cgx = cooperative_groups;
+    cgx::cluster_group cl = cgx::this_cluster();
+    __shared__ double vj[LC_MAX_K], vp[LC_MAX_K], w[LC_MAX_K], part[3][LC_CL];
+    __shared__ double sh;
+    const int rank = (int)cl.block_rank(), t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int per = (K + LC_CL - 1) / LC_CL, r0 = min(K, rank * per), r1 = min(K, r0 + per);
+    extern __shared__ double rows[];
+    for (int e = t; e < (r1 - r0) * K; e += LC_THREADS) rows[e] = A[(long long)r0 * K + e];
+    // start vector, formed by every CTA for itself
+    double s = 0.0;
+    for (int i = t; i < K; i += LC_THREADS) {
+        const double r = (double)(splitmix64(seed * 0x100000001B3ull + (unsigned long long)i) >> 11) * 0x1.0p-53 - 0.5;
+        vj[i] = r;
+        vp[i] = 0.0;
+        s += r * r;
+    }
+    s = block_sum<LC_THREADS>(s);
+    if (t == 0) sh = sqrt(s);
+    __syncthreads();
+    for (int i = t; i < K; i += LC_THREADS) vj[i] /= sh;
+    double beta = 0.0;
+    if (rank == 0 && t == 0) scal[SCAL_BETA] = 0.0;
+    // this CTA's partial sum to slot `which` of every CTA
+    auto publish = [&](double x, int which) {
+        x = block_sum<LC_THREADS>(x);
+        if (t == 0) sh = x;
+        __syncthreads();
+        if (t < LC_CL) cl.map_shared_rank(&part[which][rank], t)[0] = sh;
+    };
+    auto total = [&](int which) {
+        double x = 0.0;
+        for (int q = 0; q < LC_CL; ++q) x += part[which][q];
+        return x;
+    };
+    cl.sync();
+    for (int j = 0; j < m; ++j) {
+        s = 0.0;
+        // one row per 8 lanes: three shuffle additions per row instead of five
+        for (int r = r0 + 4 * warp + (lane >> 3); r - (lane >> 3) < r1; r += 4 * LC_THREADS / 32) {
+            const double* a = rows + (r - r0) * K;
+            double x = 0.0, y = 0.0;
+            if (r < r1)
+                for (int c = lane & 7; c < K; c += 16) {
+                    x = fma(a[c], vj[c], x);
+                    if (c + 8 < K) y = fma(a[c + 8], vj[c + 8], y);
+                }
+            x += y;
+            for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            if ((lane & 7) == 0 && r < r1) {
+                w[r] = x;
+                s = fma(x, vj[r], s);
+            }
+        }
+        publish(s, 0);
+        cl.sync();
+        double alpha = total(0);
+        s = 0.0;
+        for (int r = r0 + t; r < r1; r += LC_THREADS) {
+            const double x = w[r] - alpha * vj[r] - beta * vp[r];
+            w[r] = x;
+            s = fma(x, vj[r], s);
+        }
+        publish(s, 1);
+        cl.sync();
+        const double c = total(1);   // second pass against v_j (local orthogonality)
+        alpha += c;
+        s = 0.0;
+        for (int r = r0 + t; r < r1; r += LC_THREADS) {
+            const double x = w[r] - c * vj[r];
+            s = fma(x, x, s);
+            w[r] = x;
+            for (int q = 0; q < LC_CL; ++q)
+                if (q != rank) cl.map_shared_rank(&w[r], q)[0] = x;
+        }
+        publish(s, 2);
+        cl.sync();
+        const double bn = sqrt(total(2)), inv = bn > 0.0 ? 1.0 / bn : 0.0;
+        for (int i = t; i < K; i += LC_THREADS) {
+            vp[i] = vj[i];
+            vj[i] = w[i] * inv;
+        }
+        beta = bn;
+        if (rank == 0 && t == 0) {
+            scal[SCAL_ALPHA + j] = alpha;
+            scal[SCAL_BETA + j + 1] = bn;
+        }
+        __syncthreads();
+        // w of the next step is written by its own CTA only, and read here above by
+        // threads of this CTA; others write into it after the next two barriers
+    }
+    cl.sync();   // no CTA leaves while its shared memory may still be written
 }
 
 // number of eigenvalues of the m x m tridiagonal below x (Sturm sequence)
@@ -441,42 +550,71 @@ __device__ int sturm_count(const double* al, const double* be, int m, double x) 
     return cnt;
 }
 
-// extreme eigenvalues of the Lanczos tridiagonal by multisection on the
-// Sturm count: warp 0 seeks the smallest, warp 1 the largest; every round
-// each lane counts the eigenvalues below one of 32 interior points and the
-// bracket shrinks 33-fold to the two points around the sought one.  The
-// bounds are padded by 2% of the width on each side (the paper does not say
-// how E_min and E_max are found).
-__global__ void __launch_bounds__(64) k_tridiag_bounds(int m, double* scal) {
+// extreme eigenvalues of the Lanczos tridiagonal by multisection on the Sturm
+// count, one launch per round: TRI_BLOCKS blocks of 32 points for the smallest
+// (blocks 0 ..) and as many for the largest eigenvalue, so the bracket shrinks
+// by 32 TRI_BLOCKS + 1 per round; every warp first reduces the counts of the
+// round before to its bracket.  One warp per block and SM: the divisions of
+// the Sturm sequence keep the SM's FP64 pipe busy by themselves (both ends on
+// one SM with 32 points each took 417 us).  The last round pads the bounds
+// by 2% of the width on each side (the paper does not say how E_min and E_max
+// are found).  state: two rounds' {a, b} and counts per end.
+constexpr int TRI_BLOCKS = 32, TRI_PTS = 32 * TRI_BLOCKS, TRI_ROUNDS = 6;
+constexpr int TRI_STATE = 2 + TRI_PTS;   // doubles per end and round
+__global__ void __launch_bounds__(32) k_tridiag_round(int round, int m, double* scal, double* state) {
     const double* al = scal + SCAL_ALPHA;
     const double* be = scal + SCAL_BETA;
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double lo = 1e300, hi = -1e300;
-    for (int i = 0; i < m; ++i) {
-        double r = (i > 0 ? fabs(be[i]) : 0.0) + (i + 1 < m ? fabs(be[i + 1]) : 0.0);
-        lo = fmin(lo, al[i] - r);
-        hi = fmax(hi, al[i] + r);
+    const int lane = threadIdx.x;
+    auto bracket = [&](int end, double& a, double& b) {
+        const int target = end == 0 ? 1 : m;
+        if (round == 0) {
+            double lo = 1e300, hi = -1e300;
+            for (int i = lane; i < m; i += 32) {
+                const double r = (i > 0 ? fabs(be[i]) : 0.0) + (i + 1 < m ? fabs(be[i + 1]) : 0.0);
+                lo = fmin(lo, al[i] - r);
+                hi = fmax(hi, al[i] + r);
+            }
+            for (int o = 16; o > 0; o >>= 1) {
+                lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+                hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+            }
+            a = lo;   // count(a) < target <= count(b)
+            b = hi;
+            return;
+        }
+        const double* st = state + (((round + 1) & 1) * 2 + end) * TRI_STATE;
+        int j = TRI_PTS;   // first point with count >= target
+        for (int i = lane; i < TRI_PTS; i += 32)
+            if (st[2 + i] >= (double)target) {
+                j = i;
+                break;
+            }
+        for (int o = 16; o > 0; o >>= 1) j = min(j, __shfl_xor_sync(0xffffffffu, j, o));
+        const double w = (st[1] - st[0]) / (TRI_PTS + 1);
+        a = j == 0 ? st[0] : st[0] + w * j;
+        b = j == TRI_PTS ? st[1] : st[0] + w * (j + 1);
+    };
+    if (round == TRI_ROUNDS) {
+        double a, b, e[2];
+        for (int end = 0; end < 2; ++end) {
+            bracket(end, a, b);
+            e[end] = 0.5 * (a + b);
+        }
+        if (lane == 0) {
+            const double pad = 0.02 * (e[1] - e[0]) + 1e-3;
+            scal[SCAL_EMIN] = e[0] - pad;
+            scal[SCAL_EMAX] = e[1] + pad;
+        }
+        return;
     }
-    // invariant: count(a) < target <= count(b)
-    const int target = w == 0 ? 1 : m;
-    double a = lo, b = hi;
-    for (int it = 0; it < 64; ++it) {
-        const double x = a + (b - a) * (double)(lane + 1) / 33.0;
-        const unsigned ge = __ballot_sync(0xffffffffu, sturm_count(al, be, m, x) >= target);
-        const int j = ge ? __ffs(ge) - 1 : 32;
-        const double na = j == 0 ? a : a + (b - a) * (double)j / 33.0;
-        const double nb = j == 32 ? b : a + (b - a) * (double)(j + 1) / 33.0;
-        if (!(na > a || nb < b)) break;   // the bracket is at FP64 resolution
-        a = na;
-        b = nb;
-    }
-    __shared__ double e[2];
-    if (lane == 0) e[w] = 0.5 * (a + b);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const double pad = 0.02 * (e[1] - e[0]) + 1e-3;
-        scal[SCAL_EMIN] = e[0] - pad;
-        scal[SCAL_EMAX] = e[1] + pad;
+    const int end = blockIdx.x / TRI_BLOCKS, p = (blockIdx.x % TRI_BLOCKS) * 32 + lane;
+    double a, b;
+    bracket(end, a, b);
+    double* st = state + ((round & 1) * 2 + end) * TRI_STATE;
+    st[2 + p] = (double)sturm_count(al, be, m, a + (b - a) / (TRI_PTS + 1) * (p + 1));
+    if (p == 0) {
+        st[0] = a;
+        st[1] = b;
     }
 }
 
@@ -516,20 +654,30 @@ int cholesky_inplace(double* A, int K, int* d_flag, cudaStream_t s) {
 
 void congruence_lower(int K, const double* Linv, const double* F, double* tmp, double* out, cudaStream_t s) {
     // out = Linv F Linv^T, Linv lower triangular, F and out symmetric
-    const int nb = (K + GB - 1) / GB;
-    dim3 grid(nb, nb);
-    k_dgemm_tri<false, false, 1, false><<<grid, 256, 0, s>>>(K, Linv, F, tmp);
-    k_dgemm_tri<false, true, 2, true><<<grid, 256, 0, s>>>(K, tmp, Linv, out);
+    auto go = [&](auto tile) {
+        constexpr int TB = decltype(tile)::value;
+        const int nb = (K + TB - 1) / TB;
+        const dim3 grid(nb, nb);
+        k_dgemm_tri<TB, false, false, 1, false><<<grid, 256, 0, s>>>(K, Linv, F, tmp);
+        k_dgemm_tri<TB, false, true, 2, true><<<grid, 256, 0, s>>>(K, tmp, Linv, out);
+    };
+    if ((K + 63) / 64 * ((K + 63) / 64) < 152) go(std::integral_constant<int, 32>{});
+    else go(std::integral_constant<int, 64>{});
     k_mirror_upper<<<blocks_for((long long)K * K, 256), 256, 0, s>>>(K, out);
     check_launch("congruence_lower", 3);
 }
 
 void congruence_lower_t(int K, const double* Linv, const double* R, double* tmp, double* out, cudaStream_t s) {
     // out = Linv^T R Linv, Linv lower triangular, R and out symmetric
-    const int nb = (K + GB - 1) / GB;
-    dim3 grid(nb, nb);
-    k_dgemm_tri<true, false, 3, false><<<grid, 256, 0, s>>>(K, Linv, R, tmp);
-    k_dgemm_tri<false, false, 4, true><<<grid, 256, 0, s>>>(K, tmp, Linv, out);
+    auto go = [&](auto tile) {
+        constexpr int TB = decltype(tile)::value;
+        const int nb = (K + TB - 1) / TB;
+        const dim3 grid(nb, nb);
+        k_dgemm_tri<TB, true, false, 3, false><<<grid, 256, 0, s>>>(K, Linv, R, tmp);
+        k_dgemm_tri<TB, false, false, 4, true><<<grid, 256, 0, s>>>(K, tmp, Linv, out);
+    };
+    if ((K + 63) / 64 * ((K + 63) / 64) < 152) go(std::integral_constant<int, 32>{});
+    else go(std::integral_constant<int, 64>{});
     k_mirror_upper<<<blocks_for((long long)K * K, 256), 256, 0, s>>>(K, out);
     check_launch("congruence_lower_t", 3);
 }
@@ -658,44 +806,41 @@ void launch_identity(int K, double* X, cudaStream_t s) {
     check_launch("identity");
 }
 
-void lanczos_bounds(const Ctx& c, const double* A, int steps, cudaStream_t s) {
-    int K = c.K;
-    int m = std::max(2, std::min(steps, std::min(K, 120)));
-    double* v[3] = {c.d_vec, c.d_vec + K, c.d_vec + 2 * K};
-    double* w = c.d_vec + 3 * K;
-    k_lanczos_start<<<1, 1024, 0, s>>>(K, c.p.seed, v[0], c.d_scal);
-    check_launch("lanczos_start");
-    for (int j = 0; j < m; ++j) {
-        double* vj = v[j % 3];
-        double* vjm1 = v[(j + 2) % 3];
-        double* vn = v[(j + 1) % 3];
-        k_gemv<<<blocks_for(K, 8), 256, 0, s>>>(K, A, vj, w);
-        k_lanczos_update<<<1, 1024, 0, s>>>(K, j, w, vj, vjm1, vn, c.d_scal);
-        check_launch("lanczos_step", 2);
-    }
-    k_tridiag_bounds<<<1, 64, 0, s>>>(m, c.d_scal);
-    check_launch("lanczos");
-}
-
 // Lanczos bounds with caller-given buffers: vec holds 4 K doubles, scal
-// SCAL_COUNT doubles; the padded bounds land in scal[SCAL_EMIN], scal[SCAL_EMAX]
+// SCAL_COUNT doubles, state TRI_STATE_DOUBLES; the padded bounds land in
+// scal[SCAL_EMIN], scal[SCAL_EMAX]
 void lanczos_bounds_at(int K, const double* A, int steps, unsigned long long seed, double* vec, double* scal,
-                       cudaStream_t s) {
+                       double* state, cudaStream_t s) {
+    static_assert(4 * TRI_STATE <= TRI_STATE_DOUBLES, "scratch of the tridiagonal bounds");
     int m = std::max(2, std::min(steps, std::min(K, 120)));
     double* v[3] = {vec, vec + K, vec + 2 * K};
     double* w = vec + 3 * K;
-    k_lanczos_start<<<1, 1024, 0, s>>>(K, seed, v[0], scal);
-    check_launch("lanczos_start");
-    for (int j = 0; j < m; ++j) {
+    if (K <= LC_MAX_K) {
+        constexpr int most = (LC_MAX_K + LC_CL - 1) / LC_CL * LC_MAX_K * (int)sizeof(double);
+        static_assert(most <= 204800, "rows of a CTA in shared memory");
+        DFT_CUDA_CHECK(cudaFuncSetAttribute(k_lanczos_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+        k_lanczos_cluster<<<LC_CL, LC_THREADS, (size_t)((K + LC_CL - 1) / LC_CL) * K * sizeof(double), s>>>(K, m, seed, A, scal);
+        check_launch("lanczos_cluster");
+    } else {
+        k_lanczos_start<<<1, 1024, 0, s>>>(K, seed, v[0], scal);
+        check_launch("lanczos_start");
+    }
+    for (int j = 0; j < m && K > LC_MAX_K; ++j) {
         double* vj = v[j % 3];
         double* vjm1 = v[(j + 2) % 3];
         double* vn = v[(j + 1) % 3];
         k_gemv<<<blocks_for(K, 8), 256, 0, s>>>(K, A, vj, w);
-        k_lanczos_update<<<1, 1024, 0, s>>>(K, j, w, vj, vjm1, vn, scal);
+        // 128 threads up to K = 1024
+        if (K <= 1024) k_lanczos_update<128><<<1, 128, 0, s>>>(K, j, w, vj, vjm1, vn, scal);
+        else k_lanczos_update<256><<<1, 256, 0, s>>>(K, j, w, vj, vjm1, vn, scal);
         check_launch("lanczos_step", 2);
     }
-    k_tridiag_bounds<<<1, 64, 0, s>>>(m, scal);
-    check_launch("lanczos");
+    for (int r = 0; r <= TRI_ROUNDS; ++r) k_tridiag_round<<<r < TRI_ROUNDS ? 2 * TRI_BLOCKS : 1, 32, 0, s>>>(r, m, scal, state);
+    check_launch("lanczos", TRI_ROUNDS + 1);
+}
+
+void lanczos_bounds(const Ctx& c, const double* A, int steps, cudaStream_t s) {
+    lanczos_bounds_at(c.K, A, steps, c.p.seed, c.d_vec, c.d_scal, c.d_gram, s);
 }
 
 }  // namespace dft

@@ -24,7 +24,7 @@
 // the limit of every kernel here).  All operands are symmetric polynomials
 // of H_N, so products are formed on upper tiles and mirrored.  Whole density
 // matrix at tail 1e-10 (N_C ~ 2900), the three-term recurrence with full
-// products before and this now: K = 80 134 -> 8.8 ms, K = 370 559 -> 20.0 ms,
+// products before and this now: K = 80 133 -> 4.7 ms, K = 370 560 -> 14.2 ms,
 // error against an exact eigensolve 6e-14 relative on both sides.
 #include "dft_internal.cuh"
 #include "ps_plan.cuh"
@@ -47,16 +47,16 @@ __device__ __forceinline__ void upper_tile(int t, int nb, int& i, int& j) {
 
 // out_y = alpha sum_{f_y <= p < f_{y+1}} A_p B_p - prev_y on the upper TB x TB
 // tiles, mirrored; prev: none, a matrix (may be out itself) or the identity.
-// One tile per block, TB^2 / 8 threads (2 x 4 sums each; 2 x 2 at TB = 16):
+// One tile per block of 128 threads (2 x 4 sums each; 1 x 2 at TB = 16):
 // the FP64 pipe needs one warp per scheduler with a few independent FMAs, so
 // small tiles cost nothing and spread a small K over the SMs.  32 x 32 tiles
 // read 16 bytes per 32 FMA from L2.
 template <int TB>
-__global__ void __launch_bounds__(TB * TB / (TB == 32 ? 8 : 4)) k_ps_prod(int K, Ps64Items it, double alpha,
+__global__ void __launch_bounds__(128) k_ps_prod(int K, Ps64Items it, double alpha,
                                                                           double limit, int* __restrict__ flags) {
     constexpr int KS = 32;
-    constexpr int NT = TB * TB / (TB == 32 ? 8 : 4);
-    constexpr int MR = 2, MC = TB == 32 ? 4 : 2;     // sums per thread
+    constexpr int NT = 128;                          // four warps: one for each quarter of the SM's FP64 pipe
+    constexpr int MR = TB == 32 ? 2 : 1, MC = TB == 32 ? 4 : 2;   // sums per thread
     constexpr int TX = TB / MC;                      // threads along a row
     __shared__ double As[KS][TB + 1];
     __shared__ double Bs[KS][TB + 1];
@@ -212,20 +212,17 @@ __global__ void __launch_bounds__(256) k_ps_add(int K, int np, Ps64Out part, con
 }
 
 // partial Gram sums <G_q, T_r> over the upper 32 x 32 tiles blockIdx.x,
-// + gridDim.x, ... (off-diagonal elements twice); 64 x 64 pairs per block of
-// 256 threads, 4 x 4 each
+// + gridDim.x, ... (off-diagonal elements twice); 64 x 32 pairs per block of
+// 256 threads, 4 x 2 each
 __global__ void __launch_bounds__(256) k_ps_gram(int K, PsList G, int nq, PsList T, int s, double* __restrict__ part) {
-    __shared__ double g[32][65], t[32][65];
+    __shared__ double g[32][65], t[32][33];
     const int nb = (K + 31) / 32, nt = nb * (nb + 1) / 2;
-    const int qb = blockIdx.y * 64, rb = blockIdx.z * 64;
+    const int qb = blockIdx.y * 64, rb = blockIdx.z * 32;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    double acc[4][4] = {};
-    int ni = 0, nj = 0;   // live sums per thread along q and r
+    double acc[4][2] = {};
+    int ni = 0;   // live sums per thread along q
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        ni += qb + ty + 16 * i < nq;
-        nj += rb + tx + 16 * i < s;
-    }
+    for (int i = 0; i < 4; ++i) ni += qb + ty + 16 * i < nq;
     for (int tile = blockIdx.x; tile < nt; tile += gridDim.x) {
         int ti, tj;
         upper_tile(tile, nb, ti, tj);
@@ -235,22 +232,22 @@ __global__ void __launch_bounds__(256) k_ps_gram(int K, PsList G, int nq, PsList
                 const int c = e & 31, m = e >> 5, gc = tj * 32 + c;
                 const double w = gc >= K || gc < row ? 0.0 : (gc == row ? 1.0 : 2.0);
                 g[c][m] = (w != 0.0 && qb + m < nq) ? w * G.p[qb + m][(long long)row * K + gc] : 0.0;
-                t[c][m] = (gc < K && rb + m < s && rb + m > 0) ? T.p[rb + m][(long long)row * K + gc] : 0.0;
+                if (m < 32) t[c][m] = (gc < K && rb + m < s && rb + m > 0) ? T.p[rb + m][(long long)row * K + gc] : 0.0;
             }
             __syncthreads();
             if (ni == 0) continue;
 #pragma unroll 4
             for (int c = 0; c < 32; ++c) {
-                double a[4], b[4];
+                double a[4], b[2];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) a[i] = g[c][ty + 16 * i];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) b[j] = t[c][tx + 16 * j];
+                for (int j = 0; j < 2; ++j) b[j] = t[c][tx + 16 * j];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     if (i >= ni) break;
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+                    for (int j = 0; j < 2; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
                 }
             }
         }
@@ -259,7 +256,7 @@ __global__ void __launch_bounds__(256) k_ps_gram(int K, PsList G, int nq, PsList
     for (int i = 0; i < 4; ++i) {
         const int q = qb + ty + 16 * i;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < 2; ++j) {
             const int r = rb + tx + 16 * j;
             if (q < nq && r < s) part[((long long)blockIdx.x * nq + q) * s + r] = acc[i][j];
         }
@@ -386,7 +383,7 @@ struct Ps64 {
         if ((long long)big * n >= 2 * 152) {
             k_ps_prod<32><<<dim3(big, n), 128, 0, st>>>(c.K, it, alpha, limit, c.d_flags);
         } else {
-            k_ps_prod<16><<<dim3(upper_tiles(c.K, 16), n), 64, 0, st>>>(c.K, it, alpha, limit, c.d_flags);
+            k_ps_prod<16><<<dim3(upper_tiles(c.K, 16), n), 128, 0, st>>>(c.K, it, alpha, limit, c.d_flags);
         }
         check_launch("ps_prod");
     }
@@ -420,7 +417,7 @@ struct Ps64 {
         const int nt = upper_tiles(c.K, 32);
         const int nsplit = (int)std::max<long long>(1, std::min<long long>({(long long)nt, 2 * 152LL, c.gram_cap / ((long long)nq * s)}));
         if ((long long)nq * s > c.gram_cap) throw Error(DFT_EINTERNAL, "Gram partials exceed their buffer");
-        k_ps_gram<<<dim3(nsplit, (nq + 63) / 64, (s + 63) / 64), 256, 0, st>>>(c.K, G, nq, T, s, c.d_gram);
+        k_ps_gram<<<dim3(nsplit, (nq + 63) / 64, (s + 31) / 32), 256, 0, st>>>(c.K, G, nq, T, s, c.d_gram);
         k_ps_gram_sum<<<(nq * s + 255) / 256, 256, 0, st>>>(nsplit, nq * s, c.d_gram, D + (long long)q0 * s);
         k_ps_trace<<<nq, 128, 0, st>>>(c.K, G, D + (long long)q0 * s, s);
         check_launch("ps_gram", 3);

@@ -78,7 +78,7 @@ extern "C" dft_status dft_spectral_bounds_static(dft_ctx* ctx, const double* F, 
         // previous call's contents)
         DFT_CUDA_CHECK(cudaMemsetAsync(scal, 0, sizeof(double) * SCAL_COUNT, s));
         congruence_lower(K, c.d_Linv, F, tmp, Ft, s);
-        lanczos_bounds_at(K, Ft, c.p.lanczos_steps > 0 ? c.p.lanczos_steps : 64, c.p.seed, vec, scal, s);
+        lanczos_bounds_at(K, Ft, c.p.lanczos_steps > 0 ? c.p.lanczos_steps : 64, c.p.seed, vec, scal, tmp, s);   // tmp is free again
         DFT_CUDA_CHECK(cudaMemcpyAsync(bounds, scal + SCAL_EMIN, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
         DFT_CUDA_CHECK(cudaStreamSynchronize(s));
         c.err.clear();
