@@ -21,6 +21,8 @@
 // host checking for remaining columns between graphs.
 #include "dft_internal.cuh"
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -332,6 +334,187 @@ __global__ void k_pcg_precond(int K, int B, BJ bj, const double* __restrict__ r,
     }
 }
 
+// A whole solve of NC columns as one launch of a cluster of PC_CL CTAs (columns
+// do not depend on one another).  Each CTA owns a run of rows (whole atoms, so
+// that the preconditioner is local), keeps its rows of S in shared memory where they fit
+// (`cached`: room for that many entries), and holds all of p.  Per iteration
+// three cluster barriers: after the partial sums of p.q, after those of r.r and
+// r.z, after the new p.  The FP64 pipe bounds the product; with seven
+// launches per iteration and a host check every eight, an iteration of 32
+// columns at K = 370 took 72 us.
+constexpr int PC_CL = 8, PC_THREADS = 384, PC_WARPS = PC_THREADS / 32;
+struct PcRows {
+    int at[PC_CL + 1];   // first row of each CTA
+};
+template <int NC>
+size_t pc_smem(int K, int rows, int cached) {
+    return sizeof(double) * ((size_t)K * NC + 4 * (size_t)rows * NC + cached) + sizeof(int) * (size_t)cached;
+}
+template <int NC>
+__global__ void __cluster_dims__(PC_CL, 1, 1) __launch_bounds__(PC_THREADS)
+    k_pcg_cluster(int K, int B, PcRows pr, int max_rows, int cached, const int* __restrict__ ptr,
+                  const int* __restrict__ idx, const double* __restrict__ val, BJ bj, const double* __restrict__ b,
+                  double* __restrict__ x_out, double tol2, int limit, Cols cs) {
+    namespace cgx = cooperative_groups;
+    cgx::cluster_group cl = cgx::this_cluster();
+    extern __shared__ __align__(16) double pc_sh[];
+    double* p = pc_sh;                                  // [K][NC]
+    double* x = p + (size_t)K * NC;                     // [NC][rows], as r, z, q
+    double* r = x + (size_t)max_rows * NC;
+    double* z = r + (size_t)max_rows * NC;
+    double* q = z + (size_t)max_rows * NC;
+    double* sv = q + (size_t)max_rows * NC;             // cached rows of S
+    int* si = (int*)(sv + cached);
+    __shared__ double part[3][PC_CL][NC], red[2][PC_WARPS], alpha[NC], beta[NC], rz[NC], bn2[NC], rr[NC];
+    __shared__ int act[NC], iters[NC], any;
+    const int rank = (int)cl.block_rank(), t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int r0 = pr.at[rank], rows = pr.at[rank + 1] - r0;
+    const int c0 = (int)(blockIdx.x / PC_CL) * NC;
+    const int e0 = ptr[r0], ne = ptr[r0 + rows] - e0;
+    const bool in_sh = ne <= cached;
+    if (in_sh)
+        for (int e = t; e < ne; e += PC_THREADS) {
+            sv[e] = val[e0 + e];
+            si[e] = idx[e0 + e];
+        }
+    // element-wise steps: warp w takes column w % NC, rows 32 (w / NC) + lane, ...
+    static_assert(PC_WARPS % NC == 0, "whole warps per column");
+    const int u = warp % NC, i0 = warp / NC * 32 + lane, di = PC_WARPS / NC * 32;
+    const bool idle = warp / NC * 32 >= rows;
+    // up to two sums per column of this CTA to slots s0, s0 + 1 of every CTA
+    // (a shuffle addition of one warp holds the FP64 pipe for 16 clocks, so
+    // idle warps take no part)
+    auto publish = [&](const double (&v)[2], int s0, int n) {
+        for (int k = 0; k < n; ++k) {
+            double d = v[k];
+            if (!idle)
+                for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+            if (lane == 0) red[k][warp] = idle ? 0.0 : d;
+        }
+        __syncthreads();
+        if (t < n * NC) {
+            const int k = t / NC, u = t % NC;
+            double d = 0.0;
+            for (int w = u; w < PC_WARPS; w += NC) d += red[k][w];
+            for (int to = 0; to < PC_CL; ++to) cl.map_shared_rank(&part[s0 + k][rank][u], to)[0] = d;
+        }
+        cl.sync();
+    };
+    auto total = [&](int s, int u) {
+        double d = 0.0;
+        for (int f = 0; f < PC_CL; ++f) d += part[s][f][u];
+        return d;
+    };
+    auto precond = [&](int i, int u) {
+        if (!bj.inv) return r[u * max_rows + i];
+        const int row = r0 + i, blk = bj.fn_blk[row], first = bj.blk_idx[bj.blk_ptr[blk]] - r0;
+        const int n = bj.blk_ptr[blk + 1] - bj.blk_ptr[blk];
+        const double* a = bj.inv + bj.blk_off[blk] + (long long)bj.fn_pos[row] * n;
+        double d = 0.0;
+        for (int m = 0; m < n; ++m) d = fma(a[m], r[u * max_rows + first + m], d);
+        return d;
+    };
+    auto send_p = [&](int i, int u, double v) {
+        double* at = &p[(size_t)(r0 + i) * NC + u];
+        for (int to = 0; to < PC_CL; ++to) cl.map_shared_rank(at, to)[0] = v;
+    };
+    double v[2];
+    auto clear = [&] { v[0] = v[1] = 0.0; };
+    // x = 0, r = b, z = M r, p = z
+    for (int i = i0; i < rows; i += di) {
+        x[u * max_rows + i] = 0.0;
+        r[u * max_rows + i] = c0 + u < B ? b[(size_t)(r0 + i) * B + c0 + u] : 0.0;
+    }
+    cl.sync();   // every CTA of the cluster runs: remote shared memory may be written
+    clear();
+    for (int i = i0; i < rows; i += di) {
+        const double rv = r[u * max_rows + i], zv = precond(i, u);
+        send_p(i, u, zv);
+        v[0] = fma(rv, rv, v[0]);
+        v[1] = fma(rv, zv, v[1]);
+    }
+    publish(v, 1, 2);
+    if (t < NC) {
+        bn2[t] = rr[t] = total(1, t);
+        rz[t] = total(2, t);
+        act[t] = bn2[t] > 0.0 ? 1 : 0;   // a zero right-hand side is solved by x = 0
+        iters[t] = 0;
+    }
+    __syncthreads();
+    for (int it = 0; it < limit; ++it) {
+        if (t == 0) {
+            any = 0;
+            for (int u = 0; u < NC; ++u) any |= act[u];
+        }
+        __syncthreads();
+        if (!any) break;   // the same decision in every CTA: all hold the same sums
+        // q = S p on this CTA's rows, 8 lanes per row
+        for (int i = 4 * warp + (lane >> 3); i - (lane >> 3) < rows; i += 4 * PC_WARPS) {
+            double a[NC];
+            for (int k = 0; k < NC; ++k) a[k] = 0.0;
+            if (i < rows) {
+                const int beg = ptr[r0 + i] - e0, end = ptr[r0 + i + 1] - e0;
+#pragma unroll 4
+                for (int e = beg + (lane & 7); e < end; e += 8) {
+                    const double s = in_sh ? sv[e] : val[e0 + e];
+                    const double* pj = p + (size_t)(in_sh ? si[e] : idx[e0 + e]) * NC;
+#pragma unroll
+                    for (int k = 0; k < NC; ++k) a[k] = fma(s, pj[k], a[k]);
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < NC; ++k) {
+                for (int o = 4; o > 0; o >>= 1) a[k] += __shfl_xor_sync(0xffffffffu, a[k], o);
+                if ((lane & 7) == 0 && i < rows) q[k * max_rows + i] = a[k];
+            }
+        }
+        __syncthreads();
+        clear();
+        for (int i = i0; i < rows; i += di) {
+            v[0] = fma(p[(size_t)(r0 + i) * NC + u], q[u * max_rows + i], v[0]);
+        }
+        publish(v, 0, 1);
+        if (t < NC) {
+            const double pq = total(0, t);
+            alpha[t] = act[t] && pq > 0.0 ? rz[t] / pq : 0.0;
+            iters[t] += act[t];
+        }
+        __syncthreads();
+        for (int i = i0; i < rows; i += di) {
+            const double a = alpha[u];
+            x[u * max_rows + i] = fma(a, p[(size_t)(r0 + i) * NC + u], x[u * max_rows + i]);
+            r[u * max_rows + i] = fma(-a, q[u * max_rows + i], r[u * max_rows + i]);
+        }
+        __syncthreads();
+        clear();
+        for (int i = i0; i < rows; i += di) {
+            const double rv = r[u * max_rows + i], zv = precond(i, u);
+            z[u * max_rows + i] = zv;
+            v[0] = fma(rv, rv, v[0]);
+            v[1] = fma(rv, zv, v[1]);
+        }
+        publish(v, 1, 2);
+        if (t < NC) {
+            rr[t] = total(1, t);
+            if (act[t] && !(rr[t] > tol2 * bn2[t])) act[t] = 0;
+            const double n = total(2, t);
+            beta[t] = act[t] && rz[t] != 0.0 ? n / rz[t] : 0.0;
+            if (act[t]) rz[t] = n;
+        }
+        __syncthreads();
+        for (int i = i0; i < rows; i += di) send_p(i, u, fma(beta[u], p[(size_t)(r0 + i) * NC + u], z[u * max_rows + i]));
+        cl.sync();
+    }
+    for (int i = i0; i < rows && c0 + u < B; i += di) x_out[(size_t)(r0 + i) * B + c0 + u] = x[u * max_rows + i];
+    if (rank == 0 && t < NC && c0 + t < B) {
+        cs.bn2[c0 + t] = bn2[t];
+        cs.rr[c0 + t] = rr[t];
+        cs.act[c0 + t] = act[t];
+        cs.iters[c0 + t] = iters[t];
+    }
+    cl.sync();   // no CTA leaves while its shared memory may still be written
+}
+
 // p = z + beta p (first = 1: p = z)
 __global__ void k_pcg_p(long long n, int B, const double* __restrict__ beta, const double* __restrict__ z,
                         double* __restrict__ p, int first) {
@@ -627,8 +810,46 @@ void sparse_columns(Ctx& c, const double* F, const int* cols, int ncols, double 
         if (e != cudaSuccess) throw Error(DFT_ECUDA, std::string("cudaGraphInstantiate: ") + cudaGetErrorString(e));
         graph.width = Bb;
     };
+    // The cluster kernel takes a solve whose p (and the CTA's vectors) fit shared
+    // memory, with atoms' functions contiguous where they are preconditioned
+    // together; K <= PC_MAX_K: beyond, every cluster would read S from HBM for its
+    // few columns.  Otherwise iterations of seven kernels run as graphs.
+    constexpr int PC_MAX_K = 4096, PC_SMEM = 225 * 1024;
+    PcRows pr{};
+    int max_rows = 0;
+    bool cluster = K <= PC_MAX_K;
+    for (int i = 0; nbj > 0 && i < K; ++i) cluster = cluster && blk_idx[i] == i;
+    if (cluster) {
+        int at = 0;
+        for (int rk = 1; rk <= PC_CL; ++rk) {
+            const long long want = (long long)K * rk / PC_CL;
+            if (nbj == 0) at = (int)want;
+            else
+                while (at < want) at = blk_ptr[fn_blk[at] + 1];
+            pr.at[rk] = rk == PC_CL ? K : at;
+            max_rows = std::max(max_rows, pr.at[rk] - pr.at[rk - 1]);
+        }
+    }
+    auto solve_cluster = [&](int Bb, auto nc) {
+        constexpr int NC = decltype(nc)::value;
+        const long long room = (long long)(PC_SMEM - (long long)pc_smem<NC>(K, max_rows, 0)) / 12;
+        const int cached = (int)std::min<long long>(room, (long long)max_rows * K) & ~1;
+        auto kern = k_pcg_cluster<NC>;
+        DFT_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, PC_SMEM));
+        kern<<<PC_CL * ((Bb + NC - 1) / NC), PC_THREADS, pc_smem<NC>(K, max_rows, cached), s>>>(
+            K, Bb, pr, max_rows, cached, mS.ptr, mS.idx, mS.val, bj, q, Xs, tol2,
+            (maxit + PCG_GRAPH - 1) / PCG_GRAPH * PCG_GRAPH, cs);
+        k_pcg_stats<<<1, 256, 0, s>>>(Bb, cs, d_stats);
+        check_launch("pcg_cluster", 2);
+    };
     // S^-1 of the block in q (the right-hand sides) into Xs
     auto solve = [&](int Bb) {
+        if (cluster) {
+            // one column per cluster while that fits the SMs at once, then two
+            if (PC_CL * Bb <= 152) solve_cluster(Bb, std::integral_constant<int, 1>{});
+            else solve_cluster(Bb, std::integral_constant<int, 2>{});
+            return;
+        }
         const long long n = (long long)K * Bb;
         const unsigned cb = nblocks(Bb, 32);
         k_pcg_init<<<nrb, eb2, 0, s>>>(K, Bb, q, Xs, r, part);
