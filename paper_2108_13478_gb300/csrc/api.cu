@@ -233,7 +233,7 @@ void build_basis(Ctx& c, const dft_basis_desc* b, const dft_grid_desc* g, const 
             }
     }
     for (int d = 0; d < 3; ++d) c.Nfft[d] = fft_size(2 * c.n[d]);
-    c.nfft_r = (long long)c.Nfft[0] * c.Nfft[1] * c.Nfft[2];
+    c.nfft_r = (long long)c.Nfft[0] * c.Nfft[1] * c.n[2];   // the filled planes
     c.nfft_c = (long long)(c.Nfft[0] / 2 + 1) * c.Nfft[1] * c.Nfft[2];
     c.cheb_cap = 1 << 16;
     if (c.p.precision != DFT_PREC_FP64) {
@@ -1266,6 +1266,7 @@ dft_status dft_destroy(dft_ctx* ctx) {
     if (c->aux_done) cudaEventDestroy(c->aux_done);
     if (c->plan_f) cufftDestroy(c->plan_f);
     if (c->plan_b) cufftDestroy(c->plan_b);
+    if (c->plan_z) cufftDestroy(c->plan_z);
     if (c->kplan_f) cufftDestroy(c->kplan_f);
     if (c->kplan_b) cufftDestroy(c->kplan_b);
     delete c;

@@ -183,8 +183,8 @@ struct Ctx {
     double* d_vks = nullptr;
     double* d_nout = nullptr;
     double* d_gtmp = nullptr;
-    double* d_fft_r = nullptr;   // [nfft_r] padded transform input (zero outside the box)
-    double* d_fft_o = nullptr;   // [nfft_r] inverse transform output
+    double* d_fft_r = nullptr;   // [nfft_r] padded planes of the transform's input (zero outside the box)
+    double* d_fft_o = nullptr;   // [nfft_r] the same planes of the inverse transform's output
     double* d_ghat = nullptr;    // [nfft_c] real spectrum of the Coulomb kernel
     cufftDoubleComplex* d_fft_c = nullptr;  // [nfft_c]
     double* d_kerker = nullptr;  // Kerker weights on the unpadded box [nz][ny][nx/2+1]
@@ -249,7 +249,7 @@ struct Ctx {
     long long pl_count = 0;
     std::vector<double> pl_B;    // cached <R_i, R_j>, pl_hist x pl_hist
 
-    cufftHandle plan_f = 0, plan_b = 0;
+    cufftHandle plan_f = 0, plan_b = 0, plan_z = 0;   // x-y planes forward and back, z lines
     cufftHandle kplan_f = 0, kplan_b = 0;
     bool have_chol = false;
     // chemical potential of the last two SCF cycles (after the FP64
