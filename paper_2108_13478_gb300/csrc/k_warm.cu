@@ -161,7 +161,7 @@ __device__ double block_sum(double v) {
 
 // part[A][slab][k] = sum over the points of z slab blockIdx.y within RCUT of
 // atom A = blockIdx.x of resid * exp(-r^2/w_k^2): warps over rows, lanes along
-// x, chains of at most 8 FP32 products before they meet in FP64 (16 FP64
+// x, chains of four rows' FP32 products before they meet in FP64 (16 FP64
 // multiply-adds per point kept the FP64 pipe busy for twice the Gaussians' time)
 __global__ void __launch_bounds__(256) k_assemble_adjoint(const double* __restrict__ xyz, const double* __restrict__ resid,
                                                           int nx, int ny, int nz, double ox, double oy, double oz,
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(256) k_assemble_adjoint(const double* __restri
     const int z0 = ez > 0 ? (int)((long long)ez * blockIdx.y / gridDim.y) : 0;
     const int z1 = ez > 0 ? (int)((long long)ez * (blockIdx.y + 1) / gridDim.y) : 0;
     const int rows = ey > 0 ? (z1 - z0) * ey : 0;
-    int held = 0;
+    int held = 0;   // rows since the last flush, the same in all lanes
     for (int row = warp; row < rows; row += 8) {
         const int iz = lo[2] + z0 + row / ey, iy = lo[1] + row % ey;
         const double dy = oy + h * iy - c[1], dz = oz + h * iz - c[2];
@@ -200,13 +200,13 @@ __global__ void __launch_bounds__(256) k_assemble_adjoint(const double* __restri
             const float r2f = (float)r2, v = (float)rv[ix];
 #pragma unroll
             for (int k = 0; k < NO; ++k) f[k] = fmaf(v, expf(-r2f * wd.iw2[k]), f[k]);
-            if (++held == 8) {
-                held = 0;
+        }
+        if (++held == 4) {   // at 0.4 bohr a row has two points per lane
+            held = 0;
 #pragma unroll
-                for (int k = 0; k < NO; ++k) {
-                    acc[k] += (double)f[k];
-                    f[k] = 0.0f;
-                }
+            for (int k = 0; k < NO; ++k) {
+                acc[k] += (double)f[k];
+                f[k] = 0.0f;
             }
         }
     }
