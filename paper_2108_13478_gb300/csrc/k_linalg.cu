@@ -179,25 +179,105 @@ __global__ void __launch_bounds__(256) k_potrf_diag(double* A, int K, int kb, in
     }
 }
 
-// rows below the diagonal block: a <- a L_kk^-T (solve x L^T = a), one thread per row
-__global__ void __launch_bounds__(128) k_trsm_panel(double* A, int K, int kb, int nb) {
-    __shared__ double L[GB][GB + 1];
+// C -= P P^T on the 64 x 64 tiles on and below the diagonal (P: n x nb, nb <= GB)
+__global__ void __launch_bounds__(256) k_syrk_lower(int n, int nb, const double* __restrict__ P, double* __restrict__ C,
+                                                    int ld) {
+    __shared__ double As[GK][GB + 1];
+    __shared__ double Bs[GK][GB + 1];
+    int ti = 0, tj = blockIdx.x;   // row tile ti, column tile tj <= ti
+    while (tj > ti) {
+        tj -= ti + 1;
+        ++ti;
+    }
+    const int m0 = ti * GB, n0 = tj * GB, tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+    double acc[4][4] = {};
+    for (int k0 = 0; k0 < nb; k0 += GK) {
+        for (int e = threadIdx.x; e < GB * GK; e += 256) {
+            const int kk = e % GK, mm = e / GK;
+            As[kk][mm] = (m0 + mm < n && k0 + kk < nb) ? P[(long long)(m0 + mm) * ld + k0 + kk] : 0.0;
+            Bs[kk][mm] = (n0 + mm < n && k0 + kk < nb) ? P[(long long)(n0 + mm) * ld + k0 + kk] : 0.0;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int kk = 0; kk < GK; ++kk) {
+            double a[4], b[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int gm = m0 + ty + 16 * i;
+        if (gm >= n) continue;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int gn = n0 + tx + 16 * j;
+            if (gn < n) C[(long long)gm * ld + gn] -= acc[i][j];
+        }
+    }
+}
+
+// rows below the diagonal block: a <- a L_kk^-T (solve x L^T = a), TRSM_R rows
+// per warp, two columns per lane: x_j is passed to all lanes, which take it out
+// of the columns behind j.  (One thread per row, with its 64 unknowns in local
+// memory, took 160 us per panel.)
+constexpr int TRSM_R = 4, TRSM_W = 4;   // rows per warp, warps per block
+__global__ void __launch_bounds__(32 * TRSM_W) k_trsm_panel(double* A, int K, int kb, int nb) {
+    __shared__ double Lt[GB][GB + 1];   // Lt[j][c] = L[c][j]
+    __shared__ double inv[GB];
     for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-        int i = e / nb, j = e % nb;
-        L[i][j] = A[(long long)(kb + i) * K + kb + j];
+        const int i = e / nb, j = e % nb;
+        Lt[j][i] = A[(long long)(kb + i) * K + kb + j];
     }
     __syncthreads();
-    int r = kb + nb + blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= K) return;
-    double x[GB];
-    double* row = &A[(long long)r * K + kb];
-#pragma unroll 1
-    for (int j = 0; j < nb; ++j) {
-        double v = row[j];
-        for (int m = 0; m < j; ++m) v -= x[m] * L[j][m];
-        x[j] = v / L[j][j];
-    }
-    for (int j = 0; j < nb; ++j) row[j] = x[j];
+    for (int j = threadIdx.x; j < nb; j += blockDim.x) inv[j] = 1.0 / Lt[j][j];
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const int r0 = kb + nb + (blockIdx.x * TRSM_W + (threadIdx.x >> 5)) * TRSM_R;
+    double a[TRSM_R][2];
+#pragma unroll
+    for (int q = 0; q < TRSM_R; ++q)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int c = lane + 32 * h;
+            a[q][h] = (r0 + q < K && c < nb) ? A[(long long)(r0 + q) * K + kb + c] : 0.0;
+        }
+    auto steps = [&](int h, int j0, int j1) {   // h is a constant in each call
+        for (int j = j0; j < j1; ++j) {
+            const double l0 = lane < nb ? Lt[j][lane] : 0.0, l1 = lane + 32 < nb ? Lt[j][lane + 32] : 0.0;
+            const double d = Lt[j][j], id = inv[j];
+#pragma unroll
+            for (int q = 0; q < TRSM_R; ++q) {
+                const double v = __shfl_sync(0xffffffffu, h ? a[q][1] : a[q][0], j & 31);
+                double x = v * id;
+                x = fma(fma(-x, d, v), id, x);   // v / d to rounding
+                if (h == 0) {
+                    if (lane > j) a[q][0] = fma(-x, l0, a[q][0]);
+                    else if (lane == j) a[q][0] = x;
+                    a[q][1] = fma(-x, l1, a[q][1]);
+                } else {
+                    if (lane + 32 > j) a[q][1] = fma(-x, l1, a[q][1]);
+                    else if (lane + 32 == j) a[q][1] = x;
+                }
+            }
+        }
+    };
+    steps(0, 0, min(nb, 32));
+    steps(1, 32, nb);
+#pragma unroll
+    for (int q = 0; q < TRSM_R; ++q)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int c = lane + 32 * h;
+            if (r0 + q < K && c < nb) A[(long long)(r0 + q) * K + kb + c] = a[q][h];
+        }
 }
 
 __global__ void k_zero_upper(double* A, int K) {
@@ -211,8 +291,11 @@ constexpr int TIB = 32;  // leaf size of the recursive triangular inverse
 
 // inverse of an n x n (n <= TIB) lower-triangular block in shared memory, one
 // column per thread (forward substitution), written with leading dimension ld
-__global__ void __launch_bounds__(TIB) k_tri_inv_block(const double* __restrict__ L, double* __restrict__ X, int n,
-                                                       int ld) {
+// (block b: rows and columns b TIB ... of the K x K factor)
+__global__ void __launch_bounds__(TIB) k_tri_inv_block(const double* __restrict__ L, double* __restrict__ X, int K) {
+    const int ld = K, n = min(TIB, K - (int)blockIdx.x * TIB);
+    L += (long long)blockIdx.x * TIB * (K + 1);
+    X += (long long)blockIdx.x * TIB * (K + 1);
     __shared__ double Ls[TIB][TIB + 1];
     __shared__ double Xs[TIB][TIB + 1];
     for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
@@ -236,6 +319,62 @@ __global__ void __launch_bounds__(TIB) k_tri_inv_block(const double* __restrict_
     for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
         int i = e / n, j = e % n;
         X[(long long)i * ld + j] = Xs[i][j];
+    }
+}
+
+// One level of the triangular inverse: neighbouring diagonal blocks of b rows
+// are inverted, X_21 = -C^-1 (B A^-1) joins them, for all pairs blockIdx.z at
+// once.  Phase 1: tmp = B A^-1 (A^-1 lower triangular: k from the column tile on);
+// phase 2: X_21 = -C^-1 tmp (k up to the row tile's end).  Tiles of 64 x 64, or
+// 32 x 32 for the small blocks; tmp in a K x K scratch at X_21's place.
+template <int GB>
+__global__ void __launch_bounds__(256) k_tri_level(int K, int b, int phase, const double* __restrict__ L,
+                                                   double* __restrict__ X, double* __restrict__ tmp) {
+    constexpr int TM = GB / 16;
+    __shared__ double As[GK][GB + 1];
+    __shared__ double Bs[GK][GB + 1];
+    const int c0 = blockIdx.z * 2 * b, r0 = c0 + b;   // the pair's first column, and first row of its lower block
+    const int n2 = min(b, K - r0);
+    const int m0 = blockIdx.y * GB, n0 = blockIdx.x * GB;
+    if (n2 <= 0 || m0 >= n2) return;
+    const double* P = phase == 1 ? L + (long long)r0 * K + c0 : X + (long long)r0 * K + r0;     // n2 x (b or n2)
+    const double* Q = phase == 1 ? X + (long long)c0 * K + c0 : tmp + (long long)r0 * K + c0;   // (b or n2) x b
+    double* out = (phase == 1 ? tmp : X) + (long long)r0 * K + c0;
+    const int klo = phase == 1 ? n0 : 0, khi = phase == 1 ? b : min(n2, m0 + GB);
+    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+    double acc[TM][TM] = {};
+    for (int k0 = klo; k0 < khi; k0 += GK) {
+        for (int e = threadIdx.x; e < GB * GK; e += 256) {
+            const int kk = e % GK, mm = e / GK;
+            As[kk][mm] = (m0 + mm < n2 && k0 + kk < khi) ? P[(long long)(m0 + mm) * K + k0 + kk] : 0.0;
+            const int nn = e % GB, kb = e / GB;
+            Bs[kb][nn] = (n0 + nn < b && k0 + kb < khi) ? Q[(long long)(k0 + kb) * K + n0 + nn] : 0.0;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int kk = 0; kk < GK; ++kk) {
+            double av[TM], bv[TM];
+#pragma unroll
+            for (int i = 0; i < TM; ++i) av[i] = As[kk][ty + 16 * i];
+#pragma unroll
+            for (int j = 0; j < TM; ++j) bv[j] = Bs[kk][tx + 16 * j];
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int j = 0; j < TM; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
+        }
+        __syncthreads();
+    }
+    const double sign = phase == 1 ? 1.0 : -1.0;
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+        const int gm = m0 + ty + 16 * i;
+        if (gm >= n2) continue;
+#pragma unroll
+        for (int j = 0; j < TM; ++j) {
+            const int gn = n0 + tx + 16 * j;
+            if (gn < b) out[(long long)gm * K + gn] = sign * acc[i][j];
+        }
     }
 }
 
@@ -274,6 +413,7 @@ __global__ void k_overlap_kinetic(const Fn* __restrict__ fn, int K, double* __re
     long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (long long)K * K) return;
     int i = (int)(e / K), j = (int)(e % K);
+    if (j < i) return;   // mirrored below
     const Fn fa = fn[i], fb = fn[j];
     const double Ac[3] = {fa.cx, fa.cy, fa.cz}, Bc[3] = {fb.cx, fb.cy, fb.cz};
     const int pa[3] = {fa.px, fa.py, fa.pz}, pb[3] = {fb.px, fb.py, fb.pz};
@@ -291,8 +431,9 @@ __global__ void k_overlap_kinetic(const Fn* __restrict__ fn, int K, double* __re
         Td[d] = 0.5 * t;
     }
     double nn = fa.norm * fb.norm;
-    if (S) S[e] = nn * Sd[0] * Sd[1] * Sd[2];
-    if (T) T[e] = nn * (Td[0] * Sd[1] * Sd[2] + Sd[0] * Td[1] * Sd[2] + Sd[0] * Sd[1] * Td[2]);
+    const long long m = (long long)j * K + i;
+    if (S) S[e] = S[m] = nn * Sd[0] * Sd[1] * Sd[2];
+    if (T) T[e] = T[m] = nn * (Td[0] * Sd[1] * Sd[2] + Sd[0] * Td[1] * Sd[2] + Sd[0] * Sd[1] * Td[2]);
 }
 
 __global__ void k_axpby(long long n, double a, const double* X, double b, const double* Y, double* Z) {
@@ -641,10 +782,12 @@ int cholesky_inplace(double* A, int K, int* d_flag, cudaStream_t s) {
         check_launch("potrf_diag");
         int rows = K - kb - nb;
         if (rows > 0) {
-            k_trsm_panel<<<blocks_for(rows, 128), 128, 0, s>>>(A, K, kb, nb);
+            k_trsm_panel<<<blocks_for(rows, TRSM_R * TRSM_W), 32 * TRSM_W, 0, s>>>(A, K, kb, nb);
             check_launch("trsm_panel");
             double* P = A + (long long)(kb + nb) * K + kb;
-            dgemm('N', 'T', rows, rows, nb, -1.0, P, K, P, K, 1.0, A + (long long)(kb + nb) * K + kb + nb, K, s);
+            const int tb = (rows + GB - 1) / GB;
+            k_syrk_lower<<<tb * (tb + 1) / 2, 256, 0, s>>>(rows, nb, P, A + (long long)(kb + nb) * K + kb + nb, K);
+            check_launch("syrk_lower");
         }
     }
     k_zero_upper<<<blocks_for((long long)K * K, 256), 256, 0, s>>>(A, K);
@@ -682,31 +825,25 @@ void congruence_lower_t(int K, const double* Linv, const double* R, double* tmp,
     check_launch("congruence_lower_t", 3);
 }
 
-namespace {
-// inverse of the n x n lower-triangular block at L (leading dimension ld) into
-// X (same layout), by the block identity
-//   [A 0; B C]^-1 = [A^-1 0; -C^-1 B A^-1  C^-1]
-// with FP64 GEMMs; tmp holds at least n^2 / 4 + n TIB doubles
-void tri_inv_rec(const double* L, double* X, int n, int ld, double* tmp, cudaStream_t s) {
-    if (n <= TIB) {
-        k_tri_inv_block<<<1, TIB, 0, s>>>(L, X, n, ld);
-        check_launch("tri_inv_block");
-        return;
-    }
-    int n1 = ((n / 2) + TIB - 1) / TIB * TIB;
-    int n2 = n - n1;
-    tri_inv_rec(L, X, n1, ld, tmp, s);
-    tri_inv_rec(L + (long long)n1 * ld + n1, X + (long long)n1 * ld + n1, n2, ld, tmp, s);
-    // tmp = B A^-1 (n2 x n1); X_21 = -C^-1 tmp
-    dgemm('N', 'N', n2, n1, n1, 1.0, L + (long long)n1 * ld, ld, X, ld, 0.0, tmp, n1, s);
-    dgemm('N', 'N', n2, n1, n2, -1.0, X + (long long)n1 * ld + n1, ld, tmp, n1, 0.0, X + (long long)n1 * ld, ld, s);
-}
-}  // namespace
-
+// L^-1 by block pairs, [A 0; B C]^-1 = [A^-1 0; -C^-1 B A^-1  C^-1], from leaves
+// of TIB rows upwards: two launches per level (a recursion over single blocks
+// took 178 launches and multiplied the zeros too: 17.7 of 34.6 ms at K = 1910)
 void tri_inverse_lower(const double* L, double* Linv, int K, double* tmp, cudaStream_t s) {
     // the strictly upper part of L^-1 is zero
     DFT_CUDA_CHECK(cudaMemsetAsync(Linv, 0, sizeof(double) * (size_t)K * K, s));
-    tri_inv_rec(L, Linv, K, K, tmp, s);
+    k_tri_inv_block<<<(K + TIB - 1) / TIB, TIB, 0, s>>>(L, Linv, K);
+    check_launch("tri_inv_block");
+    for (int b = TIB; b < K; b *= 2) {
+        const int pairs = (K + 2 * b - 1) / (2 * b);
+        for (int phase = 1; phase <= 2; ++phase) {
+            const int t64 = (b + 63) / 64, t32 = (b + 31) / 32;
+            if ((long long)t64 * t64 * pairs >= 2 * 152)
+                k_tri_level<64><<<dim3(t64, t64, pairs), 256, 0, s>>>(K, b, phase, L, Linv, tmp);
+            else
+                k_tri_level<32><<<dim3(t32, t32, pairs), 256, 0, s>>>(K, b, phase, L, Linv, tmp);
+        }
+        check_launch("tri_level", 2);
+    }
 }
 
 // (M_c)_ab = N_a N_b sum_{s in a, t in b} Mt_st
