@@ -934,7 +934,7 @@ dft_status dft_init_basis(dft_ctx** ctx, const dft_basis_desc* basis, const dft_
             DFT_CUDA_CHECK(cudaMemcpyAsync(c->d_term_par, par.data(), sizeof(int) * c->Kt, cudaMemcpyHostToDevice, s));
         }
         DFT_CUDA_CHECK(cudaMemcpyAsync(c->d_tile_ptr, tp.data(), sizeof(int) * tp.size(), cudaMemcpyHostToDevice, s));
-        c->grid_split = grid_split(*c, tp.data());
+        grid_split(*c, tp.data());
         std::vector<int> order(c->n_tiles);
         for (long long t = 0; t < c->n_tiles; ++t) order[t] = (int)t;
         std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return tp[x + 1] - tp[x] > tp[y + 1] - tp[y]; });

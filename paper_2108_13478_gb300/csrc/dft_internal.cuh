@@ -140,7 +140,8 @@ struct Ctx {
     int* d_tile_ptr = nullptr;   // [n_tiles + 1]
     int* d_tile_fn = nullptr;    // [tile_nnz]
     int* d_tile_order = nullptr; // [n_tiles], longest lists first
-    int grid_split = 1;          // blocks per tile of the grid kernels
+    int grid_split = 1;          // blocks per tile of the quadrature (by chunk pairs)
+    int plane_split = 1;         // and of the collocation (by planes)
     double* d_xyz = nullptr;     // [n_atoms * 3]
     double* d_S = nullptr;       // K x K
     double* d_T = nullptr;
@@ -295,7 +296,7 @@ void launch_nonlocal(const Ctx& c, cudaStream_t s);
 // FP64 kernels on the FP64 path, FP32 arithmetic (FP64 in and out) on the mixed path
 void launch_collocate(const Ctx& c, const double* P, double* n, cudaStream_t s);
 void launch_quadrature(const Ctx& c, const double* v, double* V, cudaStream_t s);
-int grid_split(const Ctx& c, const int* tile_ptr);   // from the host's list offsets
+void grid_split(Ctx& c, const int* tile_ptr);   // blocks per tile, from the host's list offsets
 void launch_gaussian_sum(const Ctx& c, double amp, double width, double* out, cudaStream_t s);
 
 // ---- dense FP64 linear algebra (k_linalg.cu) ----

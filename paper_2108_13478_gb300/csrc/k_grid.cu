@@ -395,7 +395,7 @@ __global__ void k_gaussian_sum(const double* __restrict__ xyz, int n_atoms, int 
 // quadrature by chunk pairs) until the longest takes at most a third of what an SM
 // gets on average (K = 240 in FP64: 343 tiles, the longest lists of 432 terms
 // against 170 on average)
-int grid_split(const Ctx& c, const int* tile_ptr) {
+void grid_split(Ctx& c, const int* tile_ptr) {
     const int ch = c.p.precision == DFT_PREC_FP64 ? GridCfg<double>::CH : GridCfg<float>::CH;
     double total = 0.0, longest = 0.0;
     for (long long t = 0; t < c.n_tiles; ++t) {
@@ -403,9 +403,12 @@ int grid_split(const Ctx& c, const int* tile_ptr) {
         total += w;
         longest = std::max(longest, w);
     }
-    int s = 1;
-    while (s < 8 && longest / s > total / 152.0 / 3.0) s *= 2;
-    return s;
+    c.grid_split = c.plane_split = 1;
+    while (c.grid_split < 8 && longest / c.grid_split > total / 152.0 / 3.0) c.grid_split *= 2;
+    // every block of a plane split reads the tile's part of P again (1470
+    // functions, FP32: 2.6 ms with one block per tile, 2.95 with four), so it
+    // only keeps a tile from outlasting an SM's share; each thread group needs a plane
+    while (c.plane_split < 4 && longest / c.plane_split > total / 152.0) c.plane_split *= 2;
 }
 
 void launch_build_tables_for(const Ctx& c, const Fn* fn, int count, int W, double* tab, cudaStream_t s) {
@@ -434,7 +437,7 @@ void launch_collocate(const Ctx& c, const double* P, double* n, cudaStream_t s) 
     }
     auto go = [&](auto kern, size_t bytes) {
         allow_smem(kern, bytes);
-        const dim3 grid((unsigned)c.n_tiles, std::min(c.grid_split, 4));   // by planes, at least one per thread group
+        const dim3 grid((unsigned)c.n_tiles, c.plane_split);
         kern<<<grid, 128, bytes, s>>>(c.d_fn, c.d_tab, c.tab_w, c.d_tile_ptr, c.d_tile_fn, c.d_tile_order, c.ntile[0],
                                       c.ntile[1], c.n[0], c.n[1], c.n[2], c.Kt, P, n);
     };
