@@ -5,6 +5,7 @@ no giant, one giant, ragged last groups, plans that keep the giants and
 orders so high that they do not fit (Clenshaw)."""
 import numpy as np
 import pytest
+import scipy.fft
 
 import workloads as w
 from oracle import basis, dm
@@ -18,6 +19,22 @@ if not torch.cuda.is_available():
 import paper_2108_13478_gb300 as dft  # noqa: E402
 
 
+@pytest.fixture
+def dct_coefficients(monkeypatch):
+    """The oracle's Gauss-Chebyshev sums by SciPy's DCT-II: the direct cosine
+    sums take minutes per order at N_C of thousands."""
+    def coeffs(mu, beta, e_min, e_max, n_c, m_nodes=None):
+        m = int(m_nodes) if m_nodes else 8 * int(n_c)
+        th = np.pi * (np.arange(m) + 0.5) / m
+        f = dm.fermi(0.5 * (e_max + e_min) + 0.5 * (e_max - e_min) * np.cos(th), mu, beta)
+        a = scipy.fft.dct(f, type=2)[:n_c] / m
+        a[0] *= 0.5
+        return a
+    args = (0.1, 20.0, -1.0, 3.0, 40, 160)
+    assert np.max(np.abs(coeffs(*args) - dm.cheb_coeffs(*args))) < 1e-14
+    monkeypatch.setattr(dm, "cheb_coeffs", coeffs)
+
+
 def problem(name, seed=3):
     s = w.config_system(name)
     S, T = basis.overlap_kinetic_system(s)
@@ -29,7 +46,7 @@ def problem(name, seed=3):
 
 @pytest.mark.parametrize("name,orders", [("tiny8", (2, 3, 4, 5, 8, 33, 64, 1000, 2900, 14000)), ("tiny3", (2, 17, 700)),
                                          ("tiny37", (65, 1500))])
-def test_fp64_expansion_matches_the_oracle_at_every_grouping(name, orders):
+def test_fp64_expansion_matches_the_oracle_at_every_grouping(name, orders, dct_coefficients):
     s, F, S, lo, hi = problem(name)
     Fd = torch.from_numpy(F).cuda()
     for n_c in orders:
@@ -49,7 +66,7 @@ def test_fp64_expansion_matches_the_oracle_at_every_grouping(name, orders):
 
 @pytest.mark.parametrize("name,orders", [("tiny8", (2, 3, 5, 40, 700, 6000)), ("tiny37", (2, 33, 1500, 7000)),
                                          ("cluster64", (1400,))])
-def test_split_expansion_matches_the_oracle_at_every_grouping(name, orders):
+def test_split_expansion_matches_the_oracle_at_every_grouping(name, orders, dct_coefficients):
     """One, two and three 256-blocks per side (operands read in place and
     transposed, folded block rows, ragged last blocks), direct and Clenshaw
     plans; the gate of the mixed path's density matrices, 1e-4 of max|P|."""
