@@ -300,9 +300,9 @@ void grid_split(Ctx& c, const int* tile_ptr);   // blocks per tile, from the hos
 void launch_gaussian_sum(const Ctx& c, double amp, double width, double* out, cudaStream_t s);
 
 // ---- dense FP64 linear algebra (k_linalg.cu) ----
-// C[M x N] = alpha op(A) op(B) + beta C, row-major, op = 'N' or 'T'
-void dgemm(char ta, char tb, int M, int N, int Kd, double alpha, const double* A, int lda,
-           const double* B, int ldb, double beta, double* C, int ldc, cudaStream_t s);
+// C[M x N] = A^T B, row-major, A Kd x M, B Kd x N
+void dgemm_tn(int M, int N, int Kd, const double* A, int lda, const double* B, int ldb, double* C, int ldc,
+              cudaStream_t s);
 int cholesky_inplace(double* A, int K, int* d_flag, cudaStream_t s);
 // dft_density_matrix_columns: the sparse-operator route (k_sparse.cu)
 void sparse_columns(Ctx& c, const double* F, const int* cols, int ncols, double mu, double e_min, double e_max,
@@ -326,8 +326,6 @@ void launch_axpby_mat(int K, double a, const double* X, double b, const double* 
 void launch_normalise_h(int K, const double* Ft, const double* scal, double* H, cudaStream_t s);
 void launch_frob_dot(long long n, const double* X, const double* Y, double* part, double* out,
                      cudaStream_t s);    // out = sum X*Y (deterministic)
-void launch_trace(int K, const double* X, double* out, cudaStream_t s);
-void launch_identity(int K, double* X, cudaStream_t s);
 // Lanczos on symmetric A: writes padded bounds to scal[SCAL_EMIN], scal[SCAL_EMAX]
 void lanczos_bounds(const Ctx& c, const double* A, int steps, cudaStream_t s);
 // the same with explicit buffers (vec: 4 K doubles, scal: SCAL_COUNT doubles,

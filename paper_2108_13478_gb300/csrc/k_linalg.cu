@@ -18,11 +18,10 @@ namespace {
 constexpr int GB = 64;   // tile edge
 constexpr int GK = 16;   // k-slab
 
-// C = alpha op(A) op(B) + beta C (row-major), 256 threads, 4x4 outputs each
-template <bool TA, bool TB>
-__global__ void __launch_bounds__(256) k_dgemm(int M, int N, int Kd, double alpha, const double* __restrict__ A,
-                                               int lda, const double* __restrict__ B, int ldb, double beta,
-                                               double* __restrict__ C, int ldc) {
+// C = A^T B (row-major, A Kd x M, B Kd x N), 256 threads, 4x4 outputs each
+__global__ void __launch_bounds__(256) k_dgemm_tn(int M, int N, int Kd, const double* __restrict__ A, int lda,
+                                                  const double* __restrict__ B, int ldb, double* __restrict__ C,
+                                                  int ldc) {
     __shared__ double As[GK][GB + 1];
     __shared__ double Bs[GK][GB + 1];
     const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
@@ -30,20 +29,9 @@ __global__ void __launch_bounds__(256) k_dgemm(int M, int N, int Kd, double alph
     double acc[4][4] = {};
     for (int k0 = 0; k0 < Kd; k0 += GK) {
         for (int e = threadIdx.x; e < GB * GK; e += 256) {
-            int mm, kk;
-            if (!TA) { kk = e % GK; mm = e / GK; } else { mm = e % GB; kk = e / GB; }
-            int gm = m0 + mm, gk = k0 + kk;
-            double v = 0.0;
-            if (gm < M && gk < Kd) v = TA ? A[(long long)gk * lda + gm] : A[(long long)gm * lda + gk];
-            As[kk][mm] = v;
-        }
-        for (int e = threadIdx.x; e < GB * GK; e += 256) {
-            int nn, kk;
-            if (!TB) { nn = e % GB; kk = e / GB; } else { kk = e % GK; nn = e / GK; }
-            int gn = n0 + nn, gk = k0 + kk;
-            double v = 0.0;
-            if (gn < N && gk < Kd) v = TB ? B[(long long)gn * ldb + gk] : B[(long long)gk * ldb + gn];
-            Bs[kk][nn] = v;
+            const int mm = e % GB, kk = e / GB, gk = k0 + kk;
+            As[kk][mm] = m0 + mm < M && gk < Kd ? A[(long long)gk * lda + m0 + mm] : 0.0;
+            Bs[kk][mm] = n0 + mm < N && gk < Kd ? B[(long long)gk * ldb + n0 + mm] : 0.0;
         }
         __syncthreads();
 #pragma unroll
@@ -67,9 +55,7 @@ __global__ void __launch_bounds__(256) k_dgemm(int M, int N, int Kd, double alph
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             int gn = n0 + tx + 16 * j;
-            if (gn >= N) continue;
-            double* cp = &C[(long long)gm * ldc + gn];
-            *cp = beta == 0.0 ? alpha * acc[i][j] : fma(alpha, acc[i][j], beta * *cp);
+            if (gn < N) C[(long long)gm * ldc + gn] = acc[i][j];
         }
     }
 }
@@ -454,12 +440,6 @@ __global__ void k_normalise_h(int K, const double* __restrict__ Ft, const double
     H[e] = v / de;
 }
 
-__global__ void k_identity(int K, double* X) {
-    long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (long long)K * K) return;
-    X[e] = (e / K == e % K) ? 1.0 : 0.0;
-}
-
 template <int BS>
 __device__ double block_sum(double v) {
     __shared__ double red[BS / 32];
@@ -487,13 +467,6 @@ __global__ void __launch_bounds__(256) k_dot_part(long long n, const double* __r
 __global__ void __launch_bounds__(256) k_sum_parts(int np, const double* part, double* out) {
     double s = 0.0;
     for (int i = threadIdx.x; i < np; i += 256) s += part[i];
-    s = block_sum<256>(s);
-    if (threadIdx.x == 0) *out = s;
-}
-
-__global__ void __launch_bounds__(256) k_trace(int K, const double* X, double* out) {
-    double s = 0.0;
-    for (int i = threadIdx.x; i < K; i += 256) s += X[(long long)i * K + i];
     s = block_sum<256>(s);
     if (threadIdx.x == 0) *out = s;
 }
@@ -763,16 +736,12 @@ inline unsigned blocks_for(long long n, int bs) { return (unsigned)((n + bs - 1)
 
 }  // namespace
 
-void dgemm(char ta, char tb, int M, int N, int Kd, double alpha, const double* A, int lda, const double* B,
-           int ldb, double beta, double* C, int ldc, cudaStream_t s) {
+void dgemm_tn(int M, int N, int Kd, const double* A, int lda, const double* B, int ldb, double* C, int ldc,
+              cudaStream_t s) {
     if (M <= 0 || N <= 0) return;
     dim3 grid((N + GB - 1) / GB, (M + GB - 1) / GB);
-    bool a = ta == 'T', b = tb == 'T';
-    if (!a && !b) k_dgemm<false, false><<<grid, 256, 0, s>>>(M, N, Kd, alpha, A, lda, B, ldb, beta, C, ldc);
-    else if (!a && b) k_dgemm<false, true><<<grid, 256, 0, s>>>(M, N, Kd, alpha, A, lda, B, ldb, beta, C, ldc);
-    else if (a && !b) k_dgemm<true, false><<<grid, 256, 0, s>>>(M, N, Kd, alpha, A, lda, B, ldb, beta, C, ldc);
-    else k_dgemm<true, true><<<grid, 256, 0, s>>>(M, N, Kd, alpha, A, lda, B, ldb, beta, C, ldc);
-    check_launch("dgemm");
+    k_dgemm_tn<<<grid, 256, 0, s>>>(M, N, Kd, A, lda, B, ldb, C, ldc);
+    check_launch("dgemm_tn");
 }
 
 int cholesky_inplace(double* A, int K, int* d_flag, cudaStream_t s) {
@@ -931,16 +900,6 @@ void launch_frob_dot(long long n, const double* X, const double* Y, double* part
     k_dot_part<<<np, 256, 0, s>>>(n, X, Y, part);
     k_sum_parts<<<1, 256, 0, s>>>(np, part, out);
     check_launch("frob_dot", 2);
-}
-
-void launch_trace(int K, const double* X, double* out, cudaStream_t s) {
-    k_trace<<<1, 256, 0, s>>>(K, X, out);
-    check_launch("trace");
-}
-
-void launch_identity(int K, double* X, cudaStream_t s) {
-    k_identity<<<blocks_for((long long)K * K, 256), 256, 0, s>>>(K, X);
-    check_launch("identity");
 }
 
 // Lanczos bounds with caller-given buffers: vec holds 4 K doubles, scal

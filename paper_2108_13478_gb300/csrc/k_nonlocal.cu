@@ -51,7 +51,7 @@ void launch_nonlocal(const Ctx& c, cudaStream_t s) {
     // V^NL = B^T (E B) from the np x K_t projections of the basis terms,
     // contracted to the functions where they are sums of terms
     double* out = c.contracted ? c.d_Mt : c.d_VNL;
-    dgemm('T', 'N', c.Kt, c.Kt, np, 1.0, c.d_nlB, c.Kt, c.d_nlEB, c.Kt, 0.0, out, c.Kt, s);
+    dgemm_tn(c.Kt, c.Kt, np, c.d_nlB, c.Kt, c.d_nlEB, c.Kt, out, c.Kt, s);
     if (c.contracted) launch_contract(c, c.d_Mt, c.d_VNL, s);
 }
 
