@@ -336,37 +336,44 @@ __global__ void k_pcg_precond(int K, int B, BJ bj, const double* __restrict__ r,
 
 // A whole solve of NC columns as one launch of a cluster of PC_CL CTAs (columns
 // do not depend on one another).  Each CTA owns a run of rows (whole atoms, so
-// that the preconditioner is local), keeps its rows of S in shared memory where they fit
-// (`cached`: room for that many entries), and holds all of p.  Per iteration
-// three cluster barriers: after the partial sums of p.q, after those of r.r and
-// r.z, after the new p.  The FP64 pipe bounds the product; with seven
-// launches per iteration and a host check every eight, an iteration of 32
-// columns at K = 370 took 72 us.
+// that the preconditioner is local; runs of about equal entries of S), keeps
+// its rows of S in shared memory where they fit (`cached`: room for that many
+// entries), and holds all of p and z: p = z + beta p is formed by every CTA, so an iteration takes
+// two cluster barriers, after the partial sums of p.q and after z with the partial
+// sums of r.r and r.z.  An iteration is bound by the FP64 pipe (a warp's
+// FP64 instruction holds its quarter of the SM for 64 clocks, idle lanes or not)
+// and the latency of its serial steps, so sums over lanes exchange
+// halves first (one addition where two values are reduced), go over as few
+// warps as hold data, and two CTAs share an SM where their memory allows it.
+// 32 columns at K = 370, 100 solves: 935 ms with seven launches per iteration
+// and a host check every eight, 334 ms with three barriers, runs of equal rows and
+// whole-warp sums, 285 ms like this.
 constexpr int PC_CL = 8, PC_THREADS = 384, PC_WARPS = PC_THREADS / 32;
 struct PcRows {
     int at[PC_CL + 1];   // first row of each CTA
 };
 template <int NC>
 size_t pc_smem(int K, int rows, int cached) {
-    return sizeof(double) * ((size_t)K * NC + 4 * (size_t)rows * NC + cached) + sizeof(int) * (size_t)cached;
+    return sizeof(double) * (2 * (size_t)K * NC + 3 * (size_t)rows * NC + cached) + sizeof(int) * (size_t)cached;
 }
 template <int NC>
-__global__ void __cluster_dims__(PC_CL, 1, 1) __launch_bounds__(PC_THREADS)
+__global__ void __cluster_dims__(PC_CL, 1, 1) __launch_bounds__(PC_THREADS, 2)
     k_pcg_cluster(int K, int B, PcRows pr, int max_rows, int cached, const int* __restrict__ ptr,
                   const int* __restrict__ idx, const double* __restrict__ val, BJ bj, const double* __restrict__ b,
                   double* __restrict__ x_out, double tol2, int limit, Cols cs) {
     namespace cgx = cooperative_groups;
     cgx::cluster_group cl = cgx::this_cluster();
+    static_assert(NC == 1 || NC == 2, "lane layout of the sums");
     extern __shared__ __align__(16) double pc_sh[];
-    double* p = pc_sh;                                  // [K][NC]
-    double* x = p + (size_t)K * NC;                     // [NC][rows], as r, z, q
+    double* p = pc_sh;                                  // [K][NC], as z
+    double* z = p + (size_t)K * NC;
+    double* x = z + (size_t)K * NC;                     // [NC][rows], as r, q
     double* r = x + (size_t)max_rows * NC;
-    double* z = r + (size_t)max_rows * NC;
-    double* q = z + (size_t)max_rows * NC;
+    double* q = r + (size_t)max_rows * NC;
     double* sv = q + (size_t)max_rows * NC;             // cached rows of S
     int* si = (int*)(sv + cached);
-    __shared__ double part[3][PC_CL][NC], red[2][PC_WARPS], alpha[NC], beta[NC], rz[NC], bn2[NC], rr[NC];
-    __shared__ int act[NC], iters[NC], any;
+    __shared__ double part[3][NC][PC_CL], red[2][NC][16], alpha[NC], beta[NC], rz[NC], bn2[NC], rr[NC];
+    __shared__ int act[NC], iters[NC];
     const int rank = (int)cl.block_rank(), t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int r0 = pr.at[rank], rows = pr.at[rank + 1] - r0;
     const int c0 = (int)(blockIdx.x / PC_CL) * NC;
@@ -378,77 +385,93 @@ __global__ void __cluster_dims__(PC_CL, 1, 1) __launch_bounds__(PC_THREADS)
             si[e] = idx[e0 + e];
         }
     // element-wise steps: warp w takes column w % NC, rows 32 (w / NC) + lane, ...
-    static_assert(PC_WARPS % NC == 0, "whole warps per column");
+    static_assert(PC_WARPS % NC == 0 && PC_WARPS <= 16, "whole warps per column");
     const int u = warp % NC, i0 = warp / NC * 32 + lane, di = PC_WARPS / NC * 32;
     const bool idle = warp / NC * 32 >= rows;
-    // up to two sums per column of this CTA to slots s0, s0 + 1 of every CTA
-    // (a shuffle addition of one warp holds the FP64 pipe for 16 clocks, so
-    // idle warps take no part)
-    auto publish = [&](const double (&v)[2], int s0, int n) {
-        for (int k = 0; k < n; ++k) {
-            double d = v[k];
-            if (!idle)
-                for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-            if (lane == 0) red[k][warp] = idle ? 0.0 : d;
-        }
+    auto add = [](double d, int o) { return d + __shfl_xor_sync(0xffffffffu, d, o); };
+    // the CTA's sum of red[k][u][0 .. 15] (slots of warps without rows hold 0) to
+    // slot s0 + k of every CTA, then the cluster barrier; n sums per column
+    auto publish = [&](int s0, int n) {
         __syncthreads();
-        if (t < n * NC) {
-            const int k = t / NC, u = t % NC;
-            double d = 0.0;
-            for (int w = u; w < PC_WARPS; w += NC) d += red[k][w];
-            for (int to = 0; to < PC_CL; ++to) cl.map_shared_rank(&part[s0 + k][rank][u], to)[0] = d;
+        if (warp < n * NC) {
+            const int k = warp / NC, col = warp % NC;
+            double d = lane < 16 ? red[k][col][lane] : 0.0;
+            for (int o = 8; o > 0; o >>= 1) d = add(d, o);
+            if (lane < PC_CL) cl.map_shared_rank(&part[s0 + k][col][rank], lane)[0] = d;
         }
         cl.sync();
     };
-    auto total = [&](int s, int u) {
-        double d = 0.0;
-        for (int f = 0; f < PC_CL; ++f) d += part[s][f][u];
-        return d;
+    // first row's part of the preconditioner
+    auto block_of = [&](int i, int& first, int& n) {
+        const int row = r0 + i, blk = bj.fn_blk[row];
+        first = bj.blk_idx[bj.blk_ptr[blk]] - r0;
+        n = bj.blk_ptr[blk + 1] - bj.blk_ptr[blk];
+        return bj.inv + bj.blk_off[blk] + (long long)bj.fn_pos[row] * n;
     };
-    auto precond = [&](int i, int u) {
+    int first0 = 0, n0 = 0;
+    const double* inv0 = bj.inv && i0 < rows ? block_of(i0, first0, n0) : nullptr;
+    auto precond = [&](int i) {
         if (!bj.inv) return r[u * max_rows + i];
-        const int row = r0 + i, blk = bj.fn_blk[row], first = bj.blk_idx[bj.blk_ptr[blk]] - r0;
-        const int n = bj.blk_ptr[blk + 1] - bj.blk_ptr[blk];
-        const double* a = bj.inv + bj.blk_off[blk] + (long long)bj.fn_pos[row] * n;
+        int first = first0, n = n0;
+        const double* a = inv0;
+        if (i != i0) a = block_of(i, first, n);
         double d = 0.0;
         for (int m = 0; m < n; ++m) d = fma(a[m], r[u * max_rows + first + m], d);
         return d;
     };
-    auto send_p = [&](int i, int u, double v) {
-        double* at = &p[(size_t)(r0 + i) * NC + u];
-        for (int to = 0; to < PC_CL; ++to) cl.map_shared_rank(at, to)[0] = v;
+    // z = M r to every CTA, sums r.r and r.z to slots 1 and 2
+    auto precondition = [&] {
+        double v0 = 0.0, v1 = 0.0;
+        for (int i = i0; i < rows; i += di) {
+            const double rv = r[u * max_rows + i], zv = precond(i);
+            double* at = &z[(size_t)(r0 + i) * NC + u];
+            for (int to = 0; to < PC_CL; ++to) cl.map_shared_rank(at, to)[0] = zv;
+            v0 = fma(rv, rv, v0);
+            v1 = fma(rv, zv, v1);
+        }
+        if (!idle) {   // lanes 0 .. 15 reduce r.r, 16 .. 31 r.z
+            const double d = __shfl_xor_sync(0xffffffffu, lane < 16 ? v1 : v0, 16);
+            v0 = (lane < 16 ? v0 : v1) + d;
+            for (int o = 8; o > 0; o >>= 1) v0 = add(v0, o);
+        }
+        if ((lane & 15) == 0) red[lane >> 4][u][warp / NC] = idle ? 0.0 : v0;
+        publish(1, 2);
     };
-    double v[2];
-    auto clear = [&] { v[0] = v[1] = 0.0; };
+    // warp col: totals of r.r (lanes 0 .. 7) and r.z (8 .. 15) of its column
+    auto totals = [&](double& s_rr, double& s_rz) {
+        double d = part[1 + ((lane >> 3) & 1)][warp][lane & 7];
+        for (int o = 4; o > 0; o >>= 1) d = add(d, o);
+        s_rr = __shfl_sync(0xffffffffu, d, 0);
+        s_rz = __shfl_sync(0xffffffffu, d, 8);
+    };
+    for (int e = t; e < 2 * NC * 16; e += PC_THREADS) (&red[0][0][0])[e] = 0.0;
     // x = 0, r = b, z = M r, p = z
     for (int i = i0; i < rows; i += di) {
         x[u * max_rows + i] = 0.0;
         r[u * max_rows + i] = c0 + u < B ? b[(size_t)(r0 + i) * B + c0 + u] : 0.0;
     }
     cl.sync();   // every CTA of the cluster runs: remote shared memory may be written
-    clear();
-    for (int i = i0; i < rows; i += di) {
-        const double rv = r[u * max_rows + i], zv = precond(i, u);
-        send_p(i, u, zv);
-        v[0] = fma(rv, rv, v[0]);
-        v[1] = fma(rv, zv, v[1]);
+    precondition();
+    if (warp < NC) {
+        double s_rr, s_rz;
+        totals(s_rr, s_rz);
+        if (lane == 0) {
+            bn2[warp] = rr[warp] = s_rr;
+            rz[warp] = s_rz;
+            act[warp] = s_rr > 0.0 ? 1 : 0;   // a zero right-hand side is solved by x = 0
+            iters[warp] = 0;
+        }
     }
-    publish(v, 1, 2);
-    if (t < NC) {
-        bn2[t] = rr[t] = total(1, t);
-        rz[t] = total(2, t);
-        act[t] = bn2[t] > 0.0 ? 1 : 0;   // a zero right-hand side is solved by x = 0
-        iters[t] = 0;
-    }
+    for (int e = t; e < K * NC; e += PC_THREADS) p[e] = z[e];
     __syncthreads();
     for (int it = 0; it < limit; ++it) {
-        if (t == 0) {
-            any = 0;
-            for (int u = 0; u < NC; ++u) any |= act[u];
-        }
-        __syncthreads();
+        int any = 0;
+#pragma unroll
+        for (int k = 0; k < NC; ++k) any |= act[k];
         if (!any) break;   // the same decision in every CTA: all hold the same sums
-        // q = S p on this CTA's rows, 8 lanes per row
+        // q = S p on this CTA's rows, 8 lanes per row, and p.q
+        double pq = 0.0;
+        const int col = NC == 2 ? (lane >> 2) & 1 : 0;   // the column a lane ends up with
         for (int i = 4 * warp + (lane >> 3); i - (lane >> 3) < rows; i += 4 * PC_WARPS) {
             double a[NC];
             for (int k = 0; k < NC; ++k) a[k] = 0.0;
@@ -462,48 +485,53 @@ __global__ void __cluster_dims__(PC_CL, 1, 1) __launch_bounds__(PC_THREADS)
                     for (int k = 0; k < NC; ++k) a[k] = fma(s, pj[k], a[k]);
                 }
             }
-#pragma unroll
-            for (int k = 0; k < NC; ++k) {
-                for (int o = 4; o > 0; o >>= 1) a[k] += __shfl_xor_sync(0xffffffffu, a[k], o);
-                if ((lane & 7) == 0 && i < rows) q[k * max_rows + i] = a[k];
+            double d;
+            if (NC == 2) {
+                const double o = __shfl_xor_sync(0xffffffffu, col ? a[0] : a[NC - 1], 4);
+                d = (col ? a[NC - 1] : a[0]) + o;
+            } else {
+                d = add(a[0], 4);
+            }
+            d = add(add(d, 2), 1);
+            if (i < rows) {
+                if ((lane & (NC == 2 ? 3 : 7)) == 0) q[col * max_rows + i] = d;
+                pq = fma(p[(size_t)(r0 + i) * NC + col], d, pq);
+            }
+        }
+        pq = add(add(pq, 8), 16);
+        if (lane < 8 && (lane & (NC == 2 ? 3 : 7)) == 0) red[0][col][warp] = pq;
+        publish(0, 1);
+        if (warp < NC) {
+            double s_pq = part[0][warp][lane & 7];
+            for (int o = 4; o > 0; o >>= 1) s_pq = add(s_pq, o);
+            if (lane == 0) {
+                alpha[warp] = act[warp] && s_pq > 0.0 ? rz[warp] / s_pq : 0.0;
+                iters[warp] += act[warp];
             }
         }
         __syncthreads();
-        clear();
-        for (int i = i0; i < rows; i += di) {
-            v[0] = fma(p[(size_t)(r0 + i) * NC + u], q[u * max_rows + i], v[0]);
-        }
-        publish(v, 0, 1);
-        if (t < NC) {
-            const double pq = total(0, t);
-            alpha[t] = act[t] && pq > 0.0 ? rz[t] / pq : 0.0;
-            iters[t] += act[t];
-        }
-        __syncthreads();
+        if (t < NC * 16) (&red[0][0][0])[t] = 0.0;   // the slots of warps beyond a column's
         for (int i = i0; i < rows; i += di) {
             const double a = alpha[u];
             x[u * max_rows + i] = fma(a, p[(size_t)(r0 + i) * NC + u], x[u * max_rows + i]);
             r[u * max_rows + i] = fma(-a, q[u * max_rows + i], r[u * max_rows + i]);
         }
         __syncthreads();
-        clear();
-        for (int i = i0; i < rows; i += di) {
-            const double rv = r[u * max_rows + i], zv = precond(i, u);
-            z[u * max_rows + i] = zv;
-            v[0] = fma(rv, rv, v[0]);
-            v[1] = fma(rv, zv, v[1]);
-        }
-        publish(v, 1, 2);
-        if (t < NC) {
-            rr[t] = total(1, t);
-            if (act[t] && !(rr[t] > tol2 * bn2[t])) act[t] = 0;
-            const double n = total(2, t);
-            beta[t] = act[t] && rz[t] != 0.0 ? n / rz[t] : 0.0;
-            if (act[t]) rz[t] = n;
+        precondition();
+        if (warp < NC) {
+            double n_rr, n;
+            totals(n_rr, n);
+            if (lane == 0) {
+                const int a = act[warp] && n_rr > tol2 * bn2[warp];
+                rr[warp] = n_rr;
+                beta[warp] = a && rz[warp] != 0.0 ? n / rz[warp] : 0.0;
+                if (a) rz[warp] = n;
+                act[warp] = a;
+            }
         }
         __syncthreads();
-        for (int i = i0; i < rows; i += di) send_p(i, u, fma(beta[u], p[(size_t)(r0 + i) * NC + u], z[u * max_rows + i]));
-        cl.sync();
+        for (int e = t; e < K * NC; e += PC_THREADS) p[e] = fma(beta[e % NC], p[e], z[e]);
+        __syncthreads();
     }
     for (int i = i0; i < rows && c0 + u < B; i += di) x_out[(size_t)(r0 + i) * B + c0 + u] = x[u * max_rows + i];
     if (rank == 0 && t < NC && c0 + t < B) {
@@ -626,6 +654,7 @@ struct Csr {
     int* idx = nullptr;
     double* val = nullptr;
     long long nnz = 0;
+    std::vector<int> ptr_host;
 };
 
 void build_csr(int K, const double* A, double thr, int* cnt, Csr& m, cudaStream_t s) {
@@ -633,10 +662,10 @@ void build_csr(int K, const double* A, double thr, int* cnt, Csr& m, cudaStream_
     k_scan_rows<<<1, 1024, 0, s>>>(K, cnt, m.ptr);
     k_csr_fill<<<nblocks(K, 8), 256, 0, s>>>(K, A, thr, m.ptr, m.idx, m.val);
     check_launch("csr_build", 3);
-    int nnz = 0;
-    DFT_CUDA_CHECK(cudaMemcpyAsync(&nnz, m.ptr + K, sizeof(int), cudaMemcpyDeviceToHost, s));
+    m.ptr_host.resize(K + 1);
+    DFT_CUDA_CHECK(cudaMemcpyAsync(m.ptr_host.data(), m.ptr, sizeof(int) * (K + 1), cudaMemcpyDeviceToHost, s));
     DFT_CUDA_CHECK(cudaStreamSynchronize(s));
-    m.nnz = nnz;
+    m.nnz = m.ptr_host[K];
 }
 
 // an instantiated graph of PCG_GRAPH iterations for one block width
@@ -816,24 +845,30 @@ void sparse_columns(Ctx& c, const double* F, const int* cols, int ncols, double 
     // few columns.  Otherwise iterations of seven kernels run as graphs.
     constexpr int PC_MAX_K = 4096, PC_SMEM = 225 * 1024;
     PcRows pr{};
-    int max_rows = 0;
+    int max_rows = 0, max_nnz = 0;
     bool cluster = K <= PC_MAX_K;
     for (int i = 0; nbj > 0 && i < K; ++i) cluster = cluster && blk_idx[i] == i;
     if (cluster) {
         int at = 0;
         for (int rk = 1; rk <= PC_CL; ++rk) {
-            const long long want = (long long)K * rk / PC_CL;
-            if (nbj == 0) at = (int)want;
-            else
-                while (at < want) at = blk_ptr[fn_blk[at] + 1];
+            // runs of equal weight, two parts entries to one part rows: a run has at
+            // most 3 / 8 of the rows, whose vectors fit at PC_MAX_K
+            const auto weight = [&](int i) { return 2LL * mS.ptr_host[i] * K + mS.nnz * i; };
+            const long long want = weight(K) / PC_CL * rk;
+            while (at < K && weight(at) < want) at = nbj == 0 ? at + 1 : blk_ptr[fn_blk[at] + 1];
             pr.at[rk] = rk == PC_CL ? K : at;
             max_rows = std::max(max_rows, pr.at[rk] - pr.at[rk - 1]);
+            max_nnz = std::max(max_nnz, mS.ptr_host[pr.at[rk]] - mS.ptr_host[pr.at[rk - 1]]);
         }
     }
+    // entries of S kept in shared memory: all of a run or none
+    auto cached_for = [&](auto nc) {
+        const int want = (max_nnz + 1) & ~1;
+        return pc_smem<decltype(nc)::value>(K, max_rows, want) <= (size_t)PC_SMEM ? want : 0;
+    };
     auto solve_cluster = [&](int Bb, auto nc) {
         constexpr int NC = decltype(nc)::value;
-        const long long room = (long long)(PC_SMEM - (long long)pc_smem<NC>(K, max_rows, 0)) / 12;
-        const int cached = (int)std::min<long long>(room, (long long)max_rows * K) & ~1;
+        const int cached = cached_for(nc);
         auto kern = k_pcg_cluster<NC>;
         DFT_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, PC_SMEM));
         kern<<<PC_CL * ((Bb + NC - 1) / NC), PC_THREADS, pc_smem<NC>(K, max_rows, cached), s>>>(
@@ -846,8 +881,11 @@ void sparse_columns(Ctx& c, const double* F, const int* cols, int ncols, double 
     auto solve = [&](int Bb) {
         if (cluster) {
             // one column per cluster while that fits the SMs at once, then two
-            if (PC_CL * Bb <= 152) solve_cluster(Bb, std::integral_constant<int, 1>{});
-            else solve_cluster(Bb, std::integral_constant<int, 2>{});
+            constexpr std::integral_constant<int, 1> one{};
+            constexpr std::integral_constant<int, 2> two{};
+            const int per_sm = pc_smem<1>(K, max_rows, cached_for(one)) <= PC_SMEM / 2 ? 2 : 1;
+            if (PC_CL * Bb <= 152 * per_sm) solve_cluster(Bb, one);
+            else solve_cluster(Bb, two);
             return;
         }
         const long long n = (long long)K * Bb;
