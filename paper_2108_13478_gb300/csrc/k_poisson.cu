@@ -125,7 +125,8 @@ __device__ __forceinline__ void pw92(double rs, double& v, double& e) {
 constexpr double RS0 = 0.62035049089940001;   // (3 / (4 pi))^(1/3): r_s = RS0 n^(-1/3)
 
 // v_ks = v_loc + v_H + v_xc; energy partials sum v_loc n, v_H rho, eps_xc n
-// (v_xc: Slater exchange, plus PW92 correlation with C)
+// (v_xc: Slater exchange, plus PW92 correlation with C; pad = nullptr: no
+// potential, and the Hartree energy comes from k_spectrum_energy)
 template <bool C>
 __global__ void __launch_bounds__(256) k_vks(int nx, int ny, int nz, int Nx, int Ny, const double* __restrict__ pad,
                                              const double* __restrict__ n, const double* __restrict__ nion,
@@ -136,7 +137,7 @@ __global__ void __launch_bounds__(256) k_vks(int nx, int ny, int nz, int Nx, int
     for (int g = blockIdx.x * 256 + threadIdx.x; g < ng; g += gridDim.x * 256) {
         const int line = g / nx, ix = g - line * nx;
         const int iz = line / ny, iy = line - iz * ny;
-        double vh = pad[((long long)iz * Ny + iy) * Nx + ix];
+        double vh = pad ? pad[((long long)iz * Ny + iy) * Nx + ix] : 0.0;
         double d = n[g];
         const double cb = d > 1e-30 ? cbrt_pos(d) : 0.0;
         double c = CX * cb;
@@ -162,6 +163,29 @@ __global__ void __launch_bounds__(256) k_vks(int nx, int ny, int nz, int Nx, int
         part[3 * blockIdx.x + 1] = s1;
         part[3 * blockIdx.x + 2] = s2;
     }
+}
+
+// sum_g v_H rho without the potential: v_H is the padded circular convolution
+// and rho is zero outside the box, so by Parseval the sum is sum_k G_k |rho_k|^2 (G
+// holds the transforms' scale), each k_x but 0 and Nx / 2 standing for two.
+// Into the second slot of each block's energy partials.  Saves the energy of
+// an output density the inverse transforms, about half of a solve (6.0 ms at
+// 147^3 points)
+__global__ void __launch_bounds__(256) k_spectrum_energy(int Nx, long long n, const cufftDoubleComplex* __restrict__ c,
+                                                         const double* __restrict__ G, double* __restrict__ part) {
+    const int nxc = Nx / 2 + 1, last = Nx % 2 == 0 ? Nx / 2 : -1;
+    const long long stride = (long long)gridDim.x * 256, e0 = (long long)blockIdx.x * 256 + threadIdx.x;
+    const int step = (int)(stride % nxc);
+    int kx = (int)(e0 % nxc);
+    double s = 0.0;
+    for (long long e = e0; e < n; e += stride) {
+        const double w = kx == 0 || kx == last ? G[e] : 2.0 * G[e];
+        s = fma(w, fma(c[e].x, c[e].x, c[e].y * c[e].y), s);
+        kx += step;
+        if (kx >= nxc) kx -= nxc;
+    }
+    s = block_sum<256>(s);
+    if (threadIdx.x == 0) part[3 * blockIdx.x + 1] = s;
 }
 
 __global__ void __launch_bounds__(256) k_energy_reduce(int np, const double* part, double h3, double* scal) {
@@ -390,19 +414,26 @@ void hartree_xc(Ctx& c, const double* n, double* vks, bool energies, cudaStream_
     const long long filled = (long long)c.Nfft[1] * (c.Nfft[0] / 2 + 1) * c.n[2];
     DFT_CUDA_CHECK(cudaMemsetAsync(c.d_fft_c + filled, 0, sizeof(cufftDoubleComplex) * (c.nfft_c - filled), s));
     cufft_check(cufftExecZ2Z(c.plan_z, c.d_fft_c, c.d_fft_c, CUFFT_FORWARD), "exec Z2Z");
-    k_mul_real<<<blocks_for(c.nfft_c, 256), 256, 0, s>>>(c.nfft_c, c.d_fft_c, c.d_ghat);
-    check_launch("mul_real");
-    cufft_check(cufftExecZ2Z(c.plan_z, c.d_fft_c, c.d_fft_c, CUFFT_INVERSE), "exec Z2Z");
-    cufft_check(cufftExecZ2D(c.plan_b, c.d_fft_c, c.d_fft_o), "exec Z2D");
+    if (vks) {
+        k_mul_real<<<blocks_for(c.nfft_c, 256), 256, 0, s>>>(c.nfft_c, c.d_fft_c, c.d_ghat);
+        check_launch("mul_real");
+        cufft_check(cufftExecZ2Z(c.plan_z, c.d_fft_c, c.d_fft_c, CUFFT_INVERSE), "exec Z2Z");
+        cufft_check(cufftExecZ2D(c.plan_b, c.d_fft_c, c.d_fft_o), "exec Z2D");
+    }
+    const double* vh = vks ? c.d_fft_o : nullptr;
     int np = (int)std::min<long long>(1184, (c.ng + 255) / 256);
     if (c.p.xc == DFT_XC_PW92)
-        k_vks<true><<<np, 256, 0, s>>>(c.n[0], c.n[1], c.n[2], c.Nfft[0], c.Nfft[1], c.d_fft_o, n, nion, c.d_vloc,
+        k_vks<true><<<np, 256, 0, s>>>(c.n[0], c.n[1], c.n[2], c.Nfft[0], c.Nfft[1], vh, n, nion, c.d_vloc,
                                        vks, c.d_part);
     else
-        k_vks<false><<<np, 256, 0, s>>>(c.n[0], c.n[1], c.n[2], c.Nfft[0], c.Nfft[1], c.d_fft_o, n, nion, c.d_vloc,
+        k_vks<false><<<np, 256, 0, s>>>(c.n[0], c.n[1], c.n[2], c.Nfft[0], c.Nfft[1], vh, n, nion, c.d_vloc,
                                         vks, c.d_part);
     check_launch("vks");
     if (energies) {
+        if (!vks) {
+            k_spectrum_energy<<<np, 256, 0, s>>>(c.Nfft[0], c.nfft_c, c.d_fft_c, c.d_ghat, c.d_part);
+            check_launch("spectrum_energy");
+        }
         k_energy_reduce<<<1, 256, 0, s>>>(np, c.d_part, c.h * c.h * c.h, c.d_scal);
         check_launch("energy_reduce");
     }
