@@ -21,7 +21,7 @@
 // at a time: warp 0 lane 0 drives the TMA loads of the four operand tiles of
 // each 32-wide k-block into a 4-stage ring of 48 KB, warp 1 owns the 512
 // tensor-memory columns and lane 0 issues the MMAs, eight epilogue warps add
-// each finished unit of SUB k-blocks from one of two accumulators into FP32
+// each finished unit of one or two k-blocks from one of two accumulators into FP32
 // registers (round to nearest; the tensor core's own FP32 accumulation leans
 // towards zero with every addition, so its chains are kept short) and then
 // write x = alpha A B - prev + add straight from registers: neighbouring lanes
@@ -33,9 +33,9 @@
 // drains what it issued and returns.
 //
 // Density matrix at K = 1230, tail 1e-5 (N_C ~ 1410, direct plan): 118.9 ms
-// with the recurrence of k_cheb_tc.cu, 7.4 ms with this (error of P against
-// an exact eigensolve 3.7e-5 -> 2.5e-5); SCF cycle at K = 4650 (Clenshaw plan,
-// s = 34, 112 products) 677 -> 165 ms.
+// with the recurrence of k_cheb_tc.cu, 6.1 ms with this (error of P against
+// an exact eigensolve 3.6e-5 -> 1.7e-5); SCF step at K = 4650 (Clenshaw plan,
+// s = 34, 112 products) 668 -> 87 ms.
 #include "ps_plan.cuh"
 #include "tc_ptx.cuh"
 
@@ -323,6 +323,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
             const uint16_t* ad = w.it.add >= 0 ? (const uint16_t*)S.slot[w.it.add] + e0 : nullptr;
             uint16_t* out = (uint16_t*)S.slot[w.it.out] + e0;
             const float limit = w.it.limit;
+            const bool edge = w.i * BM + BM > K || w.j * BN + BN > K;   // rows or columns beyond K
             bool bad = false;
             constexpr int EB = 16;   // columns per batch, the next one's loads in flight
             uint32_t nh[EB / 2], nl[EB / 2], mh[EB / 2], ml[EB / 2];
@@ -380,59 +381,96 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
                     gl[k] = ml[k];
                 }
                 if (cb + EB < CPT) fetch(cb + EB);
+                // Step by step over the whole batch, the uniform branches outside: inside
+                // the loop over columns they kept the columns' chains of shuffles and
+                // conversions from overlapping.  Conversions go in pairs and neighbours exchange
+                // sums (one shuffle instead of two).  Clocks of a tile's update, without and with
+                // prev: 25,400 and 29,500 before, 14,500 and 15,900 now (the products of a tile
+                // take 57,400 at K = 1230).
+                // x[2 k], x[2 k + 1]: columns c, c + 1 of this lane's row, one from its own
+                // words, one from the neighbour's
+                float x[EB];
+#pragma unroll
+                for (int u = 0; u < EB; ++u) x[u] = alpha * __uint_as_float(av[u]);
+                if (pv) {
+#pragma unroll
+                    for (int k = 0; k < EB / 2; ++k) {
+                        const float2 h = H16<BF>::to_f2(ph[k]), l = H16<BF>::to_f2(pl[k]);
+                        const float f0 = h.x + l.x, f1 = h.y + l.y;   // rows r & ~1, r | 1
+                        const float got = __shfl_xor_sync(0xffffffffu, odd ? f0 : f1, 1);
+                        x[2 * k] = fmaf(-ISC, odd ? got : f0, x[2 * k]);
+                        x[2 * k + 1] = fmaf(-ISC, odd ? f1 : got, x[2 * k + 1]);
+                    }
+                }
+                if (ad) {
+#pragma unroll
+                    for (int k = 0; k < EB / 2; ++k) {
+                        const uint32_t f0 = __byte_perm(gl[k], gh[k], 0x5410), f1 = __byte_perm(gl[k], gh[k], 0x7632);
+                        const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? f0 : f1, 1);
+                        x[2 * k] += __uint_as_float(odd ? got : f0);
+                        x[2 * k + 1] += __uint_as_float(odd ? f1 : got);
+                    }
+                }
+                if (diag && ident) {
+#pragma unroll
+                    for (int u = 0; u < EB; ++u)
+                        if (c0 + cb + u == r) x[u] -= 1.0f;
+                }
+                if (diag || edge) {
+#pragma unroll
+                    for (int u = 0; u < EB; ++u) {
+                        const int c = c0 + cb + u;
+                        bad |= !(fabsf(x[u]) <= limit) && r < K && c < K && (!diag || c >= r);
+                    }
+                } else {
+#pragma unroll
+                    for (int u = 0; u < EB; ++u) bad |= !(fabsf(x[u]) <= limit);
+                }
+                uint32_t own[EB];
+                if (f32_out) {
+#pragma unroll
+                    for (int u = 0; u < EB; ++u) own[u] = __byte_perm(__float_as_uint(x[u]), 0, 0x1032);   // upper half first
+                } else {
+#pragma unroll
+                    for (int k = 0; k < EB / 2; ++k) {
+                        const float y0 = x[2 * k] * SC, y1 = x[2 * k + 1] * SC;
+                        const uint32_t h = H16<BF>::from_f2(y0, y1);
+                        const float2 f = H16<BF>::to_f2(h);
+                        const uint32_t l = H16<BF>::from_f2(y0 - f.x, y1 - f.y);
+                        own[2 * k] = __byte_perm(h, l, 0x5410);
+                        own[2 * k + 1] = __byte_perm(h, l, 0x7632);
+                    }
+                }
+                uint32_t eh[EB / 2], el[EB / 2];   // rows r & ~1, r | 1 of column c + (lane & 1)
 #pragma unroll
                 for (int k = 0; k < EB / 2; ++k) {
-                    // columns c, c + 1 of this lane's row: one from its own words, one from
-                    // the neighbour's
-                    uint32_t own[2];
-                    float x[2];
+                    const uint32_t mine = odd ? own[2 * k + 1] : own[2 * k];
+                    const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? own[2 * k] : own[2 * k + 1], 1);
+                    const uint32_t e = odd ? got : mine, o = odd ? mine : got;
+                    eh[k] = __byte_perm(e, o, 0x5410);
+                    el[k] = __byte_perm(e, o, 0x7632);
+                }
+                if (!diag) {
 #pragma unroll
-                    for (int u = 0; u < 2; ++u) x[u] = alpha * __uint_as_float(av[2 * k + u]);
-                    if (pv) {
-                        const uint32_t qh = __shfl_xor_sync(0xffffffffu, ph[k], 1);
-                        const uint32_t ql = __shfl_xor_sync(0xffffffffu, pl[k], 1);
-                        const uint32_t h0 = odd ? qh >> 16 : ph[k], h1 = odd ? ph[k] >> 16 : qh;
-                        const uint32_t l0 = odd ? ql >> 16 : pl[k], l1 = odd ? pl[k] >> 16 : ql;
-                        x[0] = fmaf(-ISC, H16<BF>::to_f(from_bits16<T>(h0)) + H16<BF>::to_f(from_bits16<T>(l0)), x[0]);
-                        x[1] = fmaf(-ISC, H16<BF>::to_f(from_bits16<T>(h1)) + H16<BF>::to_f(from_bits16<T>(l1)), x[1]);
+                    for (int k = 0; k < EB / 2; ++k) {
+                        const size_t at = (size_t)(cb + 2 * k) * ld;
+                        *(uint32_t*)(out + at) = eh[k];
+                        *(uint32_t*)(out + plane + at) = el[k];
                     }
-                    if (ad) {
-                        const uint32_t qh = __shfl_xor_sync(0xffffffffu, gh[k], 1);
-                        const uint32_t ql = __shfl_xor_sync(0xffffffffu, gl[k], 1);
-                        const uint32_t f0 = odd ? __byte_perm(ql, qh, 0x7632) : __byte_perm(gl[k], gh[k], 0x5410);
-                        const uint32_t f1 = odd ? __byte_perm(gl[k], gh[k], 0x7632) : __byte_perm(ql, qh, 0x5410);
-                        x[0] += __uint_as_float(f0);
-                        x[1] += __uint_as_float(f1);
-                    }
+                } else {
 #pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        const int c = c0 + cb + 2 * k + u;
-                        if (ident && c == r) x[u] -= 1.0f;
-                        bad |= !(fabsf(x[u]) <= limit) && r < K && c < K && (!diag || c >= r);
-                        if (f32_out) {
-                            own[u] = __byte_perm(__float_as_uint(x[u]), 0, 0x1032);   // upper half first
-                        } else {
-                            const float y = x[u] * SC;
-                            const T th = H16<BF>::from_f(y);
-                            own[u] = bits16(th) | (bits16(H16<BF>::from_f(y - H16<BF>::to_f(th))) << 16);
+                    for (int k = 0; k < EB / 2; ++k) {
+                        const size_t at = (size_t)(cb + 2 * k) * ld;
+                        const int c = c0 + cb + 2 * k + odd;
+                        if (c >= (r | 1)) {
+                            *(uint32_t*)(out + at) = eh[k];
+                            *(uint32_t*)(out + plane + at) = el[k];
+                        } else if (c == (r & ~1)) {
+                            out[at] = (uint16_t)eh[k];
+                            out[plane + at] = (uint16_t)el[k];
                         }
-                    }
-                    const uint32_t mine = odd ? own[1] : own[0];
-                    const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? own[0] : own[1], 1);
-                    const uint32_t e = odd ? got : mine, o = odd ? mine : got;   // even and odd row of my column
-                    const size_t at = (size_t)(cb + 2 * k) * ld;
-                    const uint32_t eh = __byte_perm(e, o, 0x5410), el = __byte_perm(e, o, 0x7632);
-                    const int c = c0 + cb + 2 * k + odd;
-                    if (!diag || c >= (r | 1)) {
-                        *(uint32_t*)(out + at) = eh;
-                        *(uint32_t*)(out + plane + at) = el;
-                    } else if (c == (r & ~1)) {
-                        out[at] = (uint16_t)eh;
-                        out[plane + at] = (uint16_t)el;
-                    }
-                    if (diag) {
-                        tr[(2 * k) * 33 + lane] = own[0];
-                        tr[(2 * k + 1) * 33 + lane] = own[1];
+                        tr[(2 * k) * 33 + lane] = own[2 * k];
+                        tr[(2 * k + 1) * 33 + lane] = own[2 * k + 1];
                     }
                 }
                 if (diag) {
