@@ -161,8 +161,10 @@ __device__ double block_sum(double v) {
 
 // part[A][slab][k] = sum over the points of z slab blockIdx.y within RCUT of
 // atom A = blockIdx.x of resid * exp(-r^2/w_k^2): warps over rows, lanes along
-// x, chains of four rows' FP32 products before they meet in FP64 (16 FP64
-// multiply-adds per point kept the FP64 pipe busy for twice the Gaussians' time)
+// x.  Four rows' products are summed in pairs of FP32 numbers (residual in two
+// parts, exact product and sum errors carried), then in FP64: 16 FP64
+// multiply-adds per point kept the FP64 pipe busy for twice the Gaussians' time,
+// and plain FP32 chains left the gradient 20% less accurate.
 __global__ void __launch_bounds__(256) k_assemble_adjoint(const double* __restrict__ xyz, const double* __restrict__ resid,
                                                           int nx, int ny, int nz, double ox, double oy, double oz,
                                                           double h, Widths wd, double* __restrict__ part) {
@@ -175,11 +177,11 @@ __global__ void __launch_bounds__(256) k_assemble_adjoint(const double* __restri
         hi[d] = min(nn[d] - 1, (int)floor((c[d] + RCUT - o[d]) / h));
     }
     double acc[NO];
-    float f[NO];
+    float f[NO], fc[NO];   // sum and its error
 #pragma unroll
     for (int k = 0; k < NO; ++k) {
         acc[k] = 0.0;
-        f[k] = 0.0f;
+        f[k] = fc[k] = 0.0f;
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ey = hi[1] - lo[1] + 1, ez = hi[2] - lo[2] + 1;
@@ -197,21 +199,28 @@ __global__ void __launch_bounds__(256) k_assemble_adjoint(const double* __restri
             const double dx = ox + h * ix - c[0];
             const double r2 = dx * dx + q;
             if (r2 >= RCUT * RCUT) continue;
-            const float r2f = (float)r2, v = (float)rv[ix];
+            const double vd = rv[ix];
+            const float r2f = (float)r2, v = (float)vd, vl = (float)(vd - (double)v);
 #pragma unroll
-            for (int k = 0; k < NO; ++k) f[k] = fmaf(v, expf(-r2f * wd.iw2[k]), f[k]);
+            for (int k = 0; k < NO; ++k) {
+                const float e = expf(-r2f * wd.iw2[k]);
+                const float p = __fmul_rn(v, e), pe = fmaf(vl, e, fmaf(v, e, -p));
+                const float t = __fadd_rn(f[k], p), b = __fsub_rn(t, f[k]);
+                fc[k] += (__fsub_rn(f[k], __fsub_rn(t, b)) + __fsub_rn(p, b)) + pe;
+                f[k] = t;
+            }
         }
         if (++held == 4) {   // at 0.4 bohr a row has two points per lane
             held = 0;
 #pragma unroll
             for (int k = 0; k < NO; ++k) {
-                acc[k] += (double)f[k];
-                f[k] = 0.0f;
+                acc[k] += (double)f[k] + (double)fc[k];
+                f[k] = fc[k] = 0.0f;
             }
         }
     }
     for (int k = 0; k < NO; ++k) {
-        const double v = block_sum<256>(acc[k] + (double)f[k]);
+        const double v = block_sum<256>(acc[k] + ((double)f[k] + (double)fc[k]));
         if (threadIdx.x == 0) part[((long long)a * gridDim.y + blockIdx.y) * NO + k] = v;
     }
 }
