@@ -17,7 +17,6 @@ rank 0 prints one JSON line.
 from __future__ import annotations
 
 import argparse
-import tempfile
 import json
 import os
 import statistics
@@ -205,9 +204,8 @@ def cpu_baseline(sysm, budget_s):
 
 def run_batched(args, rank, world):
     """Ragged batch: every SCF step advances all systems with one
-    dft_scf_step_batched call (the tensor-core recurrence of the whole batch
-    as one launch per step in a CUDA graph, or one dataflow launch per pass,
-    whichever the tuner picks).  Value = sum of K over systems x steps / time."""
+    dft_scf_step_batched call (the products of all systems' expansions merged
+    into tensor-core launches).  Value = sum of K over systems x steps / time."""
     import torch
     import torch.distributed as dist
     import paper_2108_13478_gb300 as dft
@@ -297,9 +295,6 @@ def run_dm_only(args, dft, torch, sysm, prec, local, rank):
     K = ctx.K
     t = statistics.median(ms)
     info = infos[-1]
-    flops = 3.0 * K * K * (K + 1)
-    per_launch = info.ms_stage[4] / 1000.0 / max(1, info.n_cheb - 2)
-    pk = peaks()
     line = {"metric": METRIC, "value": K / (t / 1000.0), "unit": "P-columns/s (dft_density_matrix)", "n_gpus": 1,
             "steps": args.steps, "warmup": 0, "ms_per_step": t, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": args.precision, "data": "synthetic",
@@ -307,9 +302,7 @@ def run_dm_only(args, dft, torch, sysm, prec, local, rank):
                        "n_cheb": info.n_cheb, "cheb_tail_tol": cheb_tail(args), "mode": "density matrix only",
                        "setup_s": setup_s},
             "stages_ms": [round(x, 3) for x in info.ms_stage],
-            "roofline": {"kernel": "k_cheb_step_tc", "bound": "tensor", "achieved": flops / per_launch / 1e12,
-                         "peak": pk.get("bf16_tflops_sustained", 1700.0), "unit": "TFLOP/s",
-                         "frac": flops / per_launch / 1e12 / pk.get("bf16_tflops_sustained", 1700.0)}}
+            "roofline": expansion_roofline(infos, K, False, *tensor_peak(peaks()))}
     if rank == 0:
         print(json.dumps(line), flush=True)
     ctx.close()
@@ -366,10 +359,6 @@ def dm_accuracy(dft, torch, local, name, tail):
     e_kin = 2.0 * float(torch.sum(P * T))
     e_band = 2.0 * float(torch.sum(P * F))
     n_e = 2.0 * float(torch.sum(P * S))
-    per_step = info.ms_stage[4] / 1000.0 / max(1, info.n_cheb - 2)
-    flops = 3.0 * K * K * (K + 1)
-    pk = peaks()
-    peak = pk.get("bf16_tflops_sustained", 1700.0)
     out.update({
         "ms": ms, "value": K / (ms / 1000.0), "unit": "P-columns/s (dft_density_matrix)", "n_cheb": info.n_cheb,
         "stages_ms": [round(x, 3) for x in info.ms_stage],
@@ -378,8 +367,7 @@ def dm_accuracy(dft, torch, local, name, tail):
         "n_e_trace": n_e, "n_e_uncorrected": info.n_e_uncorrected, "n_electrons": s.n_electrons,
         "mu": info.mu, "mu_oracle": g["mu"], "mu_correction": info.mu_correction,
         "gate_1e-5_Ha_per_atom": bool(abs(e_kin - g["e_kin"]) / na <= 1e-5 and abs(e_band - g["e_band"]) / na <= 1e-5),
-        "roofline": {"kernel": "k_cheb_step_tc", "bound": "tensor", "achieved": flops / per_step / 1e12,
-                     "peak": peak, "unit": "TFLOP/s", "frac": flops / per_step / 1e12 / peak},
+        "roofline": expansion_roofline([info], K, False, *tensor_peak(peaks())),
         "reference": "oracle exact traces, tests/golden/" + os.path.basename(path)})
     ctx.close()
     return out
@@ -623,25 +611,23 @@ def run_reference(args, sysm, rank, world):
     print(json.dumps(line), flush=True)
 
 
-# DRAM bytes per recurrence step of the weighted pass from ncu captures
-# (dram__bytes_read.sum + dram__bytes_write.sum of one dataflow launch over
-# its steps), keyed by workload, dataflow launch (1) or not, k-block width
-# and the SHA-256 (first 16 hex digits) of the kernel source they were taken
-# on: a changed kernel has no traffic figure until it is captured again
-MEASURED_TRAFFIC = {
-    # weighted pass of one density matrix at N_C 1414 (1412 steps), sphere25
-    ("sphere25", 1, 32, "f66dc8e82982a668"): (1176.289e9 + 281.285e9) / 1412,
-}
-TC_SOURCE = os.path.join(ROOT, "paper_2108_13478_gb300", "csrc", "k_cheb_tc.cu")
+def expansion_roofline(infos, K, fp64, peak, peak_source):
+    """Roofline of the Chebyshev expansion (moments and weighted sum): a
+    polynomial of N_C terms and its moments take at least 2 sqrt(2 N_C)
+    products of symmetric K x K matrices (the fewest products any grouping of
+    s + 2 N_C / s needs), each K^2 (K + 1) flop, three times that in split 16-bit form; over the time of
+    both passes, so that everything else in them counts as loss."""
+    per = (1.0 if fp64 else 3.0) * K * K * (K + 1.0)
+    rate = statistics.median(2.0 * (2.0 * i.n_cheb) ** 0.5 * per / ((i.ms_stage[3] + i.ms_stage[4]) / 1000.0)
+                             for i in infos if i.ms_stage[3] + i.ms_stage[4] > 0) / 1e12
+    return {"kernel": "k_ps_prod" if fp64 else "k_pst_prod", "bound": "alu" if fp64 else "tensor", "achieved": rate,
+            "peak": peak, "unit": "TFLOP/s", "frac": rate / peak, "traffic": None, "peak_source": peak_source}
 
 
-def kernel_sha16(path=TC_SOURCE):
-    import hashlib
-    try:
-        with open(path, "rb") as f:
-            return hashlib.sha256(f.read()).hexdigest()[:16]
-    except OSError:
-        return None
+def tensor_peak(pk):
+    return pk.get("bf16_tflops_sustained", 1700.0), (
+        "MEASURED_PEAKS bf16_tflops_sustained (of measured; fp16 dense rate equals bf16)"
+        if "bf16_tflops_sustained" in pk else "fallback 1700 TFLOP/s sustained (MEASURED_PEAKS.json absent)")
 
 
 def max_over_ranks(value, world, device):
@@ -659,19 +645,6 @@ def job_throughput(world, units_per_rank, steps, max_ms):
     """Units all ranks processed per second (weak scaling: every rank runs the
     same workload), timed by the slowest rank."""
     return world * units_per_rank * steps / (max_ms / 1000.0)
-
-
-def tuned_shape():
-    """Launch shape(s) the tuner picked in this process: {key: {bk, persist, bn, streamk, flow}}."""
-    path = os.environ.get("DFT_AUTOTUNE_CACHE")
-    if not path or not os.path.exists(path):
-        return None
-    try:
-        with open(path) as f:
-            d = json.load(f)
-    except (OSError, ValueError):
-        return None
-    return {k: dict(zip(("bk", "persist", "bn", "streamk", "flow"), v[:5])) for k, v in d.items()}
 
 
 def main():
@@ -692,9 +665,6 @@ def main():
         return
     import torch
     import torch.distributed as dist
-    # the library's launch-shape tuner writes its choice here (read back for the report)
-    if "DFT_AUTOTUNE_CACHE" not in os.environ:
-        os.environ["DFT_AUTOTUNE_CACHE"] = os.path.join(tempfile.mkdtemp(prefix="dft_tune_"), "autotune.json")
     import paper_2108_13478_gb300 as dft
     torch.cuda.set_device(local)
     if world > 1:
@@ -767,36 +737,16 @@ def main():
         e2e_ms += e0.elapsed_time(e1)
         n_host.copy_(out_host)
     e2e_value = job_throughput(world, K, args.steps, max_over_ranks(e2e_ms, world, f"cuda:{local}"))
-    # roofline of the dominant kernel: the Chebyshev step (one launch per term of pass 2)
     pk = peaks()
     n_c = infos[-1].n_cheb
-    # each step's weighted-pass time over its own number of recurrence launches
-    per_launch_s = statistics.median(i.ms_stage[4] / 1000.0 / max(1, i.n_cheb - 2) for i in infos)
     sm_mhz = clocks.get("sm_mhz") or pk.get("sm_max_mhz", 2070.0)
-    if prec == dft.DFT_PREC_FP64:
-        flops = 2.0 * K ** 3
-        peak = FP64_FLOP_PER_SM_CLK * N_SM * sm_mhz * 1e6 / 1e12
-        roof = {"kernel": "k_cheb_step_fp64", "bound": "alu", "achieved": flops / per_launch_s / 1e12,
-                "peak": peak, "unit": "TFLOP/s", "frac": (flops / per_launch_s / 1e12) / peak,
-                "traffic": None, "peak_source": "FP64 issue rate 4 flop/SM/clk x 152 SMs x median SM clock"}
-        dtype = "f64"
+    fp64 = prec == dft.DFT_PREC_FP64
+    if fp64:
+        roof = expansion_roofline(infos, K, True, FP64_FLOP_PER_SM_CLK * N_SM * sm_mhz * 1e6 / 1e12,
+                                  "FP64 issue rate 4 flop/SM/clk x 152 SMs x median SM clock")
     else:
-        # three 16-bit products per step on the upper triangle of the symmetric
-        # output: 3 x K(K+1)/2 outputs x 2K flop
-        flops = 3.0 * K * K * (K + 1)
-        tiles = tc_tiles(K)
-        kpad = -(-K // 64) * 64
-        executed = 3.0 * tiles * 128 * 256 * 2 * kpad
-        peak = pk.get("bf16_tflops_sustained", 1700.0)
-        ach = flops / per_launch_s / 1e12
-        roof = {"kernel": "k_cheb_step_tc", "bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
-                "frac": ach / peak, "traffic": None,
-                "executed_mma_tflops": executed / per_launch_s / 1e12,
-                "fp32_class_tflops": ach / 3.0,
-                "peak_source": ("MEASURED_PEAKS bf16_tflops_sustained (of measured; fp16 dense rate equals bf16)"
-                                if "bf16_tflops_sustained" in pk else
-                                "fallback 1700 TFLOP/s sustained (MEASURED_PEAKS.json absent)")}
-        dtype = args.precision
+        roof = expansion_roofline(infos, K, False, *tensor_peak(pk))
+    dtype = "f64" if fp64 else args.precision
     line = {"metric": METRIC, "value": value, "unit": "P-columns/s", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": total_ms / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": dtype, "data": "synthetic",
@@ -813,21 +763,6 @@ def main():
             "stages_ms_median": [round(statistics.median(i.ms_stage[k] for i in infos), 3) for k in range(8)],
             "mu_reused_steps": int(sum(i.mu_reused for i in infos)),
             "energy_per_atom": infos[-1].e_total / sysm.n_atoms}
-    shape = tuned_shape()
-    if prec != dft.DFT_PREC_FP64:
-        # which source of the tensor-core step this line measured (and the key of
-        # its DRAM traffic record)
-        line["roofline"]["kernel_source_sha16"] = kernel_sha16()
-    if shape is not None and prec != dft.DFT_PREC_FP64:
-        line["roofline"]["launch_shape"] = shape
-        shapes = {(v.get("flow", 0), v.get("bk", 32)) for v in shape.values()}
-        if len(shapes) == 1:
-            flow, bk = shapes.pop()
-            tr = MEASURED_TRAFFIC.get((sysm.name, flow, bk, kernel_sha16()))
-            if tr is not None:
-                line["roofline"]["traffic"] = tr
-                line["roofline"]["traffic_note"] = "DRAM bytes per recurrence step (ncu, dataflow launch)"
-
     if rank == 0 and not args.no_compare:
         line["mixed_vs_fp64"] = compare_precisions(dft, torch, local, cheb_tail(args))
     if rank == 0 and not args.no_sparse:
