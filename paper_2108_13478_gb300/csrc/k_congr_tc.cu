@@ -353,13 +353,18 @@ __global__ void __launch_bounds__(256) k_corr_norms(int K, const double* __restr
 // 2 beta (Tr rho - ||rho||_F^2): dmu = (N_e / 2 - Tr rho) / (beta (Tr rho -
 // ||rho||^2)).  Skipped (dmu = 0) where the first-order step is not
 // trustworthy: no states at the Fermi level, or |beta dmu| > 0.5.
-__global__ void k_corr_mu(int np, const double* __restrict__ part, double beta, double n_e, double* scal) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+__global__ void __launch_bounds__(32) k_corr_mu(int np, const double* __restrict__ part, double beta, double n_e, double* scal) {
+    // one warp, strided sums joined in a fixed order (one thread took 54 us)
     double tr = 0.0, fr = 0.0;
-    for (int i = 0; i < np; ++i) {
+    for (int i = threadIdx.x; i < np; i += 32) {
         tr += part[2 * i];
         fr += part[2 * i + 1];
     }
+    for (int o = 16; o > 0; o >>= 1) {
+        tr += __shfl_down_sync(0xffffffffu, tr, o);
+        fr += __shfl_down_sync(0xffffffffu, fr, o);
+    }
+    if (threadIdx.x != 0) return;
     const double slope = beta * (tr - fr);
     double dmu = 0.0, raw = INFINITY;
     if (slope > 1e-12 * fmax(1.0, tr)) {

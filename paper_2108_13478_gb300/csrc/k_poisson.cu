@@ -235,11 +235,13 @@ __global__ void __launch_bounds__(256) k_maxabs_part(long long n, const double* 
     }
 }
 
-__global__ void k_max_parts(int np, const double* part, double* out) {
-    if (threadIdx.x != 0) return;
+// one warp (one thread took 74 us for the 1184 parts of a step, most of it
+// latency between a batch's systems)
+__global__ void __launch_bounds__(32) k_max_parts(int np, const double* part, double* out) {
     double r = 0.0;
-    for (int i = 0; i < np; ++i) r = fmax(r, part[i]);
-    *out = r;
+    for (int i = threadIdx.x; i < np; i += 32) r = fmax(r, part[i]);
+    for (int o = 16; o > 0; o >>= 1) r = fmax(r, __shfl_down_sync(0xffffffffu, r, o));
+    if (threadIdx.x == 0) *out = r;
 }
 
 // Kerker weights g^2 / (g^2 + q0^2) over the periodic box, R2C layout
