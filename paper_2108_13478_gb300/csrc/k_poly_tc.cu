@@ -1090,11 +1090,12 @@ void pst_pass1(Ctx* const* cs, int n, const int* moments, cudaStream_t st) {
             for (int q = 1; q <= p.Q; ++q) g.push_back(v.giant(q));
             gram(c, 1, g, st);
         }
-        if (!p.direct && p.Q > 1) {
+        if (!p.direct && p.Q > 0) {
             const int r0 = v.extra(0), nring = v.nextra(), ts = v.baby(s);
             if (moments[k]) {
-                // giants G_2 .. G_Q in a ring of nring buffers; the Gram sums take up
-                // to nring - 2 at a time, so that the babies are read less often
+                // giants G_2 .. G_Q (none where Q = 1, whose G_1 = T_s has its Gram sums all
+                // the same) in a ring of nring buffers; the Gram sums take up to nring - 2
+                // at a time, so that the babies are read less often
                 std::vector<int> at(p.Q + 1, ts);
                 for (int q = 2; q <= p.Q; ++q) at[q] = r0 + (q - 2) % nring;
                 for (int q = 1; q < p.Q; ++q) {

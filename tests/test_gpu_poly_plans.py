@@ -1,0 +1,78 @@
+"""The grouped expansion on Fock matrices with a chosen spectrum: plans of a
+context whose workspace holds few expansion buffers (Clenshaw's recurrence,
+down to a single giant).
+
+F = L F~ L^T with S = L L^T and F~ = W diag(x) W^T for an orthogonal W, so the
+eigenvalues of S^-1 F are x, and the expansion of order N_C is evaluated at
+them exactly: P = L^-T W diag(p(x)) W^T L^-1."""
+import numpy as np
+import pytest
+import scipy.fft
+
+from workloads.si_clusters import diamond_sphere, jitter, make_system
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no GPU", allow_module_level=True)
+
+import paper_2108_13478_gb300 as dft  # noqa: E402
+from oracle import dm  # noqa: E402
+
+FP64, FP16 = dft.DFT_PREC_FP64, dft.DFT_PREC_FP16X3
+
+
+def few_slots():
+    """K = 3500 on a coarse grid: a mixed context has 30 expansion buffers."""
+    xyz = diamond_sphere(25.0)
+    xyz = jitter(xyz[np.argsort((xyz ** 2).sum(1), kind="stable")[:350]], 0.05, 1)
+    return make_system(xyz, h=1.0, grid_n=np.array([60, 60, 60]), grid_origin=xyz.min(0) - 7.0)
+
+
+def given_spectrum(ctx, x, W):
+    """F and L^-T W for the eigenvalues x (device)."""
+    S, _ = ctx.overlap_kinetic()
+    L = torch.linalg.cholesky(S)
+    A = L @ W
+    return ((A * x) @ A.T).contiguous(), torch.linalg.solve_triangular(L.T, W, upper=True)
+
+
+def orthogonal(K, localised=False):
+    g = torch.Generator(device="cuda").manual_seed(11)
+    if localised:   # every eigenvector close to one function
+        v = torch.randn(K, 1, generator=g, device="cuda", dtype=torch.float64)
+        return torch.eye(K, device="cuda", dtype=torch.float64) - 2.0 / float((v ** 2).sum()) * (v @ v.T)
+    return torch.linalg.qr(torch.randn(K, K, generator=g, device="cuda", dtype=torch.float64))[0]
+
+
+def coefficients(mu, beta, n_c):
+    """a_l on [-1, 1] from 4 N_C nodes, as the library takes them."""
+    m = 4 * n_c
+    a = scipy.fft.dct(dm.fermi(np.cos(np.pi * (np.arange(m) + 0.5) / m), mu, beta), type=2)[:n_c] / m
+    a[0] *= 0.5
+    return a
+
+
+@pytest.mark.parametrize("n_c", [26, 40, 46])
+def test_clenshaw_plan_with_a_single_giant(n_c):
+    """One giant, no room to keep it with its sums: its moments still come
+    from its own Gram sums (mu, and with it the electron count, depend on
+    them)."""
+    s = few_slots()
+    beta = n_c / 2.0
+    ctx = dft.Context(s, precision=FP16, e_min=-1.0, e_max=1.0, cheb_order=n_c, kT=1.0 / beta, skip_correction=1)
+    K = ctx.K
+    x = np.sort(np.random.default_rng(2).uniform(-0.95, 0.95, K))
+    F, LW = given_spectrum(ctx, torch.from_numpy(x).cuda(), orthogonal(K))
+    mom = dm.moments_from_eigs(x, n_c)
+    mu = dm.bisect(lambda m: 2.0 * float(coefficients(m, beta, n_c) @ mom), s.n_electrons, -1.0 - 40 / beta, 1.0 + 40 / beta)
+    for _ in range(2):   # the second call finds the first one's weights where its sums go
+        P, info = ctx.density_matrix(F)
+    ctx.close()
+    ref = (LW * torch.from_numpy(dm.cheb_eval(x, coefficients(mu, beta, n_c))).cuda()) @ LW.T
+    err = float((P - ref).abs().max() / ref.abs().max())
+    print(f"K {K} N_C {n_c}: dmu {info.mu - mu:.2e}, N_e {info.n_e_trace:.6f} of {s.n_electrons}, max|dP| / max|P| {err:.2e}")
+    assert abs(info.mu - mu) < 1e-5
+    assert abs(info.n_e_trace - s.n_electrons) < 1e-5 * s.n_electrons
+    assert err < 1e-4
