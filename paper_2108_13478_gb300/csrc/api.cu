@@ -635,8 +635,9 @@ void dm_prepare(Ctx& c, const double* F, cudaStream_t s, Timer* tm, int t0) {
     if (n_c > 2) launch_moment_reduce(1, c.d_scal + SCAL_TRACE, c.d_mom, 2, -1, m0, c.d_mom + 1, s);
 }
 
-// first pass of one system: the matrices of the expansion and, if wanted, the
-// moments m_l = Tr T_l(H_N), l < N_C (the plain recurrence by doubling)
+// first pass of one system: the matrices of the expansion and, if wanted (mixed
+// path; FP64 always), the moments m_l = Tr T_l(H_N), l < N_C (the plain
+// recurrence by doubling)
 void dm_pass1(Ctx& c, bool moments, cudaStream_t s) {
     if (c.p.precision != DFT_PREC_FP64 && !c.recurrence) {
         Ctx* cp = &c;
@@ -663,7 +664,7 @@ void dm_pass1(Ctx& c, bool moments, cudaStream_t s) {
         }
         return;
     }
-    ps64_pass1(c, moments, s);
+    ps64_pass1(c, s);
 }
 
 // mu from 2 sum_l a_l(mu) m_l = N_e (Eq. 2.8), then the coefficients

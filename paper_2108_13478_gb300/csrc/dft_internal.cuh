@@ -355,7 +355,7 @@ void launch_ps_moments(int K, const PsPlan& p, const double* D, double* mom, cud
 void launch_ps_coefs(const PsPlan& p, const double* a, double* c, double* work, cudaStream_t s);
 // FP64 path: babies and giants of H_N and the moments into d_mom; then
 // rho = sum_l a_l T_l into d_rho from the coefficients in d_coef
-void ps64_pass1(Ctx& c, bool moments, cudaStream_t s);
+void ps64_pass1(Ctx& c, cudaStream_t s);
 void ps64_pass2(Ctx& c, cudaStream_t s);
 
 // the same in split 16-bit form on the tensor cores, for n systems at once

@@ -410,6 +410,24 @@ struct Ps64 {
             }
         }
     }
+    // the spectrum check beyond the last giant (ps_check), in slots s0 and s0 + 1
+    void check(int s0) const {
+        const PsCheck k = ps_check(p, true);
+        const double* cur = baby(std::max(1, k.baby));
+        for (int i = 0, l = k.baby; i < k.doublings; ++i) {
+            // T_{2l} = 2 T_l^2 - I or T_{2l+1} = 2 T_l T_{l+1} - T_1
+            Ps64Items it{};
+            it.A[0] = cur;
+            it.B[0] = k.odd ? baby(l + 1) : cur;
+            it.prev[0] = k.odd ? baby(1) : nullptr;
+            it.ident[0] = k.odd ? 0 : 1;
+            it.out[0] = c.ps_slot[s0 + (i & 1)];
+            it.first[1] = 1;
+            l *= 2;
+            products(it, 1, 2.0, i + 1 == k.doublings ? growth_limit(l + k.odd, p.n_c) : 4.0);
+            cur = it.out[0];
+        }
+    }
     void gram(int q0, int nq, const PsList& G, double* D) const {
         const int s = p.s;
         PsList T{};
@@ -424,17 +442,10 @@ struct Ps64 {
     }
 };
 
-// the iterates grow like cosh(l t) when the spectrum leaves the interval: the
-// bound at l that corresponds to 4 at the last term n_c - 1
-double growth_limit(int l, int n_c) {
-    if (l >= n_c - 1 || n_c < 3) return 4.0;
-    return std::cosh(std::acosh(4.0) * (double)l / (n_c - 1));
-}
-
 }  // namespace
 
-// babies, giants and (with moments) m_l; the plan is kept in c.ps
-void ps64_pass1(Ctx& c, bool moments, cudaStream_t st) {
+// babies, giants and m_l; the plan is kept in c.ps
+void ps64_pass1(Ctx& c, cudaStream_t st) {
     const double waves = upper_tiles(c.K, 16) / 152.0;
     c.ps = ps_plan(c.n_c_cur, (int)c.ps_slot.size(), std::ceil(waves), waves, 2);
     const PsPlan& p = c.ps;
@@ -450,10 +461,10 @@ void ps64_pass1(Ctx& c, bool moments, cudaStream_t st) {
         it.ident[0] = r == 1;
         it.out[0] = const_cast<double*>(e.baby(r + 1));
         it.first[1] = 1;
-        e.products(it, 1, 2.0, 4.0);
+        e.products(it, 1, 2.0, r + 1 == s && Q == 1 ? growth_limit(s, p.n_c) : 4.0);
     }
     double* D = c.d_wk;   // (Q + 1) s doubles, consumed before the moment weights are written there
-    if (moments && s > 1) {
+    if (s > 1) {
         PsList L{};
         for (int r = 1; r < s; ++r) L.p[r - 1] = e.baby(r);
         k_ps_trace<<<s - 1, 128, 0, st>>>(c.K, L, D + 1, 1);
@@ -461,14 +472,14 @@ void ps64_pass1(Ctx& c, bool moments, cudaStream_t st) {
     }
     if (p.direct) {
         e.doubling(Q, [&](int q) { return e.giant(q); }, growth_limit(Q * s, p.n_c));
-        if (moments && Q > 0)
+        if (Q > 0)
             for (int q0 = 1; q0 <= Q; q0 += PS_MAX_S) {
                 const int nq = std::min(PS_MAX_S, Q - q0 + 1);
                 PsList G{};
                 for (int q = 0; q < nq; ++q) G.p[q] = e.giant(q0 + q);
                 e.gram(q0, nq, G, D);
             }
-    } else if (moments) {
+    } else {
         double* roll[2] = {c.ps_slot[s - 1], c.ps_slot[s]};
         const double* Ts = e.baby(s);
         const double *prev = nullptr, *cur = Ts;
@@ -490,7 +501,8 @@ void ps64_pass1(Ctx& c, bool moments, cudaStream_t st) {
             cur = it.out[0];
         }
     }
-    if (moments) launch_ps_moments(c.K, p, D, c.d_mom, st);
+    e.check(p.direct ? s - 1 + std::max(0, Q - 1) : s - 1);   // the buffers behind the giants, or those they rolled in
+    launch_ps_moments(c.K, p, D, c.d_mom, st);
 }
 
 // rho = sum_l a_l T_l with the coefficients in c.d_coef

@@ -823,11 +823,6 @@ int sys_tiles(const Ctx& c) {
     return n;
 }
 
-double growth_limit(int l, int n_c) {
-    if (l >= n_c - 1 || n_c < 3) return 4.0;
-    return std::cosh(std::acosh(4.0) * (double)l / (n_c - 1));
-}
-
 // One call's product launches: items are queued level by level (all systems
 // of the batch together) and uploaded once per flush.
 struct Queue {
@@ -1024,8 +1019,8 @@ void pst_split_h(Ctx& c, cudaStream_t st) {
 }
 
 // Babies, giants and moments of every system (T_1 in place).  moments[q] = 0:
-// the coefficients of system q are already fixed, so only the spectrum check
-// is left of the moments' giants.
+// the coefficients of system q are already fixed, so a Clenshaw plan forms no
+// giants and only the spectrum check is left of them.
 void pst_pass1(Ctx* const* cs, int n, const int* moments, cudaStream_t st) {
     Ctx& lead = *cs[0];
     std::vector<PstSys> tab(n);
@@ -1062,7 +1057,7 @@ void pst_pass1(Ctx* const* cs, int n, const int* moments, cudaStream_t st) {
             if (r >= (p.Q > 0 ? p.s : p.s - 1)) continue;
             const View v(*cs[k]);
             Q.add(k, *cs[k], {make_int2(v.baby(1), v.baby(r))}, r > 1 ? v.baby(r - 1) : -1, -1, v.baby(r + 1),
-                  PST_FINE | PST_ALPHA2 | (r == 1 ? PST_IDENT : 0), 4.0);
+                  PST_FINE | PST_ALPHA2 | (r == 1 ? PST_IDENT : 0), r + 1 == p.s && p.Q == 1 ? growth_limit(p.s, p.n_c) : 4.0);
             any = true;
         }
         Q.close();
@@ -1090,46 +1085,46 @@ void pst_pass1(Ctx* const* cs, int n, const int* moments, cudaStream_t st) {
             for (int q = 1; q <= p.Q; ++q) g.push_back(v.giant(q));
             gram(c, 1, g, st);
         }
-        if (!p.direct && p.Q > 0) {
+        if (!p.direct && moments[k] && p.Q > 0) {
             const int r0 = v.extra(0), nring = v.nextra(), ts = v.baby(s);
-            if (moments[k]) {
-                // giants G_2 .. G_Q (none where Q = 1, whose G_1 = T_s has its Gram sums all
-                // the same) in a ring of nring buffers; the Gram sums take up to nring - 2
-                // at a time, so that the babies are read less often
-                std::vector<int> at(p.Q + 1, ts);
-                for (int q = 2; q <= p.Q; ++q) at[q] = r0 + (q - 2) % nring;
-                for (int q = 1; q < p.Q; ++q) {
-                    Q.add(k, c, {make_int2(ts, at[q])}, q > 1 ? at[q - 1] : -1, -1, at[q + 1],
-                          PST_ALPHA2 | (q == 1 ? PST_IDENT : 0), q + 1 == p.Q ? growth_limit(p.Q * s, p.n_c) : 4.0);
-                    Q.close();
-                }
-                Q.upload();
-                int done = 1;   // giants 1 .. done - 1 are in the Gram sums
-                for (int q = 1; q <= p.Q; ++q) {
-                    const int have = q - done + 1;
-                    if (q == p.Q || have >= std::max(1, nring - 2)) {
-                        gram(c, done, std::vector<int>(at.begin() + done, at.begin() + q + 1), st);
-                        done = q + 1;
-                    }
-                    if (q < p.Q) Q.launch(q - 1);
-                }
-                Q.items.clear();
-                Q.pairs.clear();
-                Q.launches.clear();
-                Q.open = 0;
-            } else {
-                // T_{2^i s} up to the order of the expansion: the spectrum check
-                int cur = ts, l = s;
-                for (int i = 0; 2 * l <= p.n_c - 1; ++i) {
-                    Q.add(k, c, {make_int2(cur, cur)}, -1, -1, r0 + (i & 1), PST_ALPHA2 | PST_IDENT,
-                          growth_limit(2 * l, p.n_c));
-                    Q.close();
-                    cur = r0 + (i & 1);
-                    l *= 2;
-                }
-                Q.run();
+            // giants G_2 .. G_Q (none where Q = 1, whose G_1 = T_s has its Gram sums all
+            // the same) in a ring of nring buffers; the Gram sums take up to nring - 2
+            // at a time, so that the babies are read less often
+            std::vector<int> at(p.Q + 1, ts);
+            for (int q = 2; q <= p.Q; ++q) at[q] = r0 + (q - 2) % nring;
+            for (int q = 1; q < p.Q; ++q) {
+                Q.add(k, c, {make_int2(ts, at[q])}, q > 1 ? at[q - 1] : -1, -1, at[q + 1],
+                      PST_ALPHA2 | (q == 1 ? PST_IDENT : 0), q + 1 == p.Q ? growth_limit(p.Q * s, p.n_c) : 4.0);
+                Q.close();
             }
+            Q.upload();
+            int done = 1;   // giants 1 .. done - 1 are in the Gram sums
+            for (int q = 1; q <= p.Q; ++q) {
+                const int have = q - done + 1;
+                if (q == p.Q || have >= std::max(1, nring - 2)) {
+                    gram(c, done, std::vector<int>(at.begin() + done, at.begin() + q + 1), st);
+                    done = q + 1;
+                }
+                if (q < p.Q) Q.launch(q - 1);
+            }
+            Q.items.clear();
+            Q.pairs.clear();
+            Q.launches.clear();
+            Q.open = 0;
         }
+        // the spectrum check beyond the last giant (the giants' buffers, or those behind them, are free)
+        const PsCheck ck = ps_check(p, p.direct || moments[k]);
+        int cur = v.baby(std::max(1, ck.baby));
+        for (int i = 0, l = ck.baby; i < ck.doublings; ++i) {
+            // T_{2l} = 2 T_l^2 - I or T_{2l+1} = 2 T_l T_{l+1} - T_1
+            const int out = v.extra(i & 1);
+            l *= 2;
+            Q.add(k, c, {make_int2(cur, ck.odd ? cur + 1 : cur)}, ck.odd ? v.baby(1) : -1, -1, out,
+                  PST_ALPHA2 | (ck.odd ? 0 : PST_IDENT), i + 1 == ck.doublings ? growth_limit(l + ck.odd, p.n_c) : 4.0);
+            Q.close();
+            cur = out;
+        }
+        Q.run();
         if (moments[k]) launch_ps_moments(c.K, p, c.d_wk, c.d_mom, st);
     }
 }

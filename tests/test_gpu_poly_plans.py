@@ -1,6 +1,6 @@
 """The grouped expansion on Fock matrices with a chosen spectrum: plans of a
 context whose workspace holds few expansion buffers (Clenshaw's recurrence,
-down to a single giant).
+down to a single giant), and the refusal of a spectrum outside the interval.
 
 F = L F~ L^T with S = L L^T and F~ = W diag(x) W^T for an orthogonal W, so the
 eigenvalues of S^-1 F are x, and the expansion of order N_C is evaluated at
@@ -9,6 +9,7 @@ import numpy as np
 import pytest
 import scipy.fft
 
+import workloads as w
 from workloads.si_clusters import diamond_sphere, jitter, make_system
 
 pytestmark = pytest.mark.gpu
@@ -76,3 +77,71 @@ def test_clenshaw_plan_with_a_single_giant(n_c):
     assert abs(info.mu - mu) < 1e-5
     assert abs(info.n_e_trace - s.n_electrons) < 1e-5 * s.n_electrons
     assert err < 1e-4
+
+
+def outside(n_c, weight, at_last):
+    """The eigenvalue above 1 whose T_{n_c - 1} makes an element of `at_last`
+    with an eigenvector of largest squared component `weight`."""
+    return float(np.cosh(np.arccosh(at_last / weight) / (n_c - 1)))
+
+
+# (atoms, precision, N_C): one giant, two, a few; many (kept); Clenshaw's recurrence
+PLANS = [(8, FP64, 26), (8, FP64, 40), (8, FP64, 71), (8, FP64, 140), (8, FP64, 1400), (8, FP64, 7000),
+         (8, FP16, 26), (8, FP16, 40), (8, FP16, 71), (8, FP16, 140), (8, FP16, 1400), (8, FP16, 2900)]
+
+
+@pytest.mark.parametrize("atoms,prec,n_c", PLANS)
+def test_spectrum_outside_the_interval_is_refused(atoms, prec, n_c):
+    """An eigenvalue above the interval makes the last term's largest element
+    12: refused (the limit is 4), also where that term is never formed.  One
+    that makes it 1.5 stays accepted."""
+    s = w.config_system(f"tiny{atoms}")
+    for at_last, ok in ((12.0, False), (1.5, True)):
+        ctx = dft.Context(s, precision=prec, e_min=-1.0, e_max=1.0, cheb_order=n_c, kT=4.0 / n_c)
+        K = ctx.K
+        W = orthogonal(K)
+        x = np.sort(np.random.default_rng(2).uniform(-0.9, 0.9, K))
+        x[-1] = outside(n_c, float((W[:, -1] ** 2).max()), at_last)
+        F, _ = given_spectrum(ctx, torch.from_numpy(x).cuda(), W)
+        if ok:
+            _, info = ctx.density_matrix(F)
+            assert info.spectrum_ok == 1
+        else:
+            with pytest.raises(dft.DftError) as e:
+                ctx.density_matrix(F)
+            print(f"N_C {n_c}, x_max - 1 = {x[-1] - 1:.2e}, T_last {at_last}: {e.value}")
+            assert e.value.status == dft._binding.DFT_ESPECTRUM
+        ctx.close()
+
+
+def test_spectrum_outside_the_interval_is_refused_where_mu_is_reused():
+    """A cycle that takes over mu forms no giants: only the check itself sees
+    a spectrum that left the interval since the cycles before."""
+    s = w.config_system("tiny8")
+    ref = dft.Context(s, model=dft.DFT_MODEL_NEUTRAL)
+    S, T = ref.overlap_kinetic()
+    Li = torch.linalg.inv(torch.linalg.cholesky(S))
+
+    def edges(n):
+        e = torch.linalg.eigvalsh(Li @ (T + ref.potential_matrix(ref.hartree_xc(n)[0])) @ Li.T)
+        return float(e[0]), float(e[-1])
+    n0 = ref.initial_density()
+    n1 = 0.9 * n0
+    if edges(n1)[1] < edges(n0)[1]:
+        n0, n1 = n1, n0
+    (lo, top0), (_, top1) = edges(n0), edges(n1)
+    ref.close()
+    # top1 at cosh(12 / 2899) of the interval, top0 well inside
+    n_c, lo = 2900, lo - 1.0
+    hi = lo + 2.0 * (top1 - lo) / (1.0 + np.cosh(12.0 / (n_c - 1)))
+    assert top0 < hi - 1e-3
+    ctx = dft.Context(s, precision=FP16, model=dft.DFT_MODEL_NEUTRAL, e_min=lo, e_max=hi, cheb_order=n_c, mix_alpha=0.0,
+                      reuse_mu=1)
+    ctx.overlap_kinetic()
+    n = n0.clone()
+    assert [ctx.scf_step(n).mu_reused for _ in range(3)] == [0, 0, 1]
+    with pytest.raises(dft.DftError) as e:
+        ctx.scf_step(n1.clone())
+    print(f"top eigenvalues {top0:.4f}, {top1:.6f}, E_max {hi:.6f}: refused, {e.value}")
+    assert e.value.status == dft._binding.DFT_ESPECTRUM
+    ctx.close()
