@@ -223,7 +223,8 @@ dft_status dft_nonlocal_matrix(dft_ctx* ctx, double* VNL, void* stream);
  * rho += dmu beta (rho - rho^2), which restores 2 Tr[P S] = N_e to FP64
  * rounding; it is skipped where no states lie at the Fermi level or
  * |beta dmu| > 0.5.  DFT_EINTERNAL if a split operand leaves the FP16
- * range (|x| >= 32768). */
+ * range (|x| >= 32768; 32 for the elements of rho, where a spectrum outside
+ * the interval is reported first, as DFT_ESPECTRUM). */
 dft_status dft_density_matrix(dft_ctx* ctx, const double* F, double* P, dft_info* info, void* stream);
 
 /* Preconditioners of the sparse-operator route (dft_density_matrix_columns) */

@@ -745,6 +745,7 @@ void dm_finish(Ctx& c, double* P, dft_info* info, cudaStream_t s) {
     if (flags[FLAG_TIMEOUT]) throw Error(DFT_ETIMEOUT, "a tensor-core pipeline wait expired");
     if (flags[FLAG_RANGE]) throw Error(DFT_EINTERNAL, "a split-precision congruence left the range of the FP16 pair");
     if (flags[FLAG_SPECTRUM]) throw Error(DFT_ESPECTRUM, "Chebyshev iterates left [-1, 1]: spectral bounds too tight");
+    if (flags[FLAG_RHO]) throw Error(DFT_EINTERNAL, "the density matrix left the range of the FP16 pair");
     if (flags[FLAG_MU]) throw Error(DFT_ENOTCONV, "mu bisection: the bracket does not contain N_e");
 }
 

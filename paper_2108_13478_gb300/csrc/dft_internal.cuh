@@ -284,8 +284,10 @@ enum {
     SCAL_DMU_RAW = 303,  // its Newton step before the trust check
     SCAL_COUNT = 304
 };
-// FLAG_RANGE: a split-precision operand or product left the FP16 pair's range
-enum { FLAG_SPECTRUM = 0, FLAG_CHOL = 1, FLAG_MU = 2, FLAG_TIMEOUT = 3, FLAG_RANGE = 4, FLAG_COUNT = 8 };
+// FLAG_RANGE: a split-precision operand or product left the FP16 pair's range;
+// FLAG_RHO: the same of rho and what is formed from it (|rho| <= 1 unless the
+// expansion diverged, which FLAG_SPECTRUM reports first)
+enum { FLAG_SPECTRUM = 0, FLAG_CHOL = 1, FLAG_MU = 2, FLAG_TIMEOUT = 3, FLAG_RANGE = 4, FLAG_RHO = 5, FLAG_COUNT = 8 };
 
 // ---- grid kernels (k_grid.cu) ----
 void launch_build_tables(const Ctx& c, cudaStream_t s);

@@ -60,6 +60,7 @@ struct Out {
     __half* lo = nullptr;
     double* f64 = nullptr;  // FP64 output, K x K (ld K), symmetric when upper
     float scale = 1.0f;     // applied to the product (a power of two)
+    int range = FLAG_RANGE; // flag set when a split output leaves the pair's range
 };
 // rho's pair holds RHO_SCALE rho: most of its elements are far below 1, where
 // the low half of an unscaled FP16 pair is subnormal (2^-25 absolute, which
@@ -273,7 +274,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm3_tc(const __grid_constant_
                     *(uint4*)(ph + 8 * c8) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
                     *(uint4*)(pl + 8 * c8) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
                 }
-                if (big) atomicExch(&flags[FLAG_RANGE], 1);
+                if (big) atomicExch(&flags[out.range], 1);
             } else if (r < K) {
                 double* o = out.f64;
                 // lanes hold consecutive rows: the mirror stores (row c, column r)
@@ -299,16 +300,16 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gemm3_tc(const __grid_constant_
 }
 
 // FP64 K x K (leading dimension ld, transposed if trans) -> FP16 pair Kp x Kp,
-// zero-padded; FLAG_RANGE if an element is outside the pair's range
+// zero-padded; *flag if an element is outside the pair's range
 __global__ void k_split16(int K, int Kp, const double* __restrict__ A, int ld, int trans, double scale, __half* __restrict__ hi,
-                          __half* __restrict__ lo, int* __restrict__ flags) {
+                          __half* __restrict__ lo, int* __restrict__ flag) {
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (long long)Kp * Kp) return;
     const int i = (int)(e / Kp), j = (int)(e % Kp);
     double x = 0.0;
     if (i < K && j < K) x = scale * (trans ? A[(long long)j * ld + i] : A[(long long)i * ld + j]);
     if (!(fabs(x) < (double)SPLIT_MAX)) {
-        atomicExch(&flags[FLAG_RANGE], 1);
+        atomicExch(flag, 1);
         x = 0.0;
     }
     const __half h = __double2half(x);
@@ -414,9 +415,11 @@ void gemm(const Ctx& c, const CUtensorMap* a, const CUtensorMap* b, int kr, bool
     check_launch("gemm3_tc");
 }
 
-void split(const Ctx& c, const double* A, bool trans, void* hi, void* lo, cudaStream_t s, double scale = 1.0) {
+void split(const Ctx& c, const double* A, bool trans, void* hi, void* lo, cudaStream_t s, double scale = 1.0,
+           int flag = FLAG_RANGE) {
     const long long n = (long long)c.Kp * c.Kp;
-    k_split16<<<blocks_for(n, 256), 256, 0, s>>>(c.K, c.Kp, A, c.K, trans ? 1 : 0, scale, (__half*)hi, (__half*)lo, c.d_flags);
+    k_split16<<<blocks_for(n, 256), 256, 0, s>>>(c.K, c.Kp, A, c.K, trans ? 1 : 0, scale, (__half*)hi, (__half*)lo,
+                                             c.d_flags + flag);
     check_launch("split16");
 }
 
@@ -450,7 +453,7 @@ void cg_transform_f(const Ctx& c, const double* F, double* Ft, cudaStream_t s) {
 }
 
 void cg_split_rho(const Ctx& c, cudaStream_t s) {
-    cg::split(c, c.d_rho, false, c.d_x16[0], c.d_x16[1], s, cg::RHO_SCALE);
+    cg::split(c, c.d_rho, false, c.d_x16[0], c.d_x16[1], s, cg::RHO_SCALE, FLAG_RHO);
 }
 
 void cg_correct_rho(const Ctx& c, cudaStream_t s) {
@@ -475,6 +478,7 @@ void cg_back_transform(const Ctx& c, double* P, cudaStream_t s) {
     g2.hi = (__half*)c.d_x16[2];
     g2.lo = (__half*)c.d_x16[3];
     g2.scale = 1.0f / cg::RHO_SCALE;
+    g2.range = FLAG_RHO;
     cg::gemm(c, c.tm_lt[0], c.tm_x[0], cg::KR_ROW_START, false, g2, s);
     cg::Out p;
     p.f64 = P;

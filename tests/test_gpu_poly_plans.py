@@ -94,9 +94,10 @@ PLANS = [(8, FP64, 26), (8, FP64, 40), (8, FP64, 71), (8, FP64, 140), (8, FP64, 
 def test_spectrum_outside_the_interval_is_refused(atoms, prec, n_c):
     """An eigenvalue above the interval makes the last term's largest element
     12: refused (the limit is 4), also where that term is never formed.  One
-    that makes it 1.5 stays accepted."""
+    that makes it 1.5 stays accepted; one that drives the operands or rho out
+    of an FP16 pair is the same refusal, not an internal error."""
     s = w.config_system(f"tiny{atoms}")
-    for at_last, ok in ((12.0, False), (1.5, True)):
+    for at_last, ok in ((12.0, False), (1.5, True), (300.0, False), (1e7, False)):
         ctx = dft.Context(s, precision=prec, e_min=-1.0, e_max=1.0, cheb_order=n_c, kT=4.0 / n_c)
         K = ctx.K
         W = orthogonal(K)
@@ -144,4 +145,18 @@ def test_spectrum_outside_the_interval_is_refused_where_mu_is_reused():
         ctx.scf_step(n1.clone())
     print(f"top eigenvalues {top0:.4f}, {top1:.6f}, E_max {hi:.6f}: refused, {e.value}")
     assert e.value.status == dft._binding.DFT_ESPECTRUM
+    ctx.close()
+
+
+def test_fock_matrix_beyond_the_pair_is_an_internal_error():
+    """Elements of F beyond the FP16 pair's range: the split reports them,
+    whatever the expansion then makes of the operands."""
+    s = w.config_system("tiny8")
+    ctx = dft.Context(s, precision=FP16, e_min=-1.0, e_max=1.0, cheb_order=100, kT=0.04)
+    W = orthogonal(ctx.K)
+    F, _ = given_spectrum(ctx, torch.linspace(-0.9, 0.9, ctx.K, device="cuda", dtype=torch.float64), W)
+    F[3, 3] = 1e6
+    with pytest.raises(dft.DftError) as e:
+        ctx.density_matrix(F)
+    assert e.value.status == dft._binding.DFT_EINTERNAL
     ctx.close()
