@@ -860,6 +860,7 @@ void sparse_columns(Ctx& c, const double* F, const int* cols, int ncols, double 
             max_rows = std::max(max_rows, pr.at[rk] - pr.at[rk - 1]);
             max_nnz = std::max(max_nnz, mS.ptr_host[pr.at[rk]] - mS.ptr_host[pr.at[rk - 1]]);
         }
+        cluster = pc_smem<2>(K, max_rows, 0) <= (size_t)PC_SMEM;   // not where no entry of S is kept: one run holds all rows
     }
     // entries of S kept in shared memory: all of a run or none
     auto cached_for = [&](auto nc) {

@@ -10,6 +10,7 @@ import numpy as np
 import pytest
 
 import workloads as w
+from workloads.si_clusters import diamond_sphere, jitter, make_system
 from oracle import basis, dm
 from oracle import sparse as osp
 
@@ -164,3 +165,21 @@ def test_columns_with_contracted_d_functions(name):
     assert info.not_converged == 0
     assert np.max(np.abs(out.cpu().numpy() - ref)) < 1e-8 * np.max(np.abs(ref))
     p["ctx"].close()
+
+
+def large():
+    """K = 3500 on a coarse grid."""
+    xyz = diamond_sphere(25.0)
+    xyz = jitter(xyz[np.argsort((xyz ** 2).sum(1), kind="stable")[:350]], 0.05, 1)
+    return make_system(xyz, h=1.0, grid_n=np.array([60, 60, 60]), grid_origin=xyz.min(0) - 7.0)
+
+
+def test_no_entry_of_s_kept():
+    """A threshold above every entry leaves an empty S: the first solve does not
+    converge, the others start from zero, and the columns are zero."""
+    ctx = dft.Context(large())
+    _, T = ctx.overlap_kinetic()
+    out, info = ctx.density_matrix_columns(T, list(range(32)), 1.0, 0.0, 20.0, 3, thresh=1e9, pcg_maxit=8)
+    assert info.nnz_s == 0 and info.pcg_solves == 3 and info.not_converged == 1
+    assert float(out.abs().max()) == 0.0
+    ctx.close()
