@@ -16,9 +16,13 @@
 // Layout: a block of vectors is K x B row-major (row i holds the B columns'
 // entries i), so one sparse row times the block reads whole contiguous rows.
 // Column dot products go through per-block partial sums (4 rows per block)
-// added in a fixed order, so every result is independent of scheduling.  The
-// conjugate-gradient iterations run as CUDA graphs of 8 iterations, with the
-// host checking for remaining columns between graphs.
+// added in a fixed order, so every result is independent of scheduling.
+//
+// A solve runs on one of two routes, chosen in sparse_columns: a whole solve
+// as one launch of clusters, one or two columns each (k_pcg_cluster), or
+// iterations of seven kernels over all columns of the block, replayed as CUDA
+// graphs of 8 iterations with the host checking for remaining columns between
+// graphs.
 #include "dft_internal.cuh"
 
 #include <cooperative_groups.h>
@@ -841,9 +845,20 @@ void sparse_columns(Ctx& c, const double* F, const int* cols, int ncols, double 
     };
     // The cluster kernel takes a solve whose p (and the CTA's vectors) fit shared
     // memory, with atoms' functions contiguous where they are preconditioned
-    // together; K <= PC_MAX_K: beyond, every cluster would read S from HBM for its
-    // few columns.  Otherwise iterations of seven kernels run as graphs.
-    constexpr int PC_MAX_K = 4096, PC_SMEM = 225 * 1024;
+    // together.  Every cluster reads S for its one or two columns, and 64 columns
+    // run at a time with two CTAs per SM (K below about 2,900), 48 with one,
+    // while the graphs' sparse product reads S once per 128 columns, so beyond a
+    // few waves of clusters the graphs are faster.  Milliseconds per solve, clusters /
+    // graphs, 1e-8 threshold: K = 640 at 32, 160 columns 3.9 / 20, 12 / 25; K =
+    // 1230 at 128, 307 columns 29 / 47, 54 / 66; K = 1910 at 160, 240, 477 67 /
+    // 86, 94 / 91, 183 / 151; K = 2300 at 64, 128, 256 38 / 73, 74 / 75, 139 /
+    // 114; K = 2850 at 96, 128, 512 81 / 89, 100 / 90, 363 / 235; K = 3000 at
+    // 48, 64, 128, 512 60 / 86, 86 / 87, 145 / 90, 535 / 252; K = 4000 at 48,
+    // 64, 128 83 / 114, 122 / 117, 201 / 121.  The line is 8e8 columns x K^2
+    // with two CTAs per SM and 48 columns with one (or half of the 8e8, where
+    // cached entries of S take the room).
+    constexpr int PC_MAX_K = 4096, PC_SMEM = 225 * 1024, PC_WAVE = 48;
+    constexpr double PC_WORK = 4e8;   // columns x K^2 per CTA on an SM
     PcRows pr{};
     int max_rows = 0, max_nnz = 0;
     bool cluster = K <= PC_MAX_K;
@@ -880,10 +895,11 @@ void sparse_columns(Ctx& c, const double* F, const int* cols, int ncols, double 
     };
     // S^-1 of the block in q (the right-hand sides) into Xs
     auto solve = [&](int Bb) {
-        if (cluster) {
+        constexpr std::integral_constant<int, 1> one{};
+        constexpr std::integral_constant<int, 2> two{};
+        const int ctas = cluster && pc_smem<2>(K, max_rows, cached_for(two)) <= PC_SMEM / 2 ? 2 : 1;
+        if (cluster && (Bb <= PC_WAVE || (double)Bb * K * K <= PC_WORK * ctas)) {
             // one column per cluster while that fits the SMs at once, then two
-            constexpr std::integral_constant<int, 1> one{};
-            constexpr std::integral_constant<int, 2> two{};
             const int per_sm = pc_smem<1>(K, max_rows, cached_for(one)) <= PC_SMEM / 2 ? 2 : 1;
             if (PC_CL * Bb <= 152 * per_sm) solve_cluster(Bb, one);
             else solve_cluster(Bb, two);

@@ -183,3 +183,65 @@ def test_no_entry_of_s_kept():
     assert info.nnz_s == 0 and info.pcg_solves == 3 and info.not_converged == 1
     assert float(out.abs().max()) == 0.0
     ctx.close()
+
+
+def launches_per_step(ctx, *args, **kw):
+    """Kernels per step of the vector recurrence (graph replays not counted):
+    2 and a solve's 2 as clusters, 6 as graphs of iterations."""
+    n = []
+    for n_c in (4, 6):
+        before = dft.dft_kernel_launches()
+        out, info = ctx.density_matrix_columns(*args, n_c, **kw)
+        n.append(dft.dft_kernel_launches() - before)
+    return (n[1] - n[0]) / 2, out, info
+
+
+def test_large_basis_by_clusters_and_by_graphs():
+    """K = 3500, where a CTA does not hold its rows of S: 40 columns go to the
+    cluster kernel two at a time, 60 to the graphs; both against the dense
+    recurrence on the thresholded matrices."""
+    ctx = dft.Context(large(), kT=4.0)
+    S, T = ctx.overlap_kinetic()
+    thr, lo, hi, mu, n_c = 1e-8, -1.0, 40.0, 8.0, 6
+    St, Ft = S * (S.abs() > thr), T * (T.abs() > thr)
+    L = torch.linalg.cholesky(St)
+    cols = list(range(0, 3500, 60))[:60]
+    a = dm.cheb_coeffs(mu, 0.25, lo, hi, n_c, m_nodes=4 * n_c)
+    eb, de = 0.5 * (hi + lo), 0.5 * (hi - lo)
+    h = lambda u: (torch.cholesky_solve(Ft @ u, L) - eb * u) / de   # noqa: E731
+    u0 = torch.cholesky_solve(torch.eye(3500, device="cuda", dtype=torch.float64)[:, cols], L)
+    u1 = h(u0)
+    ref = a[0] * u0 + a[1] * u1
+    for l in range(2, n_c):
+        u0, u1 = u1, 2 * h(u1) - u0
+        ref += a[l] * u1
+    for n, kernels in ((40, 4), (60, 8)):
+        per, out, info = launches_per_step(ctx, T, cols[:n], mu, lo, hi, thresh=thr, pcg_tol=1e-12)
+        err = float((out - ref[:, :n]).abs().max() / ref.abs().max())
+        print(f"K 3500, {n} columns: {per} kernels per step, max|d| {err:.1e}, {info.pcg_iterations} iterations")
+        assert per == kernels
+        assert info.not_converged == 0 and err < 1e-9
+    ctx.close()
+
+
+def test_functions_of_an_atom_that_are_not_contiguous():
+    """Shells listed kind by kind instead of atom by atom: the preconditioner's
+    blocks are scattered, which the graphs handle; the columns are the same."""
+    s = w.config_system("tiny8")
+    order = np.argsort(np.arange(len(s.shell_atom)) % 6, kind="stable")
+    p = problem("tiny8", 48)
+    first = np.concatenate([[0], np.cumsum(2 * s.shell_l + 1)])
+    fn = np.concatenate([np.arange(first[q], first[q + 1]) for q in order])   # function i of the new order
+    s.shell_atom, s.shell_l, s.shell_exp = s.shell_atom[order], s.shell_l[order], s.shell_exp[order]
+    ctx = dft.Context(s)
+    ctx.overlap_kinetic()
+    F = p["F_g"][torch.from_numpy(fn).cuda()][:, torch.from_numpy(fn).cuda()].contiguous()
+    cols = [0, 9, 41, 79]
+    args = p["mu"], p["e_min"], p["e_max"]
+    per, out, info = launches_per_step(ctx, F, cols, *args, pcg_tol=1e-12)
+    assert per == 8 and info.not_converged == 0
+    out, _ = ctx.density_matrix_columns(F, cols, *args, p["n_c"], pcg_tol=1e-12)
+    dense = dm.dm_cheb_recurrence(p["F_o"], p["S_o"], p["a"], p["e_min"], p["e_max"], form="paper")
+    assert np.max(np.abs(out.cpu().numpy() - dense[np.ix_(fn, fn[cols])])) < 1e-9 * np.max(np.abs(dense))
+    p["ctx"].close()
+    ctx.close()
