@@ -243,7 +243,8 @@ void build_basis(Ctx& c, const dft_basis_desc* b, const dft_grid_desc* g, const 
     }
     c.part_cap = std::max<long long>({2LL * c.tile_cap, 3LL * 1184, 2048, 592LL * 16}) + 64;
     c.pl_hist = c.p.mixer == DFT_MIX_PULAY ? (c.p.mix_history > 0 ? c.p.mix_history : 8) : 0;
-    c.gram_cap = 1 << 20;
+    // partial Gram sums, and the warm start's adjoint sums (16 per atom and slab)
+    c.gram_cap = std::max(1LL << 20, 16LL * c.n_atoms);
 }
 
 // Expansion buffers beyond the scratch matrices X0, X1 and B that the FP64

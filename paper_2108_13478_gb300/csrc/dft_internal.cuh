@@ -166,7 +166,7 @@ struct Ctx {
     PstItem* d_pst_items = nullptr;
     int2* d_pst_pairs = nullptr;
     bool recurrence = false;     // this density matrix runs the plain three-term recurrence
-    double* d_gram = nullptr;    // partial Gram sums [gram_cap]
+    double* d_gram = nullptr;    // partial Gram sums, adjoint sums of the warm start [gram_cap]
     long long gram_cap = 0;
     double* d_B = nullptr;       // K x K scratch
     double* d_P = nullptr;       // K x K density matrix of the last SCF step

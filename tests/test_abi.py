@@ -346,3 +346,28 @@ def test_columns_binding_refuses_buffers_the_kernels_cannot_use(built, monkeypat
     assert called == []
     B.dft_density_matrix_columns(None, good_F, [0, 3], *args, good_out)
     assert len(called) == 1
+
+
+def test_workspace_holds_the_warm_start_sums_of_any_number_of_atoms(built):
+    """A training step keeps 16 FP64 sums per atom and slab in the buffer of the
+    partial Gram sums (2^20 doubles): beyond 65,536 atoms it has to grow with
+    them, next to the positions (24 bytes), descriptors, coefficients and their
+    gradients, and pre-activations of each atom."""
+    import paper_2108_13478_gb300 as dft
+
+    def size(n):
+        xyz, one = np.zeros((n, 3)), np.zeros(1, np.int32)
+        b = dft.dft_basis_desc()
+        b.n_atoms, b.n_shells = n, 1
+        b.xyz = xyz.ctypes.data_as(ctypes.POINTER(ctypes.c_double))
+        b.shell_atom = b.shell_l = one.ctypes.data_as(ctypes.POINTER(ctypes.c_int))
+        exp = np.ones(1)
+        b.shell_exp = exp.ctypes.data_as(ctypes.POINTER(ctypes.c_double))
+        g = dft.dft_grid_desc()
+        g.h = 1.0
+        for d in range(3):
+            g.n[d] = 8
+        return dft.dft_workspace_bytes(b, g, dft.make_params(kT=0.01, n_electrons=2.0))
+    assert size(70000) > 0
+    per_atom = 3 * 8 + 32 * 8 + 16 * 8 + 3 * 128 * 4 + 16 * 8
+    assert size(140000) - size(70000) >= 70000 * (per_atom + 16 * 8) - 4096
