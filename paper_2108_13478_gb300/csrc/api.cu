@@ -243,8 +243,12 @@ void build_basis(Ctx& c, const dft_basis_desc* b, const dft_grid_desc* g, const 
     }
     c.part_cap = std::max<long long>({2LL * c.tile_cap, 3LL * 1184, 2048, 592LL * 16}) + 64;
     c.pl_hist = c.p.mixer == DFT_MIX_PULAY ? (c.p.mix_history > 0 ? c.p.mix_history : 8) : 0;
-    // partial Gram sums, and the warm start's adjoint sums (16 per atom and slab)
-    c.gram_cap = std::max(1LL << 20, 16LL * c.n_atoms);
+    // partial Gram sums (mixed path: of 320 pairs of a giant and a baby, more
+    // than a launch has at K > 20,000, where 2^20 doubles would be too few for
+    // two columns of CTAs per block), and the warm start's adjoint sums (16 per
+    // atom and slab)
+    const long long nb = c.Kp / 256;
+    c.gram_cap = std::max({1LL << 20, 16LL * c.n_atoms, 320 * nb * (nb + 1)});
 }
 
 // Expansion buffers beyond the scratch matrices X0, X1 and B that the FP64

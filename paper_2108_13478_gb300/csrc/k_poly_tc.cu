@@ -622,8 +622,8 @@ __global__ void __launch_bounds__(256) k_pst_combine(int K, int nb, int s, PstLi
 // off-diagonal blocks count twice.  HBM-bound where few giants are at hand
 // (each baby is read once per 8 giants; the CTAs of one column, adjacent in
 // launch order, share the giants' elements in L2), so nothing is staged: every thread keeps its 64 FP32
-// FMA chains (at most GRAM_GROUPS x 4 products long) and the chains meet in
-// FP64.
+// FMA chains (GRAM_GROUPS x 4 products long, the buffer of the partial sums is
+// sized for that) and the chains meet in FP64.
 constexpr int GRAM_GROUPS = 32;   // 4-element groups per thread
 template <bool BF>
 __global__ void __launch_bounds__(256) k_pst_gram(int K, int nb, PstList G, int nq, PstList T, int s,
@@ -923,7 +923,7 @@ void gram(Ctx& c, int q0, const std::vector<int>& slots, cudaStream_t st) {
         PstList G;
         for (int q = 0; q < PS_MAX_S; ++q) G.p[q] = c.pst_slot[slots[k + std::min(q, nq - 1)]];
         if ((long long)nq * s > c.gram_cap) throw Error(DFT_EINTERNAL, "Gram partials exceed their buffer");
-        // chains of GRAM_GROUPS groups while the partial sums fit their buffer
+        // chains of GRAM_GROUPS groups (longer only if the partial sums did not fit their buffer)
         const int nsplit = (int)std::max<long long>(
             1, std::min<long long>({(long long)nb * (nb + 1) / 2 * (16384 / (256 * GRAM_GROUPS)),
                                     c.gram_cap / ((long long)nq * s), 65535LL}));
