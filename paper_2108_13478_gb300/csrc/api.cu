@@ -345,16 +345,18 @@ size_t carve(Ctx& c, char* base) {
     for (auto& o : o_ps) o = L.off(K2);
     // expansion slots of the mixed path: scratch that is free while the
     // expansion runs (T_1 = slot 0 is split from d_H, so the pairs come first),
-    // then buffers of their own, at most an eighth of the workspace, or as much
-    // again while the total stays below 1.6 GB; 2 sqrt(2 N_C) products use up
-    // to about 110
+    // then buffers of their own, at most an eighth of the workspace (none beyond
+    // a total of 240 GB, so that what fits the GPU without them still does), or
+    // as much again while the total stays below 1.6 GB; 2 sqrt(2 N_C) products
+    // use up to about 110
     std::vector<size_t> o_pst;
     size_t o_pmaps = 0, o_pslots = 0, o_psys = 0, o_pitems = 0, o_ppairs = 0;
     if (c.Kp > 0) {
-        const size_t sb = pst_slot_bytes(c.Kp), small = 1600000000;
+        const size_t sb = pst_slot_bytes(c.Kp), small = 1600000000, most = 240000000000;
         for (const auto& r : {free_tc, free_mat, free_fft})
             for (size_t o = r.first; o + sb <= r.second; o += sb) o_pst.push_back(o);
-        const size_t extra = std::max(L.total / 8, L.total < small ? std::min(L.total, small - L.total) : 0);
+        const size_t extra = std::max(std::min(L.total / 8, L.total < most ? most - L.total : 0),
+                                      L.total < small ? std::min(L.total, small - L.total) : 0);
         for (size_t used = sb; used <= extra && o_pst.size() < 112; used += sb) o_pst.push_back(L.off(sb));
         if (o_pst.size() > 160) o_pst.resize(160);
         o_pmaps = L.off(sizeof(CUtensorMap) * 4 * o_pst.size());

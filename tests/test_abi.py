@@ -371,3 +371,28 @@ def test_workspace_holds_the_warm_start_sums_of_any_number_of_atoms(built):
     assert size(70000) > 0
     per_atom = 3 * 8 + 32 * 8 + 16 * 8 + 3 * 128 * 4 + 16 * 8
     assert size(140000) - size(70000) >= 70000 * (per_atom + 16 * 8) - 4096
+
+
+@pytest.mark.parametrize("mixed", [False, True])
+def test_workspace_of_a_large_basis_fits_the_gpu(built, mixed):
+    """The expansion's buffers are extra: K = 48,000 (4,800 atoms) needs 268 GB
+    without them on the mixed path, and they must not take it beyond the 298
+    GB of the GPU, nor leave no room for F and P (18 GB each)."""
+    import paper_2108_13478_gb300 as dft
+    import workloads as w
+    n = 4800
+    i = np.arange(n)
+    xyz = np.stack([i % 50, i // 50 % 50, i // 2500], axis=1) * 2.0 + 8.0
+    s = w.make_system(xyz, h=1.0, grid_n=np.array([120] * 3), grid_origin=np.zeros(3))
+    b = dft.dft_basis_desc()
+    b.n_atoms, b.n_shells = n, len(s.shell_atom)
+    for name, t in (("xyz", ctypes.c_double), ("shell_exp", ctypes.c_double), ("shell_atom", ctypes.c_int),
+                    ("shell_l", ctypes.c_int)):
+        setattr(b, name, getattr(s, name).ctypes.data_as(ctypes.POINTER(t)))
+    g = dft.dft_grid_desc()
+    g.h = 1.0
+    for d in range(3):
+        g.n[d] = 120
+    nb = dft.dft_workspace_bytes(b, g, dft.make_params(kT=0.01, n_electrons=4.0 * n,
+                                                       precision=dft.DFT_PREC_FP16X3 if mixed else dft.DFT_PREC_FP64))
+    assert 200e9 < nb < 270e9
