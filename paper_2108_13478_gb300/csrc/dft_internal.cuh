@@ -79,6 +79,7 @@ struct TcCfg {
 struct PsPlan {
     int n_c = 0, s = 1, Q = 0;
     bool direct = false;
+    float down = 1.0f;   // C_q, q >= 1, of a Clenshaw plan in split pairs, as a power of two (k_poly_tc.cu)
 };
 
 // one system of a tensor-core product launch (k_poly_tc.cu) and one product:
@@ -353,7 +354,7 @@ void launch_moment_reduce(int nparts, const double* part, double* mom, int idx_e
 PsPlan ps_plan(int n_c, int nslot, double seq, double par, int nroll);
 // m_l, l < n_c, from the traces and Gram sums D ((Q + 1) x s)
 void launch_ps_moments(int K, const PsPlan& p, const double* D, double* mom, cudaStream_t s);
-// c_qr of the C_q from a_l; work holds (Q + 1) s doubles
+// c_qr of the C_q from a_l, times p.down for q >= 1; work holds (Q + 1) s doubles
 void launch_ps_coefs(const PsPlan& p, const double* a, double* c, double* work, cudaStream_t s);
 // FP64 path: babies and giants of H_N and the moments into d_mom; then
 // rho = sum_l a_l T_l into d_rho from the coefficients in d_coef

@@ -298,16 +298,17 @@ __global__ void __launch_bounds__(256) k_ps_moments(int K, int n_c, int s, int Q
     }
 }
 
-// c_qr from a_l (the header's top-down elimination); work holds (Q + 1) s doubles
-__global__ void __launch_bounds__(256) k_ps_coefs(int n_c, int s, int Q, const double* __restrict__ a, double* c,
-                                                  double* work) {
+// c_qr from a_l (the header's top-down elimination), times down for q >= 1;
+// work holds (Q + 1) s doubles
+__global__ void __launch_bounds__(256) k_ps_coefs(int n_c, int s, int Q, double down, const double* __restrict__ a,
+                                                  double* c, double* work) {
     const int n = (Q + 1) * s;
     for (int l = threadIdx.x; l < n; l += 256) work[l] = l < n_c ? a[l] : 0.0;
     for (int q = Q; q >= 0; --q) {
         __syncthreads();
         for (int r = threadIdx.x; r < s; r += 256) {
             const double x = work[q * s + r];
-            c[q * s + r] = (r == 0 || q == 0) ? x : 2.0 * x;
+            c[q * s + r] = q == 0 ? x : down * (r == 0 ? x : 2.0 * x);
             if (r > 0 && q > 0) work[q * s - r] -= x;
         }
     }
@@ -360,7 +361,7 @@ void launch_ps_moments(int K, const PsPlan& p, const double* D, double* mom, cud
 }
 
 void launch_ps_coefs(const PsPlan& p, const double* a, double* c, double* work, cudaStream_t s) {
-    k_ps_coefs<<<1, 256, 0, s>>>(p.n_c, p.s, p.Q, a, c, work);
+    k_ps_coefs<<<1, 256, 0, s>>>(p.n_c, p.s, p.Q, (double)p.down, a, c, work);
     check_launch("ps_coefs");
 }
 

@@ -73,8 +73,18 @@ constexpr int SMS = 152;
 // pairs hold x * SC: the low half of an FP16 pair of x itself would be a
 // subnormal number for the elements of order K^-1/2 that most of a T_l
 // consists of (2^-25 absolute); scaled, the pair keeps 22 bits down to
-// 2^-27.  |T_l| <= 4 and the b_q stay far below 65504 / SC.
+// 2^-27.  |T_l| <= 4; the b_q of Clenshaw's recurrence grow to Q / 6 for a step
+// at a multiple of pi / s (64-bit evaluation, s = 14 to 128, N_C to 65536; 1 at
+// the benchmark's Q = 41, 100 at N_C = 65536 with s = 24 and a converged tail),
+// so that beyond Q = B_Q all C_q but C_0 carry a power of two that keeps Q / 4
+// below 48 of the 64 that a pair holds.
 constexpr float SC = 1024.0f, ISC = 1.0f / SC;
+constexpr int B_Q = 192;
+float clenshaw_down(int Q) {
+    float d = 1.0f;
+    for (int q = Q; q > B_Q; q = (q + 1) / 2) d *= 0.5f;
+    return d;
+}
 
 // folded place of block (a, b), a <= b
 __device__ __forceinline__ void fold(int a, int b, int nb, int& row, int& col) {
@@ -748,10 +758,11 @@ __global__ void __launch_bounds__(128) k_pst_trace(int K, int nb, PstList L, dou
 }
 
 // rho (K x K, FP64, both triangles) = [C_0 or rho] + sum of np FP32 partial
-// products - b2: C_0 = sum_r c_0r T_r in FP32 FMA chains of 8 terms added in FP64
+// products - b2, these two times up: C_0 = sum_r c_0r T_r in FP32 FMA chains of
+// 8 terms added in FP64
 template <bool BF>
 __global__ void __launch_bounds__(256) k_pst_finish(int K, int nb, int s, PstList T, const double* __restrict__ c,
-                                                    PstOut part, int np, const uint16_t* b2, int first,
+                                                    PstOut part, int np, const uint16_t* b2, double up, int first,
                                                     double* __restrict__ rho) {
     using H = typename H16<BF>::T;
     __shared__ double sh[32][33];
@@ -790,9 +801,9 @@ __global__ void __launch_bounds__(256) k_pst_finish(int K, int nb, int s, PstLis
             }
             for (int p = 0; p < np; ++p) {
                 const uint16_t* q = (const uint16_t*)part.p[p] + e;
-                x += (double)__uint_as_float(((uint32_t)q[0] << 16) | q[plane]);
+                x = fma(up, (double)__uint_as_float(((uint32_t)q[0] << 16) | q[plane]), x);
             }
-            if (b2) x -= (double)pr(b2 + e, plane);
+            if (b2) x = fma(-up, (double)pr(b2 + e, plane), x);
             if (gc >= gr) rho[(long long)gc * K + gr] = x;
         }
         sh[lc][lr] = x;
@@ -962,8 +973,8 @@ void finish(Ctx& c, const double* cf, const std::vector<int>& part, int b2, bool
     const uint16_t* b = b2 >= 0 ? (const uint16_t*)c.pst_slot[b2] : nullptr;
     const int np = (int)part.size();
     pick(c.p.precision == DFT_PREC_BF16X3,
-         [&] { k_pst_finish<true><<<nt * (nt + 1) / 2, 256, 0, st>>>(c.K, c.Kp / 256, v.p.s, T, cf, o, np, b, first, c.d_rho); },
-         [&] { k_pst_finish<false><<<nt * (nt + 1) / 2, 256, 0, st>>>(c.K, c.Kp / 256, v.p.s, T, cf, o, np, b, first, c.d_rho); });
+         [&] { k_pst_finish<true><<<nt * (nt + 1) / 2, 256, 0, st>>>(c.K, c.Kp / 256, v.p.s, T, cf, o, np, b, 1.0 / v.p.down, first, c.d_rho); },
+         [&] { k_pst_finish<false><<<nt * (nt + 1) / 2, 256, 0, st>>>(c.K, c.Kp / 256, v.p.s, T, cf, o, np, b, 1.0 / v.p.down, first, c.d_rho); });
     check_launch("pst_finish");
 }
 
@@ -1030,6 +1041,7 @@ void pst_pass1(Ctx* const* cs, int n, const int* moments, cudaStream_t st) {
         // T_1 takes a slot here
         const double waves = sys_tiles(c) / (double)SMS;
         c.ps = ps_plan(c.n_c_cur, nslot - 1, std::ceil(waves), waves, 6);
+        c.ps.down = c.ps.direct ? 1.0f : clenshaw_down(c.ps.Q);
         tab[k] = PstSys{c.K, c.Kp / 256, c.d_pst_maps, c.d_pst_slots, c.d_flags};
     }
     DFT_CUDA_CHECK(cudaMemcpyAsync(lead.d_pst_sys, tab.data(), sizeof(PstSys) * n, cudaMemcpyHostToDevice, st));

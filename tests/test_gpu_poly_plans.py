@@ -160,3 +160,29 @@ def test_fock_matrix_beyond_the_pair_is_an_internal_error():
         ctx.density_matrix(F)
     assert e.value.status == dft._binding.DFT_EINTERNAL
     ctx.close()
+
+
+def test_clenshaw_sums_of_a_high_order_stay_in_the_pair():
+    """b_q of Clenshaw's recurrence in T_s grows with the number of giants
+    where the Fermi angle is near a multiple of pi / s: at N_C = 65536 with s
+    = 24 it reaches 100, with eigenvectors that are nearly single functions
+    also in its elements."""
+    s = few_slots()
+    n_c = 65536
+    beta = n_c / 3.0
+    ctx = dft.Context(s, precision=FP16, e_min=-1.0, e_max=1.0, cheb_order=n_c, kT=1.0 / beta, n_electrons=3500.0,
+                      skip_correction=1)
+    K = ctx.K
+    near = np.pi / n_c * np.array([0.5, 1.0, 2.0, 3.0, 4.0, 6.0])
+    x = np.concatenate([np.linspace(0.05, 0.9, K // 2 - len(near)), near])
+    x = np.concatenate([x, -x])   # symmetric: mu = 0
+    F, LW = given_spectrum(ctx, torch.from_numpy(x).cuda(), orthogonal(K, localised=True))
+    P, info = ctx.density_matrix(F)
+    ctx.close()
+    p = dm.cheb_eval(x, coefficients(0.0, beta, n_c))
+    ref = (LW * torch.from_numpy(p).cuda()) @ LW.T
+    err = float((P - ref).abs().max() / ref.abs().max())
+    # a relative error 2^-22 of H_N's pair shifts an eigenvalue, and f changes by up to beta / 4 per unit
+    bound = 8 * beta / 4 * 2.0 ** -22
+    print(f"K {K} N_C {n_c}: mu {info.mu:.2e}, N_e {info.n_e_trace:.4f}, max|dP| / max|P| {err:.2e} (bound {bound:.1e})")
+    assert err < bound
