@@ -39,10 +39,11 @@
  *    cooperative launch per recurrence pass, tiles of consecutive steps
  *    ordered by per-block counters (256-wide tiles, no stream-K).  Malformed
  *    values are ignored.
- *  - DFT_TEST_EXPIRE_WAITS: test hook of the bounded waits; any value makes
- *    every block-counter wait of the dataflow launch ask for one write more
- *    than any tile makes, so each runs out after its limit (1 s) and the call
- *    returns DFT_ETIMEOUT with the context still usable.  Never set in use.
+ *  - DFT_TEST_EXPIRE_WAITS: test hook of the bounded waits; any value makes a
+ *    warp of the grouped products keep back a release (and every block-counter
+ *    wait of the dataflow launch ask for one write more than any tile makes),
+ *    so the waits run out after their limit (1 s) and the call returns
+ *    DFT_ETIMEOUT with the context still usable.  Never set in use.
  */
 #ifndef DFT_H
 #define DFT_H

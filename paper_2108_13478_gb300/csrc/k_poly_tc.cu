@@ -29,8 +29,11 @@
 // 32-bit access and a warp whole sectors (with one row per lane and 16-byte
 // accesses along the row the epilogue took 60 of 100 us per tile at K =
 // 2000).  The ring stays with the producer, and the next tile's loads and
-// first two units run under the epilogue.  Every wait is bounded; on expiry the CTA sets FLAG_TIMEOUT,
-// drains what it issued and returns.
+// first two units run under the epilogue.  Every wait is bounded; on expiry the
+// CTA sets FLAG_TIMEOUT of the system and of the launch's leader, drains what it
+// issued and returns, and the call's later launches find the leader's flag and
+// return at once.  hold (a test, DFT_TEST_EXPIRE_WAITS) makes one epilogue warp
+// withhold the release of its first accumulator, so that the waits run out.
 //
 // Density matrix at K = 1230, tail 1e-5 (N_C ~ 1410, direct plan): 118.9 ms
 // with the recurrence of k_cheb_tc.cu, 6.1 ms with this (error of P against
@@ -41,6 +44,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
 
 namespace dft {
 namespace {
@@ -76,10 +80,10 @@ constexpr int SMS = 152;
 // 2^-27.  |T_l| <= 4; the b_q of Clenshaw's recurrence grow to Q / 6 for a step
 // at a multiple of pi / s (64-bit evaluation, s = 14 to 128, N_C to 65536; 1 at
 // the benchmark's Q = 41, 100 at N_C = 65536 with s = 24 and a converged tail),
-// so that beyond Q = B_Q all C_q but C_0 carry a power of two that keeps Q / 4
-// below 48 of the 64 that a pair holds.
+// so that beyond Q = B_Q all C_q but C_0 carry a power of two that keeps Q / 6
+// below 60 of the 64 that a pair holds.
 constexpr float SC = 1024.0f, ISC = 1.0f / SC;
-constexpr int B_Q = 192;
+constexpr int B_Q = 360;
 float clenshaw_down(int Q) {
     float d = 1.0f;
     for (int q = Q; q > B_Q; q = (q + 1) / 2) d *= 0.5f;
@@ -123,6 +127,17 @@ __device__ __forceinline__ uint64_t smem_desc_mn(const void* p) {
     return addr | ((uint64_t)(BK * 128 >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
 }
 
+// mbar_wait that also gives up when the CTA is leaving (the producer's; in the
+// MMA issuer's and the epilogue's waits the extra read cost 0.3% of a density matrix)
+__device__ __forceinline__ bool wait_or_leave(uint64_t* bar, uint32_t parity, const volatile int* leave) {
+    if (mbar_try_wait(bar, parity)) return true;
+    const unsigned long long t0 = globaltimer();
+    while (!mbar_try_wait(bar, parity)) {
+        if (*leave || globaltimer() - t0 > WAIT_NS) return false;
+    }
+    return true;
+}
+
 // one product of a launch as the roles walk it
 struct Work {
     PstItem it;
@@ -148,7 +163,8 @@ __device__ __forceinline__ Work work_at(int t, const PstItem* items, int nitems,
 template <bool BF>
 __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restrict__ sys,
                                                           const PstItem* __restrict__ items_g, int nitems,
-                                                          const int2* __restrict__ pairs, int ntiles) {
+                                                          const int2* __restrict__ pairs, int ntiles,
+                                                          int* lead_flags, int hold) {
     using T = typename H16<BF>::T;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -216,7 +232,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
                         int ar, ac, br, bc;
                         fold(min(w.p, kq), max(w.p, kq), nb, ar, ac);
                         fold(min(w.j, kq), max(w.j, kq), nb, br, bc);
-                        if (!mbar_wait(&empty[s], (uint32_t)((g / STAGES) & 1) ^ 1u)) {
+                        if (!wait_or_leave(&empty[s], (uint32_t)((g / STAGES) & 1) ^ 1u, abort_flag)) {
                             *abort_flag = 1;
                             break;
                         }
@@ -242,11 +258,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
                     }
                 }
             }
-            if (*abort_flag) {
-                // the last load issued into each stage must land before exit
-                for (long long q = (g > STAGES ? g - STAGES : 0); q < g; ++q)
-                    mbar_wait(&full[q % STAGES], (uint32_t)((q / STAGES) & 1));
-            }
+            // the last load issued into each stage must land before exit (whoever leaves
+            // the launch early, and at what point: this thread has nothing else to do)
+            for (long long q = (g > STAGES ? g - STAGES : 0); q < g; ++q)
+                mbar_wait(&full[q % STAGES], (uint32_t)((q / STAGES) & 1));
+            // wake the MMA issuer if it waits for the load that does not come (it issues one
+            // block on stale operands, whose sums nobody reads)
+            if (*abort_flag) mbar_arrive(&full[g % STAGES]);
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -299,13 +317,19 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
                     umma_commit(&accfull[a]);
                 }
             }
-            if (*abort_flag) {
-                // every MMA this thread issued must finish before tensor memory is freed
-                umma_commit(drain);
-                mbar_wait(drain, 0);
+            // every MMA this thread issued must finish before tensor memory is freed
+            umma_commit(drain);
+            mbar_wait(drain, 0);
+            if (*abort_flag) {   // wake the epilogue, which sees the abort
+                mbar_arrive(&accfull[0]);
+                mbar_arrive(&accfull[1]);
             }
         }
         __syncwarp();
+    } else if (warp == 2) {
+        // an earlier launch of this call gave up: so does this one (read by an idle
+        // warp: in front of the first loads it cost 0.6 us per launch)
+        if (lane == 0 && *(volatile int*)&lead_flags[FLAG_TIMEOUT]) *abort_flag = 1;
     }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 232;");
@@ -360,11 +384,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
                 tmem_add_groups<CPT / 16>(tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(a * BN + half * CPT), R);
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0 && q + 1 < nunit) mbar_arrive(&accempty[a]);
+                if (lane == 0 && q + 1 < nunit && !(hold && warp == 4 && u == 0)) mbar_arrive(&accempty[a]);
             }
             if (!ok) {
                 *abort_flag = 1;
-                if (lane == 0) atomicExch(&S.flags[FLAG_TIMEOUT], 1);
+                if (lane == 0) {
+                    atomicExch(&S.flags[FLAG_TIMEOUT], 1);
+                    atomicExch(&lead_flags[FLAG_TIMEOUT], 1);
+                }
                 break;
             }
             // the sums go back to the last unit's accumulator, which stays with the
@@ -845,8 +872,10 @@ struct Queue {
     struct Launch { int first, n, tiles; };
     std::vector<Launch> launches;
     int open = 0;
+    int hold;
 
-    Queue(Ctx& l, cudaStream_t s) : lead(l), st(s), bf(l.p.precision == DFT_PREC_BF16X3) {}
+    Queue(Ctx& l, cudaStream_t s)
+        : lead(l), st(s), bf(l.p.precision == DFT_PREC_BF16X3), hold(std::getenv("DFT_TEST_EXPIRE_WAITS") ? 1 : 0) {}
     void add(int sys, const Ctx& c, std::initializer_list<int2> ab, int prev, int add_, int out, int mode, double limit) {
         PstItem it{};
         it.sys = sys;
@@ -884,8 +913,12 @@ struct Queue {
     void launch(size_t k) {
         const Launch& l = launches[k];
         const int grid = std::min(l.tiles, SMS);
-        if (bf) k_pst_prod<true><<<grid, NTHREADS, SMEM_BYTES, st>>>(lead.d_pst_sys, lead.d_pst_items + l.first, l.n, lead.d_pst_pairs, l.tiles);
-        else k_pst_prod<false><<<grid, NTHREADS, SMEM_BYTES, st>>>(lead.d_pst_sys, lead.d_pst_items + l.first, l.n, lead.d_pst_pairs, l.tiles);
+        auto go = [&](auto kern) {
+            kern<<<grid, NTHREADS, SMEM_BYTES, st>>>(lead.d_pst_sys, lead.d_pst_items + l.first, l.n, lead.d_pst_pairs, l.tiles,
+                                                     lead.d_flags, hold);
+        };
+        if (bf) go(k_pst_prod<true>);
+        else go(k_pst_prod<false>);
         check_launch("pst_prod");
     }
     void run() {

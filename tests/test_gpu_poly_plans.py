@@ -186,3 +186,32 @@ def test_clenshaw_sums_of_a_high_order_stay_in_the_pair():
     bound = 8 * beta / 4 * 2.0 ** -22
     print(f"K {K} N_C {n_c}: mu {info.mu:.2e}, N_e {info.n_e_trace:.4f}, max|dP| / max|P| {err:.2e} (bound {bound:.1e})")
     assert err < bound
+
+
+def test_expired_waits_of_the_products_return_timeout_and_leave_the_context_usable(monkeypatch):
+    """With DFT_TEST_EXPIRE_WAITS one epilogue warp of every CTA keeps back the
+    release of its first accumulator: the waits of all roles run out (1 s), the
+    CTAs drain their copies and MMAs, free tensor memory and return, the later
+    launches of the call return at once, and the call reports DFT_ETIMEOUT.
+    The same context then gives the density matrix."""
+    import time
+    s = w.config_system("tiny37")
+    n_c = 300
+    beta = n_c / 4.0
+    ctx = dft.Context(s, precision=FP16, e_min=-1.0, e_max=1.0, cheb_order=n_c, kT=1.0 / beta)
+    x = np.linspace(-0.9, 0.9, ctx.K)
+    F, LW = given_spectrum(ctx, torch.from_numpy(x).cuda(), orthogonal(ctx.K))
+    monkeypatch.setenv("DFT_TEST_EXPIRE_WAITS", "1")
+    t0 = time.time()
+    with pytest.raises(dft.DftError) as e:
+        ctx.density_matrix(F)
+    took = time.time() - t0
+    print(f"expired waits: {e.value} after {took:.1f} s")
+    assert e.value.status == dft._binding.DFT_ETIMEOUT
+    assert took < 20.0
+    monkeypatch.delenv("DFT_TEST_EXPIRE_WAITS")
+    P, info = ctx.density_matrix(F)
+    ctx.close()
+    ref = (LW * torch.from_numpy(dm.cheb_eval(x, coefficients(info.mu - info.mu_correction, beta, n_c))).cuda()) @ LW.T
+    assert info.spectrum_ok == 1
+    assert float((P - ref).abs().max() / ref.abs().max()) < 1e-4
