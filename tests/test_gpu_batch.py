@@ -1,9 +1,8 @@
-"""Batched SCF steps of ragged systems (one persistent tensor-core launch per
-recurrence step for all systems) against the FP64 oracle's converged
-energies, and against the same steps run one system at a time.  Each tile's
-arithmetic is the same in both; the quadrature's FP64 atomics leave
-differences at the 1e-16 level, which two SCF cycles carry to about 1e-11 in
-the density."""
+"""Batched SCF steps of ragged systems (the expansions' products of all systems
+in launches level by level) against the FP64 oracle's converged energies, and
+against the same steps run one system at a time.  Each tile's arithmetic is
+the same in both; how many partial sums a weighted product is cut into
+depends on the whole batch, which is within the bounds below."""
 import json
 import os
 
@@ -32,8 +31,9 @@ def make(name):
 
 @pytest.mark.parametrize("shape", [None, "32,0,256,0,0,0,1"])
 def test_batched_equals_one_by_one(shape, monkeypatch):
-    """Tuned launch shape, and the dataflow shape (each pass one launch over
-    all systems' tiles, block counters per system, fixed-point moments)."""
+    """The grouped expansion, and the three-term recurrence's dataflow shape
+    (each pass one launch over all systems' tiles, block counters per system,
+    fixed-point moments)."""
     if shape:
         monkeypatch.setenv("DFT_TC_SHAPE", shape)
     solo = [make(n) for n in NAMES]
@@ -64,8 +64,9 @@ def test_batched_scf_converges_to_the_oracle(shape, monkeypatch):
     against the oracle's converged energy (tests/golden/scf_<name>.json, from
     the exact density matrix): every system must meet the stop criterion of
     the one-system test (|dE|/atom < 1e-7 between cycles and max|n_out - n_in|
-    < 1e-5) and land within 1e-5 Ha/atom.  shape None: the tuned launch
-    shape; the other: one dataflow launch per pass over all systems' tiles."""
+    < 1e-5) and land within 1e-5 Ha/atom.  shape None: the grouped expansion;
+    the other: the three-term recurrence, one dataflow launch per pass over all
+    systems' tiles."""
     gold = {}
     for n in ORACLE_NAMES:
         p = os.path.join(GOLD, f"scf_{n}.json")
@@ -93,7 +94,7 @@ def test_batched_scf_converges_to_the_oracle(shape, monkeypatch):
     for n in ORACLE_NAMES:
         assert done[n] is not None, f"{n} did not converge in the batch"
         cycles, e = done[n]
-        print(f"batched {shape or 'tuned'} {n}: {cycles} cycles, E/atom {e:.10f} vs oracle "
+        print(f"batched {shape or 'grouped'} {n}: {cycles} cycles, E/atom {e:.10f} vs oracle "
               f"{gold[n]['E_per_atom']:.10f}, |dE| {abs(e - gold[n]['E_per_atom']):.2e}")
         assert abs(e - gold[n]["E_per_atom"]) < 1e-5
     for c in ctxs:

@@ -24,11 +24,15 @@ from oracle import dm  # noqa: E402
 FP64, FP16 = dft.DFT_PREC_FP64, dft.DFT_PREC_FP16X3
 
 
+def coarse(atoms):
+    xyz = diamond_sphere(25.0)
+    xyz = jitter(xyz[np.argsort((xyz ** 2).sum(1), kind="stable")[:atoms]], 0.05, 1)
+    return make_system(xyz, h=1.0, grid_n=np.array([60, 60, 60]), grid_origin=xyz.min(0) - 7.0)
+
+
 def few_slots():
     """K = 3500 on a coarse grid: a mixed context has 30 expansion buffers."""
-    xyz = diamond_sphere(25.0)
-    xyz = jitter(xyz[np.argsort((xyz ** 2).sum(1), kind="stable")[:350]], 0.05, 1)
-    return make_system(xyz, h=1.0, grid_n=np.array([60, 60, 60]), grid_origin=xyz.min(0) - 7.0)
+    return coarse(350)
 
 
 def given_spectrum(ctx, x, W):
@@ -75,6 +79,25 @@ def test_clenshaw_plan_with_a_single_giant(n_c):
     err = float((P - ref).abs().max() / ref.abs().max())
     print(f"K {K} N_C {n_c}: dmu {info.mu - mu:.2e}, N_e {info.n_e_trace:.6f} of {s.n_electrons}, max|dP| / max|P| {err:.2e}")
     assert abs(info.mu - mu) < 1e-5
+    assert abs(info.n_e_trace - s.n_electrons) < 1e-5 * s.n_electrons
+    assert err < 1e-4
+
+
+@pytest.mark.parametrize("n_c", [90, 700, 2900])
+def test_units_of_two_k_blocks(n_c):
+    """K = 2060, above the line where accumulators take two k-blocks at a time:
+    nine blocks per side, a last one of 12 columns, 65 k-blocks (a last unit of
+    one); plans that keep few and many giants, and Clenshaw's recurrence."""
+    s = coarse(206)
+    beta = n_c / 4.0
+    ctx = dft.Context(s, precision=FP16, e_min=-1.0, e_max=1.0, cheb_order=n_c, kT=1.0 / beta, skip_correction=1)
+    x = np.sort(np.random.default_rng(3).uniform(-0.95, 0.95, ctx.K))
+    F, LW = given_spectrum(ctx, torch.from_numpy(x).cuda(), orthogonal(ctx.K))
+    P, info = ctx.density_matrix(F)
+    ctx.close()
+    ref = (LW * torch.from_numpy(dm.cheb_eval(x, coefficients(info.mu, beta, n_c))).cuda()) @ LW.T
+    err = float((P - ref).abs().max() / ref.abs().max())
+    print(f"K 2060 N_C {n_c}: N_e {info.n_e_trace:.6f} of {s.n_electrons}, max|dP| / max|P| {err:.2e}")
     assert abs(info.n_e_trace - s.n_electrons) < 1e-5 * s.n_electrons
     assert err < 1e-4
 

@@ -1,5 +1,7 @@
 """Parity at full size: the 465-atom silicon sphere (K = 4650, 147^3 grid)
-in the mixed precision and the dataflow launch shape that the benchmark times.
+in the mixed precision that the benchmark times (the grouped expansion, whose
+memory-limited Clenshaw plan this size takes), and once by the three-term
+recurrence.
 
 Inputs come from the oracle and the seeded geometry only.  The Fock matrix is
 F = T + V[v_loc]: the closed-form kinetic matrix plus the quadrature (Eq. 2.5)
@@ -40,7 +42,7 @@ if not torch.cuda.is_available():
 
 import paper_2108_13478_gb300 as dft  # noqa: E402
 
-FLOW = "32,0,256,0,0,0,1"      # one cooperative launch per recurrence pass
+FLOW = "32,0,256,0,0,0,1"      # the three-term recurrence, one cooperative launch per pass
 U32 = 2.0 ** -24
 
 
@@ -79,13 +81,10 @@ def sphere():
 
 @pytest.fixture(scope="module")
 def ctx(sphere):
-    mp = pytest.MonkeyPatch()
-    mp.setenv("DFT_TC_SHAPE", FLOW)
     c = dft.Context(sphere["s"], precision=dft.DFT_PREC_FP16X3, model=dft.DFT_MODEL_NEUTRAL,
                     cheb_tail_tol=1e-10)
     yield c
     c.close()
-    mp.undo()
 
 
 def test_overlap_kinetic(sphere, ctx):
@@ -104,7 +103,7 @@ def test_density_matrix(sphere, ctx):
     e_kin = abs(2 * np.sum(dP * T)) / s.n_atoms
     e_band = abs(2 * np.sum(dP * F)) / s.n_atoms
     n_e = 2 * np.sum(P * sphere["S"])
-    print(f"sphere25 fp16x3 {FLOW}: N_C {info.n_cheb}  max|dP| {err:.3e} (max|P| {np.max(np.abs(ex['P'])):.3f})  "
+    print(f"sphere25 fp16x3: N_C {info.n_cheb}  max|dP| {err:.3e} (max|P| {np.max(np.abs(ex['P'])):.3f})  "
           f"dEkin/atom {e_kin:.3e}  dEband/atom {e_band:.3e}  2Tr[PS] {n_e:.6f}  "
           f"mu {info.mu:.8f} vs {ex['mu']:.8f}")
     assert info.spectrum_ok == 1
@@ -113,17 +112,17 @@ def test_density_matrix(sphere, ctx):
     assert e_kin < 1e-5 and e_band < 1e-5
 
 
-@pytest.mark.parametrize("skip", [0, 1])
-def test_density_matrix_at_the_benchmark_order(sphere, skip):
+@pytest.mark.parametrize("skip,shape", [(0, None), (1, None), (0, FLOW)])
+def test_density_matrix_at_the_benchmark_order(sphere, skip, shape, monkeypatch):
     """The benchmark runs the mixed path with the Chebyshev tail 1e-5 (about
     half the steps of 1e-10; the oracle's truncated expansion against its
     exact eigensolve gives 9e-10 Ha/atom here, and the K = 640 case is
     pinned in tests/test_oracle_truncation.py): the same gates hold, with
-    the FP64 electron-count correction after the recurrence (skip = 0, the
-    default) and without it."""
+    the FP64 electron-count correction after the expansion (skip = 0, the
+    default) and without it, and by the three-term recurrence."""
     s, ex, F, T = sphere["s"], sphere["ex"], sphere["F"], sphere["T"]
-    mp = pytest.MonkeyPatch()
-    mp.setenv("DFT_TC_SHAPE", FLOW)
+    if shape:
+        monkeypatch.setenv("DFT_TC_SHAPE", shape)
     c = dft.Context(s, precision=dft.DFT_PREC_FP16X3, model=dft.DFT_MODEL_NEUTRAL, cheb_tail_tol=1e-5,
                     skip_correction=skip)
     try:
@@ -132,13 +131,12 @@ def test_density_matrix_at_the_benchmark_order(sphere, skip):
         P = host(P)
     finally:
         c.close()
-        mp.undo()
     dP = P - ex["P"]
     err = float(np.max(np.abs(dP)))
     e_kin = abs(2 * np.sum(dP * T)) / s.n_atoms
     e_band = abs(2 * np.sum(dP * F)) / s.n_atoms
     n_e = 2 * np.sum(P * sphere["S"])
-    print(f"sphere25 fp16x3 tail 1e-5 {'without' if skip else 'with'} correction: N_C {info.n_cheb}  "
+    print(f"sphere25 fp16x3 {shape or 'grouped'} tail 1e-5 {'without' if skip else 'with'} correction: N_C {info.n_cheb}  "
           f"max|dP| {err:.3e}  dEkin/atom {e_kin:.3e}  dEband/atom {e_band:.3e}  2Tr[PS] {n_e:.6f}  "
           f"dmu {info.mu_correction:+.3e}  stages {[round(x, 1) for x in info.ms_stage]}")
     assert info.spectrum_ok == 1
