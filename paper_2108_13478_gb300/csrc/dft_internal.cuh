@@ -143,6 +143,7 @@ struct Ctx {
     int* d_tile_order = nullptr; // [n_tiles], longest lists first
     int grid_split = 1;          // blocks per tile of the quadrature (by chunk pairs)
     int plane_split = 1;         // and of the collocation (by planes)
+    long long n_busy = 0;        // tiles with a list, the first of d_tile_order
     double* d_xyz = nullptr;     // [n_atoms * 3]
     double* d_S = nullptr;       // K x K
     double* d_T = nullptr;

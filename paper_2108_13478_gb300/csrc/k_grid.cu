@@ -287,6 +287,69 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 3 : 2) k_collocate(
     }
 }
 
+// The same for short lists: 256 threads of two points each, SCH functions a at a
+// time in registers, phi_b formed by each thread, P taken whole.  k_collocate
+// pads the list to chunks of 64 (32) in both indexes and pays for staging a whole
+// chunk and its 64 x y products, which a short list does not repay.  Sums as long as
+// there: at most 64 functions b, then 8 functions a, then FP64.
+constexpr int SCH = 32;
+template <typename R>
+__global__ void __launch_bounds__(256) k_collocate_short(
+    const Fn* __restrict__ fn, const double* __restrict__ tab, int W, const int* __restrict__ tile_ptr,
+    const int* __restrict__ tile_fn, const int* __restrict__ tile_order, int ntx, int nty, int nx, int ny, int nz, int K,
+    const double* __restrict__ P, double* __restrict__ n_out) {
+    __shared__ R sa[3][SCH][TILE], sb[3][SCH][TILE];
+    __shared__ __align__(16) R sP[SCH][SCH];
+    const int t = tile_order[blockIdx.x];
+    const int tx = t % ntx, ty = (t / ntx) % nty, tz = t / (ntx * nty);
+    const int t0[3] = {tx * TILE, ty * TILE, tz * TILE};
+    const int* list = tile_fn + tile_ptr[t];
+    const int n_t = tile_ptr[t + 1] - tile_ptr[t];
+    const int px = threadIdx.x & 7, py = (threadIdx.x >> 3) & 7, pz0 = threadIdx.x >> 6, pz1 = pz0 + 4;
+    double acc0 = 0.0, acc1 = 0.0;
+    for (int ca = 0; ca < n_t; ca += SCH) {
+        for (int cb = 0; cb < n_t;) {
+            R y0[SCH], y1[SCH];
+#pragma unroll
+            for (int j = 0; j < SCH; ++j) y0[j] = y1[j] = (R)0;
+            for (const int end = min(n_t, cb + 2 * SCH); cb < end; cb += SCH) {
+                __syncthreads();
+                if (cb == 0) stage_slices<R, SCH>(fn, tab, W, list, n_t, ca, t0, sa);
+                stage_slices<R, SCH>(fn, tab, W, list, n_t, cb, t0, sb);
+                for (int e = threadIdx.x; e < SCH * SCH; e += 256) {
+                    const int i = e / SCH, j = e % SCH;
+                    sP[i][j] = (R)(cb + i < n_t && ca + j < n_t ? P[(long long)list[cb + i] * K + list[ca + j]] : 0.0);
+                }
+                __syncthreads();
+                const int nb = min(SCH, n_t - cb);
+#pragma unroll 2
+                for (int i = 0; i < nb; ++i) {
+                    const R pxy = sb[0][i][px] * sb[1][i][py], pb0 = pxy * sb[2][i][pz0], pb1 = pxy * sb[2][i][pz1];
+#pragma unroll
+                    for (int j = 0; j < SCH; ++j) {
+                        y0[j] = fma(pb0, sP[i][j], y0[j]);
+                        y1[j] = fma(pb1, sP[i][j], y1[j]);
+                    }
+                }
+            }
+            R c0[4] = {}, c1[4] = {};
+#pragma unroll
+            for (int j = 0; j < SCH; ++j) {
+                const R pxy = sa[0][j][px] * sa[1][j][py];
+                c0[j % 4] = fma(pxy * sa[2][j][pz0], y0[j], c0[j % 4]);
+                c1[j % 4] = fma(pxy * sa[2][j][pz1], y1[j], c1[j % 4]);
+            }
+            acc0 += (double)((c0[0] + c0[1]) + (c0[2] + c0[3]));
+            acc1 += (double)((c1[0] + c1[1]) + (c1[2] + c1[3]));
+        }
+    }
+    const int gx = t0[0] + px, gy = t0[1] + py, gz0 = t0[2] + pz0, gz1 = t0[2] + pz1;
+    if (gx < nx && gy < ny) {
+        if (gz0 < nz) n_out[((long long)gz0 * ny + gy) * nx + gx] = 2.0 * acc0;
+        if (gz1 < nz) n_out[((long long)gz1 * ny + gy) * nx + gx] = 2.0 * acc1;
+    }
+}
+
 // V_ab += h^3 sum_{g in tile} phi_a v phi_b for all pairs of the tile's list
 // (Eq. A.6): per chunk pair and plane G_ab = sum_q (x y)_a(q) w_b(q) with w =
 // v phi_b, V_ab += z_a G_ab.  Contributions of different tiles meet as
@@ -449,6 +512,13 @@ __global__ void k_gaussian_sum(const double* __restrict__ xyz, int n_atoms, int 
 
 }  // namespace
 
+// Longest list (of a context) that k_collocate_short takes.  Density on the grid
+// in us by k_collocate / k_collocate_short, by longest list: FP32 8 terms (465
+// atoms, grid 147^3) 286 / 56, 22 380 / 85, 77 82 / 60, 113 135 / 109, 149 221 /
+// 176, 173 237 / 247, 242 397 / 461; FP64 8 2731 / 480, 29 312 / 161, 50 404 /
+// 453, 64 543 / 570, 77 1082 / 1054.
+constexpr int SHORT_F32 = 160, SHORT_F64 = 32;
+
 // Blocks per grid tile: a tile's work grows with the square of its list, and a
 // small cluster has few tiles, so tiles are split (collocation by planes,
 // quadrature by chunk pairs) until the longest takes at most a third of what an SM
@@ -457,7 +527,9 @@ __global__ void k_gaussian_sum(const double* __restrict__ xyz, int n_atoms, int 
 void grid_split(Ctx& c, const int* tile_ptr) {
     const int ch = c.p.precision == DFT_PREC_FP64 ? GridCfg<double>::CH : GridCfg<float>::CH;
     double total = 0.0, longest = 0.0;
+    c.n_busy = 0;
     for (long long t = 0; t < c.n_tiles; ++t) {
+        c.n_busy += tile_ptr[t + 1] > tile_ptr[t];
         const double n = (tile_ptr[t + 1] - tile_ptr[t] + ch - 1) / ch, w = n * (n + 1) / 2;
         total += w;
         longest = std::max(longest, w);
@@ -494,14 +566,20 @@ void launch_collocate(const Ctx& c, const double* P, double* n, cudaStream_t s) 
         launch_expand(c, P, c.d_Mt, s);
         P = c.d_Mt;
     }
-    auto go = [&](auto kern, size_t bytes) {
+    auto go = [&](auto kern, unsigned split, int threads, size_t bytes) {
         allow_smem(kern, bytes);
-        const dim3 grid((unsigned)c.n_tiles, c.plane_split);
-        kern<<<grid, 128, bytes, s>>>(c.d_fn, c.d_tab, c.tab_w, c.d_tile_ptr, c.d_tile_fn, c.d_tile_order, c.ntile[0],
-                                      c.ntile[1], c.n[0], c.n[1], c.n[2], c.Kt, P, n);
+        const dim3 grid((unsigned)c.n_tiles, split);
+        kern<<<grid, threads, bytes, s>>>(c.d_fn, c.d_tab, c.tab_w, c.d_tile_ptr, c.d_tile_fn, c.d_tile_order, c.ntile[0],
+                                          c.ntile[1], c.n[0], c.n[1], c.n[2], c.Kt, P, n);
     };
-    if (c.p.precision == DFT_PREC_FP64) go(k_collocate<double>, sizeof(CollSmem<double>));
-    else go(k_collocate<float>, sizeof(CollSmem<float>));
+    const bool f64 = c.p.precision == DFT_PREC_FP64;
+    if (c.tile_max <= (f64 ? SHORT_F64 : SHORT_F32)) {
+        if (f64) go(k_collocate_short<double>, 1, 256, 0);
+        else go(k_collocate_short<float>, 1, 256, 0);
+    } else {
+        if (f64) go(k_collocate<double>, c.plane_split, 128, sizeof(CollSmem<double>));
+        else go(k_collocate<float>, c.plane_split, 128, sizeof(CollSmem<float>));
+    }
     check_launch("collocate");
 }
 
@@ -512,7 +590,8 @@ void launch_quadrature(const Ctx& c, const double* v, double* V, cudaStream_t s)
     DFT_CUDA_CHECK(cudaMemsetAsync(Vq, 0, sizeof(double) * (size_t)K * K, s));
     auto go = [&](auto kern, size_t bytes) {
         allow_smem(kern, bytes);
-        kern<<<dim3((unsigned)c.n_tiles, c.grid_split), 128, bytes, s>>>(c.d_fn, c.d_tab, c.tab_w, c.d_tile_ptr, c.d_tile_fn, c.d_tile_order, c.ntile[0],
+        if (c.n_busy == 0) return;
+        kern<<<dim3((unsigned)c.n_busy, c.grid_split), 128, bytes, s>>>(c.d_fn, c.d_tab, c.tab_w, c.d_tile_ptr, c.d_tile_fn, c.d_tile_order, c.ntile[0],
                                                      c.ntile[1], c.n[0], c.n[1], c.n[2], K, c.h * c.h * c.h, v, Vq);
     };
     if (c.p.precision == DFT_PREC_FP64) go(k_quadrature<double>, sizeof(QuadSmem<double>));

@@ -1,7 +1,9 @@
 """Collocation and quadrature by chunk pairs: lists shorter than a chunk, of
 one chunk and a remainder, and of several chunks (chunks of 64 functions in
-FP32, 32 in FP64), ragged grid tiles, and a P that is not symmetric, against
-the oracle's plain sums."""
+FP32, 32 in FP64), ragged grid tiles, mostly empty boxes, and a P that is not
+symmetric, against the oracle's plain sums.  Collocation has a kernel for
+contexts whose longest list has at most 160 terms in FP32 (tiny19: 156, tiny20:
+161) and 32 in FP64 (tiny3: 29)."""
 import numpy as np
 import pytest
 
@@ -19,10 +21,11 @@ import paper_2108_13478_gb300 as dft  # noqa: E402
 U32 = 2.0 ** -24
 
 
-@pytest.mark.parametrize("name", ["tiny1", "tiny3", "tiny7", "tiny13", "dtiny4"])
+@pytest.mark.parametrize("name,pad", [("tiny1", 5.0), ("tiny3", 5.0), ("tiny7", 5.0), ("tiny13", 5.0), ("tiny19", 5.0),
+                                      ("tiny20", 5.0), ("dtiny4", None), ("tiny2", 24.0)])
 @pytest.mark.parametrize("mixed", [False, True])
-def test_chunk_pairs_match_the_oracle(name, mixed):
-    s = w.config_system(name)
+def test_chunk_pairs_match_the_oracle(name, pad, mixed):
+    s = w.config_system(name, pad=pad) if pad else w.config_system(name)
     rng = np.random.default_rng(21)
     v = rng.normal(size=tuple(int(t) for t in s.grid_n[::-1]))
     K = s.n_basis
