@@ -261,8 +261,11 @@ typedef struct dft_columns_info {
  * block-Jacobi (the inverse of each atom's diagonal block of S; atoms of at
  * most 48 functions) or none; the paper's incomplete Cholesky is not offered
  * (its triangular solves are sequential).  FP64 throughout, whatever the
- * context's precision.  The iterations run in groups of 8 (CUDA graphs), so
- * a solve takes at most pcg_maxit rounded up to a multiple of 8.
+ * context's precision.  Where K <= 4096, an atom's functions are contiguous
+ * and the columns are not too many for the basis (48, or columns x K^2 up to
+ * 4e8 to 8e8), a solve is one launch of thread-block clusters; otherwise its
+ * iterations run in groups of 8 (CUDA graphs).  Either way it takes at most
+ * pcg_maxit iterations rounded up to a multiple of 8.
  *   F        device, K x K Fock matrix, row-major (symmetric)
  *   cols     host, ncols column indices in [0, K) (repeats allowed)
  *   mu       chemical potential (Ha), e.g. dft_info.mu of dft_density_matrix

@@ -53,11 +53,13 @@ using namespace tc;
 
 constexpr int BM = 128, BN = 256, BK = 32, STAGES = 4;
 // k-blocks per accumulator promotion (PstItem::sub).  Longer chains lean
-// further towards zero.  Error of P at K = 370 / 1230 against an exact
-// eigensolve with 1, 2 and 4 in all products: 1.2e-5 / 2.4e-5, 1.3e-5 / 2.5e-5,
-// 1.8e-5 / 2.8e-5 (the recurrence this replaced: 2.3e-5 / 3.6e-5); a density
-// matrix at K = 2000 takes 10.7, 10.3 and 9.9 ms.  The babies' bias acts as a
-// scale of H_N on every term, so they, and everything where K is small, take 1.
+// further towards zero; the babies' bias acts as a scale of H_N on every term,
+// so they take 1.  Giants and weighted products with 1 / 2, density matrix in ms
+// (tail 1e-5, without the set-up of H_N): K = 1230 4.35 / 4.17, 2100 9.01 / 8.49,
+// 3000 26.8 / 24.4, 4650 60.1 / 54.1; the error of P against FP64 is the same to
+// 1% at all of them (relative 1.7e-5, 2.0e-5, 2.4e-5, 2.9e-5; the three-term
+// recurrence 3.1e-5, 3.6e-5, -, 4.8e-5).  Up to SUB_FINE_K, where a chain of two
+// saves 4% at most, the chains stay at one.
 constexpr int SUB_FINE = 1, SUB = 2, SUB_FINE_K = 2048;
 constexpr int A_BYTES = BM * BK * 2, B_BYTES = BN * BK * 2;
 constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;
@@ -593,7 +595,9 @@ __device__ __forceinline__ void block_at(int t, int nb, int& a, int& b) {
 }
 
 // C_q = sum_{r<s} c_qr T_r (T_0 = I) for up to 8 q at once, each to a slot, as
-// a pair (operand) or as FP32 planes.  HBM-bound: the babies are read once
+// a pair (operand) or as FP32 planes.  HBM-bound at large K (K = 4650: 1.74 GB in
+// 324 us, 0.79 of the measured copy rate; K = 1230: 160 MB in 46 us, 0.52, where the
+// launch has 12 blocks of 256 threads per SM): the babies are read once
 // per 8 q; 4 consecutive elements per thread, FP32 FMA chains of s terms.
 template <bool BF>
 __global__ void __launch_bounds__(256) k_pst_combine(int K, int nb, int s, PstList T, PstOut out, int q0, int nq,
@@ -656,11 +660,14 @@ __global__ void __launch_bounds__(256) k_pst_combine(int K, int nb, int s, PstLi
 
 // partial Gram sums <G_q, T_r>, 8 x 8 pairs per CTA (blockIdx.x: 8 babies,
 // blockIdx.z: 8 giants) over the 4-element groups of CTA column blockIdx.y;
-// off-diagonal blocks count twice.  HBM-bound where few giants are at hand
-// (each baby is read once per 8 giants; the CTAs of one column, adjacent in
-// launch order, share the giants' elements in L2), so nothing is staged: every thread keeps its 64 FP32
-// FMA chains (GRAM_GROUPS x 4 products long, the buffer of the partial sums is
-// sized for that) and the chains meet in FP64.
+// off-diagonal blocks count twice.  Each baby is read once per 8 giants; the
+// CTAs of one column, adjacent in launch order, share the giants' elements in
+// L2, so nothing is staged: every thread keeps its 64 FP32 FMA chains
+// (GRAM_GROUPS x 4 products long, the buffer of the partial sums is sized for
+// that) and the chains meet in FP64.  Bound by the latency of a group's loads
+// with one block of 8 warps per SM (164 registers): K = 4650, 4 giants, 1.73 GB
+// in 838 us, 0.30 of the measured copy rate and 34% of the issue slots; K = 1230,
+// all 58 giants, 0.62 GB in 332 us.
 constexpr int GRAM_GROUPS = 32;   // 4-element groups per thread
 template <bool BF>
 __global__ void __launch_bounds__(256) k_pst_gram(int K, int nb, PstList G, int nq, PstList T, int s,
