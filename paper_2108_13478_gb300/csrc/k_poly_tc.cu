@@ -537,6 +537,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
             if (lane == 0) mbar_arrive(&accempty[a_last]);
             if (bad && limit > 0.0f) atomicExch(&S.flags[FLAG_SPECTRUM], 1);
         }
+        if (!ok && lane == 0) {   // wake the MMA issuer, which sees the abort
+            mbar_arrive(&accempty[0]);
+            mbar_arrive(&accempty[1]);
+        }
     }
     tc_fence_before();
     __syncthreads();
