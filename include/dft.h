@@ -68,8 +68,11 @@ typedef enum dft_status {
 
 /* Precision of the Chebyshev products: FP64 throughout, or tensor cores on
  * operands split into two 16-bit floats (hi + lo) with three products per
- * step and FP32 accumulation (BF16 or FP16 pairs).  The mixed modes also run
- * collocation and quadrature in FP32 arithmetic. */
+ * step and FP32 accumulation.  BF16X3 holds the three-term recurrence's
+ * operands (DFT_TC_SHAPE) as BF16 pairs; everything else in it, the grouped
+ * expansion too, is the same FP16 pairs as in FP16X3, whose 22 bits its
+ * weighted products need.  The mixed modes also run collocation and quadrature
+ * in FP32 arithmetic. */
 enum { DFT_PREC_FP64 = 0, DFT_PREC_BF16X3 = 1, DFT_PREC_FP16X3 = 2 };
 enum { DFT_MODEL_LITERAL = 0, DFT_MODEL_NEUTRAL = 1 };
 /* Density mixing of the SCF step: linear, Kerker-preconditioned linear, or

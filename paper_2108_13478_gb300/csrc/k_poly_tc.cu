@@ -51,6 +51,12 @@ namespace {
 
 using namespace tc;
 
+// FP16 pairs in every mixed precision: the operands are bounded, and 16 bits of a
+// BF16 pair for the C_q left P 9% further from FP64 than the three-term recurrence
+// does on BF16 pairs (its sum is FP32; K = 80 to 1230, four geometries each: 9.9e-5,
+// 1.1e-4, 1.3e-4 against 9.0e-5, 1.0e-4, 1.2e-4)
+using P16 = H16<false>;
+
 constexpr int BM = 128, BN = 256, BK = 32, STAGES = 4;
 // k-blocks per accumulator promotion (PstItem::sub).  Longer chains lean
 // further towards zero; the babies' bias acts as a scale of H_N on every term,
@@ -162,12 +168,11 @@ __device__ __forceinline__ Work work_at(int t, const PstItem* items, int nitems,
     return w;
 }
 
-template <bool BF>
 __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restrict__ sys,
                                                           const PstItem* __restrict__ items_g, int nitems,
                                                           const int2* __restrict__ pairs, int ntiles,
                                                           int* lead_flags, int hold) {
-    using T = typename H16<BF>::T;
+    using T = P16::T;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint64_t* full = (uint64_t*)(smem + STAGES * STAGE_BYTES);
@@ -271,7 +276,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
         __syncwarp();
     } else if (warp == 1) {
         if (lane == 0) {
-            const uint32_t idesc0 = (1u << 4) | ((BF ? 1u : 0u) << 7) | ((BF ? 1u : 0u) << 10) |
+            const uint32_t idesc0 = (1u << 4) |
                                     ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
             long long g = 0, u = 0;   // k-blocks and units of this CTA
             for (int t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x) {
@@ -434,7 +439,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
                 if (pv) {
 #pragma unroll
                     for (int k = 0; k < EB / 2; ++k) {
-                        const float2 h = H16<BF>::to_f2(ph[k]), l = H16<BF>::to_f2(pl[k]);
+                        const float2 h = P16::to_f2(ph[k]), l = P16::to_f2(pl[k]);
                         const float f0 = h.x + l.x, f1 = h.y + l.y;   // rows r & ~1, r | 1
                         const float got = __shfl_xor_sync(0xffffffffu, odd ? f0 : f1, 1);
                         x[2 * k] = fmaf(-ISC, odd ? got : f0, x[2 * k]);
@@ -473,9 +478,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
 #pragma unroll
                     for (int k = 0; k < EB / 2; ++k) {
                         const float y0 = x[2 * k] * SC, y1 = x[2 * k + 1] * SC;
-                        const uint32_t h = H16<BF>::from_f2(y0, y1);
-                        const float2 f = H16<BF>::to_f2(h);
-                        const uint32_t l = H16<BF>::from_f2(y0 - f.x, y1 - f.y);
+                        const uint32_t h = P16::from_f2(y0, y1);
+                        const float2 f = P16::to_f2(h);
+                        const uint32_t l = P16::from_f2(y0 - f.x, y1 - f.y);
                         own[2 * k] = __byte_perm(h, l, 0x5410);
                         own[2 * k + 1] = __byte_perm(h, l, 0x7632);
                     }
@@ -551,9 +556,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_pst_prod(const PstSys* __restri
 }
 
 // FP64 symmetric matrix -> pair in a slot, zero beyond K
-template <bool BF>
 __global__ void __launch_bounds__(256) k_pst_split(int K, int nb, const double* __restrict__ A, uint16_t* slot) {
-    using T = typename H16<BF>::T;
+    using T = P16::T;
     int a = 0, t = blockIdx.x;   // block (a, b)
     while (t >= nb - a) {
         t -= nb - a;
@@ -567,8 +571,8 @@ __global__ void __launch_bounds__(256) k_pst_split(int K, int nb, const double* 
     for (int r = blockIdx.y * 16; r < (int)blockIdx.y * 16 + 16; ++r) {
         const int gr = b * 256 + r;
         const double x = gr < K && gc < K ? A[(long long)gr * K + gc] * (double)SC : 0.0;
-        const T h = H16<BF>::from_d(x);
-        const T l = H16<BF>::from_d(x - (double)H16<BF>::to_f(h));
+        const T h = P16::from_d(x);
+        const T l = P16::from_d(x - (double)P16::to_f(h));
         uint16_t* o = slot + (size_t)(fr * 256 + r) * ld + fc * 256 + c;
         o[0] = (uint16_t)bits16(h);
         o[plane] = (uint16_t)bits16(l);
@@ -576,15 +580,13 @@ __global__ void __launch_bounds__(256) k_pst_split(int K, int nb, const double* 
 }
 
 // four consecutive elements of a pair, as stored and scaled back
-template <bool BF>
 __device__ __forceinline__ float4 pair4_raw(uint2 h, uint2 l) {
-    using T = typename H16<BF>::T;
-    auto f = [](uint32_t a, uint32_t b) { return H16<BF>::to_f(from_bits16<T>(a)) + H16<BF>::to_f(from_bits16<T>(b)); };
+    using T = P16::T;
+    auto f = [](uint32_t a, uint32_t b) { return P16::to_f(from_bits16<T>(a)) + P16::to_f(from_bits16<T>(b)); };
     return make_float4(f(h.x, l.x), f(h.x >> 16, l.x >> 16), f(h.y, l.y), f(h.y >> 16, l.y >> 16));
 }
-template <bool BF>
 __device__ __forceinline__ float4 pair4(const uint16_t* p, size_t plane) {
-    const float4 x = pair4_raw<BF>(*(const uint2*)p, *(const uint2*)(p + plane));
+    const float4 x = pair4_raw(*(const uint2*)p, *(const uint2*)(p + plane));
     return make_float4(ISC * x.x, ISC * x.y, ISC * x.z, ISC * x.w);
 }
 
@@ -603,10 +605,9 @@ __device__ __forceinline__ void block_at(int t, int nb, int& a, int& b) {
 // 324 us, 0.79 of the measured copy rate; K = 1230: 160 MB in 46 us, 0.52, where the
 // launch has 12 blocks of 256 threads per SM): the babies are read once
 // per 8 q; 4 consecutive elements per thread, FP32 FMA chains of s terms.
-template <bool BF>
 __global__ void __launch_bounds__(256) k_pst_combine(int K, int nb, int s, PstList T, PstOut out, int q0, int nq,
                                                      const double* __restrict__ c, int f32) {
-    using H = typename H16<BF>::T;
+    using H = P16::T;
     __shared__ float4 cf[PS_MAX_S][2];
     const int qb = blockIdx.z * 8, n = min(8, nq - qb);
     for (int e = threadIdx.x; e < s * 8; e += 256) {
@@ -629,7 +630,7 @@ __global__ void __launch_bounds__(256) k_pst_combine(int K, int nb, int s, PstLi
         for (int k = 0; k < 4; ++k) acc[q][k] = (gr == gc + k && gr < K) ? ((const float*)cf)[q] : 0.0f;
 #pragma unroll 4
     for (int r = 1; r < s; ++r) {
-        const float4 x = pair4<BF>((const uint16_t*)T.p[r] + e0, plane);
+        const float4 x = pair4((const uint16_t*)T.p[r] + e0, plane);
         const float4 c0 = cf[r][0], c1 = cf[r][1];
         const float w[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
 #pragma unroll
@@ -651,9 +652,9 @@ __global__ void __launch_bounds__(256) k_pst_combine(int K, int nb, int s, PstLi
                 h[k] = __float_as_uint(x) >> 16;
                 l[k] = __float_as_uint(x) & 0xffffu;
             } else {
-                const H th = H16<BF>::from_f(x * SC);
+                const H th = P16::from_f(x * SC);
                 h[k] = bits16(th);
-                l[k] = bits16(H16<BF>::from_f(x * SC - H16<BF>::to_f(th)));
+                l[k] = bits16(P16::from_f(x * SC - P16::to_f(th)));
             }
         }
         uint16_t* o = (uint16_t*)out.p[qb + q] + e0;
@@ -673,7 +674,6 @@ __global__ void __launch_bounds__(256) k_pst_combine(int K, int nb, int s, PstLi
 // in 838 us, 0.30 of the measured copy rate and 34% of the issue slots; K = 1230,
 // all 58 giants, 0.62 GB in 332 us.
 constexpr int GRAM_GROUPS = 32;   // 4-element groups per thread
-template <bool BF>
 __global__ void __launch_bounds__(256) k_pst_gram(int K, int nb, PstList G, int nq, PstList T, int s,
                                                   double* __restrict__ part) {
     __shared__ double red[8][64];
@@ -722,7 +722,7 @@ __global__ void __launch_bounds__(256) k_pst_gram(int K, int nb, PstList G, int 
             fetch(0);
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
-                x[q] = pair4_raw<BF>(hx[q], lx[q]);
+                x[q] = pair4_raw(hx[q], lx[q]);
                 x[q].x *= wt;
                 x[q].y *= wt;
                 x[q].z *= wt;
@@ -738,7 +738,7 @@ __global__ void __launch_bounds__(256) k_pst_gram(int K, int nb, PstList G, int 
                 float4 y[4];
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
-                    y[r] = pair4_raw<BF>(hy[r], ly[r]);
+                    y[r] = pair4_raw(hy[r], ly[r]);
                     if (live < 4) {
                         if (live < 2) y[r].y = 0.f;
                         if (live < 3) y[r].z = 0.f;
@@ -776,9 +776,8 @@ __global__ void __launch_bounds__(256) k_pst_gram(int K, int nb, PstList G, int 
 }
 
 // out[y * stride] = Tr of matrix y of the list
-template <bool BF>
 __global__ void __launch_bounds__(128) k_pst_trace(int K, int nb, PstList L, double* __restrict__ out, int stride) {
-    using H = typename H16<BF>::T;
+    using H = P16::T;
     __shared__ double red[4];
     const size_t ld = (size_t)nb * 256, plane = (size_t)(nb / 2 + 1) * 256 * ld;
     const uint16_t* X = (const uint16_t*)L.p[blockIdx.x];
@@ -787,7 +786,7 @@ __global__ void __launch_bounds__(128) k_pst_trace(int K, int nb, PstList L, dou
         int fr, fc;
         fold(i >> 8, i >> 8, nb, fr, fc);
         const size_t e = (size_t)(fr * 256 + (i & 255)) * ld + fc * 256 + (i & 255);
-        x += (double)H16<BF>::to_f(from_bits16<H>(X[e])) + (double)H16<BF>::to_f(from_bits16<H>(X[e + plane]));
+        x += (double)P16::to_f(from_bits16<H>(X[e])) + (double)P16::to_f(from_bits16<H>(X[e + plane]));
     }
     for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
@@ -798,11 +797,10 @@ __global__ void __launch_bounds__(128) k_pst_trace(int K, int nb, PstList L, dou
 // rho (K x K, FP64, both triangles) = [C_0 or rho] + sum of np FP32 partial
 // products - b2, these two times up: C_0 = sum_r c_0r T_r in FP32 FMA chains of
 // 8 terms added in FP64
-template <bool BF>
 __global__ void __launch_bounds__(256) k_pst_finish(int K, int nb, int s, PstList T, const double* __restrict__ c,
                                                     PstOut part, int np, const uint16_t* b2, double up, int first,
                                                     double* __restrict__ rho) {
-    using H = typename H16<BF>::T;
+    using H = P16::T;
     __shared__ double sh[32][33];
     __shared__ float cf[PS_MAX_S];
     const int nt = (K + 31) / 32;
@@ -815,7 +813,7 @@ __global__ void __launch_bounds__(256) k_pst_finish(int K, int nb, int s, PstLis
     const size_t ld = (size_t)nb * 256, plane = (size_t)(nb / 2 + 1) * 256 * ld;
     const int lc = threadIdx.x & 31;
     auto pr = [](const uint16_t* p, size_t pl) {
-        return ISC * (H16<BF>::to_f(from_bits16<H>(*p)) + H16<BF>::to_f(from_bits16<H>(p[pl])));
+        return ISC * (P16::to_f(from_bits16<H>(*p)) + P16::to_f(from_bits16<H>(p[pl])));
     };
     // lanes along the row index gr (contiguous in the slots), element (gr, gc), gc >= gr
     for (int lr = threadIdx.x >> 5; lr < 32; lr += 8) {
@@ -877,7 +875,6 @@ int sys_tiles(const Ctx& c) {
 struct Queue {
     Ctx& lead;
     cudaStream_t st;
-    bool bf;
     std::vector<PstItem> items;
     std::vector<int2> pairs;
     struct Launch { int first, n, tiles; };
@@ -886,7 +883,7 @@ struct Queue {
     int hold;
 
     Queue(Ctx& l, cudaStream_t s)
-        : lead(l), st(s), bf(l.p.precision == DFT_PREC_BF16X3), hold(std::getenv("DFT_TEST_EXPIRE_WAITS") ? 1 : 0) {}
+        : lead(l), st(s), hold(std::getenv("DFT_TEST_EXPIRE_WAITS") ? 1 : 0) {}
     void add(int sys, const Ctx& c, std::initializer_list<int2> ab, int prev, int add_, int out, int mode, double limit) {
         PstItem it{};
         it.sys = sys;
@@ -924,12 +921,8 @@ struct Queue {
     void launch(size_t k) {
         const Launch& l = launches[k];
         const int grid = std::min(l.tiles, SMS);
-        auto go = [&](auto kern) {
-            kern<<<grid, NTHREADS, SMEM_BYTES, st>>>(lead.d_pst_sys, lead.d_pst_items + l.first, l.n, lead.d_pst_pairs, l.tiles,
-                                                     lead.d_flags, hold);
-        };
-        if (bf) go(k_pst_prod<true>);
-        else go(k_pst_prod<false>);
+        k_pst_prod<<<grid, NTHREADS, SMEM_BYTES, st>>>(lead.d_pst_sys, lead.d_pst_items + l.first, l.n, lead.d_pst_pairs,
+                                                       l.tiles, lead.d_flags, hold);
         check_launch("pst_prod");
     }
     void run() {
@@ -961,16 +954,9 @@ struct View {
     }
 };
 
-template <class A, class B>
-void pick(bool bf, A&& a, B&& b) {
-    if (bf) a();
-    else b();
-}
-
 void gram(Ctx& c, int q0, const std::vector<int>& slots, cudaStream_t st) {
     const View v(c);
     const int s = v.p.s, nb = c.Kp / 256;
-    const bool bf = c.p.precision == DFT_PREC_BF16X3;
     double* D = c.d_wk;
     const PstList T = v.babies();
     for (size_t k = 0; k < slots.size(); k += PS_MAX_S) {
@@ -985,12 +971,10 @@ void gram(Ctx& c, int q0, const std::vector<int>& slots, cudaStream_t st) {
         const dim3 grid((s + 7) / 8, nsplit, (nq + 7) / 8);
         double* Dq = D + (long long)(q0 + k) * s;
         if (s > 1) {
-            pick(bf, [&] { k_pst_gram<true><<<grid, 256, 0, st>>>(c.K, nb, G, nq, T, s, c.d_gram); },
-                 [&] { k_pst_gram<false><<<grid, 256, 0, st>>>(c.K, nb, G, nq, T, s, c.d_gram); });
+            k_pst_gram<<<grid, 256, 0, st>>>(c.K, nb, G, nq, T, s, c.d_gram);
             k_pst_gram_sum<<<(nq * s + 7) / 8, 256, 0, st>>>(nsplit, nq * s, c.d_gram, Dq);
         }
-        pick(bf, [&] { k_pst_trace<true><<<nq, 128, 0, st>>>(c.K, nb, G, Dq, s); },
-             [&] { k_pst_trace<false><<<nq, 128, 0, st>>>(c.K, nb, G, Dq, s); });
+        k_pst_trace<<<nq, 128, 0, st>>>(c.K, nb, G, Dq, s);
         check_launch("pst_gram", 3);
     }
 }
@@ -1002,9 +986,7 @@ void combine(Ctx& c, const double* cf, int q0, int nq, const std::vector<int>& o
     for (int q = 0; q < nq; ++q) o.p[q] = c.pst_slot[out[q]];
     const PstList T = v.babies();
     const dim3 grid(nb * (nb + 1) / 2, 64, (nq + 7) / 8);
-    pick(c.p.precision == DFT_PREC_BF16X3,
-         [&] { k_pst_combine<true><<<grid, 256, 0, st>>>(c.K, nb, v.p.s, T, o, q0, nq, cf, f32 ? 1 : 0); },
-         [&] { k_pst_combine<false><<<grid, 256, 0, st>>>(c.K, nb, v.p.s, T, o, q0, nq, cf, f32 ? 1 : 0); });
+    k_pst_combine<<<grid, 256, 0, st>>>(c.K, nb, v.p.s, T, o, q0, nq, cf, f32 ? 1 : 0);
     check_launch("pst_combine");
 }
 
@@ -1016,9 +998,7 @@ void finish(Ctx& c, const double* cf, const std::vector<int>& part, int b2, bool
     const PstList T = v.babies();
     const uint16_t* b = b2 >= 0 ? (const uint16_t*)c.pst_slot[b2] : nullptr;
     const int np = (int)part.size();
-    pick(c.p.precision == DFT_PREC_BF16X3,
-         [&] { k_pst_finish<true><<<nt * (nt + 1) / 2, 256, 0, st>>>(c.K, c.Kp / 256, v.p.s, T, cf, o, np, b, 1.0 / v.p.down, first, c.d_rho); },
-         [&] { k_pst_finish<false><<<nt * (nt + 1) / 2, 256, 0, st>>>(c.K, c.Kp / 256, v.p.s, T, cf, o, np, b, 1.0 / v.p.down, first, c.d_rho); });
+    k_pst_finish<<<nt * (nt + 1) / 2, 256, 0, st>>>(c.K, c.Kp / 256, v.p.s, T, cf, o, np, b, 1.0 / v.p.down, first, c.d_rho);
     check_launch("pst_finish");
 }
 
@@ -1059,8 +1039,7 @@ void pst_setup(Ctx& c, cudaStream_t st) {
     DFT_CUDA_CHECK(cudaMemcpyAsync(c.d_pst_maps, maps.data(), sizeof(CUtensorMap) * maps.size(), cudaMemcpyHostToDevice, st));
     DFT_CUDA_CHECK(cudaMemcpyAsync(c.d_pst_slots, c.pst_slot.data(), sizeof(void*) * n, cudaMemcpyHostToDevice, st));
     DFT_CUDA_CHECK(cudaStreamSynchronize(st));   // the host staging goes out of scope
-    DFT_CUDA_CHECK(cudaFuncSetAttribute(k_pst_prod<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-    DFT_CUDA_CHECK(cudaFuncSetAttribute(k_pst_prod<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
+    DFT_CUDA_CHECK(cudaFuncSetAttribute(k_pst_prod, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
 }
 
 // T_1 = H_N (from c.d_H, which is free afterwards)
@@ -1068,8 +1047,7 @@ void pst_split_h(Ctx& c, cudaStream_t st) {
     const int nb = c.Kp / 256;
     const dim3 grid(nb * (nb + 1) / 2, 16);
     uint16_t* t1 = (uint16_t*)c.pst_slot[0];
-    pick(c.p.precision == DFT_PREC_BF16X3, [&] { k_pst_split<true><<<grid, 256, 0, st>>>(c.K, nb, c.d_H, t1); },
-         [&] { k_pst_split<false><<<grid, 256, 0, st>>>(c.K, nb, c.d_H, t1); });
+    k_pst_split<<<grid, 256, 0, st>>>(c.K, nb, c.d_H, t1);
     check_launch("pst_split");
 }
 
@@ -1128,12 +1106,10 @@ void pst_pass1(Ctx* const* cs, int n, const int* moments, cudaStream_t st) {
         const PsPlan& p = c.ps;
         const View v(c);
         const int s = p.s, nb = c.Kp / 256;
-        const bool bf = c.p.precision == DFT_PREC_BF16X3;
         if (moments[k] && s > 1) {
             PstList L{};
             for (int r = 1; r < s; ++r) L.p[r - 1] = c.pst_slot[v.baby(r)];
-            pick(bf, [&] { k_pst_trace<true><<<s - 1, 128, 0, st>>>(c.K, nb, L, c.d_wk + 1, 1); },
-                 [&] { k_pst_trace<false><<<s - 1, 128, 0, st>>>(c.K, nb, L, c.d_wk + 1, 1); });
+            k_pst_trace<<<s - 1, 128, 0, st>>>(c.K, nb, L, c.d_wk + 1, 1);
             check_launch("pst_trace");
         }
         if (p.direct && moments[k] && p.Q > 0) {

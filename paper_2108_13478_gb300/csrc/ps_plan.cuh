@@ -43,7 +43,7 @@ inline double growth_limit(int l, int n_c) {
 // then gives T_{n_c - 1} itself (an outlier whose elements are a tenth of its
 // cosh is still below 1 at T_24 when it reaches 4 at T_39), more products an
 // order within 1 / b of it.  Each doubling multiplies rounding errors by up
-// to 4; one of 1e-5 (BF16 pairs) stays below the limit through 8 of them.
+// to 4; one of 1e-5 stays below the limit through 8 of them.
 struct PsCheck {
     int baby = 0, doublings = 0;   // 0: nothing beyond the last giant
     int odd = 0;                   // the single product is T_b T_{b+1}

@@ -238,3 +238,30 @@ def test_expired_waits_of_the_products_return_timeout_and_leave_the_context_usab
     ref = (LW * torch.from_numpy(dm.cheb_eval(x, coefficients(info.mu - info.mu_correction, beta, n_c))).cuda()) @ LW.T
     assert info.spectrum_ok == 1
     assert float((P - ref).abs().max() / ref.abs().max()) < 1e-4
+
+
+@pytest.mark.parametrize("prec", [FP16, dft.DFT_PREC_BF16X3])
+def test_grouped_expansion_is_no_further_off_than_the_recurrence(prec, monkeypatch):
+    """The distance of P from the FP64 context's (2-norm, six geometries, the
+    first Fock matrix of an SCF run), by the grouped expansion and by the
+    three-term recurrence."""
+    err = {"grouped": 0.0, "three-term": 0.0}
+    for seed in range(6):
+        s = w.config_system("tiny8", seed=seed)
+        ctx = dft.Context(s, model=dft.DFT_MODEL_NEUTRAL, cheb_tail_tol=1e-10)
+        _, T = ctx.overlap_kinetic()
+        F = (T + ctx.potential_matrix(ctx.hartree_xc(ctx.initial_density())[0])).contiguous()
+        ref, info = ctx.density_matrix(F)
+        ctx.close()
+        for form in err:
+            if form == "three-term":
+                monkeypatch.setenv("DFT_TC_SHAPE", "32,0,256")
+            else:
+                monkeypatch.delenv("DFT_TC_SHAPE", raising=False)
+            ctx = dft.Context(s, precision=prec, e_min=info.e_min, e_max=info.e_max, cheb_tail_tol=1e-6, skip_correction=1)
+            ctx.overlap_kinetic()
+            P, _ = ctx.density_matrix(F)
+            ctx.close()
+            err[form] += float(((P - ref) ** 2).sum() / (ref ** 2).sum()) / 6
+    print({k: f"{v ** 0.5:.2e}" for k, v in err.items()})
+    assert err["grouped"] <= err["three-term"]
