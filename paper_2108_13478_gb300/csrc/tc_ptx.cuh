@@ -196,11 +196,6 @@ struct H16<true> {
     static __device__ __forceinline__ float to_f(T x) { return __bfloat162float(x); }
     static __device__ __forceinline__ T from_f(float x) { return __float2bfloat16_rn(x); }
     static __device__ __forceinline__ T from_d(double x) { return __double2bfloat16(x); }
-    static __device__ __forceinline__ uint32_t from_f2(float a, float b) {
-        const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-        return *(const uint32_t*)&h;
-    }
-    static __device__ __forceinline__ float2 to_f2(uint32_t x) { return __bfloat1622float2(*(const __nv_bfloat162*)&x); }
 };
 
 // the 16 bits of a split part, and back
